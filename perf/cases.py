@@ -189,3 +189,49 @@ def tolerance(case):
     # The intermediate activations are rounded to bf16 and then ranked: a rounding that falls the other way moves single
     # indices across the threshold.  Taken in 64 bits up to that rounding, the block differs by 2.3e-2.
     return {"rel": 3e-2}
+
+
+def _kept(energy, rho):
+    """The ceil(rho K) indices of largest energy, equal energies to the lower index, ascending."""
+    k = rmm.rmm_keep_count(rho, energy.numel())
+    return torch.sort(energy, descending=True, stable=True).indices[:k].sort().values
+
+
+def _exact_attention(st):
+    Q, K, V, causal = st["Q"], st["K"], st["V"], st["causal"]
+    B, Hq, Lq, Dh = Q.shape
+    Hkv, Lk = K.shape[1], K.shape[2]
+    hidden = torch.ones(Lq, Lk, dtype=torch.bool, device=Q.device).triu(1 + Lk - Lq) if causal else None
+    O = torch.empty(B, Hq, Lq, Dh, dtype=torch.float64, device=Q.device)
+    for b in range(B):
+        for h in range(Hq):
+            q, k, v = Q[b, h].double(), K[b, h // (Hq // Hkv)].double(), V[b, h // (Hq // Hkv)].double()
+            idx = _kept(q.square().sum(0), st["rho_d"])
+            S = q[:, idx] @ k[:, idx].T / math.sqrt(Dh)
+            if st["mask"] is not None:
+                S += st["mask"][b, 0].double()
+            if causal:
+                S.masked_fill_(hidden, float("-inf"))
+            P = torch.softmax(S, -1)
+            if st["rho_t"] < 1.0:
+                # tokens are scored on the probabilities as they are stored
+                t = _kept(P.to(torch.bfloat16).double().square().sum(0), st["rho_t"])
+                P, v = P[:, t], v[t]
+            O[b, h] = P @ v
+    return O
+
+
+def exact(case, seed):
+    st, kind = prepare(case, seed), case["kind"]
+    if kind == "attention":
+        return _exact_attention(st)
+    if kind == "mlp_block":
+        # the intermediate activations are bf16 numbers: they are an output of the first call and an input of the next
+        H = (st["X"].double() @ st["up"].double()).to(torch.bfloat16).double()
+        idx = _kept(H.square().sum(0), st["rho"])
+        return H[:, idx] @ st["down"].double()[idx]
+    A = st["A"].double()
+    idx = _kept(A.square().sum(0), st["rho"])
+    if kind == "product_q8":
+        return A[:, idx] @ (st["Wq"].double()[:, idx] * st["step"]).T
+    return A[:, idx] @ st["B"][idx].double(), idx.to(torch.int32)
