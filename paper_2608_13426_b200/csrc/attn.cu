@@ -13,6 +13,7 @@
 //   rho_t = 1: one pass, O = softmax(S~ + mask) V;
 //   rho_t < 1: row normalisers (sweep 1), token scores of the bf16-rounded P (sweep 2), select T, pack K[T] and V[T],
 //              O = P[:, T] V[T, :] (sweep 3).
+// A few query rows per head (decode steps, rho_t = 1) read the caches in place instead: attn_decode.cu.
 #include <math.h>
 #include <stdlib.h>
 
@@ -83,18 +84,18 @@ __global__ void __launch_bounds__(kSoftmaxThreads) softmax_rows_kernel(const flo
 
 struct AttnPlan {
     int64_t kd, kt, ldd, ldt, ld_s, ld_p, hg, lse_ld;
-    bool fused;
+    bool fused, decode;
     size_t inner_bytes, off_idxf, off_idxt, off_qp, off_kp, off_s, off_p, off_pp, off_vp, off_lse, off_energy, off_kpt, total;
 };
 
-// up to 128 kept features of heads up to 256 wide run fused (RMM_ATTN_FUSED=0 keeps the composed form, for comparison).
-bool use_fused(const rmm_attn_desc_t *d, int64_t kd)
+// RMM_ATTN_FUSED=0 keeps the composed form, for comparison.
+bool fused_enabled()
 {
     static const bool enabled = [] {
         const char *e = getenv("RMM_ATTN_FUSED");
         return e == nullptr || e[0] != '0';
     }();
-    return enabled && fused_attn_eligible(d, kd);
+    return enabled;
 }
 
 // A batch of sequences whose (batch, head) pairs are evenly spaced in memory is one sequence with B * Hq heads on
@@ -138,6 +139,11 @@ int plan_attn(const rmm_attn_desc_t *d, AttnPlan *p)
     // V's (batch, head) pairs must form one batch axis of the tensor map used when V is read in place
     if (d->v_stride[2] < d->Dh || d->v_stride[0] != d->Hkv * d->v_stride[1])
         return fail(RMM_ERR_UNSUPPORTED, "reduced_attn: V needs batch stride = Hkv * head stride");
+    p->decode = fused_enabled() && decode_attn_eligible(d);
+    if (p->decode) {
+        p->total = RMM_WS_HEADER_BYTES + decode_attn_workspace_bytes(d);
+        return RMM_OK;
+    }
     p->ldd = (p->kd + 7) / 8 * 8;
     p->ldt = (p->kt + 7) / 8 * 8;
     p->ld_p = (d->Lk + 7) / 8 * 8;
@@ -151,7 +157,8 @@ int plan_attn(const rmm_attn_desc_t *d, AttnPlan *p)
     const bool mask_ok = d->mask == nullptr ||
                          (d->rho_t >= 1.0 && reinterpret_cast<uintptr_t>(d->mask) % 16 == 0 && d->mask_stride[0] % 4 == 0 &&
                           d->mask_stride[1] % 4 == 0 && d->mask_stride[2] % 4 == 0);
-    p->fused = mask_ok && use_fused(d, p->kd);
+    // up to 128 kept features of heads up to 256 wide run fused
+    p->fused = mask_ok && fused_enabled() && fused_attn_eligible(d, p->kd);
     if (hg > d->Hq || p->fused) hg = d->Hq;  // the fused form materialises neither S~ nor P: all heads at once
     p->hg = hg;
 
@@ -228,6 +235,7 @@ int rmm_reduced_attn(const rmm_attn_desc_t *desc, const void *Q, const void *K, 
 
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     char *w = static_cast<char *>(ws);
+    if (p.decode) return launch_decode_attn(d, p.kd, Q, K, V, O, idx_feat, w + RMM_WS_HEADER_BYTES, st);
     int *status = &reinterpret_cast<WsHeader *>(w)->status;
     const __nv_bfloat16 *q = static_cast<const __nv_bfloat16 *>(Q), *kk = static_cast<const __nv_bfloat16 *>(K),
                         *v = static_cast<const __nv_bfloat16 *>(V);

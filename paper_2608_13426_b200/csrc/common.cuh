@@ -225,6 +225,13 @@ int launch_softmax_rows(const float *S, int64_t ld_s, int64_t heads, int64_t Lq,
 // Kp [heads, Lk, ldd] (kd valid columns) and V [v_batches, Lk, Dh] (row pitch v_ld, batch pitch v_sb; head h uses
 // batch entry (h + v_off) / v_div).
 bool fused_attn_eligible(const rmm_attn_desc_t *d, int64_t kd);
+// Decode steps (attn_decode.cu): rho_t = 1, no additive mask, head_dim up to 256 and at most this many query rows; feature
+// selection included, K and V read in place, every layout that plan_attn accepts.  `scratch` holds partial sums.
+constexpr int64_t kDecodeMaxRows = 16;
+bool decode_attn_eligible(const rmm_attn_desc_t *d);
+size_t decode_attn_workspace_bytes(const rmm_attn_desc_t *d);
+int launch_decode_attn(const rmm_attn_desc_t *d, int64_t kd, const void *Q, const void *K, const void *V, void *O, int32_t *idx_feat,
+                       void *scratch, cudaStream_t stream);
 // lse == tok == NULL: O = softmax(Qp Kp^T / sqrt(Dh) + mask) V.  With lse [heads, lse_ld] and tok [heads, Lk] given,
 // Kp and V hold the kept keys only (Lk of them, at positions tok): O = P V with P = bf16(2^(x - lse)), not
 // renormalised.  diag = Lk - Lq of the unpacked problem (causal: query i sees key t iff t <= i + diag).

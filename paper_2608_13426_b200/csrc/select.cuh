@@ -88,7 +88,7 @@ __device__ __forceinline__ void find_bin(SelectSmem &sm, int nbins, unsigned rem
 // digit of up to 11 bits is histogrammed over all keys, the (few) keys that share the threshold's digit are copied
 // to a short list and finished there with 8-bit digits.  The kept indices are then emitted by warps that own
 // consecutive chunks of the index range, ranks coming from ballots.
-__device__ void block_select(const float *__restrict__ keys, int K, int k, int32_t *__restrict__ idx, float *retained,
+inline __device__ void block_select(const float *__restrict__ keys, int K, int k, int32_t *__restrict__ idx, float *retained,
                              SelectSmem &sm, unsigned *kcache)
 {
     const int tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31, warp = tid >> 5, nwarp = nthr >> 5;
