@@ -85,6 +85,8 @@ __global__ void __launch_bounds__(kSoftmaxThreads) softmax_rows_kernel(const flo
 struct AttnPlan {
     int64_t kd, kt, ldd, ldt, ld_s, ld_p, hg, lse_ld;
     bool fused, decode;
+    MaskView mask;  // fused: the additive mask of the first sequence's (or, folded, all sequences') heads
+    size_t off_kind;
     size_t inner_bytes, off_idxf, off_idxt, off_qp, off_kp, off_s, off_p, off_pp, off_vp, off_lse, off_energy, off_kpt, total;
 };
 
@@ -100,14 +102,18 @@ bool fused_enabled()
 
 // A batch of sequences whose (batch, head) pairs are evenly spaced in memory is one sequence with B * Hq heads on
 // B * Hkv kv heads (head h of sequence b reads kv head b * Hkv + h / group either way): one pass of launches
-// instead of B.
+// instead of B.  A mask whose planes are not spaced like that (one shared by the heads of a sequence) folds as well where
+// the fused kernel takes it, which keeps the sequences' own strides.
 rmm_attn_desc_t fold_batch(const rmm_attn_desc_t &d)
 {
     rmm_attn_desc_t f = d;
+    int64_t kd = 0;
+    const bool mask_kept = d.mask != nullptr && d.rho_t >= 1.0 && rmm_keep_count(d.rho_d, d.Dh, &kd) == RMM_OK && fused_enabled() &&
+                           fused_attn_eligible(&d, kd);
     const bool even = d.B > 1 && d.Hkv >= 1 && d.Hq % d.Hkv == 0 && d.B * d.Hq <= 65535 &&
                       d.q_stride[0] == d.Hq * d.q_stride[1] && d.k_stride[0] == d.Hkv * d.k_stride[1] &&
                       d.v_stride[0] == d.Hkv * d.v_stride[1] && d.o_stride[0] == d.Hq * d.o_stride[1] &&
-                      (d.mask == nullptr || d.mask_stride[0] == d.Hq * d.mask_stride[1]);
+                      (d.mask == nullptr || mask_kept || d.mask_stride[0] == d.Hq * d.mask_stride[1]);
     if (even) {
         f.B = 1;
         f.Hq = d.B * d.Hq;
@@ -121,7 +127,8 @@ rmm_attn_desc_t fold_batch(const rmm_attn_desc_t &d)
     return f;
 }
 
-int plan_attn(const rmm_attn_desc_t *d, AttnPlan *p)
+// `d` after fold_batch; `given` as the caller passed it
+int plan_attn(const rmm_attn_desc_t *d, const rmm_attn_desc_t *given, AttnPlan *p)
 {
     if (d == nullptr) return fail(RMM_ERR_INVALID_ARG, "reduced_attn: NULL description");
     if (d->B < 1 || d->Hq < 1 || d->Hkv < 1 || d->Lq < 1 || d->Lk < 1 || d->Dh < 1)
@@ -152,11 +159,9 @@ int plan_attn(const rmm_attn_desc_t *d, AttnPlan *p)
     const double per_head = (double)d->Lq * ((double)p->ld_s * 4 + (double)p->ld_p * 2 + (double)p->ldt * 2);
     int64_t hg = (int64_t)(6.0 * 1073741824.0 / per_head);
     if (hg < 1) hg = 1;
-    // the one-pass fused kernel also takes the caller's additive mask (rows 16-byte aligned); the three sweeps of the
-    // token reduction take the causal mask only (their second sweep walks the mask by columns)
-    const bool mask_ok = d->mask == nullptr ||
-                         (d->rho_t >= 1.0 && reinterpret_cast<uintptr_t>(d->mask) % 16 == 0 && d->mask_stride[0] % 4 == 0 &&
-                          d->mask_stride[1] % 4 == 0 && d->mask_stride[2] % 4 == 0);
+    // the one-pass fused kernel also takes the caller's additive mask; the three sweeps of the token reduction take the
+    // causal mask only (their second sweep walks the mask by columns)
+    const bool mask_ok = d->mask == nullptr || d->rho_t >= 1.0;
     // up to 128 kept features of heads up to 256 wide run fused
     p->fused = mask_ok && fused_enabled() && fused_attn_eligible(d, p->kd);
     if (hg > d->Hq || p->fused) hg = d->Hq;  // the fused form materialises neither S~ nor P: all heads at once
@@ -187,6 +192,18 @@ int plan_attn(const rmm_attn_desc_t *d, AttnPlan *p)
     p->off_lse = off; off += tokf * align_up((size_t)hg * p->lse_ld * 4, 256);
     p->off_energy = off; off += tokf * align_up((size_t)hg * d->Lk * 4, 256);
     p->off_kpt = off; off += tokf * align_up((size_t)hg * p->kt * p->ldd * 2, 256);
+    p->off_kind = off;
+    if (p->fused && d->mask != nullptr) {
+        const int64_t *ms = given->mask_stride;
+        MaskView &m = p->mask;
+        m.p = d->mask;
+        m.sb = ms[0]; m.sh = ms[1]; m.sr = ms[2];
+        m.seq_heads = given->Hq;
+        m.plane_heads = ms[1] == 0 ? 1 : given->Hq;
+        m.plane_step = ms[0] == 0 ? 0 : m.plane_heads;
+        m.vec = reinterpret_cast<uintptr_t>(d->mask) % 16 == 0 && ms[0] % 4 == 0 && ms[1] % 4 == 0 && ms[2] % 4 == 0;
+        off += align_up(mask_tiles_bytes(m, d->Hq / given->Hq, d->Lq, d->Lk), 256);
+    }
     p->total = off;
     return RMM_OK;
 }
@@ -214,7 +231,7 @@ size_t rmm_reduced_attn_workspace_bytes(const rmm_attn_desc_t *desc)
     AttnPlan p;
     if (desc == nullptr) return 0;
     const rmm_attn_desc_t folded = fold_batch(*desc);
-    if (plan_attn(&folded, &p) != RMM_OK) return 0;
+    if (plan_attn(&folded, desc, &p) != RMM_OK) return 0;
     return p.total;
 }
 
@@ -225,7 +242,7 @@ int rmm_reduced_attn(const rmm_attn_desc_t *desc, const void *Q, const void *K, 
     if (desc == nullptr) return fail(RMM_ERR_INVALID_ARG, "reduced_attn: NULL description");
     const rmm_attn_desc_t folded = fold_batch(*desc);
     const rmm_attn_desc_t *d = &folded;
-    int rc = plan_attn(d, &p);
+    int rc = plan_attn(d, desc, &p);
     if (rc != RMM_OK) return rc;
     if (Q == nullptr || K == nullptr || V == nullptr || O == nullptr) return fail(RMM_ERR_INVALID_ARG, "reduced_attn: NULL tensor");
     for (const void *ptr : {Q, K, V, (const void *)O})
@@ -272,11 +289,12 @@ int rmm_reduced_attn(const rmm_attn_desc_t *desc, const void *Q, const void *K, 
             if (p.fused) {
                 __nv_bfloat16 *og = o + b * d->o_stride[0] + h0 * d->o_stride[1];
                 if (!tok) {
+                    MaskView mask = p.mask;
+                    if (d->mask != nullptr) mask.p += b * d->mask_stride[0];
                     rc = launch_fused_attn(Qp, Kp, p.ldd, p.kd, v, d->v_stride[2], d->v_stride[1], d->B * d->Hkv, b * d->Hq + h0, group,
                                            og, d->o_stride[1], d->o_stride[2], hg, d->Lq, d->Lk, d->Dh, d->causal, d->Lk - d->Lq,
-                                           nullptr, 0, nullptr,
-                                           d->mask != nullptr ? d->mask + b * d->mask_stride[0] + h0 * d->mask_stride[1] : nullptr,
-                                           d->mask_stride[1], d->mask_stride[2], status, st);
+                                           nullptr, 0, nullptr, d->mask != nullptr ? &mask : nullptr,
+                                           reinterpret_cast<uint8_t *>(w + p.off_kind), status, st);
                     if (rc != RMM_OK) return rc;
                     continue;
                 }
@@ -294,7 +312,7 @@ int rmm_reduced_attn(const rmm_attn_desc_t *desc, const void *Q, const void *K, 
                 if ((rc = launch_pack(kv, 2, status, st)) != RMM_OK) return rc;
                 // sweep 3: O = P[:, T] V[T, :] against the full-row normalisers
                 rc = launch_fused_attn(Qp, KpT, p.ldd, p.kd, Vp, d->Dh, p.kt * d->Dh, hg, 0, 1, og, d->o_stride[1], d->o_stride[2], hg,
-                                       d->Lq, p.kt, d->Dh, d->causal, d->Lk - d->Lq, lse, p.lse_ld, It, nullptr, 0, 0, status, st);
+                                       d->Lq, p.kt, d->Dh, d->causal, d->Lk - d->Lq, lse, p.lse_ld, It, nullptr, nullptr, status, st);
                 if (rc != RMM_OK) return rc;
                 continue;
             }

@@ -80,13 +80,89 @@ struct FusedArgs {
     float *energy;               // ENERGY: [heads, Lr] squared token scores
     const int32_t *tok;          // GATHERED: [heads, Lc] kept key positions, ascending
     float scale_log2;            // (1 / sqrt(Dh)) * log2(e)
-    const float *mask;           // MASK: additive mask M of softmax(S~ + M), fp32, row (head, i) at mask + head m_sh + i m_sr
-    int64_t m_sh, m_sr;
+    MaskView mask;               // MASK: the caller's additive mask
+    const uint8_t *tile_kind;    // MASK: what the mask does to a 128 x 128 tile: [plane][row block][tile], see mask_tiles_kernel
+    int64_t kind_rb, kind_ld;    // row blocks per plane (even), bytes per row block (a multiple of 8)
     float mask_gain;             // sqrt(Dh): M is added to the unscaled S~ tile as M * sqrt(Dh)
     int *status;
     unsigned long long wait_ns;  // bound of every device-side wait
     int withhold;                // test switch: block 0 never requests its first key tile
 };
+
+// What the additive mask does to each tile of 128 queries x 128 keys, once per mask plane (the heads that share a plane
+// share the answer): hides it all (the tile is skipped like one beyond the causal diagonal), leaves it alone (the
+// ordinary softmax step), or has to be added.  Padding, causal, block and window masks are nearly all of the first
+// two kinds, and the additions were what bound the masked kernel: each thread reads its own row of the mask, 32 rows a
+// load.  2 sequences x 16 heads x 2048 x 128, padded: 2 x 244 us with every tile added, 80 us in one launch with this
+// pass (6 us) in front; a mask whose every value is added: 254 -> 224 us on 16 heads x 2048 (one launch for all sequences).
+// Bound by reading the mask once; a warp stops reading a tile once it knows that its values have to be added.
+// A value counts as hiding when mask x sqrt(Dh) is -inf in fp32, which is what the softmax step would make of it.
+enum { TILE_HIDDEN = 0, TILE_CLEAR = 1, TILE_ADD = 2 };
+constexpr int kMaskThreads = 128;
+
+struct MaskTileArgs {
+    MaskView mask;
+    int64_t Lq, Lk, diag;
+    int causal, vec;   // vec: rows are 16-byte aligned
+    float gain;
+    uint8_t *kind;
+    int64_t kind_rb, kind_ld;
+};
+
+__global__ void __launch_bounds__(kMaskThreads) mask_tiles_kernel(const MaskTileArgs a)
+{
+    __shared__ int s_some[kMaskThreads / 32], s_live[kMaskThreads / 32];
+    pdl_wait();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t t0 = (int64_t)blockIdx.x * FN, r0 = (int64_t)blockIdx.y * FM, plane = blockIdx.z;
+    const float *m = a.mask.p + (plane / a.mask.plane_heads) * a.mask.sb + (plane % a.mask.plane_heads) * a.mask.sh;
+    const int64_t rows = a.mask.sr == 0 ? 1 : min((int64_t)FM, a.Lq - r0);   // one row stands for all of them
+    const bool beyond = t0 >= a.Lk || r0 >= a.Lq || (a.causal && t0 > min(a.Lq, r0 + FM) - 1 + a.diag);
+    bool some = false, live = false;  // some value is not zero; some value does not hide
+    auto look = [&](float v) {
+        some |= !(v == 0.f);
+        live |= !(v * a.gain == -INFINITY);
+    };
+    for (int64_t rr = warp * 8; rr < rows && !beyond; rr += kMaskThreads / 32 * 8) {
+        float4 v[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {  // rows and columns past the end repeat the tile's first value
+            const float *row = m + (r0 + (rr + i < rows ? rr + i : 0)) * a.mask.sr + t0;
+            const int64_t c = t0 + lane * 4;
+            if (a.vec && c + 3 < a.Lk) {
+                v[i] = __ldg(reinterpret_cast<const float4 *>(row) + lane);
+            } else {
+                v[i].x = __ldg(row + (c < a.Lk ? lane * 4 : 0));
+                v[i].y = __ldg(row + (c + 1 < a.Lk ? lane * 4 + 1 : 0));
+                v[i].z = __ldg(row + (c + 2 < a.Lk ? lane * 4 + 2 : 0));
+                v[i].w = __ldg(row + (c + 3 < a.Lk ? lane * 4 + 3 : 0));
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            look(v[i].x);
+            look(v[i].y);
+            look(v[i].z);
+            look(v[i].w);
+        }
+        if (__any_sync(0xffffffffu, some) && __any_sync(0xffffffffu, live)) break;
+    }
+    some = __any_sync(0xffffffffu, some);
+    live = __any_sync(0xffffffffu, live);
+    if (lane == 0) {
+        s_some[warp] = some;
+        s_live[warp] = live;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int any_some = 0, any_live = 0;
+        for (int w = 0; w < kMaskThreads / 32; ++w) {
+            any_some |= s_some[w];
+            any_live |= s_live[w];
+        }
+        a.kind[(plane * a.kind_rb + blockIdx.y) * a.kind_ld + blockIdx.x] = !any_live ? TILE_HIDDEN : (any_some ? TILE_ADD : TILE_CLEAR);
+    }
+}
 
 template <int MODE, bool MASK>
 __global__ void __launch_bounds__(kFusedThreads, 1)
@@ -183,6 +259,28 @@ fused_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         else if (e1 <= b1) { *jb = b0; *je = e0; }
         else { *jb = min(b0, b1); *je = max(e0, e1); }
     };
+    // MASK: the next tile >= j, before je, that is not hidden from the rows of group g (both groups: g < 0), else je
+    auto kinds_of = [&](int64_t head, int64_t row) -> const uint8_t * {
+        const int64_t plane = (head / a.mask.seq_heads) * a.mask.plane_step + (head % a.mask.seq_heads) % a.mask.plane_heads;
+        return a.tile_kind + (plane * a.kind_rb + row / FM) * a.kind_ld;
+    };
+    auto next_tile = [&](int64_t head, int64_t r0, int g, int j, int je) -> int {
+        if constexpr (!MASK) return j;
+        const uint8_t *k0 = kinds_of(head, r0 + (g < 0 ? 0 : g) * FM);
+        while (j < je) {
+            unsigned long long u = __ldg(reinterpret_cast<const unsigned long long *>(k0 + (j & ~7)));
+            if (g < 0) {  // tiles past a group's causal range are hidden in its list
+                u |= __ldg(reinterpret_cast<const unsigned long long *>(k0 + a.kind_ld + (j & ~7)));
+            }
+            u >>= 8 * (j & 7);
+            if (u != 0) {
+                const int at = j + ((__ffsll((long long)u) - 1) >> 3);
+                return at < je ? at : je;
+            }
+            j = (j | 7) + 1;
+        }
+        return je;
+    };
     // The n-th item of this block: heaviest row blocks first (the last ones when causal; in ENERGY mode, where early
     // keys are seen by most queries, the first ones), and the direction alternates from round to round, so that the
     // block that drew the heaviest item of one round draws the lightest of the next.
@@ -218,6 +316,7 @@ fused_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             if (!item_of(n, &head, &r0)) continue;
             int jb, je;
             block_range(head, r0, &jb, &je);
+            jb = next_tile(head, r0, -1, jb, je);
             if (je <= jb) continue;
             const int vb = (int)((head + a.v_off) / a.v_div);
             if (!mbar_wait_sleepy(q_empty, (n_item & 1u) ^ 1u, abort_flag, a.status, a.wait_ns)) { ok = false; break; }
@@ -226,8 +325,9 @@ fused_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                 for (int c = 0; c < kq; ++c)
                     tma_load_3d(base + kOffQ + g * kQTile + c * kQChunk, &map_q, c * 64, (int)(r0 + g * FM), (int)head, q_full);
             ok = load_kv(&map_k, kq, (int64_t)jb * FN, (int)head);
-            for (int j = jb; j < je && ok; ++j) {
-                if (j + 1 < je) ok = load_kv(&map_k, kq, (int64_t)(j + 1) * FN, (int)head);
+            for (int j = jb, nj; j < je && ok; j = nj) {
+                nj = next_tile(head, r0, -1, j + 1, je);
+                if (nj < je) ok = load_kv(&map_k, kq, (int64_t)nj * FN, (int)head);
                 if constexpr (kHasV) {
                     if (ok) ok = load_kv(&map_v, nv, (int64_t)j * FN, vb);
                 }
@@ -252,12 +352,13 @@ fused_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         uint32_t ks = 0, kph = 0, n_item = 0, s_it = 0, p_it = 0, o_it = 0;
         bool ok = true;
         int gb = 0, ge = 0;  // this group's tile range in the current item
+        int gn = 0;          // MASK: the first tile from the current one on that this group needs
         ASTAMP_DECL(blockIdx.x == 0 && lane == 0 && g == 0);
         auto step_s = [&](int j) -> bool {  // S~ of tile j (if this group needs it); consumes one ring entry
             ASTAMP(7);
             if (!mbar_wait(kv_full(ks), kph, abort_flag, a.status, a.wait_ns)) return false;
             ASTAMP(0);
-            if (j >= gb && j < ge) {
+            if (MASK ? j == gn && gn < ge : (j >= gb && j < ge)) {
                 // S~ is single-buffered: the softmax warps release it as soon as they hold the tile in registers
                 if (!mbar_wait(s_empty(g, 0), (s_it & 1u) ^ 1u, abort_flag, a.status, a.wait_ns)) return false;
                 ASTAMP(1);
@@ -284,18 +385,24 @@ fused_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             if (!item_of(n, &head, &r0)) continue;
             int jb, je;
             block_range(head, r0, &jb, &je);
+            jb = next_tile(head, r0, -1, jb, je);
             if (je <= jb) continue;
             tile_range(head, r0 + g * FM, &gb, &ge);
+            gn = gb = next_tile(head, r0, g, gb, ge);
             if (!mbar_wait(q_full, n_item & 1u, abort_flag, a.status, a.wait_ns)) { ok = false; break; }
             ok = step_s(jb);
-            for (int j = jb; j < je && ok; ++j) {
-                if (j + 1 < je) ok = step_s(j + 1);                        // S~ of the next tile runs ahead of this P V
+            for (int j = jb, nj; j < je && ok; j = nj) {
+                nj = next_tile(head, r0, -1, j + 1, je);
+                const bool use = MASK ? j == gn && gn < ge : (j >= gb && j < ge);  // this group needs the tile
+                if (MASK && use) gn = next_tile(head, r0, g, j + 1, ge);
+                const bool last_use = MASK ? gn >= ge : j == ge - 1;
+                if (nj < je) ok = step_s(nj);                              // S~ of the next tile runs ahead of this P V
                 if (!ok) break;
                 if constexpr (kHasV) {
                     ASTAMP(7);
                     if (!mbar_wait(kv_full(ks), kph, abort_flag, a.status, a.wait_ns)) { ok = false; break; }
                     ASTAMP(3);
-                    if (j >= gb && j < ge) {
+                    if (use) {
                         if (j == gb && !mbar_wait(o_empty(g), (o_it & 1u) ^ 1u, abort_flag, a.status, a.wait_ns)) { ok = false; break; }
                         ASTAMP(4);
                         if (!mbar_wait(p_full(g), p_it & 1u, abort_flag, a.status, a.wait_ns)) { ok = false; break; }
@@ -308,10 +415,10 @@ fused_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                                 umma_bf16_lohi<1>(t_o, p_lo + (st >> 2) * (kPChunk >> 4) + (st & 3) * 2, p_hi, vl + st * (2048 >> 4), v_hi, idesc_o,
                                                   (j != gb || st != 0) ? 1u : 0u);
                             umma_commit<1>(p_empty(g));   // "P V of this tile is complete": P may be rewritten, O may be rescaled
-                            if (j == ge - 1) umma_commit<1>(o_full(g));
+                            if (last_use) umma_commit<1>(o_full(g));
                         }
                         ++p_it;
-                        if (j == ge - 1) ++o_it;
+                        if (last_use) ++o_it;
                     }
                     if (elect_one()) umma_commit<1>(kv_empty(ks));
                     __syncwarp();
@@ -344,6 +451,7 @@ fused_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             if (r0 >= a.Lr) continue;                  // this group has no rows in the last block
             int jb, je;
             tile_range(head, r0, &jb, &je);
+            jb = next_tile(head, r0, 0, jb, je);
             const int64_t i = r0 + r;                  // this thread's row
             __nv_bfloat16 *orow = a.O + head * a.o_sh + i * a.o_sr;
             if (je <= jb) {  // nothing visible for any row of this group
@@ -370,6 +478,7 @@ fused_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
 
             // 64 logits of the current tile (columns c_off .. c_off + 63) into registers; hidden columns become -inf on
             // boundary tiles (the diagonal and the ragged end)
+            [[maybe_unused]] bool add_mask = false;  // MASK: the mask has to be added to the current tile
             auto load_chunk = [&](int j, int c_off, uint32_t (&v0)[32], uint32_t (&v1)[32]) {
                 tmem_ld32_issue(t_s + c_off, v0);
                 tmem_ld32_issue(t_s + c_off + 32, v1);
@@ -388,18 +497,18 @@ fused_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                 if constexpr (MASK) {
                     // the caller's additive mask for this row's 64 columns (-inf hides a key); rows past the end and
                     // columns past the last key read nothing
-                    if (i < a.Lr) {
-                        const float *mrow = a.mask + head * a.m_sh + i * a.m_sr + c0;
+                    if (add_mask && i < a.Lr) {
+                        const float *mrow = a.mask.p + (head / a.mask.seq_heads) * a.mask.sb + (head % a.mask.seq_heads) * a.mask.sh + i * a.mask.sr + c0;
                         const float gain = a.mask_gain;
                         auto add4 = [&](uint32_t (&v)[32], int e, int col) {
                             float4 m4;
-                            if (c0 + col + 3 < a.Lc) {
+                            if (a.mask.vec && c0 + col + 3 < a.Lc) {
                                 m4 = __ldg(reinterpret_cast<const float4 *>(mrow + col));
                             } else {
                                 m4.x = c0 + col < a.Lc ? __ldg(mrow + col) : 0.f;
                                 m4.y = c0 + col + 1 < a.Lc ? __ldg(mrow + col + 1) : 0.f;
                                 m4.z = c0 + col + 2 < a.Lc ? __ldg(mrow + col + 2) : 0.f;
-                                m4.w = 0.f;
+                                m4.w = c0 + col + 3 < a.Lc ? __ldg(mrow + col + 3) : 0.f;
                             }
                             v[e] = __float_as_uint(fmaf(m4.x, gain, __uint_as_float(v[e])));
                             v[e + 1] = __float_as_uint(fmaf(m4.y, gain, __uint_as_float(v[e + 1])));
@@ -473,7 +582,8 @@ fused_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                 return alpha;
             };
 
-            for (int j = jb; j < je; ++j, ++s_it) {
+            for (int j = jb; j < je; j = next_tile(head, r0, 0, j + 1, je), ++s_it) {
+                if constexpr (MASK) add_mask = __ldg(kinds_of(head, r0) + j) == TILE_ADD;
                 if constexpr (MODE == MODE_ENERGY) {
                     // the 128 normalisers of the next tile (512 bytes, the same for every thread) are pulled into L1
                     // one step ahead; the first tile's are fetched cold
@@ -681,19 +791,34 @@ bool fused_attn_eligible(const rmm_attn_desc_t *d, int64_t kd)
     return d->Dh % 8 == 0 && d->Dh <= 256 && kd <= 128 && d->Lq <= INT32_MAX && d->Lk <= INT32_MAX;
 }
 
+size_t mask_tiles_bytes(const MaskView &m, int64_t seqs, int64_t Lq, int64_t Lk)
+{
+    const int64_t planes = (m.plane_step > 0 ? seqs : 1) * m.plane_heads;
+    return (size_t)planes * (2 * ceil_div(Lq, kGroups * FM)) * (ceil_div(Lk, FN * 8) * 8);
+}
+
 // FULL (lse NULL, tok NULL): O = softmax(Qp Kp^T / sqrt(Dh) + mask) V; `mask` (or NULL) is the caller's additive fp32 mask on
-// top of the causal one, row (head, i) at mask + head m_sh + i m_sr (16-byte aligned rows).
+// top of the causal one, and tile_kind room for mask_tiles_bytes().
 // GATHERED (lse and tok given): Kp and V hold the kept keys only (Lk = their count, tok their positions); O = P V with
 // P = bf16(2^(x - lse)), no renormalisation.  `diag` = Lk - Lq of the unpacked problem.
 // Qp [heads, Lq, ldd], Kp [heads, Lk, ldd] packed; V [v_batches, Lk, Dh] with row pitch v_ld and batch pitch v_sb.
 int launch_fused_attn(const __nv_bfloat16 *Qp, const __nv_bfloat16 *Kp, int64_t ldd, int64_t kd, const __nv_bfloat16 *V,
                       int64_t v_ld, int64_t v_sb, int64_t v_batches, int64_t v_off, int64_t v_div, __nv_bfloat16 *O,
                       int64_t o_sh, int64_t o_sr, int64_t heads, int64_t Lq, int64_t Lk, int64_t Dh, int causal, int64_t diag,
-                      const float *lse, int64_t lse_ld, const int32_t *tok, const float *mask, int64_t m_sh, int64_t m_sr,
+                      const float *lse, int64_t lse_ld, const int32_t *tok, const MaskView *mask, uint8_t *tile_kind,
                       int *status, cudaStream_t stream)
 {
     CUtensorMap mq, mk, mv;
     int rc;
+    const int64_t kind_rb = 2 * ceil_div(Lq, kGroups * FM), kind_ld = ceil_div(Lk, FN * 8) * 8;
+    if (mask != nullptr) {
+        const int64_t planes = (mask->plane_step > 0 ? heads / mask->seq_heads : 1) * mask->plane_heads;
+        if (kind_rb > 65535 || planes > 65535) return fail(RMM_ERR_UNSUPPORTED, "fused_attn: mask too large");
+        MaskTileArgs t = {*mask, Lq, Lk, diag, causal, mask->vec, (float)sqrt((double)Dh), tile_kind, kind_rb, kind_ld};
+        prof_begin("mask_tiles_kernel", stream);
+        launch_kernel(mask_tiles_kernel, dim3((unsigned)kind_ld, (unsigned)kind_rb, (unsigned)planes), dim3(kMaskThreads), 0, stream, 1, t);
+        if ((rc = check_launch("mask_tiles_kernel", stream)) != RMM_OK) return rc;
+    }
     if ((rc = packed_map(&mq, Qp, kd, Lq, heads, ldd, FM)) != RMM_OK) return rc;
     if ((rc = packed_map(&mk, Kp, kd, Lk, heads, ldd, FN)) != RMM_OK) return rc;
     // The O accumulators of a block hold 128 columns per query group: a wider head (up to 256 columns) is produced in
@@ -719,7 +844,7 @@ int launch_fused_attn(const __nv_bfloat16 *Qp, const __nv_bfloat16 *Kp, int64_t 
         if (tok != nullptr) {
             rc = launch_mode<MODE_GATHERED>(mq, mk, mv, a, "fused_attn_gathered_kernel", stream);
         } else if (mask != nullptr) {
-            a.mask = mask; a.m_sh = m_sh; a.m_sr = m_sr;
+            a.mask = *mask; a.tile_kind = tile_kind; a.kind_rb = kind_rb; a.kind_ld = kind_ld;
             a.mask_gain = (float)sqrt((double)Dh);
             rc = launch_mode<MODE_FULL, true>(mq, mk, mv, a, "fused_attn_masked_kernel", stream);
         } else {

@@ -221,6 +221,15 @@ int launch_gather_q8(bool quantise, const void *src, int64_t rows, int64_t s_row
 // (row (h, i) at mask + h m_sh + i m_sr, fp32); writes bf16 P [heads, Lq, ld_p] (columns Lk .. ld_p zeroed).
 int launch_softmax_rows(const float *S, int64_t ld_s, int64_t heads, int64_t Lq, int64_t Lk, int causal, const float *mask,
                         int64_t m_sh, int64_t m_sr, __nv_bfloat16 *P, int64_t ld_p, cudaStream_t stream);
+// The caller's additive fp32 mask as a launch sees it: row (head h, i) at p + (h / seq_heads) sb + (h % seq_heads) sh + i sr.
+// Heads and sequences that share a plane are described by plane_heads (distinct planes per sequence) and plane_step
+// (planes from one sequence to the next, 0: all sequences share).
+struct MaskView {
+    const float *p;
+    int64_t sb, sh, sr, seq_heads, plane_heads, plane_step;
+    int vec;  // every row starts on a 16-byte boundary
+};
+size_t mask_tiles_bytes(const MaskView &m, int64_t seqs, int64_t Lq, int64_t Lk);
 // Fused forms (S~ and P stay on the SM; head_dim and kept features up to 128) on packed Qp [heads, Lq, ldd],
 // Kp [heads, Lk, ldd] (kd valid columns) and V [v_batches, Lk, Dh] (row pitch v_ld, batch pitch v_sb; head h uses
 // batch entry (h + v_off) / v_div).
@@ -238,7 +247,7 @@ int launch_decode_attn(const rmm_attn_desc_t *d, int64_t kd, const void *Q, cons
 int launch_fused_attn(const __nv_bfloat16 *Qp, const __nv_bfloat16 *Kp, int64_t ldd, int64_t kd, const __nv_bfloat16 *V,
                       int64_t v_ld, int64_t v_sb, int64_t v_batches, int64_t v_off, int64_t v_div, __nv_bfloat16 *O,
                       int64_t o_sh, int64_t o_sr, int64_t heads, int64_t Lq, int64_t Lk, int64_t Dh, int causal, int64_t diag,
-                      const float *lse, int64_t lse_ld, const int32_t *tok, const float *mask, int64_t m_sh, int64_t m_sr, int *status, cudaStream_t stream);
+                      const float *lse, int64_t lse_ld, const int32_t *tok, const MaskView *mask, uint8_t *tile_kind, int *status, cudaStream_t stream);
 // Two sweeps: lse [heads, lse_ld] (lse_ld a multiple of 64, >= Lq) = log2-domain row normalisers of softmax(S~ + mask);
 // energy [heads, Lk] = squared token scores sum_i bf16(P_it)^2.
 int launch_fused_attn_scores(const __nv_bfloat16 *Qp, const __nv_bfloat16 *Kp, int64_t ldd, int64_t kd, int64_t heads,

@@ -1,0 +1,84 @@
+"""Additive masks whose 128 x 128 tiles are skipped, left alone or added (attn_fused.cu)."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2608_13426_b200 as rmm
+from paper_2608_13426_b200 import synth
+from test_gpu_parity import check_attention, dev
+
+pytestmark = pytest.mark.gpu
+HIDE = -float("inf")
+
+
+def padded(B, Lq, Lk, lengths, value=HIDE):
+    M = torch.zeros(B, 1, Lq, Lk)
+    for b, n in enumerate(lengths):
+        M[b, :, :, n:] = value
+    return M
+
+
+def blocks(L, size):
+    """Block-diagonal: whole tiles hidden between visible ones, left and right of the diagonal."""
+    i = torch.arange(L) // size
+    return torch.where(i[:, None] == i[None, :], 0.0, HIDE)
+
+
+def sliding(L, width):
+    i = torch.arange(L)
+    return torch.where((i[:, None] - i[None, :]).abs() <= width, 0.0, HIDE)
+
+
+CASES = {
+    # B, Hq, Hkv, Lq, Lk, Dh, causal, mask
+    "padding per sequence, shared by heads": (2, 4, 2, 300, 300, 128, True, padded(2, 300, 300, [300, 129])),
+    "rows of odd length": (2, 4, 2, 261, 261, 64, True, padded(2, 261, 261, [131, 256])),
+    "no value is zero or hides": (1, 2, 2, 257, 263, 64, False, torch.randn(1, 1, 257, 263, generator=torch.Generator().manual_seed(1))),
+    "an odd pitch per head": (2, 2, 1, 140, 275, 128, False, torch.randn(2, 2, 140, 275, generator=torch.Generator().manual_seed(2)).round()),
+    "one row for all queries": (2, 4, 4, 400, 385, 128, False, padded(2, 1, 385, [128, 300])),
+    "the lowest finite value": (2, 4, 2, 300, 300, 128, True, padded(2, 300, 300, [140, 256], torch.finfo(torch.float32).min)),
+    "first sequence sees nothing": (2, 4, 2, 300, 300, 128, False, padded(2, 300, 300, [0, 200])),
+    "blocks": (1, 4, 2, 1280, 1280, 128, False, blocks(1280, 320)),
+    "window": (1, 2, 1, 1500, 1500, 64, True, sliding(1500, 150)),
+    "wide heads": (1, 2, 1, 700, 700, 256, True, sliding(700, 200)),
+    "all zero": (1, 2, 1, 513, 513, 128, False, torch.zeros(513, 513)),
+    "every second key block, over more than eight tiles": (1, 2, 2, 256, 2300, 64, False,
+                                                             torch.where((torch.arange(2300) // 128) % 2 == 1, 0.0, HIDE).expand(256, 2300)),
+}
+
+
+@pytest.mark.parametrize("name", sorted(CASES))
+def test_masked_attention_by_tiles(oracle, name):
+    B, Hq, Hkv, Lq, Lk, Dh, causal, M = CASES[name]
+    M = M.contiguous()
+    mask = M if M.dim() == 4 else M[None, None]
+    assert check_attention_or_zero(oracle, B, Hq, Hkv, Lq, Lk, Dh, causal, mask)
+    assert rmm.rmm_status_read() == 0
+
+
+def check_attention_or_zero(oracle, B, Hq, Hkv, Lq, Lk, Dh, causal, mask):
+    if not (mask[0] < -1e30).all():
+        low = mask.clone()
+        low[low < -1e30] = HIDE          # the lowest finite value hides a key as -inf does
+        Q, K, V = synth.attention_qkv(B, Hq, Hkv, Lq, Lk, Dh, seed=171)
+        O, feat, _ = rmm.rmm_reduced_attn(dev(Q), dev(K), dev(V), causal, 0.5, 1.0, want_idx=True, mask=dev(mask))
+        want = oracle.attn(Q, K, V, causal, 0.5, 1.0, idx_feat=feat.cpu().numpy(), mask=low.numpy().astype(np.float64))[0]
+        got = O.float().cpu().numpy()
+        assert np.isfinite(got).all()
+        return bool((np.linalg.norm(got - want, axis=(2, 3)) <= 1e-2 * np.linalg.norm(want, axis=(2, 3))).all())
+    Q, K, V = synth.attention_qkv(B, Hq, Hkv, Lq, Lk, Dh, seed=171)
+    O = rmm.rmm_reduced_attn(dev(Q), dev(K), dev(V), causal, 0.5, 1.0, mask=dev(mask))
+    alone = rmm.rmm_reduced_attn(dev(Q[1:]), dev(K[1:]), dev(V[1:]), causal, 0.5, 1.0, mask=dev(mask[1:]))
+    return torch.count_nonzero(O[0]) == 0 and torch.equal(O[1:], alone)
+
+
+def test_masked_attention_folds_only_even_sequences(oracle):
+    """Sequences that are not evenly spaced in memory run one by one against their own planes of the mask."""
+    M = padded(3, 200, 200, [200, 90, 140])
+    Q, K, V = synth.attention_qkv(3, 4, 2, 200, 200, 64, seed=172)
+    wide = torch.zeros(3, 5, 200, 64, dtype=torch.bfloat16)
+    wide[:, :4] = Q
+    a = rmm.rmm_reduced_attn(dev(wide)[:, :4], dev(K), dev(V), True, 0.5, 1.0, mask=dev(M))
+    b = rmm.rmm_reduced_attn(dev(Q), dev(K), dev(V), True, 0.5, 1.0, mask=dev(M))
+    assert torch.equal(a, b)
+    assert check_attention(oracle, 3, 4, 2, 200, 200, 64, True, 0.5, 1.0, seed=172, mask=M)
