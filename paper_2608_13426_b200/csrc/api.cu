@@ -240,7 +240,7 @@ size_t rmm_reduced_gemm_workspace_bytes(const rmm_mat_t *A, const rmm_mat_t *B, 
     if (gemv_eligible(A, &b, k, Y, &gplan)) return gplan.total_bytes;
     TcPlan plan;
     if (tc_eligible(A, &b, k, Y, &plan)) return plan.total_bytes;
-    return RMM_WS_HEADER_BYTES;
+    return gemm_simt_workspace_bytes(A, &b, k);
 }
 
 int rmm_reduced_gemm(const rmm_mat_t *A, const rmm_mat_t *B, const int32_t *idx, int64_t k, float scale,
@@ -261,7 +261,7 @@ int rmm_reduced_gemm(const rmm_mat_t *A, const rmm_mat_t *B, const int32_t *idx,
         if (rc != RMM_OK) return rc;
         return launch_gemm_tc(A, &b, idx, k, scale, Y, plan, ws, static_cast<cudaStream_t>(stream));
     }
-    rc = check_ws(ws, ws_bytes, RMM_WS_HEADER_BYTES, "reduced_gemm");
+    rc = check_ws(ws, ws_bytes, gemm_simt_workspace_bytes(A, &b, k), "reduced_gemm");
     if (rc != RMM_OK) return rc;
     return launch_gemm_simt(A, &b, idx, k, scale, Y, ws, static_cast<cudaStream_t>(stream));
 }

@@ -126,6 +126,7 @@ int launch_front(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k, int32_t *idx
 // Plain FMA kernel: any strides, bf16 or fp32 operands, fp32 accumulation, bf16 or fp32 output.
 int launch_gemm_simt(const rmm_mat_t *A, const rmm_mat_t *B, const int32_t *idx, int64_t k, float scale,
                      const rmm_mat_t *Y, void *ws, cudaStream_t stream);
+size_t gemm_simt_workspace_bytes(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k);
 
 // Decode-step path (M <= 4 rows of bf16 activations, B rows contiguous): HBM-bound gathered GEMV, no packing.
 struct GemvPlan {
