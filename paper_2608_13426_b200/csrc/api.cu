@@ -342,7 +342,7 @@ size_t rmm_reduced_gemm_scored_workspace_bytes(const rmm_mat_t *A, const rmm_mat
     TcPlan plan;
     size_t need;
     if (!gemv_eligible(A, &b, k, Y, &gplan) && tc_eligible(A, &b, k, Y, &plan, true)) {
-        if (plan.epilogue_energy) return plan.total_bytes;
+        if (plan.epilogue_energy && !plan.gathers) return plan.total_bytes;
         need = plan.total_bytes;
     } else {
         need = rmm_reduced_gemm_workspace_bytes(A, B, k, Y);
@@ -361,7 +361,7 @@ int rmm_reduced_gemm_scored(const rmm_mat_t *A, const rmm_mat_t *B, const int32_
     rmm_mat_t b = shared_b(A, B);
     GemvPlan gplan;
     TcPlan plan;
-    if (!gemv_eligible(A, &b, k, Y, &gplan) && tc_eligible(A, &b, k, Y, &plan, true) && plan.epilogue_energy) {
+    if (!gemv_eligible(A, &b, k, Y, &gplan) && tc_eligible(A, &b, k, Y, &plan, true) && plan.epilogue_energy && !(plan.gathers && idx != nullptr)) {
         rc = check_ws(ws, ws_bytes, plan.total_bytes, "reduced_gemm_scored");
         if (rc != RMM_OK) return rc;
         return launch_gemm_tc(A, &b, idx, k, scale, Y, plan, ws, static_cast<cudaStream_t>(stream), energy_out);

@@ -38,34 +38,6 @@ struct DecodeArgs {
     float *part_o, *part_ml;     // pieces > 1: [blocks][row tile][Dh padded], [blocks][row tile][2]
 };
 
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, bool live)
-{
-    const int n = live ? 16 : 0;  // 0: the 16 bytes are zero-filled and src is not read
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(n) : "memory");
-}
-__device__ __forceinline__ void ldm4(uint32_t (&r)[4], uint32_t addr)
-{
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
-}
-__device__ __forceinline__ void ldm4_trans(uint32_t (&r)[4], uint32_t addr)
-{
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
-}
-__device__ __forceinline__ uint32_t transpose8x8(uint32_t x)
-{
-    uint32_t y;
-    asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(y) : "r"(x));
-    return y;
-}
-__device__ __forceinline__ void mma16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
-{
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-
 constexpr int kDecodeWarps = 4, kDecodeBlocks = 2;  // warps per block, blocks per SM
 
 template <int DH, int NT>
@@ -112,7 +84,7 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, kDecodeBlocks) attn_decode_
             for (int i = 0; i < 16 * CPR / 32; ++i) {
                 const int r = lane / CPR + i * (32 / CPR);
                 const bool live = key0 + r < a.Lk && c * 8 < a.Dh;
-                cp_async16(dst + r * (DH * 2) + ((c ^ (r & 7)) << 4), live ? src + (int64_t)(key0 + r) * pitch + c * 8 : a.k, live);
+                ptx::cp_async_16(dst + r * (DH * 2) + ((c ^ (r & 7)) << 4), live ? src + (int64_t)(key0 + r) * pitch + c * 8 : a.k, live ? 16u : 0u);
             }
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
@@ -221,9 +193,9 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, kDecodeBlocks) attn_decode_
 #pragma unroll
         for (int ks = 0; ks < DH / 16; ++ks) {
             uint32_t ka[4];
-            ldm4(ka, kst + k_lane + (((2 * ks + (lane >> 4)) ^ k_x) << 4));
+            ptx::ldmatrix_x4(ka, kst + k_lane + (((2 * ks + (lane >> 4)) ^ k_x) << 4));
 #pragma unroll
-            for (int nt = 0; nt < NT; ++nt) mma16816(ks & 1 ? s2[nt] : s[nt], ka, qf[nt][ks][0], qf[nt][ks][1]);
+            for (int nt = 0; nt < NT; ++nt) ptx::mma_bf16_16816(ks & 1 ? s2[nt] : s[nt], ka, qf[nt][ks][0], qf[nt][ks][1]);
         }
 #pragma unroll
         for (int nt = 0; nt < NT; ++nt)
@@ -285,8 +257,8 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, kDecodeBlocks) attn_decode_
             l[nt][0] += p0 + p2;
             l[nt][1] += p1 + p3;
             __nv_bfloat162 x = __floats2bfloat162_rn(p0, p1), y = __floats2bfloat162_rn(p2, p3);
-            pb[nt][0] = transpose8x8(*reinterpret_cast<uint32_t *>(&x));  // (key g, rows 2t) -> (row g, keys 2t)
-            pb[nt][1] = transpose8x8(*reinterpret_cast<uint32_t *>(&y));
+            pb[nt][0] = ptx::transpose8x8(*reinterpret_cast<uint32_t *>(&x));  // (key g, rows 2t) -> (row g, keys 2t)
+            pb[nt][1] = ptx::transpose8x8(*reinterpret_cast<uint32_t *>(&y));
         }
         landed();
         load(2 * n + U);
@@ -294,9 +266,9 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, kDecodeBlocks) attn_decode_
 #pragma unroll
         for (int mt = 0; mt < DH / 16; ++mt) {
             uint32_t va[4];
-            ldm4_trans(va, vst + v_row * (DH * 2) + (((2 * mt + ((lane >> 3) & 1)) ^ (v_row & 7)) << 4));
+            ptx::ldmatrix_x4_trans(va, vst + v_row * (DH * 2) + (((2 * mt + ((lane >> 3) & 1)) ^ (v_row & 7)) << 4));
 #pragma unroll
-            for (int nt = 0; nt < NT; ++nt) mma16816(o[nt][mt], va, pb[nt][0], pb[nt][1]);
+            for (int nt = 0; nt < NT; ++nt) ptx::mma_bf16_16816(o[nt][mt], va, pb[nt][0], pb[nt][1]);
         }
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");

@@ -141,6 +141,7 @@ int launch_gemv(const rmm_mat_t *A, const rmm_mat_t *B, const int32_t *idx, int6
 struct TcPlan {
     int b_kmajor;       // 0: B rows (contraction slices) contiguous, kept rows copied; 1: B is K-contiguous, packed like A
     int64_t ldp;        // leading dimension of the packed operands (multiple of 8)
+    bool gathers;       // with an index list the kernel fetches the kept rows of B itself (no column energies in that form)
     size_t off_ap, off_bp, off_colen, total_bytes;
     bool epilogue_energy;  // the plan reserves the per-group column energies of Y and the epilogue fills them
 };
@@ -162,6 +163,7 @@ struct TcProblem {
     // kept rows b_idx[i * b_idx_stride + 0 .. k-1] itself (no packed copy of B; outputs of up to 128 rows)
     const int32_t *b_idx;
     int64_t b_idx_stride, b_rows;
+    float *partials;         // with b_idx: [2 x SMs][min(M, 128)][256] fp32 for the tiles whose contraction is cut
     void *y;
     int y_bf16;
     int64_t y_sb, y_sr;
@@ -176,6 +178,10 @@ struct TcProblem {
     float *col_energy;
 };
 int launch_gemm_tc_problem(const TcProblem &p, cudaStream_t stream);
+// The same for at most kSkinnyRows rows with b_idx set (gemm_skinny.cu).
+constexpr int64_t kSkinnyRows = 32;
+size_t gemm_skinny_partial_bytes(int64_t batch, int64_t M, int64_t N, int64_t k);
+int launch_gemm_skinny(const TcProblem &p, cudaStream_t stream);
 // energy[b, c] = sum over the 32-row groups of col_energy (fp64, in group order), rounded to fp32
 int launch_energy_combine(const float *col_energy, int64_t batch, int64_t groups, int64_t N, float *energy, cudaStream_t stream);
 

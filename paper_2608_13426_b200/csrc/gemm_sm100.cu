@@ -9,10 +9,11 @@
 //             K-contiguous (K^T in attention) it is packed like A and loaded as K-major tiles.  (Fetching the
 //             kept rows inside the producer with TMA gather4 was measured first: at 512 bytes per instruction
 //             the copy engine sustained about one instruction per 70 clocks, 2.5x slower than this form.)
-//             Outputs of up to 256 rows (small decode batches) skip the packed copy of B: eight gather warps fetch
+//             Outputs of 33 to 256 rows (fewer: gemm_skinny.cu) skip the packed copy of B: eight gather warps fetch
 //             the kept rows straight from B with 16-byte cp.async into the same swizzled layout (one row of the tile
 //             = one 512-byte warp request).  There every tile of B is used once, the product is bound by reading the
-//             kept rows from HBM, and the copy would triple that traffic.  (For taller outputs the same gather was
+//             kept rows from HBM, and the copy would triple that traffic; where whole tiles leave SMs idle the
+//             contraction is cut into equal shares (launch_gemm_tc_problem).  (For taller outputs the same gather was
 //             measured at 1480 clocks per k-block against 590 for TMA tiles of the packed copy: the load/store path
 //             does not sustain the L2-to-SM rate that re-used tiles need.)
 //   MMA       one elected thread issues tcgen05.mma (bf16 x bf16 -> fp32, M=128, N=BN, K=16 per instruction);
@@ -71,6 +72,8 @@ struct TcArgs {
     const __nv_bfloat16 *b_src;
     const int32_t *b_idx;
     int64_t b_ld, b_sb, b_idx_stride, b_rows;
+    int64_t seg_kb;              // k-blocks per block: the k-blocks of all tiles form one axis that is cut into equal shares
+    float *partials;             // [2 x blocks][min(M, 128)][256] unscaled sums of the tiles that were cut
 };
 
 // BN = tile columns (MMA N, accumulator columns); CTAS = CTAs per tile.  With CTAS == 2 a pair of CTAs on one TPC
@@ -130,11 +133,29 @@ reduced_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) { GSTAMP_MIN(0); }
     const int64_t num_tiles = a.batch * a.tiles_m * a.tiles_n;  // tiles of (128 * CTAS) x BN
-    const int64_t tile0 = blockIdx.x / CTAS, tile_step = gridDim.x / CTAS;
+    const int64_t tile_step = gridDim.x / CTAS;
     constexpr int BKE = FP8 ? 2 * BK : BK;          // contraction indices per stage (128 bytes per row either way)
     constexpr int UK = FP8 ? 2 * UMMA_K : UMMA_K;   // contraction indices per MMA instruction (32 bytes per row)
     static_assert(!FP8 || (B_KMAJOR && !B_GATHER), "8-bit operands: both K-major, packed");
     const int num_kb = (int)((a.k + BKE - 1) / BKE);
+    // The n-th piece of work of this block: k-blocks [kb0, kb1) of a tile.  Whole tiles, round robin; in the gather form
+    // what its share of the joint (tile, k-block) axis holds (only the first and the last of its tiles can be cut).
+    auto piece = [&](int64_t n, int64_t &tile, int &kb0, int &kb1) -> bool {
+        if constexpr (B_GATHER) {
+            const int64_t begin = (int64_t)blockIdx.x * a.seg_kb, end = min(num_tiles * num_kb, begin + a.seg_kb);
+            const int64_t pos = n == 0 ? begin : (begin / num_kb + n) * num_kb;
+            if (pos >= end) return false;
+            tile = pos / num_kb;
+            kb0 = (int)(pos - tile * num_kb);
+            kb1 = (int)min((int64_t)num_kb, kb0 + (end - pos));
+            return true;
+        } else {
+            tile = blockIdx.x / CTAS + n * tile_step;
+            kb0 = 0;
+            kb1 = num_kb;
+            return tile < num_tiles;
+        }
+    };
 
     if (threadIdx.x == 32) {  // descriptor fetch overlaps barrier set-up and the TMEM allocation
         asm volatile("prefetch.tensormap [%0];" ::"l"(&map_a) : "memory");
@@ -178,7 +199,9 @@ reduced_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
         unsigned wave_target = 0;
         bool meeting = a.wave_ctr != nullptr;
         int64_t wave_first = 0;  // first tile of the current wave
-        for (int64_t tile = tile0; lane == 0 && tile < num_tiles && ok; tile += tile_step, wave_first += tile_step) {
+        int64_t tile;
+        int kb0, kb1;
+        for (int64_t n = 0; lane == 0 && ok && piece(n, tile, kb0, kb1); ++n, wave_first += tile_step) {
             const int64_t in_wave = num_tiles - wave_first < tile_step ? num_tiles - wave_first : tile_step;
             auto meet = [&]() {
                 wave_target += (unsigned)(in_wave * CTAS);
@@ -201,10 +224,10 @@ reduced_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
             tile_coords(tile - b * ((int64_t)a.tiles_n * a.tiles_m), a.tiles_m, a.tiles_n, a.raster, tm, tn);
             int64_t bb = (b + a.b_batch_off) / a.b_batch_div;
             if (bb >= a.b_batches) bb = a.b_batches - 1;
-            for (int kb = 0; kb < num_kb; ++kb) {
+            for (int kb = kb0; kb < kb1; ++kb) {
                 if (meeting && a.sync_kb > 0 && kb > 0 && kb % a.sync_kb == 0) meet();
                 if (!mbar_wait_lane(empty_bar(s), ph ^ 1u, abort_flag, a.status, a.wait_ns)) { ok = false; break; }
-                if (a.withhold && blockIdx.x == 0 && tile == tile0 && kb == 0) {
+                if (a.withhold && blockIdx.x == 0 && n == 0 && kb == 0) {
                     // (test switch) this stage is never requested: its barrier stays incomplete
                 } else {
                     const uint32_t sa = base + s * L::kStageBytes;
@@ -268,17 +291,19 @@ reduced_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
         const int last_steps = (int)((a.k - (int64_t)(num_kb - 1) * BKE + UK - 1) / UK);  // MMAs of the last k-block
         uint32_t stage = 0, phase = 0, tcount = 0;
         bool ok = true;
-        for (int64_t tile = tile0; lane == 0 && tile < num_tiles && ok; tile += tile_step, ++tcount) {
+        int64_t tile;
+        int kb0, kb1;
+        for (int64_t n = 0; lane == 0 && ok && piece(n, tile, kb0, kb1); ++n, ++tcount) {
             const uint32_t acc = tcount & 1u, acc_ph = (tcount >> 1) & 1u;
             if (!mbar_wait_lane(tempty_bar(acc), acc_ph ^ 1u, abort_flag, a.status, a.wait_ns)) { ok = false; break; }
             tc_fence_after();
             const uint32_t d_tmem = tmem_base + acc * BN;
             uint32_t accumulate = 0;
-            for (int kb = 0; kb < num_kb; ++kb) {
+            for (int kb = kb0; kb < kb1; ++kb) {
                 if (!mbar_wait_lane(full_bar(stage), phase, abort_flag, a.status, a.wait_ns)) { ok = false; break; }
                 if constexpr (B_GATHER) fence_proxy_async();  // B arrived through the generic proxy (cp.async)
                 tc_fence_after();
-                if (kb == 0 && tcount == 0) { GSTAMP_MAX(2); }
+                if (kb == kb0 && tcount == 0) { GSTAMP_MAX(2); }
                 const uint32_t a_lo = a_lo0 + stage * kStageUnits, b_lo = b_lo0 + stage * kStageUnits;
                 if (kb + 1 < num_kb || last_steps == BK / UMMA_K) {
 #pragma unroll
@@ -305,13 +330,15 @@ reduced_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
         // unit (l % 8) ^ (r % 8) -- the layout a 128-byte-swizzled TMA tile load would have produced.  The thread does
         // not wait for its copies: the stage's barrier receives this thread's arrival when they have landed, so every
         // free stage has copies in flight.  The MMA thread orders the landed data before the tensor cores'
-        // (asynchronous-proxy) reads with a proxy fence.  Row numbers are fetched one k-block ahead.
+        // (asynchronous-proxy) reads with a proxy fence.
         static_assert(!B_GATHER || (!B_KMAJOR && CTAS == 1 && BN == 256), "gather form: single-CTA 128 x 256 tiles, row-contiguous B");
         constexpr int kRowsPerWarp = BK / kGatherWarps;
         const int gw = warp - 6;
         uint32_t s = 0, ph = 0;
         bool ok = true;
-        for (int64_t tile = tile0; tile < num_tiles && ok; tile += tile_step) {
+        int64_t tile;
+        int kb0, kb1;
+        for (int64_t n = 0; ok && piece(n, tile, kb0, kb1); ++n) {
             int tm, tn;
             const int64_t b = tile / ((int64_t)a.tiles_n * a.tiles_m);
             tile_coords(tile - b * ((int64_t)a.tiles_n * a.tiles_m), a.tiles_m, a.tiles_n, a.raster, tm, tn);
@@ -322,25 +349,24 @@ reduced_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
             const __nv_bfloat16 *bcol = a.b_src + bb * a.b_sb + (col < a.N ? col : 0);
             const uint32_t col_bytes = col < a.N ? 16u : 0u;
             const uint32_t lane_off = (uint32_t)(lane >> 3) * (BK * 128);
-            int rows[kRowsPerWarp], rows_next[kRowsPerWarp];
-            auto fetch_rows = [&](int kb, int (&out)[kRowsPerWarp]) {
-#pragma unroll
-                for (int i = 0; i < kRowsPerWarp; ++i) {
-                    const int64_t kk = (int64_t)kb * BK + gw + kGatherWarps * i;
-                    out[i] = kk < a.k ? __ldg(ix + kk) : -1;
-                }
+            // row numbers: one load covers this warp's rows of four k-blocks (lane = k-block x row) and is issued four ahead
+            static_assert(kRowsPerWarp == 8, "eight lanes per k-block");
+            auto fetch_rows = [&](int kb) -> int {
+                const int64_t kk = (int64_t)(kb + (lane >> 3)) * BK + gw + kGatherWarps * (lane & 7);
+                return kb + (lane >> 3) < kb1 && kk < a.k ? __ldg(ix + kk) : -1;
             };
-            fetch_rows(0, rows_next);
-            for (int kb = 0; kb < num_kb; ++kb) {
-#pragma unroll
-                for (int i = 0; i < kRowsPerWarp; ++i) rows[i] = rows_next[i];
-                if (kb + 1 < num_kb) fetch_rows(kb + 1, rows_next);
+            int rows = -1, rows_next = fetch_rows(kb0);
+            for (int kb = kb0; kb < kb1; ++kb) {
+                if (((kb - kb0) & 3) == 0) {
+                    rows = rows_next;
+                    rows_next = fetch_rows(kb + 4);
+                }
                 if (!mbar_wait(empty_bar(s), ph ^ 1u, abort_flag, a.status, a.wait_ns)) { ok = false; break; }
                 const uint32_t sb = base + s * L::kStageBytes + L::kABytes + lane_off;
 #pragma unroll
                 for (int i = 0; i < kRowsPerWarp; ++i) {
                     const int r = gw + kGatherWarps * i;
-                    int row = rows[i];
+                    int row = __shfl_sync(0xffffffffu, rows, ((kb - kb0) & 3) * 8 + i);
                     if (row >= a.b_rows || (row < 0 && (int64_t)kb * BK + r < a.k)) {
                         atomicExch(a.status, (int)RMM_ERR_BOUNDS);
                         row = -1;
@@ -366,7 +392,9 @@ reduced_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
         const int slab_id = a.epi_sets == 2 ? eset * 4 + q : q * 2;        // 4 KB slabs; a single set has two per warp
         uint8_t *slab = base_ptr + L::kEpiOffset + slab_id * 4096 + lane * 128;   // this thread's row of the warp's staging slabs
         const uint32_t slab_s = base + L::kEpiOffset + slab_id * 4096;
-        for (int64_t tile = tile0; tile < num_tiles && ok; tile += tile_step, ++tcount) {
+        int64_t tile;
+        int kb0, kb1;
+        for (int64_t n = 0; ok && piece(n, tile, kb0, kb1); ++n, ++tcount) {
             int tm, tn;
             const int64_t b = tile / ((int64_t)a.tiles_n * a.tiles_m);
             tile_coords(tile - b * ((int64_t)a.tiles_n * a.tiles_m), a.tiles_m, a.tiles_n, a.raster, tm, tn);
@@ -381,7 +409,23 @@ reduced_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
             if constexpr (FP8) {
                 if (a.row_scale != nullptr && m < a.M) scale_r *= __ldg(a.row_scale + b * a.M + m);
             }
-            if constexpr (OUT_BF16) {
+            if (B_GATHER && kb1 - kb0 < num_kb) {
+                // part of the contraction: the unscaled sums go to the block's first or last slot (gemm_meet_kernel adds them up)
+                const int64_t slot_rows = a.M < BM ? a.M : BM;
+                float *dst = a.partials + ((2 * (int64_t)blockIdx.x + (n > 0 ? 1 : 0)) * slot_rows + q * 32 + lane) * BN;
+#pragma unroll 1
+                for (int c = 0; c < BN / 32 && m_warp < a.M; ++c) {
+                    uint32_t r[32];
+                    tmem_ld32_issue(t_row + c * 32, r);
+                    tmem_ld_wait();
+                    if (m < a.M) {
+#pragma unroll
+                        for (int v = 0; v < 8; ++v)
+                            __stcg(reinterpret_cast<float4 *>(dst + c * 32) + v,
+                                   make_float4(__uint_as_float(r[4 * v]), __uint_as_float(r[4 * v + 1]), __uint_as_float(r[4 * v + 2]), __uint_as_float(r[4 * v + 3])));
+                    }
+                }
+            } else if constexpr (OUT_BF16) {
                 // 64 columns at a time: two TMEM loads, scale and round, one 32 x 64 slab per warp through a TMA store
 #pragma unroll 1
                 for (int c = eset; c < BN / 64; c += a.epi_sets) {
@@ -505,6 +549,47 @@ reduced_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
     if (threadIdx.x == 0) { GSTAMP_MAX(6); }
 }
 
+// The tiles whose contraction was cut: the pieces of a tile are added in order of their k-blocks, scaled and rounded.
+// One warp per output row of a 256-column tile.
+constexpr int kMeetRows = 4;
+template <bool OUT_BF16>
+__global__ void __launch_bounds__(32 * kMeetRows) gemm_meet_kernel(const TcArgs a, int num_kb)
+{
+    pdl_wait();
+    const int64_t tile = blockIdx.x, per_batch = (int64_t)a.tiles_n * a.tiles_m, b = tile / per_batch;
+    const int64_t b0 = tile * num_kb / a.seg_kb, b1 = ((tile + 1) * num_kb - 1) / a.seg_kb;
+    if (b0 == b1) return;  // written by its only block
+    int tm, tn;
+    tile_coords(tile - b * per_batch, a.tiles_m, a.tiles_n, a.raster, tm, tn);
+    const int r = blockIdx.y * kMeetRows + (threadIdx.x >> 5);
+    const int64_t m = (int64_t)tm * BM + r, n = (int64_t)tn * 256 + (threadIdx.x & 31) * 8;
+    if (r >= BM || m >= a.M || n >= a.N) return;
+    const int64_t slot_rows = a.M < BM ? a.M : BM;
+    float v[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll 4
+    for (int64_t blk = b0; blk <= b1; ++blk) {  // only a tile's first block can hold it as its last piece
+        const int64_t slot = 2 * blk + (blk == b0 && b0 * a.seg_kb < tile * num_kb ? 1 : 0);
+        const float4 *src = reinterpret_cast<const float4 *>(a.partials + (slot * slot_rows + r) * 256 + (threadIdx.x & 31) * 8);
+        const float4 x = __ldcg(src), y = __ldcg(src + 1);
+        v[0] += x.x; v[1] += x.y; v[2] += x.z; v[3] += x.w;
+        v[4] += y.x; v[5] += y.y; v[6] += y.z; v[7] += y.w;
+    }
+    const int64_t off = b * a.y_sb + m * a.y_sr + n;  // N is a multiple of 8, rows of Y start on 16 bytes
+    if constexpr (OUT_BF16) {
+        uint32_t w[4];
+#pragma unroll
+        for (int p = 0; p < 4; ++p) {
+            __nv_bfloat162 h = __floats2bfloat162_rn(v[2 * p] * a.scale, v[2 * p + 1] * a.scale);
+            w[p] = *reinterpret_cast<uint32_t *>(&h);
+        }
+        *reinterpret_cast<uint4 *>(static_cast<__nv_bfloat16 *>(a.Y) + off) = make_uint4(w[0], w[1], w[2], w[3]);
+    } else {
+        float4 *y = reinterpret_cast<float4 *>(static_cast<float *>(a.Y) + off);
+        y[0] = make_float4(v[0] * a.scale, v[1] * a.scale, v[2] * a.scale, v[3] * a.scale);
+        y[1] = make_float4(v[4] * a.scale, v[5] * a.scale, v[6] * a.scale, v[7] * a.scale);
+    }
+}
+
 // ----------------------------------------------------------------------------------------------
 // host side
 // ----------------------------------------------------------------------------------------------
@@ -518,15 +603,24 @@ int launch_variant(const CUtensorMap &ma, const CUtensorMap &mb, const CUtensorM
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kTotal);
         if (e != cudaSuccess) return fail(RMM_ERR_CUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e));
     }
-    const int64_t tiles = a.batch * a.tiles_m * a.tiles_n;
+    const int64_t tiles = a.batch * a.tiles_m * a.tiles_n, num_kb = ceil_div(a.k, FP8 ? 2 * BK : BK);
     const int64_t slots = sm_count() / CTAS;
+    const int64_t blocks = B_GATHER ? ceil_div(tiles * num_kb, a.seg_kb) : (tiles < slots ? tiles : slots);
     prof_begin("reduced_gemm_tc_kernel", stream);
-    cudaError_t e = launch_kernel(kern, dim3((unsigned)((tiles < slots ? tiles : slots) * CTAS)),
+    cudaError_t e = launch_kernel(kern, dim3((unsigned)(blocks * CTAS)),
                                   dim3(B_GATHER ? kThreadsTc + 32 * kGatherWarps : (a.epi_sets == 2 ? kThreadsTc2 : kThreadsTc)), L::kTotal, stream,
                                   CTAS, ma, mb, my, a);
     if (e != cudaSuccess) return fail(RMM_ERR_CUDA, "reduced_gemm_tc_kernel: launch: %s", cudaGetErrorString(e));
-    return check_launch("reduced_gemm_tc_kernel", stream);
+    int rc = check_launch("reduced_gemm_tc_kernel", stream);
+    if (!B_GATHER || rc != RMM_OK || a.seg_kb % num_kb == 0) return rc;
+    prof_begin("gemm_meet_kernel", stream);
+    launch_kernel(gemm_meet_kernel<OUT_BF16>, dim3((unsigned)tiles, (unsigned)ceil_div(a.M < BM ? a.M : BM, kMeetRows)), dim3(32 * kMeetRows), 0,
+                  stream, 1, a, (int)num_kb);
+    return check_launch("gemm_meet_kernel", stream);
 }
+
+// Products of few rows fetch the kept rows of B inside the kernel (see the file header)
+bool gathers_b(const TcPlan &plan, int64_t M, int64_t N) { return !plan.b_kmajor && M <= 2 * BM && N > 128; }
 
 }  // namespace
 
@@ -556,8 +650,11 @@ bool tc_eligible(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k, const rmm_ma
         size_t off = RMM_WS_HEADER_BYTES;
         plan->off_ap = off;
         off += align_up((size_t)batch * M * plan->ldp * 2, 256);
-        plan->off_bp = off;
-        off += align_up(b_kmajor ? (size_t)batch * N * plan->ldp * 2 : (size_t)batch * k * N * 2, 256);
+        plan->off_bp = off;  // packed B, or the sums of cut tiles
+        plan->gathers = gathers_b(*plan, M, N);
+        if (plan->gathers && M <= kSkinnyRows) off += gemm_skinny_partial_bytes(batch, M, N, k);
+        else if (plan->gathers) off += (size_t)2 * sm_count() * (M < BM ? M : BM) * 256 * 4;
+        else off += align_up(b_kmajor ? (size_t)batch * N * plan->ldp * 2 : (size_t)batch * k * N * 2, 256);
         // column energies from the epilogue: bf16 output with an even number of columns (the pairs are stored as float2)
         plan->epilogue_energy = with_energy && Y->dtype == RMM_BF16 && N % 2 == 0;
         plan->off_colen = off;
@@ -618,7 +715,7 @@ int launch_gemm_tc_problem(const TcProblem &p, cudaStream_t stream)
         // wave synchronisation: products with several waves of long tiles (measurement switch RMM_GEMM_WAVE_SYNC=0|1)
         static const int forced_sync = []() { const char *e = getenv("RMM_GEMM_WAVE_SYNC"); return e ? atoi(e) : -1; }();
         const int64_t tiles = (int64_t)a.batch * a.tiles_m * a.tiles_n, per_wave = sm_count() / ctas;
-        const bool want = forced_sync >= 0 ? forced_sync != 0 : (tiles > per_wave && p.k * es >= 8192);
+        const bool want = p.b_idx == nullptr && (forced_sync >= 0 ? forced_sync != 0 : (tiles > per_wave && p.k * es >= 8192));
         static const int sync_kb = []() { const char *e = getenv("RMM_GEMM_SYNC_KB"); return e ? atoi(e) : 128; }();
         a.sync_kb = sync_kb;
         a.wave_ctr = (want && p.status != nullptr)
@@ -634,6 +731,20 @@ int launch_gemm_tc_problem(const TcProblem &p, cudaStream_t stream)
     a.b_src = p.b; a.b_idx = p.b_idx; a.b_ld = p.b_ld; a.b_sb = p.b_batches > 1 ? p.b_sb : 0; a.b_idx_stride = p.b_idx_stride;
     a.b_rows = p.b_rows;
     if (p.b_idx != nullptr) {
+        // A product of few rows is bound by how fast the SMs pull rows of B, so none may idle: equal shares of all tiles'
+        // k-blocks, one per SM (at least two k-blocks each), where whole tiles would leave too many without work.  Cutting
+        // costs the partial sums (measured, in k-blocks of 0.94 us: 2 + 15 for 128 rows) and a k-block takes 1.27 times as
+        // long with every SM pulling.  48 x 28672 (half kept) x 8192, 32 tiles: 216 us whole, 70 cut; 128 x 8192 (a quarter)
+        // x 28672, 112 tiles: 41.6 whole, 54 cut.
+        const int64_t num_kb = ceil_div(p.k, (int64_t)BK), sms = sm_count();
+        a.seg_kb = ceil_div(n_tiles * num_kb, sms);
+        if (a.seg_kb < 2) a.seg_kb = 2;
+        const double whole = (double)(ceil_div(n_tiles, sms) * num_kb), cut = 1.27 * (double)a.seg_kb + 2.0 + 15.0 * (double)(p.M < BM ? p.M : BM) / BM;
+        if (whole <= cut) a.seg_kb = ceil_div(n_tiles, sms) * num_kb;
+        a.partials = p.partials;
+        if (p.col_energy != nullptr || p.partials == nullptr)
+            return fail(RMM_ERR_INVALID_ARG, "reduced_gemm_tc: the in-kernel row gather cuts tiles: it needs partial sums and leaves no column energies");
+        a.partials = p.partials;
         if (p.b_kmajor || ctas != 1 || BN != 256)
             return fail(RMM_ERR_UNSUPPORTED, "reduced_gemm_tc: in-kernel row gather needs single-CTA 128 x 256 tiles and row-contiguous B");
         CUtensorMap my_g = ma;  // (the tensor map of B is unused in this form; A's stands in)
@@ -725,15 +836,17 @@ int launch_gemm_tc(const rmm_mat_t *A, const rmm_mat_t *B, const int32_t *idx, i
     PackSpec specs[2];
     specs[0] = pack_cols_spec(a_src, batch, M, K, A->stride_batch, A->stride_row, 0, 1, idx, k, k, Ap, plan.ldp);
     p.a = Ap; p.a_ld = plan.ldp; p.a_sb = M * plan.ldp;
-    if (!plan.b_kmajor && M <= 2 * BM && N > 128) {
+    if (plan.gathers) {
         // one or two tile rows: a tile of B is used once or twice (the second time from L2), so the kernel fetches the
         // kept rows itself and only A[:, I] is packed
         p.b = b_src; p.b_ld = B->stride_row; p.b_rows = K;
         if (B->stride_batch == 0) { p.b_batches = 1; p.b_sb = 0; }
         else { p.b_sb = B->stride_batch; }
         p.b_idx = idx; p.b_idx_stride = k;
+        p.partials = reinterpret_cast<float *>(w + plan.off_bp);
         rc = launch_pack(specs, 1, status, stream);
         if (rc != RMM_OK) return rc;
+        if (idx != nullptr && M <= kSkinnyRows) return launch_gemm_skinny(p, stream);
         return launch_gemm_tc_problem(p, stream);
     }
     if (plan.b_kmajor) {
