@@ -432,12 +432,22 @@ int rmm_product(const rmm_mat_t *A, const rmm_mat_t *B, double rho, int64_t k, f
         if (rc != RMM_OK) return rc;
         return rmm_reduced_gemm(A, B, nullptr, kk, scale, Y, ws, ws_bytes, stream);
     }
+    rmm_mat_t b = shared_b(A, B);
     if (!pp.fused) {
+        // few rows: the kernel that scores and selects also gathers A, where the product fetches the rows of B itself
+        ScorePlan sp;
+        TcPlan tc;
+        if (!gemv_eligible(A, &b, kk, Y, nullptr) && tc_eligible(A, &b, kk, Y, &tc) && tc.gathers && plan_score(A, 1, &sp) == RMM_OK &&
+            few_rows_eligible(A, sp)) {
+            rc = launch_few_rows(A, sp, kk, idx, nullptr, nullptr, retained,
+                                 reinterpret_cast<__nv_bfloat16 *>(static_cast<char *>(ws) + tc.off_ap), tc.ldp, st);
+            if (rc != RMM_OK) return rc;
+            return launch_gemm_tc(A, &b, idx, kk, scale, Y, tc, ws, st, nullptr, true);
+        }
         rc = rmm_score_select(A, 1, rho, kk, idx, nullptr, nullptr, retained, ws, ws_bytes, stream);
         if (rc != RMM_OK) return rc;
         return rmm_reduced_gemm(A, B, idx, kk, scale, Y, ws, ws_bytes, stream);
     }
-    rmm_mat_t b = shared_b(A, B);
     rc = launch_front(A, &b, kk, idx, nullptr, retained, pp.front, ws, st);
     if (rc != RMM_OK) return rc;
     char *w = static_cast<char *>(ws);

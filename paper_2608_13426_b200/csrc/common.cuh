@@ -109,6 +109,13 @@ struct ScorePlan {
 int plan_score(const rmm_mat_t *A, int axis, ScorePlan *plan);
 int launch_score_select(const rmm_mat_t *A, const ScorePlan &p, bool do_select, int64_t k, int32_t *idx,
                         float *scores, float *energy, float *retained, void *ws, cudaStream_t stream);
+// Scores, selection and, where Ap is given, the packed columns A[:, I] ([batch, m, ldp], zeros from k on) of a bf16 matrix
+// of a few rows with contiguous scored axis, in one launch.  Level with the separate passes at 64 rows of 512 columns (9.8 us
+// against 9.5) and behind with the gather (18.5 against 15.2), ahead at 32 rows of every width.
+constexpr int64_t kFewRows = 32;
+bool few_rows_eligible(const rmm_mat_t *A, const ScorePlan &p);
+int launch_few_rows(const rmm_mat_t *A, const ScorePlan &p, int64_t k, int32_t *idx, float *scores, float *energy, float *retained,
+                    __nv_bfloat16 *Ap, int64_t ldp, cudaStream_t stream);
 int launch_select(const float *keys, int64_t batch, int64_t K, int64_t k, int32_t *idx, float *retained, void *ws,
                   cudaStream_t stream);
 
@@ -146,9 +153,10 @@ struct TcPlan {
     bool epilogue_energy;  // the plan reserves the per-group column energies of Y and the epilogue fills them
 };
 bool tc_eligible(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k, const rmm_mat_t *Y, TcPlan *plan, bool with_energy = false);
+// a_packed (plans that gather rows of B): A[:, I] is already in the workspace at plan.off_ap.
 // energy_out (with a plan made with_energy): also energy_out[b, c] = sum_i Y[b, i, c]^2 of the rounded outputs
 int launch_gemm_tc(const rmm_mat_t *A, const rmm_mat_t *B, const int32_t *idx, int64_t k, float scale,
-                   const rmm_mat_t *Y, const TcPlan &plan, void *ws, cudaStream_t stream, float *energy_out = nullptr);
+                   const rmm_mat_t *Y, const TcPlan &plan, void *ws, cudaStream_t stream, float *energy_out = nullptr, bool a_packed = false);
 
 // A tensor-core problem on operands that are already in TMA-loadable form.
 struct TcProblem {

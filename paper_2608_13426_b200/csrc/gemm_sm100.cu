@@ -799,7 +799,7 @@ int launch_gemm_tc_problem(const TcProblem &p, cudaStream_t stream)
 }
 
 int launch_gemm_tc(const rmm_mat_t *A, const rmm_mat_t *B, const int32_t *idx, int64_t k, float scale,
-                   const rmm_mat_t *Y, const TcPlan &plan, void *ws, cudaStream_t stream, float *energy_out)
+                   const rmm_mat_t *Y, const TcPlan &plan, void *ws, cudaStream_t stream, float *energy_out, bool a_packed)
 {
     if (energy_out != nullptr && plan.epilogue_energy) {
         // the product writes per-group column energies, a small kernel adds the groups up
@@ -844,8 +844,7 @@ int launch_gemm_tc(const rmm_mat_t *A, const rmm_mat_t *B, const int32_t *idx, i
         else { p.b_sb = B->stride_batch; }
         p.b_idx = idx; p.b_idx_stride = k;
         p.partials = reinterpret_cast<float *>(w + plan.off_bp);
-        rc = launch_pack(specs, 1, status, stream);
-        if (rc != RMM_OK) return rc;
+        if (!a_packed && (rc = launch_pack(specs, 1, status, stream)) != RMM_OK) return rc;
         if (idx != nullptr && M <= kSkinnyRows) return launch_gemm_skinny(p, stream);
         return launch_gemm_tc_problem(p, stream);
     }

@@ -755,38 +755,119 @@ __global__ void __launch_bounds__(kThreads, 1) rmm_front_kernel(const __grid_con
 // reads a block and digit; three digits of 11, 11 and 10 bits, 64 KB, took 14.7 / 16.2 us), then one exchange of the
 // blocks' counts for the ordered emission.  Measured on 14336 / 28672 keys: 8.8 / 9.9 us; one block with the keys in
 // shared memory 24.5 / 37, with the keys in registers 13.3 / 24.4.  8192 keys take one block 7.5 to 9 us.
+//
+// FROM_A: the keys are the energies of a bf16 matrix of at most kFewRows rows, which the same kernel sums (fp64 sums of
+// exact squares), and the kept columns may be copied out (Ap) as well: a decode step's scores, selection and gather in one
+// launch.  The separate score pass hands its energies to the last of 128 blocks: 1 / 24 x 8192 took 16 / 14.4 us with the
+// selection, 9.1 / 11.2 here, and 24 x 8192 with the gather 19.6, 15 here; 1 / 24 x 28672 28 us, 11.2 / 16.8.  Narrow
+// matrices (and up to eight rows of 4096 columns) take one block, CTAS = 1: 1 x 512 10.5 us, 5.3.
 constexpr int kSelCtas = 8, kSelThreads = 512;
 constexpr int64_t kClusterSelectMax = (int64_t)kSelCtas * kSelThreads * 16;
 
-template <int ITEMS>
-__global__ void __launch_bounds__(kSelThreads) select_cluster_kernel(const float *__restrict__ keys_all, int K, int k, int32_t *__restrict__ idx_all,
-                                                                     float *retained)
+struct ClusterSelectArgs {
+    const float *keys;       // [batch, K], or
+    const __nv_bfloat16 *A;  // FROM_A: row r of batch entry b at A + b s_batch + r s_row
+    int64_t s_batch, s_row, ldp;
+    int m, K, k, vec;        // vec: a thread's columns of a row are one aligned load
+    int32_t *idx;
+    float *energy, *scores, *retained;   // or NULL
+    __nv_bfloat16 *Ap;       // FROM_A: [batch, m, ldp] kept columns, zeros from k on, or NULL
+};
+
+template <int ITEMS, int CTAS, bool FROM_A>
+__global__ void __launch_bounds__(kSelThreads) select_cluster_kernel(const ClusterSelectArgs a)
 {
     constexpr int kWarps = kSelThreads / 32;
     __shared__ __align__(16) unsigned s_hist[4][256];
     __shared__ unsigned s_warp[kWarps], s_bin, s_left, s_total;
     __shared__ double s_sum[2 * kWarps], s_mass[2];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const uint32_t rank = ptx::cluster_rank();
-    const int64_t b = blockIdx.x / kSelCtas;
-    const float *keys = keys_all + b * K;
-    int32_t *idx = idx_all + b * (int64_t)k;
+    const int K = a.K, k = a.k;
+    const uint32_t rank = CTAS > 1 ? ptx::cluster_rank() : 0u;
+    const int64_t b = blockIdx.x / CTAS;
+    int32_t *idx = a.idx + b * (int64_t)k;
+    auto meet = [&]() {
+        if constexpr (CTAS > 1) ptx::cluster_sync_all();
+        else __syncthreads();
+    };
+    auto remote = [&](const void *p, int r) -> uint32_t {
+        const uint32_t local = ptx::smem_u32(p);
+        return CTAS > 1 ? ptx::map_to_cta(local, r) : local;
+    };
     if (tid < 256) reinterpret_cast<uint4 *>(s_hist)[tid] = make_uint4(0, 0, 0, 0);
     pdl_wait();
 
-    const int span = ((K + kSelCtas - 1) / kSelCtas + 3) / 4 * 4;    // keys of a block, <= kSelThreads * ITEMS
+    const int span = ((K + CTAS - 1) / CTAS + 7) / 8 * 8;    // keys of a block, <= kSelThreads * ITEMS
     const int j0 = (int)rank * span + tid * ITEMS, j_end = min(K, ((int)rank + 1) * span);
-    const int nvalid = max(0, min(ITEMS, min(j_end, (int)rank * span + span) - j0));
+    const int nvalid = max(0, min(ITEMS, j_end - j0));
     unsigned u[ITEMS];
-    if (nvalid == ITEMS && (reinterpret_cast<uintptr_t>(keys) & 15) == 0) {
+    const __nv_bfloat16 *col = nullptr;
+    constexpr int kBatch = ITEMS == 2 ? 16 : (ITEMS <= 8 ? 8 : 4);  // rows in flight per thread: a row at a time is one memory latency a row
+    auto each_row = [&](auto &&use) {  // use(r, x): this thread's columns of row r, zeros past the last column
+        const bool wide = a.vec && nvalid == ITEMS;
+        for (int r0 = 0; r0 < a.m; r0 += kBatch) {
+            unsigned w[kBatch][ITEMS / 2];
+            if (wide) {
 #pragma unroll
-        for (int v = 0; v < ITEMS / 4; ++v) {
-            const float4 q = __ldcg(reinterpret_cast<const float4 *>(keys + j0) + v);
-            u[4 * v] = key_image(q.x); u[4 * v + 1] = key_image(q.y); u[4 * v + 2] = key_image(q.z); u[4 * v + 3] = key_image(q.w);
+                for (int q = 0; q < kBatch; ++q) {
+                    const __nv_bfloat16 *p = col + (r0 + q < a.m ? r0 + q : r0) * a.s_row;
+                    if constexpr (ITEMS == 2) {
+                        w[q][0] = __ldg(reinterpret_cast<const unsigned *>(p));
+                    } else if constexpr (ITEMS == 4) {
+                        const uint2 v = __ldg(reinterpret_cast<const uint2 *>(p));
+                        w[q][0] = v.x; w[q][1] = v.y;
+                    } else {
+#pragma unroll
+                        for (int h = 0; h < ITEMS / 8; ++h) {
+                            const uint4 v = __ldg(reinterpret_cast<const uint4 *>(p) + h);
+                            w[q][4 * h] = v.x; w[q][4 * h + 1] = v.y; w[q][4 * h + 2] = v.z; w[q][4 * h + 3] = v.w;
+                        }
+                    }
+                }
+            } else {
+#pragma unroll
+                for (int q = 0; q < kBatch; ++q) {
+                    const unsigned short *p = reinterpret_cast<const unsigned short *>(col + (r0 + q < a.m ? r0 + q : r0) * a.s_row);
+#pragma unroll
+                    for (int i = 0; i < ITEMS / 2; ++i)
+                        w[q][i] = (2 * i < nvalid ? (unsigned)__ldg(p + 2 * i) : 0u) | (2 * i + 1 < nvalid ? (unsigned)__ldg(p + 2 * i + 1) << 16 : 0u);
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < kBatch; ++q)
+                if (r0 + q < a.m) use(r0 + q, w[q]);
+        }
+    };
+    if constexpr (FROM_A) {
+        col = a.A + b * a.s_batch + j0;
+        double e[ITEMS];
+#pragma unroll
+        for (int i = 0; i < ITEMS; ++i) e[i] = 0.0;
+        each_row([&](int, const unsigned (&w)[ITEMS / 2]) {
+#pragma unroll
+            for (int i = 0; i < ITEMS; ++i) {
+                const float x = __uint_as_float(i & 1 ? w[i / 2] & 0xffff0000u : w[i / 2] << 16);
+                e[i] += (double)(x * x);  // the square of a bf16 number is exact in fp32
+            }
+        });
+#pragma unroll
+        for (int i = 0; i < ITEMS; ++i) {
+            u[i] = i < nvalid ? key_image((float)e[i]) : 0u;
+            if (i < nvalid && a.energy != nullptr) a.energy[b * K + j0 + i] = (float)e[i];
+            if (i < nvalid && a.scores != nullptr) a.scores[b * K + j0 + i] = (float)sqrt(e[i]);
         }
     } else {
+        const float *keys = a.keys + b * K;
+        if (ITEMS >= 4 && nvalid == ITEMS && (reinterpret_cast<uintptr_t>(keys) & 15) == 0) {
 #pragma unroll
-        for (int i = 0; i < ITEMS; ++i) u[i] = i < nvalid ? key_image(__ldcg(keys + j0 + i)) : 0u;
+            for (int v = 0; v < ITEMS / 4; ++v) {
+                const float4 q = __ldcg(reinterpret_cast<const float4 *>(keys + j0) + v);
+                u[4 * v] = key_image(q.x); u[4 * v + 1] = key_image(q.y); u[4 * v + 2] = key_image(q.z); u[4 * v + 3] = key_image(q.w);
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < ITEMS; ++i) u[i] = i < nvalid ? key_image(__ldcg(keys + j0 + i)) : 0u;
+        }
     }
     __syncthreads();
 
@@ -798,17 +879,16 @@ __global__ void __launch_bounds__(kSelThreads) select_cluster_kernel(const float
 #pragma unroll
         for (int i = 0; i < ITEMS; ++i)
             if (i < nvalid && (pass == 0 || (u[i] >> (shift + 8)) == prefix)) atomicAdd(&s_hist[pass][(u[i] >> shift) & 255u], 1u);
-        ptx::cluster_sync_all();
+        meet();
         // threads 0 .. 255: bin 255 - tid over the whole cluster, and the keys in the bins above it
         unsigned sum = 0;
         if (tid < 256) {
-            const uint32_t mine = ptx::smem_u32(&s_hist[pass][255 - tid]);
-            unsigned h[kSelCtas];
+            unsigned h[CTAS];
 #pragma unroll
-            for (int r = 0; r < kSelCtas; ++r)
-                asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(h[r]) : "r"(ptx::map_to_cta(mine, r)) : "memory");
+            for (int r = 0; r < CTAS; ++r)
+                asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(h[r]) : "r"(remote(&s_hist[pass][255 - tid], r)) : "memory");
 #pragma unroll
-            for (int r = 0; r < kSelCtas; ++r) sum += h[r];
+            for (int r = 0; r < CTAS; ++r) sum += h[r];
         }
         unsigned incl = sum;
 #pragma unroll
@@ -854,22 +934,26 @@ __global__ void __launch_bounds__(kSelThreads) select_cluster_kernel(const float
     }
     const unsigned before = __shfl_sync(0xffffffffu, wi - own, warp) + incl - cnt;
     if (tid == kSelThreads - 1) s_total = before + cnt;
-    ptx::cluster_sync_all();
+    meet();
     unsigned gt_before = before >> 16, eq_before = before & 0xffffu;
-    {
+    if constexpr (CTAS > 1) {
         unsigned t = 0;
-        if (lane < (int)rank)
-            asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(t) : "r"(ptx::map_to_cta(ptx::smem_u32(&s_total), lane)) : "memory");
+        if (lane < (int)rank) asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(t) : "r"(remote(&s_total, lane)) : "memory");
         gt_before += __reduce_add_sync(0xffffffffu, t >> 16);
         eq_before += __reduce_add_sync(0xffffffffu, t & 0xffffu);
     }
     double sum_kept = 0.0, sum_all = 0.0;
+    int pos[ITEMS];  // position of a kept key in the list, or -1
 #pragma unroll
     for (int i = 0; i < ITEMS; ++i) {
+        pos[i] = -1;
         if (i < nvalid) {
             const bool gt = u[i] > tau, eq = u[i] == tau, keep = gt || (eq && eq_before < need_eq);
-            if (keep) idx[gt_before + min(eq_before, need_eq)] = j0 + i;
-            if (retained != nullptr) {
+            if (keep) {
+                pos[i] = (int)(gt_before + min(eq_before, need_eq));
+                idx[pos[i]] = j0 + i;
+            }
+            if (a.retained != nullptr) {
                 const double f = (double)key_value(u[i]);
                 sum_all += f;
                 if (keep) sum_kept += f;
@@ -878,7 +962,19 @@ __global__ void __launch_bounds__(kSelThreads) select_cluster_kernel(const float
             eq_before += eq ? 1u : 0u;
         }
     }
-    if (retained != nullptr) {
+    if constexpr (FROM_A) {
+        if (a.Ap != nullptr) {
+            unsigned short *dst = reinterpret_cast<unsigned short *>(a.Ap) + b * a.m * a.ldp;
+            each_row([&](int r, const unsigned (&w)[ITEMS / 2]) {
+#pragma unroll
+                for (int i = 0; i < ITEMS; ++i)
+                    if (pos[i] >= 0) dst[r * a.ldp + pos[i]] = (unsigned short)(i & 1 ? w[i / 2] >> 16 : w[i / 2]);
+            });
+            const int pad = (int)(a.ldp - k);
+            for (int i = tid; rank == 0 && i < a.m * pad; i += kSelThreads) dst[i / pad * a.ldp + k + i % pad] = 0;
+        }
+    }
+    if (a.retained != nullptr) {
 #pragma unroll
         for (int d = 16; d > 0; d >>= 1) {
             sum_kept += __shfl_down_sync(0xffffffffu, sum_kept, d);
@@ -894,19 +990,38 @@ __global__ void __launch_bounds__(kSelThreads) select_cluster_kernel(const float
             for (int w = 0; w < kWarps; ++w) s += s_sum[tid * kWarps + w];
             s_mass[tid] = s;
         }
-        ptx::cluster_sync_all();
+        meet();
         if (rank == 0 && tid == 0) {
             double m[2] = {0.0, 0.0};
-            for (int r = 0; r < kSelCtas; ++r)
+            for (int r = 0; r < CTAS; ++r)
                 for (int e = 0; e < 2; ++e) {
                     double v;
-                    asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(ptx::map_to_cta(ptx::smem_u32(&s_mass[e]), r)) : "memory");
+                    asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(remote(&s_mass[e], r)) : "memory");
                     m[e] += v;
                 }
-            retained[b] = m[1] > 0.0 ? (float)(m[0] / m[1]) : 1.0f;
+            a.retained[b] = m[1] > 0.0 ? (float)(m[0] / m[1]) : 1.0f;
         }
     }
-    ptx::cluster_sync_all();  // a block's shared memory stays until every block has read it
+    if constexpr (CTAS > 1) ptx::cluster_sync_all();  // a block's shared memory stays until every block has read it
+}
+
+template <bool FROM_A>
+int launch_cluster_select(const ClusterSelectArgs &a, int64_t batch, const char *name, cudaStream_t stream)
+{
+    void (*kern)(ClusterSelectArgs) = nullptr;
+    int ctas = kSelCtas;
+    if (FROM_A && (a.K <= 1024 || (a.K <= 4096 && a.m <= 8))) {
+        ctas = 1;
+        kern = a.K <= 1024 ? select_cluster_kernel<2, 1, FROM_A> : select_cluster_kernel<8, 1, FROM_A>;
+    } else if (FROM_A && a.K <= 8192) {
+        kern = select_cluster_kernel<2, kSelCtas, FROM_A>;
+    } else {
+        kern = a.K <= 16384 ? select_cluster_kernel<4, kSelCtas, FROM_A>
+                            : (a.K <= 32768 ? select_cluster_kernel<8, kSelCtas, FROM_A> : select_cluster_kernel<16, kSelCtas, FROM_A>);
+    }
+    prof_begin(name, stream);
+    launch_kernel(kern, dim3((unsigned)(batch * ctas)), dim3(kSelThreads), 0, stream, ctas, a);
+    return check_launch(name, stream);
 }
 
 __global__ void __launch_bounds__(1024) select_kernel(const float *keys, int K, int k, int32_t *idx, float *retained)
@@ -979,9 +1094,27 @@ int plan_score(const rmm_mat_t *A, int axis, ScorePlan *p)
     return RMM_OK;
 }
 
+bool few_rows_eligible(const rmm_mat_t *A, const ScorePlan &p)
+{
+    return A->dtype == RMM_BF16 && p.s_n == 1 && p.m <= kFewRows && p.n <= kClusterSelectMax;
+}
+
+int launch_few_rows(const rmm_mat_t *A, const ScorePlan &p, int64_t k, int32_t *idx, float *scores, float *energy, float *retained,
+                    __nv_bfloat16 *Ap, int64_t ldp, cudaStream_t stream)
+{
+    ClusterSelectArgs c = {};
+    c.A = static_cast<const __nv_bfloat16 *>(A->ptr);
+    c.s_batch = p.s_batch; c.s_row = p.s_red; c.ldp = ldp;
+    c.m = (int)p.m; c.K = (int)p.n; c.k = (int)k;
+    c.vec = reinterpret_cast<uintptr_t>(A->ptr) % 16 == 0 && p.s_red % 8 == 0 && p.s_batch % 8 == 0;
+    c.idx = idx; c.energy = energy; c.scores = scores; c.retained = retained; c.Ap = Ap;
+    return launch_cluster_select<true>(c, A->batch, "few_rows_kernel", stream);
+}
+
 int launch_score_select(const rmm_mat_t *A, const ScorePlan &p, bool do_select, int64_t k, int32_t *idx,
                         float *scores, float *energy, float *retained, void *ws, cudaStream_t stream)
 {
+    if (do_select && few_rows_eligible(A, p)) return launch_few_rows(A, p, k, idx, scores, energy, retained, nullptr, 0, stream);
     char *w = static_cast<char *>(ws);
     WsHeader *hdr = reinterpret_cast<WsHeader *>(w);
     ScoreArgs a;
@@ -1126,10 +1259,9 @@ int launch_select(const float *keys, int64_t batch, int64_t K, int64_t k, int32_
 {
     (void)ws;
     if (K > kFusedSelectMax && K <= kClusterSelectMax) {
-        auto kern = K <= 16384 ? select_cluster_kernel<4> : (K <= 32768 ? select_cluster_kernel<8> : select_cluster_kernel<16>);
-        prof_begin("select_kernel", stream);
-        launch_kernel(kern, dim3((unsigned)batch * kSelCtas), dim3(kSelThreads), 0, stream, kSelCtas, keys, (int)K, (int)k, idx, retained);
-        return check_launch("select_kernel", stream);
+        ClusterSelectArgs c = {};
+        c.keys = keys; c.K = (int)K; c.k = (int)k; c.idx = idx; c.retained = retained;
+        return launch_cluster_select<false>(c, batch, "select_kernel", stream);
     }
     prof_begin("select_kernel", stream);
     launch_kernel(select_kernel, dim3((unsigned)batch), dim3(1024), 0, stream, 1, keys, (int)K, (int)k, idx, retained);
