@@ -140,7 +140,8 @@ def as_mat(t: torch.Tensor) -> rmm_mat_t:
 
 
 def _stream() -> int:
-    return torch.cuda.current_stream().cuda_stream
+    # the current stream's handle without the torch.cuda.Stream object around it (3.3 us a call, 0.1 this way)
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 _poison = os.environ.get("RMM_POISON_OUTPUTS", "0") not in ("", "0")
@@ -153,8 +154,8 @@ def poison_outputs(on: bool) -> None:
     _poison = bool(on)
 
 
-def _out(shape, dtype: torch.dtype, device) -> torch.Tensor:
-    t = torch.empty(shape, dtype=dtype, device=device)
+def _out(shape, dtype: torch.dtype, like: torch.Tensor) -> torch.Tensor:
+    t = like.new_empty(shape, dtype=dtype)
     if _poison:
         t.fill_(float("nan") if dtype.is_floating_point else torch.iinfo(dtype).min)
     return t
@@ -252,8 +253,8 @@ def rmm_score(A: torch.Tensor, axis: int = 1, want_scores: bool = True, want_ene
     ws = workspace(need, A.device) if ws is None else ws
     p, nb = _ws_ptr(ws)
     shape = (m.batch, n) if A.dim() == 3 else (n,)
-    scores = _out(shape, torch.float32, A.device) if want_scores else None
-    energy = _out(shape, torch.float32, A.device) if want_energy else None
+    scores = _out(shape, torch.float32, A) if want_scores else None
+    energy = _out(shape, torch.float32, A) if want_energy else None
     _check(lib().rmm_score(ctypes.byref(m), axis, scores.data_ptr() if want_scores else None,
                            energy.data_ptr() if want_energy else None, p, nb, _stream()))
     return scores, energy
@@ -268,8 +269,8 @@ def rmm_select(keys: torch.Tensor, rho: float = 0.0, k: int = 0, want_retained: 
     kk = int(k) if k > 0 else rmm_keep_count(rho, K)
     ws = workspace(lib().rmm_select_workspace_bytes(batch, K), keys.device) if ws is None else ws
     p, nb = _ws_ptr(ws)
-    idx = _out((batch, kk) if keys.dim() == 2 else (kk,), torch.int32, keys.device)
-    ret = _out((batch,), torch.float32, keys.device) if want_retained else None
+    idx = _out((batch, kk) if keys.dim() == 2 else (kk,), torch.int32, keys)
+    ret = _out((batch,), torch.float32, keys) if want_retained else None
     _check(lib().rmm_select(keys.data_ptr(), batch, K, float(rho), int(k), idx.data_ptr(),
                             ret.data_ptr() if want_retained else None, p, nb, _stream()))
     return (idx, ret) if want_retained else idx
@@ -287,11 +288,11 @@ def rmm_score_select(A: torch.Tensor, rho: float = 0.0, k: int = 0, axis: int = 
     p, nb = _ws_ptr(ws)
     three = A.dim() == 3
     if idx is None:
-        idx = _out((m.batch, kk) if three else (kk,), torch.int32, A.device)
+        idx = _out((m.batch, kk) if three else (kk,), torch.int32, A)
     shape = (m.batch, n) if three else (n,)
-    scores = _out(shape, torch.float32, A.device) if want_scores else None
-    energy = _out(shape, torch.float32, A.device) if want_energy else None
-    ret = _out((m.batch,), torch.float32, A.device) if want_retained else None
+    scores = _out(shape, torch.float32, A) if want_scores else None
+    energy = _out(shape, torch.float32, A) if want_energy else None
+    ret = _out((m.batch,), torch.float32, A) if want_retained else None
     _check(lib().rmm_score_select(ctypes.byref(m), axis, float(rho), int(k), idx.data_ptr(),
                                   scores.data_ptr() if want_scores else None,
                                   energy.data_ptr() if want_energy else None,
@@ -352,13 +353,13 @@ def rmm_reduced_gemm(A: torch.Tensor, B: torch.Tensor, idx: Optional[torch.Tenso
     if out is None:
         dt = out_dtype if out_dtype is not None else A.dtype
         shape = (ma.batch, ma.rows, mb.cols) if A.dim() == 3 else (ma.rows, mb.cols)
-        out = _out(shape, dt, A.device)
+        out = _out(shape, dt, A)
     my = as_mat(out)
     if want_energy:
         need = lib().rmm_reduced_gemm_scored_workspace_bytes(ctypes.byref(ma), ctypes.byref(mb), k, ctypes.byref(my))
         ws = workspace(need, A.device) if ws is None else ws
         p, nb = _ws_ptr(ws)
-        energy = _out((ma.batch, mb.cols) if A.dim() == 3 else (mb.cols,), torch.float32, A.device)
+        energy = _out((ma.batch, mb.cols) if A.dim() == 3 else (mb.cols,), torch.float32, A)
         _check(lib().rmm_reduced_gemm_scored(ctypes.byref(ma), ctypes.byref(mb), idx.data_ptr() if idx is not None else None, k,
                                              float(scale), ctypes.byref(my), energy.data_ptr(), p, nb, _stream()))
         return out, energy
@@ -383,14 +384,14 @@ def rmm_reduced_gemm_q8(A: torch.Tensor, Bq_nk: torch.Tensor, b_scale: float, id
     ma, mb = as_mat(A), as_mat(Bq_nk.t())          # B as a [K, N] matrix whose rows (contraction slices) have stride 1
     k = idx.numel()
     if out is None:
-        out = _out((ma.rows, mb.cols), out_dtype if out_dtype is not None else torch.bfloat16, A.device)
+        out = _out((ma.rows, mb.cols), out_dtype if out_dtype is not None else torch.bfloat16, A)
     my = as_mat(out)
     need = lib().rmm_reduced_gemm_q8_workspace_bytes(ctypes.byref(ma), ctypes.byref(mb), k, ctypes.byref(my))
     if need == 0:
         raise RmmError(RMM_ERR_UNSUPPORTED, lib().rmm_last_error().decode())
     ws = workspace(need, A.device) if ws is None else ws
     p, nb = _ws_ptr(ws)
-    a_scale = _out((ma.rows,), torch.float32, A.device) if want_scales else None
+    a_scale = _out((ma.rows,), torch.float32, A) if want_scales else None
     _check(lib().rmm_reduced_gemm_q8(ctypes.byref(ma), ctypes.byref(mb), float(b_scale), idx.data_ptr(), k, float(scale), ctypes.byref(my),
                                      a_scale.data_ptr() if want_scales else None, p, nb, _stream()))
     return (out, a_scale) if want_scales else out
@@ -406,7 +407,7 @@ def rmm_reduced_attn(Q: torch.Tensor, K: torch.Tensor, V: torch.Tensor, causal: 
             raise RmmError(RMM_ERR_UNSUPPORTED, "Q, K, V must be 4-D bf16 CUDA tensors with a contiguous last dim")
     B, Hq, Lq, Dh = Q.shape
     _, Hkv, Lk, _ = K.shape
-    O = _out((B, Hq, Lq, Dh), torch.bfloat16, Q.device)
+    O = _out((B, Hq, Lq, Dh), torch.bfloat16, Q)
     d = rmm_attn_desc_t(B, Hq, Hkv, Lq, Lk, Dh, int(bool(causal)), float(rho_d), float(rho_t),
                         (ctypes.c_int64 * 3)(*Q.stride()[:3]), (ctypes.c_int64 * 3)(*K.stride()[:3]),
                         (ctypes.c_int64 * 3)(*V.stride()[:3]), (ctypes.c_int64 * 3)(*O.stride()[:3]),
@@ -427,9 +428,9 @@ def rmm_reduced_attn(Q: torch.Tensor, K: torch.Tensor, V: torch.Tensor, causal: 
     p, nb = _ws_ptr(ws)
     idx_feat = idx_tok = None
     if want_idx:
-        idx_feat = _out((B, Hq, rmm_keep_count(rho_d, Dh)), torch.int32, Q.device)
+        idx_feat = _out((B, Hq, rmm_keep_count(rho_d, Dh)), torch.int32, Q)
         if rho_t < 1.0:
-            idx_tok = _out((B, Hq, rmm_keep_count(rho_t, Lk)), torch.int32, Q.device)
+            idx_tok = _out((B, Hq, rmm_keep_count(rho_t, Lk)), torch.int32, Q)
     _check(lib().rmm_reduced_attn(ctypes.byref(d), Q.data_ptr(), K.data_ptr(), V.data_ptr(), O.data_ptr(),
                                   idx_feat.data_ptr() if idx_feat is not None else None,
                                   idx_tok.data_ptr() if idx_tok is not None else None, p, nb, _stream()))
@@ -459,12 +460,12 @@ def rmm_product(A: torch.Tensor, B: torch.Tensor, rho: float = 0.0, k: int = 0, 
     kk = int(k) if k > 0 else rmm_keep_count(rho, ma.cols)
     three = A.dim() == 3
     if out is None:
-        out = _out((ma.batch, ma.rows, mb.cols) if three else (ma.rows, mb.cols), A.dtype, A.device)
+        out = _out((ma.batch, ma.rows, mb.cols) if three else (ma.rows, mb.cols), A.dtype, A)
     if idx is None:
-        idx = _out((ma.batch, kk) if three else (kk,), torch.int32, A.device)
+        idx = _out((ma.batch, kk) if three else (kk,), torch.int32, A)
     elif idx.dtype != torch.int32 or not idx.is_cuda or not idx.is_contiguous() or idx.numel() != ma.batch * kk:
         raise RmmError(RMM_ERR_INVALID_ARG, "idx must be a contiguous int32 CUDA tensor of batch * k elements")
-    ret = _out((ma.batch,), torch.float32, A.device) if want_retained else None
+    ret = _out((ma.batch,), torch.float32, A) if want_retained else None
     my = as_mat(out)
     need = lib().rmm_product_workspace_bytes(ctypes.byref(ma), ctypes.byref(mb), ctypes.byref(my))
     if need == 0:
