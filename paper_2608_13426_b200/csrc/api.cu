@@ -316,9 +316,13 @@ int rmm_reduced_gemm_q8(const rmm_mat_t *A, const rmm_mat_t *B, float b_scale, c
     int *status = &reinterpret_cast<WsHeader *>(w)->status;
     uint8_t *Aq = reinterpret_cast<uint8_t *>(w + q.off_aq), *Bq = reinterpret_cast<uint8_t *>(w + q.off_bq);
     float *row_scale = a_scale != nullptr ? a_scale : reinterpret_cast<float *>(w + q.off_scale);
-    rc = launch_gather_q8(true, A->ptr, A->rows, A->stride_row, A->cols, idx, k, Aq, q.ldq, row_scale, status, st);
-    if (rc != RMM_OK) return rc;
-    rc = launch_gather_q8(false, B->ptr, B->cols, B->stride_col, B->rows, idx, k, Bq, q.ldq, nullptr, status, st);
+    if (gather_q8_streams(A->cols, q.ldq)) {
+        rc = launch_gather_q8_pair(A->ptr, A->rows, A->stride_row * 2, B->ptr, B->cols, B->stride_col, A->cols, idx, k, Aq, Bq, q.ldq, row_scale,
+                                   status, st);
+    } else {
+        rc = launch_gather_q8(true, A->ptr, A->rows, A->stride_row, A->cols, idx, k, Aq, q.ldq, row_scale, status, st);
+        if (rc == RMM_OK) rc = launch_gather_q8(false, B->ptr, B->cols, B->stride_col, B->rows, idx, k, Bq, q.ldq, nullptr, status, st);
+    }
     if (rc != RMM_OK) return rc;
     TcProblem p = {};
     p.batch = 1; p.M = A->rows; p.N = B->cols; p.k = k;

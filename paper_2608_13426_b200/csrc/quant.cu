@@ -4,7 +4,8 @@
 //                only, so the step adapts to what survives the selection; an all-zero row gets s_i = 1)
 //   weight       given as e4m3 codes with one scale for the tensor, stored [N, K] (contraction axis contiguous): the kept
 //                bytes of every row are gathered
-// One block per row: the row is staged in shared memory with 16-byte loads, then gathered (and quantised) from there.
+// Both gathers run as one streaming launch (gather_q8_stream_kernel); operands it does not take (rows above 110 KB, more than
+// 32768 kept columns) as one block per row, the row staged in shared memory with 16-byte loads.
 // Every decision that produces a code is taken in fp32 (IEEE division, round-to-nearest-even conversion, saturating).
 #include <cuda_fp8.h>
 
@@ -84,177 +85,257 @@ __global__ void __launch_bounds__(kThreadsQ) gather_q8_kernel(const void *__rest
 }
 
 
-// The same gather as a streaming kernel: one persistent 1024-thread block per SM owns a contiguous range of rows, which
-// arrive through two shared-memory buffers by bulk asynchronous copies (the next row lands while the current one is
-// worked on).  Thread t owns the output words t, t + 1024, ... (four codes each) and keeps the byte offsets of their
-// source columns in registers for all its rows, so the index list is read once per block instead of once per row.
+// Both gathers of a product as one streaming kernel: one persistent 1024-thread block per SM owns a contiguous range of the
+// rows of A and one of the rows of B, which share the index list.  Rows arrive by bulk asynchronous copies, several at a
+// time (up to 8 rows of up to 4096 kept columns; the next ones land while these are worked on), so that the barriers, the
+// wait and the row maxima's meeting are paid per handful of rows: with one 8 KB row at a time they were most of the time.
+// 4096 x 8192 activations and 8192 x 8192 weights, half kept: 33 + 35 us in two launches of a row at a time, 54 us here,
+// 185 MB.
+//
+// Quotients: a code is e4m3(a / s) with the quotient rounded as IEEE division rounds it.  q = a x (1 / s), both roundings
+// to nearest, is within 3 units in the last place of that quotient, so it yields the same code unless it lies that close to
+// a point where codes change: those sit 20 bits below the leading bit for |q| >= 2^-6 (three mantissa bits, ties), and
+// everything smaller is divided.  Divisions are thus taken for a few elements in 10^4.
 constexpr int kThreadsS = 1024;
-constexpr int kWordsS = 8;                       // output words per thread: k <= 4 * 8 * 1024
+constexpr int kUnitsS = 8;                       // (rows at a time) x (groups of 4096 outputs of a row): k <= 8 * 4096
 constexpr int kStreamMaxRowBytes = 110 * 1024;   // two such rows (and their zero pads) fit in shared memory
-constexpr int kStreamBuffers = 3;                // rows staged at once where three fit (rows up to 73 KB), else two
+constexpr int kStreamStages = 3;
 
-template <bool QUANT>
-__global__ void __launch_bounds__(kThreadsS, 1) gather_q8_stream_kernel(const void *__restrict__ src, int64_t s_row, int K, const int32_t *__restrict__ idx,
-                                                                         int k, uint8_t *__restrict__ dst, int64_t ld_dst, float *__restrict__ row_scale,
-                                                                         int64_t rows, int64_t per_block, int nbuf, int *status, unsigned long long wait_ns)
+struct StreamQ8 {
+    const unsigned char *src[2];   // A (bf16), B (codes)
+    int64_t pitch[2], rows[2], per_block[2];   // bytes between rows; rows; rows per block
+    uint8_t *dst[2];
+    int64_t ld_dst;
+    const int32_t *idx;
+    float *row_scale;
+    int K, k, rows_at_once[2], stages[2];
+    int *status;
+    unsigned long long wait_ns;
+};
+
+__device__ __forceinline__ uint32_t e4m3_code2(float x0, float x1, float step, float inv)
+{
+    auto quotient = [&](float x) -> float {
+        const float q = x * inv;
+        const uint32_t bits = __float_as_uint(q);
+        const bool near_tie = ((bits + 0x80008u) & 0xfffffu) < 16u;              // within 8 of the 20 bits' middle
+        const bool small = (bits & 0x7fffffffu) < 0x3c800000u;                   // |q| < 2^-6
+        return near_tie || small ? __fdiv_rn(x, step) : q;
+    };
+    return __nv_cvt_float2_to_fp8x2(make_float2(quotient(x0), quotient(x1)), __NV_SATFINITE, __NV_E4M3);
+}
+
+// One operand's rows of this block.  `stage` and `parity` run on from one operand to the next.
+template <bool QUANT, int G>
+__device__ __forceinline__ bool stream_rows(const StreamQ8 &a, unsigned char *smem, uint64_t *full, int *abort_flag, unsigned (*s_red)[kThreadsS / 32],
+                                            const uint32_t (&cb)[2 * G], int &turn)
+{
+    using namespace ptx;
+    constexpr int ES = QUANT ? 2 : 1, W = QUANT ? 0 : 1, R = kUnitsS / G;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int at_once = a.rows_at_once[W], nst = a.stages[W];
+    const uint32_t pad = (uint32_t)(a.K + 15) / 16 * 16 * ES, pitch = pad + 16, copied = (uint32_t)(a.K * ES + 15) / 16 * 16;
+    const int64_t lo = (int64_t)blockIdx.x * a.per_block[W], hi = min(a.rows[W], lo + a.per_block[W]);
+    if (lo >= hi) return true;
+    // 16 zero bytes after each staged row: where missing indices point
+    for (int i = tid; i < 4 * nst * at_once; i += kThreadsS) reinterpret_cast<uint32_t *>(smem + (size_t)(i >> 2) * pitch + pad)[i & 3] = 0;
+    __syncthreads();
+    const uint32_t base = smem_u32(smem);
+    // turns of this operand: turn t0 + n uses buffer n % nst; a barrier completes once per use
+    uint32_t parity_of = 0;  // bit b: parity that the next wait on buffer b expects
+#pragma unroll
+    for (int b = 0; b < kStreamStages; ++b) parity_of |= ((uint32_t)(turn >> (8 * b)) & 1u) << b;
+    auto issue = [&](int64_t r, int b) {  // the first warp: rows r .. of one turn, a copy per lane
+        const int n = (int)min((int64_t)at_once, hi - r);
+        if (lane == 0) mbar_arrive_expect_tx(smem_u32(&full[b]), copied * (uint32_t)n);
+        __syncwarp();
+        if (lane < n)
+            asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                         ::"r"(base + (uint32_t)(b * at_once + lane) * pitch), "l"(a.src[W] + (r + lane) * a.pitch[W]), "r"(copied),
+                           "r"(smem_u32(&full[b])) : "memory");
+    };
+    if (warp == 0)
+        for (int b = 0; b < nst && lo + (int64_t)b * at_once < hi; ++b) issue(lo + (int64_t)b * at_once, b);
+    const int words = (int)(a.ld_dst / 4);
+    const int rr = lane & 3, word_in_warp = 8 * rr + (lane >> 2);  // after the transpose lane 4 m + rr holds word 8 rr + m
+    auto offset = [&](int sl) -> uint32_t { return ((cb[sl >> 1] >> (16 * (sl & 1))) & 0xffffu) * ES; };
+    bool ok = true;
+    int b = 0;
+    for (int64_t r = lo; r < hi; r += at_once) {
+        const int n = (int)min((int64_t)at_once, hi - r);
+        const bool landed = mbar_wait(smem_u32(&full[b]), (parity_of >> b) & 1u, abort_flag, a.status, a.wait_ns);
+        if (!__syncthreads_and(landed)) { ok = false; break; }
+        parity_of ^= 1u << b;
+        const unsigned char *rows = smem + (size_t)(b * at_once) * pitch;
+        uint32_t val[R][QUANT ? 2 * G : G];   // this thread's inputs: bf16 pairs, or four bytes to a register
+        [[maybe_unused]] unsigned top[R];
+#pragma unroll
+        for (int q = 0; q < R; ++q) {
+            if (q < n) {
+                const unsigned char *row = rows + (size_t)q * pitch;
+                if constexpr (QUANT) {
+                    float amax = 0.f;
+#pragma unroll
+                    for (int h = 0; h < 2 * G; ++h) {
+                        const uint32_t x0 = *reinterpret_cast<const unsigned short *>(row + offset(2 * h));
+                        const uint32_t x1 = *reinterpret_cast<const unsigned short *>(row + offset(2 * h + 1));
+                        val[q][h] = x0 | (x1 << 16);
+                        amax = fmaxf(amax, fmaxf(fabsf(__uint_as_float(x0 << 16)), fabsf(__uint_as_float(x1 << 16))));
+                    }
+                    top[q] = __reduce_max_sync(0xffffffffu, __float_as_uint(amax));  // non-negative: ordered as its bits are
+                    if (lane == 0) s_red[q][warp] = top[q];
+                } else {
+#pragma unroll
+                    for (int g = 0; g < G; ++g) {
+                        uint32_t word = 0;
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) word |= (uint32_t)row[offset(4 * g + e)] << (8 * e);
+                        val[q][g] = word;
+                    }
+                }
+            }
+        }
+        __syncthreads();
+        // every thread holds what it needs of this buffer: refill it.  (s_red is read before the next turn's barrier and
+        // written after it.)
+        if (warp == 0 && r + (int64_t)nst * at_once < hi) issue(r + (int64_t)nst * at_once, b);
+#pragma unroll
+        for (int q = 0; q < R; ++q) {
+            if (q < n) {
+                float step = 1.f, inv = 1.f;
+                if constexpr (QUANT) {
+                    const float amax = __uint_as_float(__reduce_max_sync(0xffffffffu, s_red[q][lane]));
+                    step = amax > 0.f ? __fdiv_rn(amax, 448.f) : 1.f;
+                    inv = __frcp_rn(step);
+                    if (!(inv < INFINITY) || !(amax < INFINITY)) inv = 0.f;  // every quotient then counts as small: divided
+                    if (tid == 0) a.row_scale[r + q] = step;
+                }
+                uint32_t *drow = reinterpret_cast<uint32_t *>(a.dst[W] + (r + q) * a.ld_dst);
+#pragma unroll
+                for (int g = 0; g < G; ++g) {
+                    uint32_t mine;  // codes of this thread's slots 4 g .. 4 g + 3
+                    if constexpr (QUANT) {
+                        const uint32_t v0 = val[q][2 * g], v1 = val[q][2 * g + 1];
+                        mine = e4m3_code2(__uint_as_float(v0 << 16), __uint_as_float(v0 & 0xffff0000u), step, inv) |
+                               (e4m3_code2(__uint_as_float(v1 << 16), __uint_as_float(v1 & 0xffff0000u), step, inv) << 16);
+                    } else {
+                        mine = val[q][g];
+                    }
+                    // 4 x 4 byte transpose among the four lanes of a quad: lane rr ends up with the word of slot 4 g + rr
+                    uint32_t other = __shfl_xor_sync(0xffffffffu, mine, 1);
+                    mine = (rr & 1) ? __byte_perm(mine, other, 0x3715) : __byte_perm(mine, other, 0x6240);
+                    other = __shfl_xor_sync(0xffffffffu, mine, 2);
+                    mine = (rr & 2) ? __byte_perm(mine, other, 0x3276) : __byte_perm(mine, other, 0x5410);
+                    const int w = (g * (kThreadsS / 32) + warp) * 32 + word_in_warp;
+                    if (w < words) drow[w] = mine;
+                }
+            }
+        }
+        if (++b == nst) b = 0;
+    }
+    turn = 0;
+#pragma unroll
+    for (int s = 0; s < kStreamStages; ++s) turn |= (int)((parity_of >> s) & 1u) << (8 * s);
+    return ok;
+}
+
+// Output j of a row comes from column idx[j].  A warp takes 128 consecutive outputs at a time (group g of the block's
+// 32 x 128): in slot e = 0 .. 3 lane l reads the source of output 32 e + l of them, so the lanes of one instruction read
+// neighbouring kept columns (output words owned whole by a thread made the lanes' reads 16 bytes apart at rho = 1/2:
+// four lanes per bank).  The four bytes of an output word then sit in the four lanes of a quad and are brought together by
+// two shuffle rounds; the warp's 32 words leave as one 128-byte store.  Column numbers (the zero pad: K rounded up to 16)
+// stay in registers for all rows, two to a register.
+template <int G>
+__global__ void __launch_bounds__(kThreadsS, 1) gather_q8_stream_kernel(const __grid_constant__ StreamQ8 a)
 {
     using namespace ptx;
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ uint64_t full[kStreamBuffers];
+    __shared__ uint64_t full[kStreamStages];
     __shared__ int abort_flag;
-    __shared__ float s_red[kThreadsS / 32];
-    constexpr int ES = QUANT ? 2 : 1;
+    __shared__ unsigned s_red[kUnitsS / G][kThreadsS / 32];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const uint32_t row_bytes = (uint32_t)K * ES;           // a multiple of 16
-    const uint32_t pitch = row_bytes + 16;                  // 16 zero bytes after each staged row: where missing indices point
     if (tid == 0) {
-        for (int b = 0; b < kStreamBuffers; ++b) mbar_init(smem_u32(&full[b]), 1);
+        for (int b = 0; b < kStreamStages; ++b) mbar_init(smem_u32(&full[b]), 1);
         abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (tid < 4 * nbuf) reinterpret_cast<uint32_t *>(smem + (size_t)(tid >> 2) * pitch + row_bytes)[tid & 3] = 0;
     __syncthreads();
     pdl_wait();
-    const int64_t lo = (int64_t)blockIdx.x * per_block, hi = min(rows, lo + per_block);
-    auto issue = [&](int64_t r, int stage) {  // thread 0: one row, global -> shared
-        const unsigned char *g = static_cast<const unsigned char *>(src) + r * s_row * ES;
-        const uint32_t bar = smem_u32(&full[stage]), d = smem_u32(smem) + (uint32_t)stage * pitch;
-        mbar_arrive_expect_tx(bar, row_bytes);
-        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                     ::"r"(d), "l"(g), "r"(row_bytes), "r"(bar) : "memory");
-    };
-    if (tid == 0)
-        for (int b = 0; b < nbuf && lo + b < hi; ++b) issue(lo + b, b);
-    // Output j of a row comes from column idx[j].  A warp takes 128 consecutive outputs at a time (group g of the block's
-    // 32 x 128): in slot e = 0 .. 3 lane l reads the source of output 32 e + l of them, so the lanes of one instruction read
-    // neighbouring kept columns (output words owned whole by a thread made the lanes' reads 16 bytes apart at rho = 1/2:
-    // four lanes per bank).  The four bytes of an output word then sit in the four lanes of a quad and are brought
-    // together by two shuffle rounds; the warp's 32 words leave as one 128-byte store.
-    // Column numbers (column K = the zero pad): bf16 rows hold at most 55 K columns, so two share a register; byte rows
-    // keep one per register.
-    constexpr int kSlots = 4 * kWordsS;
-    constexpr int kRegs = QUANT ? kSlots / 2 : kSlots;
-    uint32_t cb[kRegs];
-    const int words = (int)(ld_dst / 4);
+    uint32_t cb[2 * G];
 #pragma unroll
-    for (int sl = 0; sl < kSlots; ++sl) {
+    for (int sl = 0; sl < 4 * G; ++sl) {
         const int j = ((sl >> 2) * (kThreadsS / 32) + warp) * 128 + 32 * (sl & 3) + lane;
-        uint32_t col = (uint32_t)K;
-        if (j < k) {
-            const int c = __ldg(idx + j);
-            if (c < 0 || c >= K) atomicExch(status, (int)RMM_ERR_BOUNDS);
+        uint32_t col = (uint32_t)(a.K + 15) / 16 * 16;
+        if (j < a.k) {
+            const int c = __ldg(a.idx + j);
+            if (c < 0 || c >= a.K) atomicExch(a.status, (int)RMM_ERR_BOUNDS);
             else col = (uint32_t)c;
         }
-        if constexpr (QUANT) {
-            if (sl & 1) cb[sl >> 1] |= col << 16;
-            else cb[sl >> 1] = col;
-        } else {
-            cb[sl] = col;
-        }
+        if (sl & 1) cb[sl >> 1] |= col << 16;
+        else cb[sl >> 1] = col;
     }
-    auto offset = [&](int sl) -> uint32_t {  // byte offset of the source of slot sl inside the staged row
-        if constexpr (QUANT) return ((cb[sl >> 1] >> (16 * (sl & 1))) & 0xffffu) * 2u;
-        else return cb[sl];
-    };
-    const int groups = (int)((ld_dst + 4095) / 4096);  // groups of 4096 outputs (32 warps x 128) that hold any
-    const int rr = lane & 3, word_in_warp = 8 * rr + (lane >> 2);  // after the transpose lane 4 m + rr holds word 8 rr + m
-    int stage = 0;
-    uint32_t parity = 0;
-    for (int64_t r = lo; r < hi; ++r) {
-        const bool landed = mbar_wait(smem_u32(&full[stage]), parity, &abort_flag, status, wait_ns);
-        if (!__syncthreads_and(landed)) break;
-        const unsigned char *row = smem + (size_t)stage * pitch;
-        // this thread's 32 inputs, read once: bf16 pairs (QUANT) or the bytes themselves, four to a register
-        uint32_t val[QUANT ? kSlots / 2 : kSlots / 4];
-        float step = 1.f;
-        if constexpr (QUANT) {
-            float amax = 0.f;
-#pragma unroll
-            for (int h = 0; h < kSlots / 2; ++h) {
-                if ((h >> 1) < groups) {  // (block-uniform: groups of 4096 outputs past k hold nothing)
-                    const uint32_t x0 = *reinterpret_cast<const unsigned short *>(row + offset(2 * h));
-                    const uint32_t x1 = *reinterpret_cast<const unsigned short *>(row + offset(2 * h + 1));
-                    val[h] = x0 | (x1 << 16);
-                    amax = fmaxf(amax, fmaxf(fabsf(__uint_as_float(x0 << 16)), fabsf(__uint_as_float(x1 << 16))));
-                }
-            }
-#pragma unroll
-            for (int d = 16; d > 0; d >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, d));
-            if (lane == 0) s_red[warp] = amax;
-            __syncthreads();
-            amax = s_red[lane];
-#pragma unroll
-            for (int d = 16; d > 0; d >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, d));
-            step = amax > 0.f ? __fdiv_rn(amax, 448.f) : 1.f;
-            if (tid == 0) row_scale[r] = step;
-        } else {
-#pragma unroll
-            for (int g = 0; g < kSlots / 4; ++g) {
-                if (g < groups) {
-                    uint32_t word = 0;
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) word |= (uint32_t)row[offset(4 * g + e)] << (8 * e);
-                    val[g] = word;
-                }
-            }
-            __syncthreads();
-        }
-        // every thread holds what it needs of this buffer (the barrier above): refill it with the row nbuf ahead.  (With
-        // rows quantised, s_red is read before the next iteration's barrier and written after it.)
-        if (tid == 0 && r + nbuf < hi) issue(r + nbuf, stage);
-        uint32_t *drow = reinterpret_cast<uint32_t *>(dst + r * ld_dst);
-#pragma unroll
-        for (int g = 0; g < kSlots / 4; ++g) {
-            if (g >= groups) break;
-            uint32_t mine;  // codes of this thread's slots 4 g .. 4 g + 3
-            if constexpr (QUANT) {
-                // slots 4 g .. 4 g + 3 are val[2 g] (low, high half) and val[2 g + 1]; two codes per conversion
-                const float x0 = __uint_as_float(val[2 * g] << 16), x1 = __uint_as_float(val[2 * g] & 0xffff0000u);
-                const float x2 = __uint_as_float(val[2 * g + 1] << 16), x3 = __uint_as_float(val[2 * g + 1] & 0xffff0000u);
-                const uint32_t lo2 = __nv_cvt_float2_to_fp8x2(make_float2(__fdiv_rn(x0, step), __fdiv_rn(x1, step)), __NV_SATFINITE, __NV_E4M3);
-                const uint32_t hi2 = __nv_cvt_float2_to_fp8x2(make_float2(__fdiv_rn(x2, step), __fdiv_rn(x3, step)), __NV_SATFINITE, __NV_E4M3);
-                mine = lo2 | (hi2 << 16);
-            } else {
-                mine = val[g];
-            }
-            // 4 x 4 byte transpose among the four lanes of a quad: lane rr ends up with the word of slot 4 g + rr
-            uint32_t other = __shfl_xor_sync(0xffffffffu, mine, 1);
-            mine = (rr & 1) ? __byte_perm(mine, other, 0x3715) : __byte_perm(mine, other, 0x6240);
-            other = __shfl_xor_sync(0xffffffffu, mine, 2);
-            mine = (rr & 2) ? __byte_perm(mine, other, 0x3276) : __byte_perm(mine, other, 0x5410);
-            const int w = (g * (kThreadsS / 32) + warp) * 32 + word_in_warp;
-            if (w < words) drow[w] = mine;
-        }
-        if (++stage == nbuf) { stage = 0; parity ^= 1u; }
+    int turn = 0;
+    if (stream_rows<true, G>(a, smem, full, &abort_flag, s_red, cb, turn)) {
+        __syncthreads();
+        stream_rows<false, G>(a, smem, full, &abort_flag, s_red, cb, turn);
     }
 }
 
 }  // namespace
 
+bool gather_q8_streams(int64_t K, int64_t ld_dst)
+{
+    return K <= 65520 && (K + 15) / 16 * 32 + 16 <= kStreamMaxRowBytes && ld_dst <= 4096 * kUnitsS;
+}
+
+int launch_gather_q8_pair(const void *A, int64_t a_rows, int64_t a_pitch, const void *B, int64_t b_rows, int64_t b_pitch, int64_t K,
+                          const int32_t *idx, int64_t k, uint8_t *Aq, uint8_t *Bq, int64_t ld_dst, float *row_scale, int *status,
+                          cudaStream_t stream)
+{
+    StreamQ8 a = {};
+    a.src[0] = static_cast<const unsigned char *>(A); a.src[1] = static_cast<const unsigned char *>(B);
+    a.pitch[0] = a_pitch; a.pitch[1] = b_pitch;
+    a.rows[0] = a_rows; a.rows[1] = b_rows;
+    a.dst[0] = Aq; a.dst[1] = Bq;
+    a.ld_dst = ld_dst; a.idx = idx; a.row_scale = row_scale;
+    a.K = (int)K; a.k = (int)k;
+    a.status = status;
+    a.wait_ns = wait_limit_ns();
+    const int64_t groups = ceil_div(ld_dst, 4096);
+    const int g = groups <= 1 ? 1 : (groups <= 2 ? 2 : (groups <= 4 ? 4 : 8));
+    int64_t blocks = 0;
+    size_t smem = 0;
+    for (int w = 0; w < 2; ++w) {
+        const size_t pitch = (size_t)(K + 15) / 16 * 16 * (w == 0 ? 2 : 1) + 16, room = 2 * (size_t)(kStreamMaxRowBytes + 16);
+        a.per_block[w] = ceil_div(a.rows[w], sm_count());
+        // as many rows at a time as the registers hold, three buffers of them where they fit, no more than a block has
+        int64_t n = kUnitsS / g;
+        while (n > 1 && (kStreamStages * n * pitch > room || n > a.per_block[w])) n /= 2;
+        a.rows_at_once[w] = (int)n;
+        a.stages[w] = kStreamStages * n * pitch <= room ? kStreamStages : 2;
+        if (a.stages[w] * n * pitch > smem) smem = a.stages[w] * n * pitch;
+        const int64_t nb = ceil_div(a.rows[w], a.per_block[w]);
+        if (nb > blocks) blocks = nb;
+    }
+    auto kern = g == 1 ? gather_q8_stream_kernel<1> : (g == 2 ? gather_q8_stream_kernel<2> : (g == 4 ? gather_q8_stream_kernel<4> : gather_q8_stream_kernel<8>));
+    static PerDeviceOnce configured;
+    if (configured.first()) {
+        const int most = 2 * (kStreamMaxRowBytes + 16);
+        cudaError_t e = cudaFuncSetAttribute(gather_q8_stream_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(gather_q8_stream_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(gather_q8_stream_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(gather_q8_stream_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+        if (e != cudaSuccess) return fail(RMM_ERR_CUDA, "gather_q8: cudaFuncSetAttribute: %s", cudaGetErrorString(e));
+    }
+    prof_begin("gather_q8_stream_kernel", stream);
+    launch_kernel(kern, dim3((unsigned)blocks), dim3(kThreadsS), smem, stream, 1, a);
+    return check_launch("gather_q8_stream_kernel", stream);
+}
+
 int launch_gather_q8(bool quantise, const void *src, int64_t rows, int64_t s_row, int64_t K, const int32_t *idx, int64_t k, uint8_t *dst,
                      int64_t ld_dst, float *row_scale, int *status, cudaStream_t stream)
 {
     const size_t row_bytes = (size_t)K * (quantise ? 2 : 1);
-    if (row_bytes % 16 == 0 && row_bytes <= (size_t)kStreamMaxRowBytes && ld_dst <= 4 * kWordsS * kThreadsS && rows >= 32 * (int64_t)sm_count()) {  // (few rows: one block per row keeps every SM busy)
-        static PerDeviceOnce stream_configured;
-        if (stream_configured.first()) {
-            cudaError_t e = cudaFuncSetAttribute(gather_q8_stream_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * (kStreamMaxRowBytes + 16));
-            if (e == cudaSuccess)
-                e = cudaFuncSetAttribute(gather_q8_stream_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * (kStreamMaxRowBytes + 16));
-            if (e != cudaSuccess) return fail(RMM_ERR_CUDA, "gather_q8: cudaFuncSetAttribute: %s", cudaGetErrorString(e));
-        }
-        const int64_t per_block = ceil_div(rows, sm_count());
-        const unsigned grid = (unsigned)ceil_div(rows, per_block);
-        const int nbuf = kStreamBuffers * (row_bytes + 16) <= 2 * (size_t)(kStreamMaxRowBytes + 16) ? kStreamBuffers : 2;
-        prof_begin("gather_q8_stream_kernel", stream);
-        if (quantise)
-            launch_kernel(gather_q8_stream_kernel<true>, dim3(grid), dim3(kThreadsS), nbuf * (row_bytes + 16), stream, 1, src, s_row, (int)K, idx,
-                          (int)k, dst, ld_dst, row_scale, rows, per_block, nbuf, status, wait_limit_ns());
-        else
-            launch_kernel(gather_q8_stream_kernel<false>, dim3(grid), dim3(kThreadsS), nbuf * (row_bytes + 16), stream, 1, src, s_row, (int)K, idx,
-                          (int)k, dst, ld_dst, row_scale, rows, per_block, nbuf, status, wait_limit_ns());
-        return check_launch("gather_q8_stream_kernel", stream);
-    }
     const size_t smem = align_up(row_bytes, 16);
     if (smem > 200 * 1024 || K > INT32_MAX / 4 || rows > INT32_MAX) return fail(RMM_ERR_UNSUPPORTED, "gather_q8: row too long");
     static PerDeviceOnce configured;
