@@ -93,8 +93,8 @@ struct FusedArgs {
 // share the answer): hides it all (the tile is skipped like one beyond the causal diagonal), leaves it alone (the
 // ordinary softmax step), or has to be added.  Padding, causal, block and window masks are nearly all of the first
 // two kinds, and the additions were what bound the masked kernel: each thread reads its own row of the mask, 32 rows a
-// load.  2 sequences x 16 heads x 2048 x 128, padded: 2 x 244 us with every tile added, 80 us in one launch with this
-// pass (6 us) in front; a mask whose every value is added: 254 -> 224 us on 16 heads x 2048 (one launch for all sequences).
+// load.  2 sequences x 16 heads x 2048 x 128, padded: 2 x 244 us with every tile added, 52 us in one launch with this
+// pass (6 us) in front; a mask whose every value is added: 254 -> 136 us a call on 16 heads x 2048.
 // Bound by reading the mask once; a warp stops reading a tile once it knows that its values have to be added.
 // A value counts as hiding when mask x sqrt(Dh) is -inf in fp32, which is what the softmax step would make of it.
 enum { TILE_HIDDEN = 0, TILE_CLEAR = 1, TILE_ADD = 2 };
@@ -259,27 +259,39 @@ fused_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         else if (e1 <= b1) { *jb = b0; *je = e0; }
         else { *jb = min(b0, b1); *je = max(e0, e1); }
     };
-    // MASK: the next tile >= j, before je, that is not hidden from the rows of group g (both groups: g < 0), else je
-    auto kinds_of = [&](int64_t head, int64_t row) -> const uint8_t * {
-        const int64_t plane = (head / a.mask.seq_heads) * a.mask.plane_step + (head % a.mask.seq_heads) % a.mask.plane_heads;
-        return a.tile_kind + (plane * a.kind_rb + row / FM) * a.kind_ld;
-    };
-    auto next_tile = [&](int64_t head, int64_t r0, int g, int j, int je) -> int {
-        if constexpr (!MASK) return j;
-        const uint8_t *k0 = kinds_of(head, r0 + (g < 0 ? 0 : g) * FM);
-        while (j < je) {
-            unsigned long long u = __ldg(reinterpret_cast<const unsigned long long *>(k0 + (j & ~7)));
-            if (g < 0) {  // tiles past a group's causal range are hidden in its list
-                u |= __ldg(reinterpret_cast<const unsigned long long *>(k0 + a.kind_ld + (j & ~7)));
+    // MASK: the tiles that are not hidden from the rows of one group, or of both (tiles past a group's causal range are hidden
+    // in its list).  Eight tiles' kinds are held at a time, so a step costs a load only every eight tiles.
+    struct Tiles {
+        const uint8_t *k0, *k1;     // kinds of the group, and of the other one or NULL
+        int at;                     // tiles 8 at .. 8 at + 7 are in `w`
+        unsigned long long w;
+        __device__ __forceinline__ int next(int j, int je)  // the first tile from j on, before je, that is not hidden, else je
+        {
+            if constexpr (MASK) {
+                for (; j < je; j = (j | 7) + 1) {
+                    if ((j >> 3) != at) {
+                        at = j >> 3;
+                        w = __ldg(reinterpret_cast<const unsigned long long *>(k0) + at);
+                        if (k1 != nullptr) w |= __ldg(reinterpret_cast<const unsigned long long *>(k1) + at);
+                    }
+                    const unsigned long long u = w >> (8 * (j & 7));
+                    if (u != 0) return min(j + ((__ffsll((long long)u) - 1) >> 3), je);
+                }
+                return je;
+            } else {
+                return j;
             }
-            u >>= 8 * (j & 7);
-            if (u != 0) {
-                const int at = j + ((__ffsll((long long)u) - 1) >> 3);
-                return at < je ? at : je;
-            }
-            j = (j | 7) + 1;
         }
-        return je;
+        __device__ __forceinline__ bool add(int j) const { return ((w >> (8 * (j & 7))) & 0xffu) == TILE_ADD; }  // j = the last next()
+    };
+    auto tiles_of = [&](int64_t head, int64_t row, bool both) -> Tiles {
+        Tiles t = {nullptr, nullptr, -1, 0ull};
+        if constexpr (MASK) {
+            const int64_t plane = (head / a.mask.seq_heads) * a.mask.plane_step + (head % a.mask.seq_heads) % a.mask.plane_heads;
+            t.k0 = a.tile_kind + (plane * a.kind_rb + row / FM) * a.kind_ld;
+            if (both) t.k1 = t.k0 + a.kind_ld;
+        }
+        return t;
     };
     // The n-th item of this block: heaviest row blocks first (the last ones when causal; in ENERGY mode, where early
     // keys are seen by most queries, the first ones), and the direction alternates from round to round, so that the
@@ -316,7 +328,8 @@ fused_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             if (!item_of(n, &head, &r0)) continue;
             int jb, je;
             block_range(head, r0, &jb, &je);
-            jb = next_tile(head, r0, -1, jb, je);
+            Tiles tiles = tiles_of(head, r0, true);
+            jb = tiles.next(jb, je);
             if (je <= jb) continue;
             const int vb = (int)((head + a.v_off) / a.v_div);
             if (!mbar_wait_sleepy(q_empty, (n_item & 1u) ^ 1u, abort_flag, a.status, a.wait_ns)) { ok = false; break; }
@@ -326,7 +339,7 @@ fused_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                     tma_load_3d(base + kOffQ + g * kQTile + c * kQChunk, &map_q, c * 64, (int)(r0 + g * FM), (int)head, q_full);
             ok = load_kv(&map_k, kq, (int64_t)jb * FN, (int)head);
             for (int j = jb, nj; j < je && ok; j = nj) {
-                nj = next_tile(head, r0, -1, j + 1, je);
+                nj = tiles.next(j + 1, je);
                 if (nj < je) ok = load_kv(&map_k, kq, (int64_t)nj * FN, (int)head);
                 if constexpr (kHasV) {
                     if (ok) ok = load_kv(&map_v, nv, (int64_t)j * FN, vb);
@@ -385,16 +398,17 @@ fused_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             if (!item_of(n, &head, &r0)) continue;
             int jb, je;
             block_range(head, r0, &jb, &je);
-            jb = next_tile(head, r0, -1, jb, je);
+            Tiles tiles = tiles_of(head, r0, true), own = tiles_of(head, r0 + g * FM, false);
+            jb = tiles.next(jb, je);
             if (je <= jb) continue;
             tile_range(head, r0 + g * FM, &gb, &ge);
-            gn = gb = next_tile(head, r0, g, gb, ge);
+            gn = gb = own.next(gb, ge);
             if (!mbar_wait(q_full, n_item & 1u, abort_flag, a.status, a.wait_ns)) { ok = false; break; }
             ok = step_s(jb);
             for (int j = jb, nj; j < je && ok; j = nj) {
-                nj = next_tile(head, r0, -1, j + 1, je);
+                nj = tiles.next(j + 1, je);
                 const bool use = MASK ? j == gn && gn < ge : (j >= gb && j < ge);  // this group needs the tile
-                if (MASK && use) gn = next_tile(head, r0, g, j + 1, ge);
+                if (MASK && use) gn = own.next(j + 1, ge);
                 const bool last_use = MASK ? gn >= ge : j == ge - 1;
                 if (nj < je) ok = step_s(nj);                              // S~ of the next tile runs ahead of this P V
                 if (!ok) break;
@@ -451,9 +465,10 @@ fused_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             if (r0 >= a.Lr) continue;                  // this group has no rows in the last block
             int jb, je;
             tile_range(head, r0, &jb, &je);
-            jb = next_tile(head, r0, 0, jb, je);
-            const int64_t i = r0 + r;                  // this thread's row
-            __nv_bfloat16 *orow = a.O + head * a.o_sh + i * a.o_sr;
+            Tiles tiles = tiles_of(head, r0, false);
+            jb = tiles.next(jb, je);
+            const int i = (int)r0 + r;                 // this thread's row (rows, columns and their sums stay below 2^31)
+            __nv_bfloat16 *orow = a.O + head * a.o_sh + (int64_t)i * a.o_sr;
             if (je <= jb) {  // nothing visible for any row of this group
                 if constexpr (kHasV) {
                     if (i < a.Lr)
@@ -466,11 +481,11 @@ fused_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                 continue;
             }
             // columns this row sees: [first_col, last_col]
-            int64_t first_col = 0, last_col = a.Lc - 1;
+            int first_col = 0, last_col = (int)a.Lc - 1;
             if (a.causal) {
-                if constexpr (MODE == MODE_ENERGY) first_col = max((int64_t)0, i - a.diag);
-                else if constexpr (MODE == MODE_GATHERED) last_col = kept_upto(a.tok + head * a.Lc, i + a.diag) - 1;
-                else last_col = min(a.Lc - 1, i + a.diag);
+                if constexpr (MODE == MODE_ENERGY) first_col = max(0, i - (int)a.diag);
+                else if constexpr (MODE == MODE_GATHERED) last_col = (int)kept_upto(a.tok + head * a.Lc, i + a.diag) - 1;
+                else last_col = min((int)a.Lc - 1, i + (int)a.diag);
             }
             float m = -INFINITY, l = 0.f;  // FULL / STATS: the maximum that p is taken against (log2 domain), the row sum
             float row_lse = 0.f;           // GATHERED: this row's normaliser
@@ -478,15 +493,11 @@ fused_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
 
             // 64 logits of the current tile (columns c_off .. c_off + 63) into registers; hidden columns become -inf on
             // boundary tiles (the diagonal and the ragged end)
-            [[maybe_unused]] bool add_mask = false;  // MASK: the mask has to be added to the current tile
             auto load_chunk = [&](int j, int c_off, uint32_t (&v0)[32], uint32_t (&v1)[32]) {
                 tmem_ld32_issue(t_s + c_off, v0);
                 tmem_ld32_issue(t_s + c_off + 32, v1);
                 tmem_ld_wait();
-                const int64_t c0 = (int64_t)j * FN + c_off;
-                const int64_t rel_hi = last_col - c0, rel_lo = first_col - c0;
-                const int hi = rel_hi > 63 ? 63 : (rel_hi < -1 ? -1 : (int)rel_hi);
-                const int lo = rel_lo < 0 ? 0 : (rel_lo > 64 ? 64 : (int)rel_lo);
+                const int c0 = j * FN + c_off, hi = max(-1, min(63, last_col - c0)), lo = MODE == MODE_ENERGY ? max(0, min(64, first_col - c0)) : 0;
                 if (!__all_sync(0xffffffffu, hi >= 63 && lo <= 0)) {
 #pragma unroll
                     for (int e = 0; e < 32; ++e) {
@@ -494,34 +505,35 @@ fused_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                         if (e + 32 > hi || e + 32 < lo) v1[e] = 0xff800000u;
                     }
                 }
-                if constexpr (MASK) {
-                    // the caller's additive mask for this row's 64 columns (-inf hides a key); rows past the end and
-                    // columns past the last key read nothing
-                    if (add_mask && i < a.Lr) {
-                        const float *mrow = a.mask.p + (head / a.mask.seq_heads) * a.mask.sb + (head % a.mask.seq_heads) * a.mask.sh + i * a.mask.sr + c0;
-                        const float gain = a.mask_gain;
-                        auto add4 = [&](uint32_t (&v)[32], int e, int col) {
-                            float4 m4;
-                            if (a.mask.vec && c0 + col + 3 < a.Lc) {
-                                m4 = __ldg(reinterpret_cast<const float4 *>(mrow + col));
-                            } else {
-                                m4.x = c0 + col < a.Lc ? __ldg(mrow + col) : 0.f;
-                                m4.y = c0 + col + 1 < a.Lc ? __ldg(mrow + col + 1) : 0.f;
-                                m4.z = c0 + col + 2 < a.Lc ? __ldg(mrow + col + 2) : 0.f;
-                                m4.w = c0 + col + 3 < a.Lc ? __ldg(mrow + col + 3) : 0.f;
-                            }
-                            v[e] = __float_as_uint(fmaf(m4.x, gain, __uint_as_float(v[e])));
-                            v[e + 1] = __float_as_uint(fmaf(m4.y, gain, __uint_as_float(v[e + 1])));
-                            v[e + 2] = __float_as_uint(fmaf(m4.z, gain, __uint_as_float(v[e + 2])));
-                            v[e + 3] = __float_as_uint(fmaf(m4.w, gain, __uint_as_float(v[e + 3])));
-                        };
+            };
+            // MASK: the caller's additive mask (-inf hides a key) added to this warp's rows of the S~ tile where they lie, 16
+            // columns at a time, so that the steps above hold no mask values in registers; rows past the end and columns
+            // past the last key read nothing
+            [[maybe_unused]] auto add_mask_tile = [&](int j) {
+                const int64_t c0 = (int64_t)j * FN;
+                const float *mrow = a.mask.p + (head / a.mask.seq_heads) * a.mask.sb + (head % a.mask.seq_heads) * a.mask.sh + (int64_t)i * a.mask.sr + c0;
+                const float gain = a.mask_gain;
+#pragma unroll 1
+                for (int c = 0; c < FN; c += 16) {
+                    float m4[16];
+                    if (i < a.Lr && a.mask.vec && c0 + c + 15 < a.Lc) {
 #pragma unroll
-                        for (int e = 0; e < 32; e += 4) {
-                            add4(v0, e, e);
-                            add4(v1, e, e + 32);
+                        for (int v = 0; v < 4; ++v) {
+                            const float4 q = __ldg(reinterpret_cast<const float4 *>(mrow + c) + v);
+                            m4[4 * v] = q.x; m4[4 * v + 1] = q.y; m4[4 * v + 2] = q.z; m4[4 * v + 3] = q.w;
                         }
+                    } else {
+#pragma unroll
+                        for (int e = 0; e < 16; ++e) m4[e] = i < a.Lr && c0 + c + e < a.Lc ? __ldg(mrow + c + e) : 0.f;
                     }
+                    uint32_t s16[16];
+                    tmem_ld16_issue(t_s + c, s16);
+                    tmem_ld_wait();
+#pragma unroll
+                    for (int e = 0; e < 16; ++e) s16[e] = __float_as_uint(fmaf(m4[e], gain, __uint_as_float(s16[e])));
+                    tmem_st16_issue(t_s + c, s16);
                 }
+                tmem_st_wait();
             };
             auto release_s = [&]() {  // this warp holds what it needs of the S~ tile
                 tc_fence_before();
@@ -582,8 +594,9 @@ fused_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                 return alpha;
             };
 
-            for (int j = jb; j < je; j = next_tile(head, r0, 0, j + 1, je), ++s_it) {
-                if constexpr (MASK) add_mask = __ldg(kinds_of(head, r0) + j) == TILE_ADD;
+            for (int j = jb, nj; j < je; j = nj, ++s_it) {
+                [[maybe_unused]] const bool add_mask = MASK && tiles.add(j);
+                nj = tiles.next(j + 1, je);
                 if constexpr (MODE == MODE_ENERGY) {
                     // the 128 normalisers of the next tile (512 bytes, the same for every thread) are pulled into L1
                     // one step ahead; the first tile's are fetched cold
@@ -595,6 +608,9 @@ fused_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                 if (!mbar_wait(s_full(g, 0), s_it & 1u, abort_flag, a.status, a.wait_ns)) { ok = false; break; }
                 ASTAMP(0);
                 tc_fence_after();
+                if constexpr (MASK) {
+                    if (add_mask) add_mask_tile(j);
+                }
                 uint32_t v0[32], v1[32];
 
                 if constexpr (MODE == MODE_ENERGY) {
