@@ -75,7 +75,7 @@ struct FusedArgs {
     int64_t v_off, v_div;        // V batch entry of head h = (h + v_off) / v_div
     __nv_bfloat16 *O;
     int64_t o_sh, o_sr;          // element strides of O: head, row
-    float *lse;                  // [heads, lse_ld] log2-domain normalisers: written by STATS, read by ENERGY / GATHERED
+    float *lse;                  // [heads, lse_ld] negated log2-domain normalisers: written by STATS, read by ENERGY / GATHERED
     int64_t lse_ld;              // multiple of 64, >= Lq
     float *energy;               // ENERGY: [heads, Lr] squared token scores
     const int32_t *tok;          // GATHERED: [heads, Lc] kept key positions, ascending
@@ -474,7 +474,7 @@ fused_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                     if (i < a.Lr)
                         for (int c = 0; c < a.Dh; c += 8) *reinterpret_cast<uint4 *>(orow + c) = make_uint4(0, 0, 0, 0);
                 } else if constexpr (MODE == MODE_STATS) {
-                    if (i < a.lse_ld) a.lse[head * a.lse_ld + i] = INFINITY;  // 2^(x - inf) = 0 for every later use
+                    if (i < a.lse_ld) a.lse[head * a.lse_ld + i] = -INFINITY;  // 2^(x - inf) = 0 for every later use
                 } else {
                     if (i < a.Lr) a.energy[head * a.Lr + i] = 0.f;
                 }
@@ -488,8 +488,8 @@ fused_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                 else last_col = min((int)a.Lc - 1, i + (int)a.diag);
             }
             float m = -INFINITY, l = 0.f;  // FULL / STATS: the maximum that p is taken against (log2 domain), the row sum
-            float row_lse = 0.f;           // GATHERED: this row's normaliser
-            if constexpr (MODE == MODE_GATHERED) row_lse = i < a.lse_ld ? a.lse[head * a.lse_ld + i] : INFINITY;
+            float neg_lse = 0.f;           // GATHERED: this row's negated normaliser
+            if constexpr (MODE == MODE_GATHERED) neg_lse = i < a.lse_ld ? a.lse[head * a.lse_ld + i] : -INFINITY;
 
             // 64 logits of the current tile (columns c_off .. c_off + 63) into registers; hidden columns become -inf on
             // boundary tiles (the diagonal and the ragged end)
@@ -614,32 +614,34 @@ fused_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                 uint32_t v0[32], v1[32];
 
                 if constexpr (MODE == MODE_ENERGY) {
-                    // p = bf16(2^(x - lse_i)); this key's score accumulates p^2 over the tile's 128 queries
-                    float acc0 = 0.f, acc1 = 0.f;
+                    // p = bf16(2^(x - lse_i)); this key's score accumulates p^2 over the tile's 128 queries, queries of even
+                    // and of odd number apart (the two halves of the packed fp32 operations: 3.5 instructions a logit where
+                    // single ones took 4.5; 148 against 154 us on 8 heads x 8000)
+                    uint64_t acc = 0;
                     for (int c_off = 0; c_off < FN; c_off += 64) {
-                        float4 cl[16];  // the normalisers of these 64 queries (the same for every thread)
-                        const float4 *lp = reinterpret_cast<const float4 *>(a.lse + head * a.lse_ld + (int64_t)j * FN + c_off);
+                        ulonglong2 cl[16];  // the negated normalisers of these 64 queries (the same for every thread), in pairs
+                        const ulonglong2 *lp = reinterpret_cast<const ulonglong2 *>(a.lse + head * a.lse_ld + (int64_t)j * FN + c_off);
 #pragma unroll
-                        for (int u = 0; u < 16; ++u) cl[u] = (int64_t)j * FN + c_off + 4 * u < a.lse_ld ? __ldg(lp + u) : make_float4(0.f, 0.f, 0.f, 0.f);
+                        for (int u = 0; u < 16; ++u) cl[u] = (int64_t)j * FN + c_off + 4 * u < a.lse_ld ? __ldg(lp + u) : make_ulonglong2(0, 0);
                         load_chunk(j, c_off, v0, v1);
                         if (c_off == 64) release_s();
                         auto fold = [&](const uint32_t (&v)[32], int c) {
 #pragma unroll
-                            for (int e = 0; e < 32; e += 4) {
-                                const float4 ls = cl[(c + e) >> 2];
-                                const float p0 = ex2(fmaf(__uint_as_float(v[e]), c2, -ls.x)), p1 = ex2(fmaf(__uint_as_float(v[e + 1]), c2, -ls.y));
-                                const float p2 = ex2(fmaf(__uint_as_float(v[e + 2]), c2, -ls.z)), p3 = ex2(fmaf(__uint_as_float(v[e + 3]), c2, -ls.w));
-                                const float2 ra = __bfloat1622float2(__floats2bfloat162_rn(p0, p1));
-                                const float2 rb = __bfloat1622float2(__floats2bfloat162_rn(p2, p3));
-                                acc0 = fmaf(ra.x, ra.x, acc0);
-                                acc1 = fmaf(ra.y, ra.y, acc1);
-                                acc0 = fmaf(rb.x, rb.x, acc0);
-                                acc1 = fmaf(rb.y, rb.y, acc1);
+                            for (int e = 0; e < 32; e += 2) {
+                                const ulonglong2 ls = cl[(c + e) >> 2];
+                                float x0, x1;
+                                unpack2(ffma2(pack2(__uint_as_float(v[e]), __uint_as_float(v[e + 1])), c22, e & 2 ? ls.y : ls.x), x0, x1);
+                                const __nv_bfloat162 h = __floats2bfloat162_rn(ex2(x0), ex2(x1));
+                                const uint32_t hw = *reinterpret_cast<const uint32_t *>(&h);
+                                const uint64_t p2 = pack2(__uint_as_float(hw << 16), __uint_as_float(hw & 0xffff0000u));
+                                acc = ffma2(p2, p2, acc);
                             }
                         };
                         fold(v0, 0);
                         fold(v1, 32);
                     }
+                    float acc0, acc1;
+                    unpack2(acc, acc0, acc1);
                     l += acc0 + acc1;
                     continue;
                 }
@@ -659,7 +661,7 @@ fused_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
 
                 uint32_t w[kHasV ? 32 : 1];
                 if constexpr (MODE == MODE_GATHERED) {
-                    const float neg_m = -row_lse;   // +inf normaliser (row sees nothing): p = 0
+                    const float neg_m = neg_lse;   // -inf (row sees nothing): p = 0
                     load_chunk(j, 0, v0, v1);
                     emit_chunk(v0, v1, neg_m, w);
                     if (!mbar_wait(p_empty(g), (p_it & 1u) ^ 1u, abort_flag, a.status, a.wait_ns)) { ok = false; break; }
@@ -712,7 +714,7 @@ fused_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             }
             if (!ok) break;
             if constexpr (MODE == MODE_STATS) {
-                if (i < a.lse_ld) a.lse[head * a.lse_ld + i] = l > 0.f ? m + log2f(l) : INFINITY;
+                if (i < a.lse_ld) a.lse[head * a.lse_ld + i] = l > 0.f ? -(m + log2f(l)) : -INFINITY;
             } else if constexpr (MODE == MODE_ENERGY) {
                 if (i < a.Lr) a.energy[head * a.Lr + i] = l;
             } else {
@@ -816,7 +818,7 @@ size_t mask_tiles_bytes(const MaskView &m, int64_t seqs, int64_t Lq, int64_t Lk)
 // FULL (lse NULL, tok NULL): O = softmax(Qp Kp^T / sqrt(Dh) + mask) V; `mask` (or NULL) is the caller's additive fp32 mask on
 // top of the causal one, and tile_kind room for mask_tiles_bytes().
 // GATHERED (lse and tok given): Kp and V hold the kept keys only (Lk = their count, tok their positions); O = P V with
-// P = bf16(2^(x - lse)), no renormalisation.  `diag` = Lk - Lq of the unpacked problem.
+// P = bf16(2^(x + lse)) (lse negated), no renormalisation.  `diag` = Lk - Lq of the unpacked problem.
 // Qp [heads, Lq, ldd], Kp [heads, Lk, ldd] packed; V [v_batches, Lk, Dh] with row pitch v_ld and batch pitch v_sb.
 int launch_fused_attn(const __nv_bfloat16 *Qp, const __nv_bfloat16 *Kp, int64_t ldd, int64_t kd, const __nv_bfloat16 *V,
                       int64_t v_ld, int64_t v_sb, int64_t v_batches, int64_t v_off, int64_t v_div, __nv_bfloat16 *O,
@@ -872,7 +874,7 @@ int launch_fused_attn(const __nv_bfloat16 *Qp, const __nv_bfloat16 *Kp, int64_t 
 }
 
 // Sweeps 1 and 2 of the token reduction on packed Qp [heads, Lq, ldd], Kp [heads, Lk, ldd]:
-//   lse [heads, lse_ld] (lse_ld a multiple of 64, >= Lq): log2-domain row normalisers of softmax(S~ + mask);
+//   lse [heads, lse_ld] (lse_ld a multiple of 64, >= Lq): negated log2-domain row normalisers of softmax(S~ + mask);
 //   energy [heads, Lk]: squared token scores sum_i bf16(P_it)^2.
 int launch_fused_attn_scores(const __nv_bfloat16 *Qp, const __nv_bfloat16 *Kp, int64_t ldd, int64_t kd, int64_t heads,
                              int64_t Lq, int64_t Lk, int64_t Dh, int causal, float *lse, int64_t lse_ld, float *energy,

@@ -264,13 +264,13 @@ size_t decode_attn_workspace_bytes(const rmm_attn_desc_t *d);
 int launch_decode_attn(const rmm_attn_desc_t *d, int64_t kd, const void *Q, const void *K, const void *V, void *O, int32_t *idx_feat,
                        void *scratch, cudaStream_t stream);
 // lse == tok == NULL: O = softmax(Qp Kp^T / sqrt(Dh) + mask) V.  With lse [heads, lse_ld] and tok [heads, Lk] given,
-// Kp and V hold the kept keys only (Lk of them, at positions tok): O = P V with P = bf16(2^(x - lse)), not
+// Kp and V hold the kept keys only (Lk of them, at positions tok): O = P V with P = bf16(2^(x + lse)), not
 // renormalised.  diag = Lk - Lq of the unpacked problem (causal: query i sees key t iff t <= i + diag).
 int launch_fused_attn(const __nv_bfloat16 *Qp, const __nv_bfloat16 *Kp, int64_t ldd, int64_t kd, const __nv_bfloat16 *V,
                       int64_t v_ld, int64_t v_sb, int64_t v_batches, int64_t v_off, int64_t v_div, __nv_bfloat16 *O,
                       int64_t o_sh, int64_t o_sr, int64_t heads, int64_t Lq, int64_t Lk, int64_t Dh, int causal, int64_t diag,
                       const float *lse, int64_t lse_ld, const int32_t *tok, const MaskView *mask, uint8_t *tile_kind, int *status, cudaStream_t stream);
-// Two sweeps: lse [heads, lse_ld] (lse_ld a multiple of 64, >= Lq) = log2-domain row normalisers of softmax(S~ + mask);
+// Two sweeps: lse [heads, lse_ld] (lse_ld a multiple of 64, >= Lq) = negated log2-domain row normalisers of softmax(S~ + mask);
 // energy [heads, Lk] = squared token scores sum_i bf16(P_it)^2.
 int launch_fused_attn_scores(const __nv_bfloat16 *Qp, const __nv_bfloat16 *Kp, int64_t ldd, int64_t kd, int64_t heads,
                              int64_t Lq, int64_t Lk, int64_t Dh, int causal, float *lse, int64_t lse_ld, float *energy,
