@@ -8,9 +8,10 @@
 //                writes 4 bytes; the index pairs are read once per thread and reused for the R rows.  Rows too long
 //                for shared memory, or not 16-byte aligned, take the direct form (2-byte gathers from global memory).
 //                Long rows (a staged row above 36 KB, e.g. a 28672-wide intermediate axis) take pack_long_kernel: one
-//                persistent 1024-thread block per SM streams whole rows through two shared-memory buffers with bulk
-//                async copies, so the next row lands while the current one is gathered; every thread keeps its index
-//                pairs in registers across all rows (3.1 -> about 5 TB/s on 32768 x 28672).
+//                persistent 1024-thread block per SM streams whole rows through three shared-memory buffers (two where
+//                three do not fit) with bulk async copies; every thread keeps its index pairs in registers across all
+//                rows, and a buffer is refilled as soon as the row's kept elements are in registers, before they are
+//                written (32768 x 28672, half kept: 568 us with two buffers refilled a row later, 515 here, 2.8 GB).
 // Row gather     dst[b, j, :] = src[sb, idx[b, j], :]    16-byte vectors, 8 kept rows per block.
 // sb = (b + b_off) / b_div maps a batch entry to its source (grouped-query heads share K and V).
 #include "common.cuh"
@@ -22,7 +23,8 @@ namespace {
 constexpr int kThreadsPack = 256;
 constexpr int kThreadsLong = 1024;          // pack_long_kernel
 constexpr int kLongPairs = 16;              // output pairs per thread and row it can hold: k <= 2 * 16 * 1024
-constexpr int kLongMaxRowBytes = 110 * 1024;  // two such rows (and their zero pads) must fit in shared memory
+constexpr int kLongMaxRowBytes = 110 * 1024;  // two such rows (and their zero pads) must fit in shared memory (so K < 65536)
+constexpr int kLongBuffers = 3;
 constexpr int kMaxStageBytes = 96 * 1024;  // longest source row that is staged in shared memory
 constexpr int kStageTarget = 36 * 1024;    // preferred staging size (two 8192-column rows with their zero pads): several blocks per SM stay resident
 constexpr int kDirectRows = 4;
@@ -261,26 +263,22 @@ __device__ void pack_rows_short(const PackJob &p, int64_t blk, int *status)
 
 // Column gather of long rows: see the file header.  Block b owns the contiguous (batch, row) range
 // [b * per_block, (b + 1) * per_block); rows stream through two buffers filled by cp.async.bulk.
-__global__ void __launch_bounds__(kThreadsLong, 1) pack_long_kernel(const __grid_constant__ PackJob p, int64_t per_block, int *status,
+__global__ void __launch_bounds__(kThreadsLong, 1) pack_long_kernel(const __grid_constant__ PackJob p, int64_t per_block, int nbuf, int *status,
                                                                     unsigned long long wait_ns, int withhold)
 {
     using namespace ptx;
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ uint64_t full[2];
+    __shared__ uint64_t full[kLongBuffers];
     __shared__ int abort_flag;
     const int tid = threadIdx.x;
     const int K = (int)p.K, k = (int)p.k, half = (int)(p.ld_dst / 2);
     const uint32_t pitch = (uint32_t)(K + 8) * 2u;   // 8 zero elements after each staged row: where missing indices point
     if (tid == 0) {
-        mbar_init(smem_u32(&full[0]), 1);
-        mbar_init(smem_u32(&full[1]), 1);
+        for (int b = 0; b < kLongBuffers; ++b) mbar_init(smem_u32(&full[b]), 1);
         abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (tid < 8) {
-        reinterpret_cast<uint32_t *>(smem + (size_t)K * 2)[tid & 3] = 0;
-        reinterpret_cast<uint32_t *>(smem + pitch + (size_t)K * 2)[tid & 3] = 0;
-    }
+    if (tid < 4 * nbuf) reinterpret_cast<uint32_t *>(smem + (size_t)(tid >> 2) * pitch + (size_t)K * 2)[tid & 3] = 0;
     __syncthreads();
     pdl_wait();
     const int64_t total = p.batch * p.rows;
@@ -293,13 +291,14 @@ __global__ void __launch_bounds__(kThreadsLong, 1) pack_long_kernel(const __grid
         asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                      ::"r"(dst), "l"(src), "r"((uint32_t)K * 2u), "r"(bar) : "memory");
     };
-    if (tid == 0 && lo < hi && !(withhold && blockIdx.x == 0)) issue(lo, 0);  // (test switch: block 0's first row is never requested)
-    uint32_t cb[2 * kLongPairs];   // byte offsets of this thread's source columns inside a staged row
+    if (tid == 0)
+        for (int b = 0; b < nbuf && lo + b < hi; ++b)
+            if (!(withhold && blockIdx.x == 0 && b == 0)) issue(lo + b, b);  // (test switch: block 0's first row is never requested)
+    uint32_t cb[kLongPairs];   // column numbers of this thread's pairs, low and high half (column K: the zero pad)
+    int stage = 0;
+    uint32_t parity = 0;
     int64_t cur_batch = -1;
     for (int64_t g = lo; g < hi; ++g) {
-        const int it = (int)(g - lo), stage = it & 1;
-        // the other buffer was last read in the previous iteration, which ended with a block-wide barrier
-        if (tid == 0 && g + 1 < hi) issue(g + 1, stage ^ 1);
         const int64_t b = g / p.rows, r = g - b * p.rows;
         if (b != cur_batch) {
             cur_batch = b;
@@ -318,21 +317,27 @@ __global__ void __launch_bounds__(kThreadsLong, 1) pack_long_kernel(const __grid
                             c = K;
                         }
                     }
-                    cb[2 * i + h] = (uint32_t)c * 2u;
+                    cb[i] = h == 0 ? (uint32_t)c : cb[i] | (uint32_t)c << 16;
                 }
             }
         }
         // every thread comes out of the wait (landed, timed out, or told to abort) and the block decides together
-        const bool landed = mbar_wait(smem_u32(&full[stage]), (uint32_t)(it >> 1) & 1u, &abort_flag, status, wait_ns);
+        const bool landed = mbar_wait(smem_u32(&full[stage]), parity, &abort_flag, status, wait_ns);
         if (!__syncthreads_and(landed)) break;
         const uint32_t row_s = smem_u32(smem) + (uint32_t)stage * pitch;
         unsigned *d = reinterpret_cast<unsigned *>(p.dst + b * p.rows * p.ld_dst + r * p.ld_dst);
+        uint32_t val[kLongPairs];
+#pragma unroll
+        for (int i = 0; i < kLongPairs; ++i)
+            if (tid + i * kThreadsLong < half) val[i] = lds_u16(row_s + (cb[i] & 0xffffu) * 2u) | (lds_u16(row_s + (cb[i] >> 16) * 2u) << 16);
+        __syncthreads();
+        if (tid == 0 && g + nbuf < hi) issue(g + nbuf, stage);
 #pragma unroll
         for (int i = 0; i < kLongPairs; ++i) {
             const int jp = tid + i * kThreadsLong;
-            if (jp < half) d[jp] = lds_u16(row_s + cb[2 * i]) | (lds_u16(row_s + cb[2 * i + 1]) << 16);
+            if (jp < half) d[jp] = val[i];
         }
-        __syncthreads();
+        if (++stage == nbuf) { stage = 0; parity ^= 1u; }
     }
 }
 
@@ -427,8 +432,9 @@ int launch_pack(const PackSpec *specs, int n, int *status, cudaStream_t stream)
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         const int64_t total = p.batch * p.rows, per_block = ceil_div(total, sms);
         prof_begin("pack_long_kernel", stream);
-        launch_kernel(pack_long_kernel, dim3((unsigned)ceil_div(total, per_block)), dim3(kThreadsLong), 2 * row_bytes, stream, 1, p,
-                      per_block, status, wait_limit_ns(), debug_withhold() == WITHHOLD_PACK ? 1 : 0);
+        const int nbuf = kLongBuffers * row_bytes <= 2 * (size_t)kLongMaxRowBytes ? kLongBuffers : 2;
+        launch_kernel(pack_long_kernel, dim3((unsigned)ceil_div(total, per_block)), dim3(kThreadsLong), nbuf * row_bytes, stream, 1, p,
+                      per_block, nbuf, status, wait_limit_ns(), debug_withhold() == WITHHOLD_PACK ? 1 : 0);
         int rc = check_launch("pack_long_kernel", stream);
         if (rc != RMM_OK) return rc;
         blocks -= p.blocks;
