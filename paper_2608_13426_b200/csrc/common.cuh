@@ -105,6 +105,7 @@ struct ScorePlan {
     size_t off_counters, off_partials, off_energy, total_bytes;
     bool counters_in_header;
     bool use_tma;    // rows streamed through shared memory by TMA (bf16, 64-column blocks)
+    bool use_shift;  // bf16 rows off 16 bytes, read in aligned words (64-column blocks)
 };
 int plan_score(const rmm_mat_t *A, int axis, ScorePlan *plan);
 int launch_score_select(const rmm_mat_t *A, const ScorePlan &p, bool do_select, int64_t k, int32_t *idx,

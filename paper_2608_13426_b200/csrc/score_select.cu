@@ -75,41 +75,14 @@ __device__ __forceinline__ void load_vec(const void *A, int64_t off, int64_t s_n
     }
 }
 
-// Everything after a block's row loop: combine the row lanes, hand the column sums over (fp64 partials and an arrival
+// From a block's column sums on: hand them over (fp64 partials and an arrival
 // counter when the rows are split), write energies and scores, and let the last block of a batch element select.
-template <int VEC>
-__device__ __forceinline__ void score_finish(const ScoreArgs &a, const double (&dacc)[VEC], unsigned char *s_dyn,
-                                             SelectSmem &s_sel, int &s_flag)
+// `owner` threads hold the sum of column mycol.
+__device__ __forceinline__ void score_publish(const ScoreArgs &a, double colsum, bool owner, int64_t mycol, SelectSmem &s_sel, int &s_flag)
 {
-    double *s_part = reinterpret_cast<double *>(s_dyn);
     const int tid = threadIdx.x;
-    const int tx = tid % a.tx, ty = tid / a.tx;
     const int64_t b = blockIdx.z;
     const int split = blockIdx.y;
-    const int width = a.tx * VEC;  // columns per block
-    const int64_t col0 = (int64_t)blockIdx.x * width;
-#pragma unroll
-    for (int e = 0; e < VEC; ++e) s_part[ty * width + tx * VEC + e] = dacc[e];
-    __syncthreads();
-
-    // combine the row lanes in a fixed order, in two levels so that every thread helps: thread (part, c) adds the
-    // lanes part, part + parts, ... of column c, then thread c < width (the column's owner) adds the parts in order
-    double colsum = 0.0;
-    const int64_t mycol = col0 + tid;
-    const bool owner = tid < width && mycol < a.n;
-    {
-        const int parts = kThreads / width;  // width and ty are powers of two with width * ty == kThreads
-        const int c = tid % width, part = tid / width;
-        double sub = 0.0;
-        for (int y = part; y < a.ty; y += parts) sub += s_part[y * width + c];
-        __syncthreads();
-        s_part[part * width + c] = sub;
-        __syncthreads();
-        const int np = parts < a.ty ? parts : a.ty;
-        if (owner)
-            for (int q = 0; q < np; ++q) colsum += s_part[q * width + tid];
-    }
-
     bool finalize = true;
     if (a.row_splits > 1) {
         if (owner) a.partials[(b * a.row_splits + split) * a.n + mycol] = colsum;
@@ -155,6 +128,41 @@ __device__ __forceinline__ void score_finish(const ScoreArgs &a, const double (&
     __threadfence();
     block_select_any(a.energy + b * a.n, (int)a.n, a.k, a.idx + b * (int64_t)a.k,
                      a.retained ? a.retained + b : nullptr, s_sel);
+}
+
+// Everything after a block's row loop: combine the row lanes, then publish.
+template <int VEC>
+__device__ __forceinline__ void score_finish(const ScoreArgs &a, const double (&dacc)[VEC], unsigned char *s_dyn,
+                                             SelectSmem &s_sel, int &s_flag)
+{
+    double *s_part = reinterpret_cast<double *>(s_dyn);
+    const int tid = threadIdx.x;
+    const int tx = tid % a.tx, ty = tid / a.tx;
+    const int width = a.tx * VEC;  // columns per block
+    const int64_t col0 = (int64_t)blockIdx.x * width;
+#pragma unroll
+    for (int e = 0; e < VEC; ++e) s_part[ty * width + tx * VEC + e] = dacc[e];
+    __syncthreads();
+
+    // combine the row lanes in a fixed order, in two levels so that every thread helps: thread (part, c) adds the
+    // lanes part, part + parts, ... of column c, then thread c < width (the column's owner) adds the parts in order
+    double colsum = 0.0;
+    const int64_t mycol = col0 + tid;
+    const bool owner = tid < width && mycol < a.n;
+    {
+        const int parts = kThreads / width;  // width and ty are powers of two with width * ty == kThreads
+        const int c = tid % width, part = tid / width;
+        double sub = 0.0;
+        for (int y = part; y < a.ty; y += parts) sub += s_part[y * width + c];
+        __syncthreads();
+        s_part[part * width + c] = sub;
+        __syncthreads();
+        const int np = parts < a.ty ? parts : a.ty;
+        if (owner)
+            for (int q = 0; q < np; ++q) colsum += s_part[q * width + tid];
+    }
+
+    score_publish(a, colsum, owner, mycol, s_sel, s_flag);
 }
 
 template <int VEC, bool BF16>
@@ -209,6 +217,94 @@ __global__ void __launch_bounds__(kThreads, 1) score_select_kernel(ScoreArgs a)
         for (int e = 0; e < VEC; ++e) dacc[e] += (double)facc[e];
     }
     score_finish<VEC>(a, dacc, s_dyn, s_sel, s_flag);
+}
+
+// ---- the same pass for bf16 rows that do not start on 16 bytes ----------------------------------------------------------
+// A block owns 64 columns; a thread reads aligned 16-byte words all the same.  The word that holds a block's first column
+// starts `shift` elements before it, and since a thread's rows are a multiple of eight apart its shift is the same in all of
+// them: nine words cover the 64 columns of any row, and which column each of a thread's eight sums belongs to is settled
+// once, at the end.  Words that reach over the ends of a row are read element by element.  Single-element loads moved
+// 1.4 TB/s whatever the rows in flight (20000 x 20001: 572 us with four a thread, 710 with sixteen), 318 us here.
+constexpr int kShiftWords = 9, kShiftLanes = 112, kShiftCols = 64;
+
+__global__ void __launch_bounds__(kThreads, 1) score_shift_kernel(const ScoreArgs a)
+{
+    extern __shared__ __align__(128) unsigned char s_dyn[];  // [row lane][column] sums
+    __shared__ SelectSmem s_sel;
+    __shared__ int s_flag;
+    static_assert(kShiftWords * kShiftLanes <= kThreads && kShiftLanes % 8 == 0, "layout");
+    pdl_wait();
+    double *s_part = reinterpret_cast<double *>(s_dyn);
+    const int tid = threadIdx.x, tx = tid % kShiftWords, ty = tid / kShiftWords;
+    const int64_t b = blockIdx.z, col0 = (int64_t)blockIdx.x * kShiftCols;
+    const int64_t r_begin = (int64_t)blockIdx.y * a.rows_per_split, r_end = min(a.m, r_begin + a.rows_per_split);
+    const __nv_bfloat16 *first = static_cast<const __nv_bfloat16 *>(a.A) + b * a.s_batch + (r_begin + ty) * a.s_red + col0;
+    const int shift = (int)(reinterpret_cast<uintptr_t>(first) >> 1 & 7);
+    const int64_t c_first = col0 + 8 * tx - shift;   // column of this thread's first element
+    const bool whole = c_first >= 0 && c_first + 8 <= a.n;
+    double dacc[8];
+    float facc[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) { dacc[e] = 0.0; facc[e] = 0.f; }
+    if (ty < kShiftLanes && c_first < a.n) {
+        int trips = 0;
+        for (int64_t r = r_begin + ty; r < r_end; r += (int64_t)kShiftLanes * kUnroll) {
+            uint4 v[kUnroll];
+#pragma unroll
+            for (int u = 0; u < kUnroll; ++u) {
+                const int64_t rr = r + (int64_t)u * kShiftLanes;
+                const __nv_bfloat16 *p = first + (rr - r_begin - ty) * a.s_red + 8 * tx - shift;
+                v[u] = make_uint4(0, 0, 0, 0);
+                if (rr < r_end) {
+                    if (whole) {
+                        v[u] = __ldg(reinterpret_cast<const uint4 *>(p));
+                    } else {
+                        unsigned w[4] = {0, 0, 0, 0};
+                        const unsigned short *q = reinterpret_cast<const unsigned short *>(p);
+#pragma unroll
+                        for (int e = 0; e < 8; ++e)
+                            if (c_first + e >= 0 && c_first + e < a.n) w[e >> 1] |= (unsigned)__ldg(q + e) << (16 * (e & 1));
+                        v[u] = make_uint4(w[0], w[1], w[2], w[3]);
+                    }
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < kUnroll; ++u) {
+                const unsigned w[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const float lo = __uint_as_float(w[i] << 16), hi = __uint_as_float(w[i] & 0xffff0000u);
+                    facc[2 * i] = fmaf(lo, lo, facc[2 * i]);
+                    facc[2 * i + 1] = fmaf(hi, hi, facc[2 * i + 1]);
+                }
+            }
+            if (++trips == kFlushEvery) {
+                trips = 0;
+#pragma unroll
+                for (int e = 0; e < 8; ++e) { dacc[e] += (double)facc[e]; facc[e] = 0.f; }
+            }
+        }
+    }
+    if (ty < kShiftLanes) {
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            const int c = 8 * tx - shift + e;   // every column of the block in exactly one word of every row lane
+            if (c >= 0 && c < kShiftCols) s_part[ty * kShiftCols + c] = dacc[e] + (double)facc[e];
+        }
+    }
+    __syncthreads();
+    // row lanes in a fixed order: sixteen threads per column add every sixteenth lane, then the sixteen
+    const int c = tid % kShiftCols, part = tid / kShiftCols;
+    double sub = 0.0;
+    for (int y = part; y < kShiftLanes; y += kThreads / kShiftCols) sub += s_part[y * kShiftCols + c];
+    __syncthreads();
+    s_part[part * kShiftCols + c] = sub;
+    __syncthreads();
+    double colsum = 0.0;
+    const bool owner = tid < kShiftCols && col0 + tid < a.n;
+    if (owner)
+        for (int q = 0; q < kThreads / kShiftCols; ++q) colsum += s_part[q * kShiftCols + tid];
+    score_publish(a, colsum, owner, col0 + tid, s_sel, s_flag);
 }
 
 // ---- the same pass with the rows streamed through shared memory by TMA ------------------------------------------------
@@ -1066,12 +1162,14 @@ int plan_score(const rmm_mat_t *A, int axis, ScorePlan *p)
     while (tx > tx_min && ceil_div(groups, tx / 2) * A->batch <= sms) tx /= 2;
     // bf16 matrices that meet the TMA rules stream through shared memory in 64-column blocks (score_tma_kernel)
     p->use_tma = p->vec == 8 && A->dtype == RMM_BF16 && p->n >= kTmaCols && p->m <= INT32_MAX;
-    if (p->use_tma) tx = 8;
+    // bf16 rows that start off 16 bytes are read in aligned words all the same (score_shift_kernel)
+    p->use_shift = p->vec == 1 && A->dtype == RMM_BF16 && p->s_n == 1 && p->n >= kShiftCols;
+    if (p->use_tma || p->use_shift) tx = 8;
     p->tx = tx;
     p->ty = kThreads / tx;
-    p->col_blocks = (int)ceil_div(p->n, (int64_t)tx * p->vec);
+    p->col_blocks = (int)ceil_div(p->n, p->use_shift ? (int64_t)kShiftCols : (int64_t)tx * p->vec);
     int64_t splits = sms / ((int64_t)p->col_blocks * A->batch);
-    int64_t min_rows = p->use_tma ? 2 * kTmaRows : (int64_t)p->ty * kUnroll * 2;
+    int64_t min_rows = p->use_tma ? 2 * kTmaRows : (p->use_shift ? (int64_t)kShiftLanes * kUnroll : (int64_t)p->ty * kUnroll * 2);
     int64_t max_splits = p->m / min_rows;
     if (max_splits < 1) max_splits = 1;
     if (splits > max_splits) splits = max_splits;
@@ -1159,6 +1257,19 @@ int launch_score_select(const rmm_mat_t *A, const ScorePlan &p, bool do_select, 
         launch_kernel(score_tma_kernel, grid, dim3(kThreads), kTmaStages * kTmaStageBytes, stream, 1, map, a, &hdr->status);
         int rc2 = check_launch("score_tma_kernel", stream);
         if (rc2 != RMM_OK || !do_select || fused) return rc2;
+        return launch_select(a.energy, A->batch, p.n, k, idx, retained, ws, stream);
+    }
+    if (p.use_shift) {
+        static PerDeviceOnce shift_configured;
+        const int shift_smem = kShiftLanes * kShiftCols * (int)sizeof(double);
+        if (shift_configured.first()) {
+            cudaError_t e = cudaFuncSetAttribute(score_shift_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, shift_smem);
+            if (e != cudaSuccess) return fail(RMM_ERR_CUDA, "score: cudaFuncSetAttribute: %s", cudaGetErrorString(e));
+        }
+        prof_begin("score_shift_kernel", stream);
+        launch_kernel(score_shift_kernel, grid, dim3(kThreads), (size_t)shift_smem, stream, 1, a);
+        int rc = check_launch("score_shift_kernel", stream);
+        if (rc != RMM_OK || !do_select || fused) return rc;
         return launch_select(a.energy, A->batch, p.n, k, idx, retained, ws, stream);
     }
     static PerDeviceOnce configured;
