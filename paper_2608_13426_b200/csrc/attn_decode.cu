@@ -312,7 +312,7 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, kDecodeBlocks) attn_decode_
             const int row = row0 + r;
             if (c < a.Dh)
                 a.o[b * a.o_sb + (hk * a.group + row / a.Lq) * a.o_sh + (int64_t)(row % a.Lq) * a.o_sr + c] =
-                    __float2bfloat16_rn(lsum > 0.f ? sum * (1.f / lsum) : 0.f);
+                    __float2bfloat16_rn(lsum == 0.f ? 0.f : sum * (1.f / lsum));  // (0: the row sees no key; a NaN stays one)
         } else {
             a.part_o[((int64_t)blockIdx.x * kRows + r) * DH + c] = sum;
             if (c == 0) {
@@ -365,7 +365,7 @@ __global__ void __launch_bounds__(kCombineWarps * 32) attn_decode_combine_kernel
     lsum = 0.f;
 #pragma unroll
     for (int w = 0; w < kCombineWarps; ++w) lsum += s_l[w];
-    const float inv = lsum > 0.f ? 1.f / lsum : 0.f;
+    const float inv = lsum == 0.f ? 0.f : 1.f / lsum;  // 0: the row sees no key; a NaN stays one
     const int64_t bh = job / a.chunks, b = bh / a.Hkv, hk = bh % a.Hkv;
     __nv_bfloat16 *o = a.o + b * a.o_sb + (hk * a.group + row / a.Lq) * a.o_sh + (int64_t)(row % a.Lq) * a.o_sr;
     for (int c = threadIdx.x; c < a.Dh; c += kCombineWarps * 32) {

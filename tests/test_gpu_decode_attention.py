@@ -53,3 +53,26 @@ def test_decode_attention_ignores_what_dropped_features_hold(oracle):
     assert torch.isfinite(got.float()).all()
     # the steps that hold such a key sum their products in another order: fp32 rounding before the bf16 rounding of P
     assert ((got.float() - want.float()).norm() / want.float().norm()).item() <= 4e-3
+
+
+@pytest.mark.parametrize("B, Hkv, Lk", [(40, 8, 60), (1, 1, 6000)])   # whole jobs per block; one job over many blocks
+def test_decode_attention_shows_a_nan(B, Hkv, Lk):
+    """A NaN (or an infinity's inf - inf) among a row's logits makes the row NaN, wherever its key lies; rows that see no
+    key stay zero and the other heads are untouched."""
+    Q, K, V = synth.attention_qkv(B, Hkv, Hkv, 2, Lk, 64, seed=16)
+    want = rmm.rmm_reduced_attn(dev(Q), dev(K), dev(V), True, 1.0)
+    for key in (0, Lk // 2, Lk - 2):
+        for bad in (float("nan"), float("inf")):
+            Kb, Qb = K.clone(), Q.clone()
+            Kb[0, 0, key, 5], Qb[0, 0, :, 5] = bad, 1.0
+            got = rmm.rmm_reduced_attn(dev(Qb), dev(Kb), dev(V), True, 1.0)
+            assert torch.isnan(got[0, 0]).all(), (key, bad)
+            assert torch.equal(got.flatten(0, 1)[1:], want.flatten(0, 1)[1:])
+    Qb = Q.clone()
+    Qb[0, 0, 1, 7] = float("nan")                 # every logit of this row
+    got = rmm.rmm_reduced_attn(dev(Qb), dev(K), dev(V), True, 1.0)
+    assert torch.isnan(got[0, 0, 1]).all() and torch.isfinite(got[0, 0, 0].float()).all()
+    Qb = Q.repeat(1, 1, 2, 1)                     # four queries on two keys: the first two see nothing
+    Qb[0, 0] = float("nan")
+    got = rmm.rmm_reduced_attn(dev(Qb), dev(K[:, :, :2]), dev(V[:, :, :2]), True, 1.0)
+    assert torch.count_nonzero(got[:, :, :2]) == 0 and torch.isnan(got[0, 0, 2:]).all()
