@@ -111,6 +111,7 @@ struct StreamQ8 {
     int K, k, rows_at_once[2], stages[2];
     int *status;
     unsigned long long wait_ns;
+    int withhold;
 };
 
 __device__ __forceinline__ uint32_t e4m3_code2(float x0, float x1, float step, float inv)
@@ -139,6 +140,8 @@ __device__ __forceinline__ bool stream_rows(const StreamQ8 &a, unsigned char *sm
     if (lo >= hi) return true;
     // 16 zero bytes after each staged row: where missing indices point
     for (int i = tid; i < 4 * nst * at_once; i += kThreadsS) reinterpret_cast<uint32_t *>(smem + (size_t)(i >> 2) * pitch + pad)[i & 3] = 0;
+    // B's rows land where A's pads and rows were: this thread's own accesses come before the copies (which are another proxy's)
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     __syncthreads();
     const uint32_t base = smem_u32(smem);
     // turns of this operand: turn t0 + n uses buffer n % nst; a barrier completes once per use
@@ -155,7 +158,8 @@ __device__ __forceinline__ bool stream_rows(const StreamQ8 &a, unsigned char *sm
                            "r"(smem_u32(&full[b])) : "memory");
     };
     if (warp == 0)
-        for (int b = 0; b < nst && lo + (int64_t)b * at_once < hi; ++b) issue(lo + (int64_t)b * at_once, b);
+        for (int b = 0; b < nst && lo + (int64_t)b * at_once < hi; ++b)
+            if (!(a.withhold && blockIdx.x == 0 && b == 0)) issue(lo + (int64_t)b * at_once, b);  // (test switch: block 0's first rows are never requested)
     const int words = (int)(a.ld_dst / 4);
     const int rr = lane & 3, word_in_warp = 8 * rr + (lane >> 2);  // after the transpose lane 4 m + rr holds word 8 rr + m
     auto offset = [&](int sl) -> uint32_t { return ((cb[sl >> 1] >> (16 * (sl & 1))) & 0xffffu) * ES; };
@@ -164,7 +168,11 @@ __device__ __forceinline__ bool stream_rows(const StreamQ8 &a, unsigned char *sm
     for (int64_t r = lo; r < hi; r += at_once) {
         const int n = (int)min((int64_t)at_once, hi - r);
         const bool landed = mbar_wait(smem_u32(&full[b]), (parity_of >> b) & 1u, abort_flag, a.status, a.wait_ns);
-        if (!__syncthreads_and(landed)) { ok = false; break; }
+        if (!__syncthreads_and(landed)) {
+            drain_copies();
+            ok = false;
+            break;
+        }
         parity_of ^= 1u << b;
         const unsigned char *rows = smem + (size_t)(b * at_once) * pitch;
         uint32_t val[R][QUANT ? 2 * G : G];   // this thread's inputs: bf16 pairs, or four bytes to a register
@@ -301,6 +309,7 @@ int launch_gather_q8_pair(const void *A, int64_t a_rows, int64_t a_pitch, const 
     a.K = (int)K; a.k = (int)k;
     a.status = status;
     a.wait_ns = wait_limit_ns();
+    a.withhold = debug_withhold() == WITHHOLD_QUANT;
     const int64_t groups = ceil_div(ld_dst, 4096);
     const int g = groups <= 1 ? 1 : (groups <= 2 ? 2 : (groups <= 4 ? 4 : 8));
     int64_t blocks = 0;
