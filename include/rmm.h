@@ -219,8 +219,9 @@ int rmm_status_read(void *ws, int *device_status);
  * is bounded: 2 s by default, RMM_SPIN_LIMIT_MS milliseconds if that environment variable is set when the library is
  * first used.  rmm_debug_control("wait_limit_ms", x) overrides the bound for later launches (0 = back to the default);
  * rmm_debug_control("withhold", w) makes block 0 of one kernel family never request its first tile (w = 1 tensor-core
- * product, 2 score pass, 3 fused attention, 4 one-launch front end of rmm_product, 5 streaming column gather; 0 = off,
- * -1 = back to the environment variable RMM_TEST_WITHHOLD = gemm | score | attn | front | pack), so that the waits behind
+ * product, 2 score pass, 3 fused attention, 4 one-launch front end of rmm_product, 5 streaming column gather, 6 streaming
+ * 8-bit gather; 0 = off, -1 = back to the environment variable RMM_TEST_WITHHOLD = gemm | score | attn | front | pack | quant),
+ * so that the waits behind
  * that tile run out: the kernel must then report RMM_ERR_TIMEOUT in the status word, release what it holds and return.
  * Results of such a call are undefined; rmm_status_read clears the workspace header, after which the workspace is
  * usable again.  Not thread-safe against concurrent launches. */

@@ -90,6 +90,7 @@ int debug_withhold()
         if (strcmp(e, "attn") == 0) return (int)WITHHOLD_ATTN;
         if (strcmp(e, "front") == 0) return (int)WITHHOLD_FRONT;
         if (strcmp(e, "pack") == 0) return (int)WITHHOLD_PACK;
+        if (strcmp(e, "quant") == 0) return (int)WITHHOLD_QUANT;
         return 0;
     }();
     return which;
@@ -560,7 +561,7 @@ int rmm_debug_control(const char *key, double value)
     }
     if (strcmp(key, "withhold") == 0) {
         const int w = (int)value;
-        if (w < -1 || w > WITHHOLD_PACK) return fail(RMM_ERR_INVALID_ARG, "debug_control: withhold must be -1 .. %d", (int)WITHHOLD_PACK);
+        if (w < -1 || w > WITHHOLD_QUANT) return fail(RMM_ERR_INVALID_ARG, "debug_control: withhold must be -1 .. %d", (int)WITHHOLD_QUANT);
         g_withhold_override.store(w, std::memory_order_relaxed);
         return RMM_OK;
     }

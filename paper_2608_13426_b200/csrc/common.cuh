@@ -70,9 +70,9 @@ struct PerDeviceOnce {
 
 int sm_count();                      // multiprocessors of the current device
 unsigned long long wait_limit_ns();  // bound of every device-side wait: 2 s, or RMM_SPIN_LIMIT_MS from the environment
-// Test switch (environment RMM_TEST_WITHHOLD = gemm | score | attn | front | pack, read once): block 0 of that kernel
+// Test switch (environment RMM_TEST_WITHHOLD = gemm | score | attn | front | pack | quant, read once): block 0 of that kernel
 // family never requests its first tile, so the waits behind it run out and the kernel's give-up path runs.  0 = off.
-enum { WITHHOLD_GEMM = 1, WITHHOLD_SCORE = 2, WITHHOLD_ATTN = 3, WITHHOLD_FRONT = 4, WITHHOLD_PACK = 5 };
+enum { WITHHOLD_GEMM = 1, WITHHOLD_SCORE = 2, WITHHOLD_ATTN = 3, WITHHOLD_FRONT = 4, WITHHOLD_PACK = 5, WITHHOLD_QUANT = 6 };
 int debug_withhold();
 
 static inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }

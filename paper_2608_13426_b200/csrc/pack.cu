@@ -262,7 +262,7 @@ __device__ void pack_rows_short(const PackJob &p, int64_t blk, int *status)
 }
 
 // Column gather of long rows: see the file header.  Block b owns the contiguous (batch, row) range
-// [b * per_block, (b + 1) * per_block); rows stream through two buffers filled by cp.async.bulk.
+// [b * per_block, (b + 1) * per_block); rows stream through nbuf buffers filled by cp.async.bulk.
 __global__ void __launch_bounds__(kThreadsLong, 1) pack_long_kernel(const __grid_constant__ PackJob p, int64_t per_block, int nbuf, int *status,
                                                                     unsigned long long wait_ns, int withhold)
 {
@@ -323,7 +323,10 @@ __global__ void __launch_bounds__(kThreadsLong, 1) pack_long_kernel(const __grid
         }
         // every thread comes out of the wait (landed, timed out, or told to abort) and the block decides together
         const bool landed = mbar_wait(smem_u32(&full[stage]), parity, &abort_flag, status, wait_ns);
-        if (!__syncthreads_and(landed)) break;
+        if (!__syncthreads_and(landed)) {
+            drain_copies();
+            break;
+        }
         const uint32_t row_s = smem_u32(smem) + (uint32_t)stage * pitch;
         unsigned *d = reinterpret_cast<unsigned *>(p.dst + b * p.rows * p.ld_dst + r * p.ld_dst);
         uint32_t val[kLongPairs];

@@ -57,6 +57,13 @@ __device__ __forceinline__ unsigned long long global_ns()
     return t;
 }
 
+// For a block that gives up: copies still in flight get time to land before its shared memory is released.
+__device__ __forceinline__ void drain_copies()
+{
+    const unsigned long long t0 = global_ns();
+    while (global_ns() - t0 < 200000ull) __nanosleep(1000);
+}
+
 // Bounded wait.  Returns false when the block is aborting (this or another thread ran out of time).
 __device__ __forceinline__ bool mbar_wait_lane(uint32_t bar, uint32_t parity, volatile int *abort_flag, int *status,
                                           unsigned long long limit_ns = kWaitLimitNs)

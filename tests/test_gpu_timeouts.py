@@ -85,6 +85,17 @@ assert np.array_equal(idx.cpu().numpy(), oracle.select(e64, 1280)[0])
 assert rel(Y.float().cpu().numpy(), oracle.reduced_gemm(A, B, idx.cpu().numpy())) <= 1e-2
 assert rmm.rmm_status_read() == 0
 """,
+    "quant": """
+A = synth.heavy_tailed_activations(2000, 8192, seed=8)
+W = (synth.weight(256, 8192, seed=9, dtype=torch.float32) * 64).to(torch.float8_e4m3fn)
+Ad, Wd = A.cuda(), W.cuda()
+idx = torch.arange(0, 8192, 2, dtype=torch.int32, device="cuda")
+expect_timeout(lambda: rmm.rmm_reduced_gemm_q8(Ad, Wd, 1.0 / 64, idx), 6)
+Y = rmm.rmm_reduced_gemm_q8(Ad, Wd, 1.0 / 64, idx)
+want = oracle.reduced_gemm_q8(A, W.float().numpy(), 1.0 / 64, idx.cpu().numpy())[0]
+assert rel(Y.float().cpu().numpy(), want) <= 1e-2
+assert rmm.rmm_status_read() == 0
+""",
     "pack": """
 A = synth.heavy_tailed_activations(40, 20000, seed=6)
 B = synth.weight(20000, 256, seed=7)
