@@ -415,10 +415,7 @@ int launch_shape(const DecodeArgs &a, const DecodeGrid &g, cudaStream_t stream)
     using S = DecodeShape<DH, NT>;
     auto kern = attn_decode_kernel<DH, NT>;
     static PerDeviceOnce configured;
-    if (configured.first()) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, S::kSmem);
-        if (e != cudaSuccess) return fail(RMM_ERR_CUDA, "attn_decode: cudaFuncSetAttribute: %s", cudaGetErrorString(e));
-    }
+    if (cudaError_t e = configured.smem(S::kSmem, kern)) return fail(RMM_ERR_CUDA, "attn_decode: cudaFuncSetAttribute: %s", cudaGetErrorString(e));
     prof_begin("attn_decode_kernel", stream);
     launch_kernel(kern, dim3((unsigned)g.blocks), dim3(kDecodeWarps * 32), S::kSmem, stream, 1, a);
     int rc = check_launch("attn_decode_kernel", stream);

@@ -56,15 +56,21 @@ __device__ __forceinline__ void pdl_wait()
 }
 #endif
 
-// Function attributes (the opt-in to more than 48 KB of dynamic shared memory) belong to a device: a flag per device
-// and call site says whether the current device has been set up.  Returns true exactly once per device.
+// The opt-in to more than 48 KB of dynamic shared memory belongs to a device: a flag per device and call site says whether
+// the current device has been set up.  It is set after the attribute is, so a thread that arrives meanwhile sets it once
+// more (which changes nothing) instead of launching without it.
 struct PerDeviceOnce {
     std::atomic<bool> done[64];
-    bool first()
+    template <typename... Kernel>
+    cudaError_t smem(int bytes, Kernel... kernels)
     {
         int dev = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return true;  // unknown: set up every time
-        return !done[dev].exchange(true);
+        const bool known = cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64;  // unknown: set up every time
+        if (known && done[dev].load(std::memory_order_acquire)) return cudaSuccess;
+        cudaError_t e = cudaSuccess;
+        ((e = e == cudaSuccess ? cudaFuncSetAttribute(kernels, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) : e), ...);
+        if (known && e == cudaSuccess) done[dev].store(true, std::memory_order_release);
+        return e;
     }
 };
 

@@ -225,10 +225,7 @@ int launch_shape(const SkinnyArgs &a, int64_t batch, cudaStream_t stream)
     using S = SkinnyShape<NT>;
     auto kern = gemm_skinny_kernel<NT>;
     static PerDeviceOnce configured;
-    if (configured.first()) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, S::kSmem);
-        if (e != cudaSuccess) return fail(RMM_ERR_CUDA, "gemm_skinny: cudaFuncSetAttribute: %s", cudaGetErrorString(e));
-    }
+    if (cudaError_t e = configured.smem(S::kSmem, kern)) return fail(RMM_ERR_CUDA, "gemm_skinny: cudaFuncSetAttribute: %s", cudaGetErrorString(e));
     prof_begin("gemm_skinny_kernel", stream);
     launch_kernel(kern, dim3((unsigned)ceil_div(a.N, CW), (unsigned)a.pieces, (unsigned)batch), dim3(kSkWarps * 32), S::kSmem, stream, 1, a);
     int rc = check_launch("gemm_skinny_kernel", stream);

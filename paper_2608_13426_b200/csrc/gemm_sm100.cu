@@ -599,10 +599,7 @@ int launch_variant(const CUtensorMap &ma, const CUtensorMap &mb, const CUtensorM
     auto kern = reduced_gemm_tc_kernel<BN, B_KMAJOR, OUT_BF16, CTAS, B_GATHER, FP8>;
     using L = SmemLayout<BN, CTAS>;
     static PerDeviceOnce configured;
-    if (configured.first()) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kTotal);
-        if (e != cudaSuccess) return fail(RMM_ERR_CUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e));
-    }
+    if (cudaError_t e = configured.smem(L::kTotal, kern)) return fail(RMM_ERR_CUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e));
     const int64_t tiles = a.batch * a.tiles_m * a.tiles_n, num_kb = ceil_div(a.k, FP8 ? 2 * BK : BK);
     const int64_t slots = sm_count() / CTAS;
     const int64_t blocks = B_GATHER ? ceil_div(tiles * num_kb, a.seg_kb) : (tiles < slots ? tiles : slots);

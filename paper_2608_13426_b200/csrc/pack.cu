@@ -426,10 +426,8 @@ int launch_pack(const PackSpec *specs, int n, int *status, cudaStream_t stream)
             p.ld_dst > 2 * kLongPairs * kThreadsLong)
             continue;
         static PerDeviceOnce long_configured;
-        if (long_configured.first()) {
-            cudaError_t e = cudaFuncSetAttribute(pack_long_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * kLongMaxRowBytes);
-            if (e != cudaSuccess) return fail(RMM_ERR_CUDA, "pack: cudaFuncSetAttribute: %s", cudaGetErrorString(e));
-        }
+        if (cudaError_t e = long_configured.smem(2 * kLongMaxRowBytes, pack_long_kernel))
+            return fail(RMM_ERR_CUDA, "pack: cudaFuncSetAttribute: %s", cudaGetErrorString(e));
         int dev = 0, sms = 148;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -452,10 +450,8 @@ int launch_pack(const PackSpec *specs, int n, int *status, cudaStream_t stream)
     }
     if (blocks > INT32_MAX) return fail(RMM_ERR_UNSUPPORTED, "pack: too many blocks");
     static PerDeviceOnce configured;
-    if (configured.first()) {
-        cudaError_t e = cudaFuncSetAttribute(pack_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxStageBytes);
-        if (e != cudaSuccess) return fail(RMM_ERR_CUDA, "pack: cudaFuncSetAttribute: %s", cudaGetErrorString(e));
-    }
+    if (cudaError_t e = configured.smem(kMaxStageBytes, pack_kernel))
+        return fail(RMM_ERR_CUDA, "pack: cudaFuncSetAttribute: %s", cudaGetErrorString(e));
     prof_begin("pack_kernel", stream);
     launch_kernel(pack_kernel, dim3((unsigned)blocks), dim3(kThreadsPack), smem, stream, 1, a);
     return check_launch("pack_kernel", stream);

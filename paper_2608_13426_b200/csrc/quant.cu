@@ -328,14 +328,9 @@ int launch_gather_q8_pair(const void *A, int64_t a_rows, int64_t a_pitch, const 
     }
     auto kern = g == 1 ? gather_q8_stream_kernel<1> : (g == 2 ? gather_q8_stream_kernel<2> : (g == 4 ? gather_q8_stream_kernel<4> : gather_q8_stream_kernel<8>));
     static PerDeviceOnce configured;
-    if (configured.first()) {
-        const int most = 2 * (kStreamMaxRowBytes + 16);
-        cudaError_t e = cudaFuncSetAttribute(gather_q8_stream_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(gather_q8_stream_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(gather_q8_stream_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(gather_q8_stream_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-        if (e != cudaSuccess) return fail(RMM_ERR_CUDA, "gather_q8: cudaFuncSetAttribute: %s", cudaGetErrorString(e));
-    }
+    const int most = 2 * (kStreamMaxRowBytes + 16);
+    if (cudaError_t e = configured.smem(most, gather_q8_stream_kernel<1>, gather_q8_stream_kernel<2>, gather_q8_stream_kernel<4>, gather_q8_stream_kernel<8>))
+        return fail(RMM_ERR_CUDA, "gather_q8: cudaFuncSetAttribute: %s", cudaGetErrorString(e));
     prof_begin("gather_q8_stream_kernel", stream);
     launch_kernel(kern, dim3((unsigned)blocks), dim3(kThreadsS), smem, stream, 1, a);
     return check_launch("gather_q8_stream_kernel", stream);
@@ -348,11 +343,8 @@ int launch_gather_q8(bool quantise, const void *src, int64_t rows, int64_t s_row
     const size_t smem = align_up(row_bytes, 16);
     if (smem > 200 * 1024 || K > INT32_MAX / 4 || rows > INT32_MAX) return fail(RMM_ERR_UNSUPPORTED, "gather_q8: row too long");
     static PerDeviceOnce configured;
-    if (configured.first()) {
-        cudaError_t e = cudaFuncSetAttribute(gather_q8_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(gather_q8_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-        if (e != cudaSuccess) return fail(RMM_ERR_CUDA, "gather_q8: cudaFuncSetAttribute: %s", cudaGetErrorString(e));
-    }
+    if (cudaError_t e = configured.smem(200 * 1024, gather_q8_kernel<true>, gather_q8_kernel<false>))
+        return fail(RMM_ERR_CUDA, "gather_q8: cudaFuncSetAttribute: %s", cudaGetErrorString(e));
     prof_begin("gather_q8_kernel", stream);
     if (quantise)
         launch_kernel(gather_q8_kernel<true>, dim3((unsigned)rows), dim3(kThreadsQ), smem, stream, 1, src, s_row, (int)K, idx, (int)k, dst, ld_dst,

@@ -1249,10 +1249,8 @@ int launch_score_select(const rmm_mat_t *A, const ScorePlan &p, bool do_select, 
         int rc = make_map(&map, const_cast<void *>(a.A), 3, dims, st, box, false);
         if (rc != RMM_OK) return rc;
         static PerDeviceOnce tma_configured;
-        if (tma_configured.first()) {
-            cudaError_t e = cudaFuncSetAttribute(score_tma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kTmaStages * kTmaStageBytes);
-            if (e != cudaSuccess) return fail(RMM_ERR_CUDA, "score: cudaFuncSetAttribute: %s", cudaGetErrorString(e));
-        }
+        if (cudaError_t e = tma_configured.smem(kTmaStages * kTmaStageBytes, score_tma_kernel))
+            return fail(RMM_ERR_CUDA, "score: cudaFuncSetAttribute: %s", cudaGetErrorString(e));
         prof_begin("score_tma_kernel", stream);
         launch_kernel(score_tma_kernel, grid, dim3(kThreads), kTmaStages * kTmaStageBytes, stream, 1, map, a, &hdr->status);
         int rc2 = check_launch("score_tma_kernel", stream);
@@ -1262,10 +1260,8 @@ int launch_score_select(const rmm_mat_t *A, const ScorePlan &p, bool do_select, 
     if (p.use_shift) {
         static PerDeviceOnce shift_configured;
         const int shift_smem = kShiftLanes * kShiftCols * (int)sizeof(double);
-        if (shift_configured.first()) {
-            cudaError_t e = cudaFuncSetAttribute(score_shift_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, shift_smem);
-            if (e != cudaSuccess) return fail(RMM_ERR_CUDA, "score: cudaFuncSetAttribute: %s", cudaGetErrorString(e));
-        }
+        if (cudaError_t e = shift_configured.smem(shift_smem, score_shift_kernel))
+            return fail(RMM_ERR_CUDA, "score: cudaFuncSetAttribute: %s", cudaGetErrorString(e));
         prof_begin("score_shift_kernel", stream);
         launch_kernel(score_shift_kernel, grid, dim3(kThreads), (size_t)shift_smem, stream, 1, a);
         int rc = check_launch("score_shift_kernel", stream);
@@ -1273,14 +1269,9 @@ int launch_score_select(const rmm_mat_t *A, const ScorePlan &p, bool do_select, 
         return launch_select(a.energy, A->batch, p.n, k, idx, retained, ws, stream);
     }
     static PerDeviceOnce configured;
-    if (configured.first()) {
-        const int big = kThreads * 8 * (int)sizeof(double);
-        cudaError_t e = cudaFuncSetAttribute(score_select_kernel<8, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(score_select_kernel<4, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(score_select_kernel<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(score_select_kernel<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
-        if (e != cudaSuccess) return fail(RMM_ERR_CUDA, "score: cudaFuncSetAttribute: %s", cudaGetErrorString(e));
-    }
+    const int big = kThreads * 8 * (int)sizeof(double);
+    if (cudaError_t e = configured.smem(big, score_select_kernel<8, true>, score_select_kernel<4, false>, score_select_kernel<1, true>, score_select_kernel<1, false>))
+        return fail(RMM_ERR_CUDA, "score: cudaFuncSetAttribute: %s", cudaGetErrorString(e));
     prof_begin("score_select_kernel", stream);
     if (bf16 && p.vec == 8) launch_kernel(score_select_kernel<8, true>, grid, dim3(kThreads), smem, stream, 1, a);
     else if (bf16) launch_kernel(score_select_kernel<1, true>, grid, dim3(kThreads), smem, stream, 1, a);
@@ -1355,10 +1346,8 @@ int launch_front(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k, int32_t *idx
     fa.rows_per_chunk = (int)(kChunkBytes / (a.n * 2));
     if (fa.rows_per_chunk < 1) return fail(RMM_ERR_UNSUPPORTED, "front: row too long");
     static PerDeviceOnce configured;
-    if (configured.first()) {
-        cudaError_t e = cudaFuncSetAttribute(rmm_front_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kFrontSmemBytes);
-        if (e != cudaSuccess) return fail(RMM_ERR_CUDA, "front: cudaFuncSetAttribute: %s", cudaGetErrorString(e));
-    }
+    if (cudaError_t e = configured.smem(kFrontSmemBytes, rmm_front_kernel))
+        return fail(RMM_ERR_CUDA, "front: cudaFuncSetAttribute: %s", cudaGetErrorString(e));
     prof_begin("rmm_front_kernel", stream);
     launch_kernel(rmm_front_kernel, dim3((unsigned)plan.col_blocks), dim3(kThreads), kFrontSmemBytes, stream, 1, map, fa,
                   &hdr->status);
