@@ -25,6 +25,7 @@
 // Warp 0 feeds TMA, warps 2-5 and 6-9 are the softmax/epilogue warps of the two groups (every scheduler has two of
 // them to switch between), and one thread of warp 1 and of warp 10 issues the tcgen05.mma of group 0 and 1: a single
 // issuing thread for both groups was the bottleneck.  Every wait is bounded.
+#include <float.h>
 #include <math.h>
 
 #include "common.cuh"
@@ -83,7 +84,6 @@ struct FusedArgs {
     MaskView mask;               // MASK: the caller's additive mask
     const uint8_t *tile_kind;    // MASK: what the mask does to a 128 x 128 tile: [plane][row block][tile], see mask_tiles_kernel
     int64_t kind_rb, kind_ld;    // row blocks per plane (even), bytes per row block (a multiple of 8)
-    float mask_gain;             // sqrt(Dh): M is added to the unscaled S~ tile as M * sqrt(Dh)
     int *status;
     unsigned long long wait_ns;  // bound of every device-side wait
     int withhold;                // test switch: block 0 never requests its first key tile
@@ -96,32 +96,34 @@ struct FusedArgs {
 // load.  2 sequences x 16 heads x 2048 x 128, padded: 2 x 244 us with every tile added, 52 us in one launch with this
 // pass (6 us) in front; a mask whose every value is added: 254 -> 136 us a call on 16 heads x 2048.
 // Bound by reading the mask once; a warp stops reading a tile once it knows that its values have to be added.
-// A value counts as hiding when mask x sqrt(Dh) is -inf in fp32, which is what the softmax step would make of it.
+// Only -inf hides a key.  A tile of the lowest finite values (masks are written with them too) is skipped all the same where
+// each of its rows sees some ordinary key, next to which such values weigh exactly nothing; a row that sees no other keep
+// them (its weights are then equal, whatever the logits: fp32 sums).
 enum { TILE_HIDDEN = 0, TILE_CLEAR = 1, TILE_ADD = 2 };
 constexpr int kMaskThreads = 128;
+constexpr float kMaskLow = -2e38f, kMaskOrdinary = -1e38f;  // 1e38 apart: e^-1e38 = 0 for any sum of logits below that
 
 struct MaskTileArgs {
     MaskView mask;
     int64_t Lq, Lk, diag;
     int causal, vec;   // vec: rows are 16-byte aligned
-    float gain;
     uint8_t *kind;
     int64_t kind_rb, kind_ld;
 };
 
 __global__ void __launch_bounds__(kMaskThreads) mask_tiles_kernel(const MaskTileArgs a)
 {
-    __shared__ int s_some[kMaskThreads / 32], s_live[kMaskThreads / 32];
     pdl_wait();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t t0 = (int64_t)blockIdx.x * FN, r0 = (int64_t)blockIdx.y * FM, plane = blockIdx.z;
+    const int64_t rb = blockIdx.y, tile = blockIdx.x, t0 = tile * FN, r0 = rb * FM, plane = blockIdx.z;
     const float *m = a.mask.p + (plane / a.mask.plane_heads) * a.mask.sb + (plane % a.mask.plane_heads) * a.mask.sh;
     const int64_t rows = a.mask.sr == 0 ? 1 : min((int64_t)FM, a.Lq - r0);   // one row stands for all of them
     const bool beyond = t0 >= a.Lk || r0 >= a.Lq || (a.causal && t0 > min(a.Lq, r0 + FM) - 1 + a.diag);
-    bool some = false, live = false;  // some value is not zero; some value does not hide
+    bool some = false, live = false, low = false;  // some value is not zero; is not low; is low but does not hide
     auto look = [&](float v) {
         some |= !(v == 0.f);
-        live |= !(v * a.gain == -INFINITY);
+        live |= !(v <= kMaskLow);
+        low |= v <= kMaskLow && v > -INFINITY;
     };
     for (int64_t rr = warp * 8; rr < rows && !beyond; rr += kMaskThreads / 32 * 8) {
         float4 v[8];
@@ -147,21 +149,23 @@ __global__ void __launch_bounds__(kMaskThreads) mask_tiles_kernel(const MaskTile
         }
         if (__any_sync(0xffffffffu, some) && __any_sync(0xffffffffu, live)) break;
     }
-    some = __any_sync(0xffffffffu, some);
-    live = __any_sync(0xffffffffu, live);
-    if (lane == 0) {
-        s_some[warp] = some;
-        s_live[warp] = live;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int any_some = 0, any_live = 0;
-        for (int w = 0; w < kMaskThreads / 32; ++w) {
-            any_some |= s_some[w];
-            any_live |= s_live[w];
+    const bool any_some = __syncthreads_or(some), any_live = __syncthreads_or(live), any_low = __syncthreads_or(low);
+    bool lone = false;  // a row of a low tile that sees no ordinary key
+    if (!any_live && any_low) {
+        const int64_t last = min((int64_t)FM, a.Lq - r0);
+        for (int64_t r = warp; r < last && !lone; r += kMaskThreads / 32) {
+            const float *row = m + (r0 + r) * a.mask.sr;
+            const int64_t seen = a.causal ? min(a.Lk, r0 + r + a.diag + 1) : a.Lk;
+            if (seen <= 0) continue;
+            bool ordinary = __any_sync(0xffffffffu, __ldg(row + (seen - 1) * lane / 31) >= kMaskOrdinary);  // 32 keys spread evenly, then all
+            for (int64_t c = 0; c < seen && !ordinary; c += 32)
+                ordinary = __any_sync(0xffffffffu, c + lane < seen && __ldg(row + c + lane) >= kMaskOrdinary);
+            lone = !ordinary;
         }
-        a.kind[(plane * a.kind_rb + blockIdx.y) * a.kind_ld + blockIdx.x] = !any_live ? TILE_HIDDEN : (any_some ? TILE_ADD : TILE_CLEAR);
     }
+    lone = __syncthreads_or(lone);
+    if (threadIdx.x == 0)
+        a.kind[(plane * a.kind_rb + rb) * a.kind_ld + tile] = any_live ? (any_some ? TILE_ADD : TILE_CLEAR) : (lone ? TILE_ADD : TILE_HIDDEN);
 }
 
 template <int MODE, bool MASK>
@@ -452,8 +456,8 @@ fused_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         const int g = (warp - 2) >> 2, q = warp & 3, r = q * 32 + lane;
         const uint32_t t_lane = tmem_base + ((uint32_t)(q * 32) << 16);
         const uint32_t t_s = t_lane + g * FN, t_o = t_lane + kTmemO + g * 128;
-        const float c2 = a.scale_log2;
-        const uint64_t c22 = pack2(c2, c2);
+        float c2 = a.scale_log2;        // (1 for tiles that hold x already)
+        uint64_t c22 = pack2(c2, c2);
         uint8_t *prow = base_ptr + kOffP + g * kPTile + r * 128;  // row r of each 64-key chunk: 128 bytes, 16-byte units swizzled
         uint32_t s_it = 0, p_it = 0, o_it = 0;
         bool ok = true;
@@ -507,12 +511,18 @@ fused_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                 }
             };
             // MASK: the caller's additive mask (-inf hides a key) added to this warp's rows of the S~ tile where they lie, 16
-            // columns at a time, so that the steps above hold no mask values in registers; rows past the end and columns
-            // past the last key read nothing
+            // columns at a time, so that the steps below hold no mask values in registers; rows past the end and columns
+            // past the last key read nothing.  The tile then holds x = scaled logit + M in the log2 domain, rounded: equal
+            // sums give equal x, however large M is, so that x - max is what it would be in exact arithmetic (the product
+            // with the scale taken inside the subtraction leaves 2^-24 of x, which an M of -1e30 turns into infinities).
+            // A finite M stays finite.
             [[maybe_unused]] auto add_mask_tile = [&](int j) {
                 const int64_t c0 = (int64_t)j * FN;
                 const float *mrow = a.mask.p + (head / a.mask.seq_heads) * a.mask.sb + (head % a.mask.seq_heads) * a.mask.sh + (int64_t)i * a.mask.sr + c0;
-                const float gain = a.mask_gain;
+                auto log2_of = [&](float v) -> float {
+                    const float t = v * 1.4426950408889634f;
+                    return fabsf(t) < INFINITY || !(fabsf(v) < INFINITY) ? t : copysignf(FLT_MAX, t);
+                };
 #pragma unroll 1
                 for (int c = 0; c < FN; c += 16) {
                     float m4[16];
@@ -530,7 +540,7 @@ fused_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                     tmem_ld16_issue(t_s + c, s16);
                     tmem_ld_wait();
 #pragma unroll
-                    for (int e = 0; e < 16; ++e) s16[e] = __float_as_uint(fmaf(m4[e], gain, __uint_as_float(s16[e])));
+                    for (int e = 0; e < 16; ++e) s16[e] = __float_as_uint(fmaf(__uint_as_float(s16[e]), a.scale_log2, log2_of(m4[e])));
                     tmem_st16_issue(t_s + c, s16);
                 }
                 tmem_st_wait();
@@ -610,6 +620,8 @@ fused_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                 tc_fence_after();
                 if constexpr (MASK) {
                     if (add_mask) add_mask_tile(j);
+                    c2 = add_mask ? 1.f : a.scale_log2;
+                    c22 = pack2(c2, c2);
                 }
                 uint32_t v0[32], v1[32];
 
@@ -829,7 +841,7 @@ int launch_fused_attn(const __nv_bfloat16 *Qp, const __nv_bfloat16 *Kp, int64_t 
     if (mask != nullptr) {
         const int64_t planes = (mask->plane_step > 0 ? heads / mask->seq_heads : 1) * mask->plane_heads;
         if (kind_rb > 65535 || planes > 65535) return fail(RMM_ERR_UNSUPPORTED, "fused_attn: mask too large");
-        MaskTileArgs t = {*mask, Lq, Lk, diag, causal, mask->vec, (float)sqrt((double)Dh), tile_kind, kind_rb, kind_ld};
+        MaskTileArgs t = {*mask, Lq, Lk, diag, causal, mask->vec, tile_kind, kind_rb, kind_ld};
         prof_begin("mask_tiles_kernel", stream);
         launch_kernel(mask_tiles_kernel, dim3((unsigned)kind_ld, (unsigned)kind_rb, (unsigned)planes), dim3(kMaskThreads), 0, stream, 1, t);
         if ((rc = check_launch("mask_tiles_kernel", stream)) != RMM_OK) return rc;
@@ -860,7 +872,6 @@ int launch_fused_attn(const __nv_bfloat16 *Qp, const __nv_bfloat16 *Kp, int64_t 
             rc = launch_mode<MODE_GATHERED>(mq, mk, mv, a, "fused_attn_gathered_kernel", stream);
         } else if (mask != nullptr) {
             a.mask = *mask; a.tile_kind = tile_kind; a.kind_rb = kind_rb; a.kind_ld = kind_ld;
-            a.mask_gain = (float)sqrt((double)Dh);
             rc = launch_mode<MODE_FULL, true>(mq, mk, mv, a, "fused_attn_masked_kernel", stream);
         } else {
             rc = launch_mode<MODE_FULL>(mq, mk, mv, a, "fused_attn_kernel", stream);

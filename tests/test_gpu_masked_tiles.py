@@ -82,3 +82,49 @@ def test_masked_attention_folds_only_even_sequences(oracle):
     b = rmm.rmm_reduced_attn(dev(Q), dev(K), dev(V), True, 0.5, 1.0, mask=dev(M))
     assert torch.equal(a, b)
     assert check_attention(oracle, 3, 4, 2, 200, 200, 64, True, 0.5, 1.0, seed=172, mask=M)
+
+
+@pytest.mark.parametrize("L", [300, 301, 2052])                 # rows of whole vectors, rows of odd length, more than eight tiles
+@pytest.mark.parametrize("value", [torch.finfo(torch.float32).min, -1e30, -1e9, -1e4])
+def test_rows_that_see_nothing_but_large_finite_values(oracle, L, value):
+    """A finite mask value hides no key: rows that hold nothing else weigh their keys by the sums S~ + M as fp32 has them,
+    and rows with one ordinary key are as if -inf stood there.  Left padding: rows before n see padding keys only."""
+    n, B, Hq, Dh = 140, 2, 4, 64
+    M = torch.zeros(B, 1, L, L)
+    M[1, :, :, :n] = value
+    Q, K, V = synth.attention_qkv(B, Hq, 2, L, L, Dh, seed=173)
+    O, feat, _ = rmm.rmm_reduced_attn(dev(Q), dev(K), dev(V), True, 0.5, 1.0, want_idx=True, mask=dev(M))
+    low = M.double()
+    if value < -1e8:
+        low[low < 0] = HIDE
+    want = oracle.attn(Q, K, V, True, 0.5, 1.0, idx_feat=feat.cpu().numpy(), mask=low.numpy())[0]
+    if value < -1e10:                                            # S~ is lost next to the mask: equal weights
+        mean = (torch.cumsum(V[1].double(), 1) / torch.arange(1, L + 1)[:, None]).numpy()
+        want[1, :, :n] = np.repeat(mean, 2, axis=0)[:, :n]
+    got = O.float().cpu().numpy()
+    assert np.isfinite(got).all()
+    rows = np.linalg.norm(got - want, axis=3) / np.linalg.norm(want, axis=3)
+    if -1e10 < value < -1e8:                                     # S~ + M in steps of 64: not compared
+        rows[1, :, :n] = 0.0
+    # one rounding of P and one of O, 2^-9 each, over the row's norm; S~ + M in steps of 2^-10 at -1e4
+    assert rows.max() <= 2.5e-2, np.unravel_index(rows.argmax(), rows.shape)
+    assert rmm.rmm_status_read() == 0
+
+
+def test_low_tiles_are_skipped_only_where_every_row_has_another_key(oracle):
+    """One row of a block keeps its low values while the other rows' tiles could go."""
+    L, low = 384, torch.finfo(torch.float32).min
+    M = torch.zeros(1, 1, L, L)
+    M[..., :128] = low
+    M[0, 0, 200] = low                                           # the only row of its block without an ordinary key
+    M[0, 0, 300, 1:] = low                                       # its ordinary key: outside the evenly spread look
+    M[0, 0, 300, 0] = low
+    M[0, 0, 300, 131] = 0.5
+    Q, K, V = synth.attention_qkv(1, 2, 1, L, L, 128, seed=174)
+    O, feat, _ = rmm.rmm_reduced_attn(dev(Q), dev(K), dev(V), False, 0.5, 1.0, want_idx=True, mask=dev(M))
+    hide = M.double()
+    hide[hide < -1e30] = HIDE
+    want = oracle.attn(Q, K, V, False, 0.5, 1.0, idx_feat=feat.cpu().numpy(), mask=hide.numpy())[0]
+    want[0, :, 200] = V[0, 0].double().mean(0).numpy()
+    got = O.float().cpu().numpy()
+    assert (np.linalg.norm(got - want, axis=3) <= 2.5e-2 * np.linalg.norm(want, axis=3)).all()
