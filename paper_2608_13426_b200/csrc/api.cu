@@ -244,6 +244,17 @@ size_t rmm_reduced_gemm_workspace_bytes(const rmm_mat_t *A, const rmm_mat_t *B, 
     return gemm_simt_workspace_bytes(A, &b, k);
 }
 
+// What a call needs: the forms that cut the contraction axis do with fewer pieces in a smaller workspace.  (A caller's one
+// workspace may have been sized for another shape.)
+static size_t gemm_least_bytes(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k, const rmm_mat_t *Y)
+{
+    rmm_mat_t b = shared_b(A, B);
+    GemvPlan gplan;
+    if (gemv_eligible(A, &b, k, Y, &gplan)) return gplan.total_bytes;
+    TcPlan plan;
+    return tc_eligible(A, &b, k, Y, &plan) ? plan.least_bytes : (size_t)RMM_WS_HEADER_BYTES;
+}
+
 int rmm_reduced_gemm(const rmm_mat_t *A, const rmm_mat_t *B, const int32_t *idx, int64_t k, float scale,
                      const rmm_mat_t *Y, void *ws, size_t ws_bytes, void *stream)
 {
@@ -258,13 +269,13 @@ int rmm_reduced_gemm(const rmm_mat_t *A, const rmm_mat_t *B, const int32_t *idx,
     }
     TcPlan plan;
     if (tc_eligible(A, &b, k, Y, &plan)) {
-        rc = check_ws(ws, ws_bytes, plan.total_bytes, "reduced_gemm");
+        rc = check_ws(ws, ws_bytes, plan.least_bytes, "reduced_gemm");
         if (rc != RMM_OK) return rc;
-        return launch_gemm_tc(A, &b, idx, k, scale, Y, plan, ws, static_cast<cudaStream_t>(stream));
+        return launch_gemm_tc(A, &b, idx, k, scale, Y, plan, ws, ws_bytes, static_cast<cudaStream_t>(stream));
     }
-    rc = check_ws(ws, ws_bytes, gemm_simt_workspace_bytes(A, &b, k), "reduced_gemm");
+    rc = check_ws(ws, ws_bytes, RMM_WS_HEADER_BYTES, "reduced_gemm");
     if (rc != RMM_OK) return rc;
-    return launch_gemm_simt(A, &b, idx, k, scale, Y, ws, static_cast<cudaStream_t>(stream));
+    return launch_gemm_simt(A, &b, idx, k, scale, Y, ws, ws_bytes, static_cast<cudaStream_t>(stream));
 }
 
 // ---- 8-bit operands -------------------------------------------------------------------------------------
@@ -369,10 +380,11 @@ int rmm_reduced_gemm_scored(const rmm_mat_t *A, const rmm_mat_t *B, const int32_
     if (!gemv_eligible(A, &b, k, Y, &gplan) && tc_eligible(A, &b, k, Y, &plan, true) && plan.epilogue_energy && !(plan.gathers && idx != nullptr)) {
         rc = check_ws(ws, ws_bytes, plan.total_bytes, "reduced_gemm_scored");
         if (rc != RMM_OK) return rc;
-        return launch_gemm_tc(A, &b, idx, k, scale, Y, plan, ws, static_cast<cudaStream_t>(stream), energy_out);
+        return launch_gemm_tc(A, &b, idx, k, scale, Y, plan, ws, ws_bytes, static_cast<cudaStream_t>(stream), energy_out);
     }
     // every other form of the product: the output is scored by the ordinary pass once it has been written
-    rc = check_ws(ws, ws_bytes, rmm_reduced_gemm_scored_workspace_bytes(A, B, k, Y), "reduced_gemm_scored");
+    const size_t s1 = rmm_score_workspace_bytes(Y, 1), s2 = gemm_least_bytes(A, B, k, Y);
+    rc = check_ws(ws, ws_bytes, s1 > s2 ? s1 : s2, "reduced_gemm_scored");
     if (rc != RMM_OK) return rc;
     rc = rmm_reduced_gemm(A, B, idx, k, scale, Y, ws, ws_bytes, stream);
     if (rc != RMM_OK) return rc;
@@ -395,8 +407,8 @@ static int plan_product(const rmm_mat_t *A, const rmm_mat_t *B, const rmm_mat_t 
         return RMM_OK;
     }
     const size_t s1 = rmm_score_select_workspace_bytes(A, 1);
-    const size_t s2 = rmm_reduced_gemm_workspace_bytes(A, B, k, Y);
-    if (s1 == 0 || s2 == 0) return RMM_ERR_UNSUPPORTED;
+    const size_t s2 = gemm_least_bytes(A, B, k, Y);
+    if (s1 == 0) return RMM_ERR_UNSUPPORTED;
     pp->total = s1 > s2 ? s1 : s2;
     return RMM_OK;
 }
@@ -447,7 +459,7 @@ int rmm_product(const rmm_mat_t *A, const rmm_mat_t *B, double rho, int64_t k, f
             rc = launch_few_rows(A, sp, kk, idx, nullptr, nullptr, retained,
                                  reinterpret_cast<__nv_bfloat16 *>(static_cast<char *>(ws) + tc.off_ap), tc.ldp, st);
             if (rc != RMM_OK) return rc;
-            return launch_gemm_tc(A, &b, idx, kk, scale, Y, tc, ws, st, nullptr, true);
+            return launch_gemm_tc(A, &b, idx, kk, scale, Y, tc, ws, ws_bytes, st, nullptr, true);
         }
         rc = rmm_score_select(A, 1, rho, kk, idx, nullptr, nullptr, retained, ws, ws_bytes, stream);
         if (rc != RMM_OK) return rc;

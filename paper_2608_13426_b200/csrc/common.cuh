@@ -139,7 +139,8 @@ int launch_front(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k, int32_t *idx
 // ---- reduced GEMM ------------------------------------------------------------------------------------
 // Plain FMA kernel: any strides, bf16 or fp32 operands, fp32 accumulation, bf16 or fp32 output.
 int launch_gemm_simt(const rmm_mat_t *A, const rmm_mat_t *B, const int32_t *idx, int64_t k, float scale,
-                     const rmm_mat_t *Y, void *ws, cudaStream_t stream);
+                     const rmm_mat_t *Y, void *ws, size_t ws_bytes, cudaStream_t stream);
+// What the slices of the contraction axis want; a smaller workspace (down to the header) gets fewer slices.
 size_t gemm_simt_workspace_bytes(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k);
 
 // Decode-step path (M <= 4 rows of bf16 activations, B rows contiguous): HBM-bound gathered GEMV, no packing.
@@ -157,13 +158,16 @@ struct TcPlan {
     int64_t ldp;        // leading dimension of the packed operands (multiple of 8)
     bool gathers;       // with an index list the kernel fetches the kept rows of B itself (no column energies in that form)
     size_t off_ap, off_bp, off_colen, total_bytes;
+    size_t least_bytes;    // what a call needs: where the kernel gathers B, a workspace without room for all partial sums does with
+                           // fewer pieces, from the size on that the packed rows of B would take
     bool epilogue_energy;  // the plan reserves the per-group column energies of Y and the epilogue fills them
 };
 bool tc_eligible(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k, const rmm_mat_t *Y, TcPlan *plan, bool with_energy = false);
 // a_packed (plans that gather rows of B): A[:, I] is already in the workspace at plan.off_ap.
 // energy_out (with a plan made with_energy): also energy_out[b, c] = sum_i Y[b, i, c]^2 of the rounded outputs
 int launch_gemm_tc(const rmm_mat_t *A, const rmm_mat_t *B, const int32_t *idx, int64_t k, float scale,
-                   const rmm_mat_t *Y, const TcPlan &plan, void *ws, cudaStream_t stream, float *energy_out = nullptr, bool a_packed = false);
+                   const rmm_mat_t *Y, const TcPlan &plan, void *ws, size_t ws_bytes, cudaStream_t stream, float *energy_out = nullptr,
+                   bool a_packed = false);
 
 // A tensor-core problem on operands that are already in TMA-loadable form.
 struct TcProblem {
@@ -178,7 +182,8 @@ struct TcProblem {
     // kept rows b_idx[i * b_idx_stride + 0 .. k-1] itself (no packed copy of B; outputs of up to 128 rows)
     const int32_t *b_idx;
     int64_t b_idx_stride, b_rows;
-    float *partials;         // with b_idx: [2 x SMs][min(M, 128)][256] fp32 for the tiles whose contraction is cut
+    float *partials;         // with b_idx: room for the fp32 sums of pieces of the contraction; what does not fit is not cut
+    size_t partials_bytes;
     void *y;
     int y_bf16;
     int64_t y_sb, y_sr;

@@ -315,7 +315,8 @@ struct SimtPlan {
 // two and three blocks of 64 rows (three fit), 0.9, 1.9, 2.1, 2.2 and 2.3 us for one to five of 32 rows.  A round of blocks
 // costs about 2 us outside its steps, slices another 1.5 for their meeting.  (777 x 1500 kept x 1500: 230 us with one
 // slice, 134 with two, 119 with three, which the rule takes; 1500 x 2000 x 700: 231, 169, 120.)
-SimtPlan plan_simt(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k)
+// Slices whose partial sums take more than `room` bytes are not considered.
+SimtPlan plan_simt(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k, size_t room)
 {
     static const double step_us[2][5] = {{1.15, 2.4, 2.7}, {0.9, 1.9, 2.1, 2.2, 2.3}};
     SimtPlan best = {8, 1, ceil_div(k, BK) * BK};
@@ -327,6 +328,7 @@ SimtPlan plan_simt(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k)
         const double *t = step_us[tm == 8 ? 0 : 1];
         const int64_t tiles = simt_tiles(A, B, tm), most = simt_slices_max(tiles, k);
         for (int64_t s = 1; s <= most; ++s) {
+            if (s > 1 && (size_t)(tiles * s) * kHi * tm * BN * sizeof(float) > room) break;
             const int64_t per = ceil_div(steps, s), blocks = tiles * ceil_div(steps, per), full = blocks / (sms * fit);
             const int64_t rest = ceil_div(blocks - full * sms * fit, sms);
             const double cost = (double)full * ((double)per * t[fit - 1] + 2.0) + (rest > 0 ? (double)per * t[rest - 1] + 2.0 : 0.0) + (s > 1 ? 1.5 : 0.0);
@@ -362,9 +364,9 @@ size_t gemm_simt_workspace_bytes(const rmm_mat_t *A, const rmm_mat_t *B, int64_t
 }
 
 int launch_gemm_simt(const rmm_mat_t *A, const rmm_mat_t *B, const int32_t *idx, int64_t k, float scale,
-                     const rmm_mat_t *Y, void *ws, cudaStream_t stream)
+                     const rmm_mat_t *Y, void *ws, size_t ws_bytes, cudaStream_t stream)
 {
-    const SimtPlan plan = plan_simt(A, B, k);
+    const SimtPlan plan = plan_simt(A, B, k, ws_bytes - RMM_WS_HEADER_BYTES);
     SimtArgs a;
     a.A = A->ptr; a.B = B->ptr; a.Y = Y->ptr; a.idx = idx;
     a.M = A->rows; a.K = A->cols; a.N = B->cols; a.k = k;

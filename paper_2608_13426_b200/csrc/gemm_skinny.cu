@@ -199,15 +199,16 @@ struct SkinnyGrid {
 
 // Slices of the kept rows: the least (rounds of blocks over the GPU) x (groups a warp walks, and about four more for what
 // a block spends outside them) and, with more than one slice, four for their meeting; among one slice and the most that
-// make one or two rounds.
-SkinnyGrid skinny_grid(int64_t batch, int64_t N, int64_t k)
+// make one or two rounds.  No more than `fit` slices, which is what the workspace holds.
+SkinnyGrid skinny_grid(int64_t batch, int64_t N, int64_t k, int64_t fit)
 {
     SkinnyGrid g = {1, 1};
     const int64_t groups = ceil_div(k, 16), tiles = batch * ceil_div(N, CW), slots = (int64_t)sm_count() * kSkBlocks;
     int64_t best = INT64_MAX;
     for (int64_t rounds = 0; rounds <= 2; ++rounds) {
         int64_t s = rounds * slots / tiles;
-        const int64_t most = ceil_div(groups, 4 * kSkWarps);  // at least four groups a warp
+        int64_t most = ceil_div(groups, 4 * kSkWarps);  // at least four groups a warp
+        if (most > fit) most = fit > 1 ? fit : 1;
         s = s < 1 ? 1 : (s > most ? most : s);
         const int64_t per = ceil_div(groups, s), cost = ceil_div(tiles * ceil_div(groups, per), slots) * (ceil_div(per, kSkWarps) + 4) + (per < groups ? 4 : 0);
         if (cost < best) {
@@ -247,11 +248,10 @@ size_t gemm_skinny_partial_bytes(int64_t batch, int64_t M, int64_t N, int64_t k)
     return s <= 1 ? 0 : align_up((size_t)(batch * s * M * N) * 4, 256);
 }
 
-// p.a packed rows (zero between k and the pitch), p.b the unpacked B with the list p.b_idx, p.partials
-// gemm_skinny_partial_bytes().
+// p.a packed rows (zero between k and the pitch), p.b the unpacked B with the list p.b_idx.
 int launch_gemm_skinny(const TcProblem &p, cudaStream_t stream)
 {
-    const SkinnyGrid g = skinny_grid(p.batch, p.N, p.k);
+    const SkinnyGrid g = skinny_grid(p.batch, p.N, p.k, (int64_t)(p.partials_bytes / (size_t)(p.batch * p.M * p.N * 4)));
     SkinnyArgs a = {};
     a.ap = p.a; a.b = p.b; a.idx = p.b_idx; a.y = p.y;
     a.M = p.M; a.N = p.N; a.k = p.k; a.K = p.b_rows;

@@ -619,6 +619,14 @@ int launch_variant(const CUtensorMap &ma, const CUtensorMap &mb, const CUtensorM
 // Products of few rows fetch the kept rows of B inside the kernel (see the file header)
 bool gathers_b(const TcPlan &plan, int64_t M, int64_t N) { return !plan.b_kmajor && M <= 2 * BM && N > 128; }
 
+// Two slots (first and last piece) per block, and no more blocks than SMs or pairs of k-blocks: enough for every cut of up
+// to k kept rows.
+size_t gather_partial_bytes(int64_t batch, int64_t M, int64_t N, int64_t k)
+{
+    const int64_t pairs = ceil_div(batch * ceil_div(M, BM) * ceil_div(N, 256) * ceil_div(k, BK), 2), sms = sm_count();
+    return (size_t)(2 * (pairs < sms ? pairs : sms) * (M < BM ? M : BM)) * 256 * 4;
+}
+
 }  // namespace
 
 bool tc_eligible(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k, const rmm_mat_t *Y, TcPlan *plan, bool with_energy)
@@ -649,14 +657,17 @@ bool tc_eligible(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k, const rmm_ma
         off += align_up((size_t)batch * M * plan->ldp * 2, 256);
         plan->off_bp = off;  // packed B, or the sums of cut tiles
         plan->gathers = gathers_b(*plan, M, N);
-        if (plan->gathers && M <= kSkinnyRows) off += gemm_skinny_partial_bytes(batch, M, N, k);
-        else if (plan->gathers) off += (size_t)2 * sm_count() * (M < BM ? M : BM) * 256 * 4;
-        else off += align_up(b_kmajor ? (size_t)batch * N * plan->ldp * 2 : (size_t)batch * k * N * 2, 256);
+        const size_t packed_b = align_up(b_kmajor ? (size_t)batch * N * plan->ldp * 2 : (size_t)batch * k * N * 2, 256);
+        size_t third = packed_b;
+        if (plan->gathers && M <= kSkinnyRows) third = gemm_skinny_partial_bytes(batch, M, N, k);
+        else if (plan->gathers) third = gather_partial_bytes(batch, M, N, k);
+        off += third;
         // column energies from the epilogue: bf16 output with an even number of columns (the pairs are stored as float2)
         plan->epilogue_energy = with_energy && Y->dtype == RMM_BF16 && N % 2 == 0;
         plan->off_colen = off;
         if (plan->epilogue_energy) off += align_up((size_t)batch * ceil_div(M, 32) * N * 4, 256);
         plan->total_bytes = off;
+        plan->least_bytes = off - third + (third < packed_b ? third : packed_b);
     }
     return true;
 }
@@ -737,11 +748,11 @@ int launch_gemm_tc_problem(const TcProblem &p, cudaStream_t stream)
         a.seg_kb = ceil_div(n_tiles * num_kb, sms);
         if (a.seg_kb < 2) a.seg_kb = 2;
         const double whole = (double)(ceil_div(n_tiles, sms) * num_kb), cut = 1.27 * (double)a.seg_kb + 2.0 + 15.0 * (double)(p.M < BM ? p.M : BM) / BM;
-        if (whole <= cut) a.seg_kb = ceil_div(n_tiles, sms) * num_kb;
+        const size_t sums = (size_t)(2 * ceil_div(n_tiles * num_kb, a.seg_kb) * (p.M < BM ? p.M : BM)) * 256 * 4;
+        if (whole <= cut || sums > p.partials_bytes) a.seg_kb = ceil_div(n_tiles, sms) * num_kb;
         a.partials = p.partials;
-        if (p.col_energy != nullptr || p.partials == nullptr)
-            return fail(RMM_ERR_INVALID_ARG, "reduced_gemm_tc: the in-kernel row gather cuts tiles: it needs partial sums and leaves no column energies");
-        a.partials = p.partials;
+        if (p.col_energy != nullptr)
+            return fail(RMM_ERR_INVALID_ARG, "reduced_gemm_tc: the in-kernel row gather cuts tiles and leaves no column energies");
         if (p.b_kmajor || ctas != 1 || BN != 256)
             return fail(RMM_ERR_UNSUPPORTED, "reduced_gemm_tc: in-kernel row gather needs single-CTA 128 x 256 tiles and row-contiguous B");
         CUtensorMap my_g = ma;  // (the tensor map of B is unused in this form; A's stands in)
@@ -796,11 +807,11 @@ int launch_gemm_tc_problem(const TcProblem &p, cudaStream_t stream)
 }
 
 int launch_gemm_tc(const rmm_mat_t *A, const rmm_mat_t *B, const int32_t *idx, int64_t k, float scale,
-                   const rmm_mat_t *Y, const TcPlan &plan, void *ws, cudaStream_t stream, float *energy_out, bool a_packed)
+                   const rmm_mat_t *Y, const TcPlan &plan, void *ws, size_t ws_bytes, cudaStream_t stream, float *energy_out, bool a_packed)
 {
     if (energy_out != nullptr && plan.epilogue_energy) {
         // the product writes per-group column energies, a small kernel adds the groups up
-        int rc0 = launch_gemm_tc(A, B, idx, k, scale, Y, plan, ws, stream, nullptr);
+        int rc0 = launch_gemm_tc(A, B, idx, k, scale, Y, plan, ws, ws_bytes, stream, nullptr);
         if (rc0 != RMM_OK) return rc0;
         return launch_energy_combine(reinterpret_cast<const float *>(static_cast<char *>(ws) + plan.off_colen), A->batch,
                                      ceil_div(A->rows, 32), B->cols, energy_out, stream);
@@ -841,6 +852,7 @@ int launch_gemm_tc(const rmm_mat_t *A, const rmm_mat_t *B, const int32_t *idx, i
         else { p.b_sb = B->stride_batch; }
         p.b_idx = idx; p.b_idx_stride = k;
         p.partials = reinterpret_cast<float *>(w + plan.off_bp);
+        p.partials_bytes = ws_bytes > plan.off_bp ? ws_bytes - plan.off_bp : 0;
         if (!a_packed && (rc = launch_pack(specs, 1, status, stream)) != RMM_OK) return rc;
         if (idx != nullptr && M <= kSkinnyRows) return launch_gemm_skinny(p, stream);
         return launch_gemm_tc_problem(p, stream);
