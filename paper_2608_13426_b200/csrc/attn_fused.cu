@@ -115,7 +115,8 @@ __global__ void __launch_bounds__(kMaskThreads) mask_tiles_kernel(const MaskTile
 {
     pdl_wait();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t rb = blockIdx.y, tile = blockIdx.x, t0 = tile * FN, r0 = rb * FM, plane = blockIdx.z;
+    const unsigned rb = blockIdx.x / (unsigned)a.kind_ld, tile = blockIdx.x % (unsigned)a.kind_ld;
+    const int64_t t0 = (int64_t)tile * FN, r0 = (int64_t)rb * FM, plane = blockIdx.z;
     const float *m = a.mask.p + (plane / a.mask.plane_heads) * a.mask.sb + (plane % a.mask.plane_heads) * a.mask.sh;
     const int64_t rows = a.mask.sr == 0 ? 1 : min((int64_t)FM, a.Lq - r0);   // one row stands for all of them
     const bool beyond = t0 >= a.Lk || r0 >= a.Lq || (a.causal && t0 > min(a.Lq, r0 + FM) - 1 + a.diag);
@@ -840,10 +841,10 @@ int launch_fused_attn(const __nv_bfloat16 *Qp, const __nv_bfloat16 *Kp, int64_t 
     const int64_t kind_rb = 2 * ceil_div(Lq, kGroups * FM), kind_ld = ceil_div(Lk, FN * 8) * 8;
     if (mask != nullptr) {
         const int64_t planes = (mask->plane_step > 0 ? heads / mask->seq_heads : 1) * mask->plane_heads;
-        if (kind_rb > 65535 || planes > 65535) return fail(RMM_ERR_UNSUPPORTED, "fused_attn: mask too large");
+        if (kind_ld * kind_rb > INT32_MAX || planes > 65535) return fail(RMM_ERR_UNSUPPORTED, "fused_attn: mask too large");
         MaskTileArgs t = {*mask, Lq, Lk, diag, causal, mask->vec, tile_kind, kind_rb, kind_ld};
         prof_begin("mask_tiles_kernel", stream);
-        launch_kernel(mask_tiles_kernel, dim3((unsigned)kind_ld, (unsigned)kind_rb, (unsigned)planes), dim3(kMaskThreads), 0, stream, 1, t);
+        launch_kernel(mask_tiles_kernel, dim3((unsigned)(kind_ld * kind_rb), 1, (unsigned)planes), dim3(kMaskThreads), 0, stream, 1, t);
         if ((rc = check_launch("mask_tiles_kernel", stream)) != RMM_OK) return rc;
     }
     if ((rc = packed_map(&mq, Qp, kd, Lq, heads, ldd, FM)) != RMM_OK) return rc;

@@ -103,7 +103,7 @@ def test_rows_that_see_nothing_but_large_finite_values(oracle, L, value):
         want[1, :, :n] = np.repeat(mean, 2, axis=0)[:, :n]
     got = O.float().cpu().numpy()
     assert np.isfinite(got).all()
-    rows = np.linalg.norm(got - want, axis=3) / np.linalg.norm(want, axis=3)
+    rows = np.linalg.norm(got - want, axis=3) / np.maximum(np.linalg.norm(want, axis=3), 1e-30)
     if -1e10 < value < -1e8:                                     # S~ + M in steps of 64: not compared
         rows[1, :, :n] = 0.0
     # one rounding of P and one of O, 2^-9 each, over the row's norm; S~ + M in steps of 2^-10 at -1e4
@@ -128,3 +128,19 @@ def test_low_tiles_are_skipped_only_where_every_row_has_another_key(oracle):
     want[0, :, 200] = V[0, 0].double().mean(0).numpy()
     got = O.float().cpu().numpy()
     assert (np.linalg.norm(got - want, axis=3) <= 2.5e-2 * np.linalg.norm(want, axis=3)).all()
+
+
+def test_a_mask_over_more_row_blocks_than_a_grid_has_rows():
+    """65536 blocks of 128 queries; one mask row stands for all of them.  Every row's result is its own."""
+    Lq, Lk = 65536 * 128 + 5, 200
+    g = torch.Generator(device="cuda").manual_seed(175)
+    Q = torch.randn(1, 1, Lq, 8, generator=g, device="cuda").to(torch.bfloat16)
+    K, V = (torch.randn(1, 1, Lk, 8, generator=g, device="cuda").to(torch.bfloat16) for _ in range(2))
+    M = torch.zeros(1, 1, 1, Lk, device="cuda")
+    M[..., 130:] = HIDE
+    M[..., 7] = 1.5
+    O = rmm.rmm_reduced_attn(Q, K, V, False, 1.0, 1.0, mask=M)
+    for lo, hi in ((0, 300), (Lq // 2, Lq // 2 + 300), (Lq - 261, Lq)):
+        part = rmm.rmm_reduced_attn(Q[:, :, lo:hi], K, V, False, 1.0, 1.0, mask=M)
+        assert ((O[:, :, lo:hi].float() - part.float()).abs().max() <= 2.0 ** -7 * part.float().abs().max()).item()
+    assert rmm.rmm_status_read() == 0
