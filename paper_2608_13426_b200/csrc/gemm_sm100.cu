@@ -72,7 +72,7 @@ struct TcArgs {
     const __nv_bfloat16 *b_src;
     const int32_t *b_idx;
     int64_t b_ld, b_sb, b_idx_stride, b_rows;
-    int64_t seg_kb;              // k-blocks per block: the k-blocks of all tiles form one axis that is cut into equal shares
+    int64_t seg_kb;              // k-blocks per block: the k-blocks of all tiles form one axis that is cut into equal shares; 0: whole tiles
     float *partials;             // [2 x blocks][min(M, 128)][256] unscaled sums of the tiles that were cut
 };
 
@@ -138,10 +138,10 @@ reduced_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
     constexpr int UK = FP8 ? 2 * UMMA_K : UMMA_K;   // contraction indices per MMA instruction (32 bytes per row)
     static_assert(!FP8 || (B_KMAJOR && !B_GATHER), "8-bit operands: both K-major, packed");
     const int num_kb = (int)((a.k + BKE - 1) / BKE);
-    // The n-th piece of work of this block: k-blocks [kb0, kb1) of a tile.  Whole tiles, round robin; in the gather form
-    // what its share of the joint (tile, k-block) axis holds (only the first and the last of its tiles can be cut).
+    // The n-th piece of work of this block: k-blocks [kb0, kb1) of a tile.  Whole tiles, round robin; where the gather form
+    // cuts them, what its share of the joint (tile, k-block) axis holds (only the first and the last of its tiles are cut).
     auto piece = [&](int64_t n, int64_t &tile, int &kb0, int &kb1) -> bool {
-        if constexpr (B_GATHER) {
+        if (B_GATHER && a.seg_kb > 0) {
             const int64_t begin = (int64_t)blockIdx.x * a.seg_kb, end = min(num_tiles * num_kb, begin + a.seg_kb);
             const int64_t pos = n == 0 ? begin : (begin / num_kb + n) * num_kb;
             if (pos >= end) return false;
@@ -349,7 +349,9 @@ reduced_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
             const __nv_bfloat16 *bcol = a.b_src + bb * a.b_sb + (col < a.N ? col : 0);
             const uint32_t col_bytes = col < a.N ? 16u : 0u;
             const uint32_t lane_off = (uint32_t)(lane >> 3) * (BK * 128);
-            // row numbers: one load covers this warp's rows of four k-blocks (lane = k-block x row) and is issued four ahead
+            // row numbers: one load covers this warp's rows of four k-blocks (lane = k-block x row) and is issued four ahead;
+            // the lane that holds a number checks it.  Everything but the copies themselves is done before the wait for the
+            // stage: what runs between the wait and the copies is time in which the stage's bytes are not in flight
             static_assert(kRowsPerWarp == 8, "eight lanes per k-block");
             auto fetch_rows = [&](int kb) -> int {
                 const int64_t kk = (int64_t)(kb + (lane >> 3)) * BK + gw + kGatherWarps * (lane & 7);
@@ -360,19 +362,26 @@ reduced_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
                 if (((kb - kb0) & 3) == 0) {
                     rows = rows_next;
                     rows_next = fetch_rows(kb + 4);
+                    if (rows >= a.b_rows || (rows < 0 && kb + (lane >> 3) < kb1 && (int64_t)(kb + (lane >> 3)) * BK + gw + kGatherWarps * (lane & 7) < a.k)) {
+                        atomicExch(a.status, (int)RMM_ERR_BOUNDS);
+                        rows = -1;
+                    }
+                }
+                const __nv_bfloat16 *src[kRowsPerWarp];
+                unsigned live = 0;
+#pragma unroll
+                for (int i = 0; i < kRowsPerWarp; ++i) {
+                    const int row = __shfl_sync(0xffffffffu, rows, ((kb - kb0) & 3) * 8 + i);
+                    live |= row >= 0 ? 1u << i : 0u;
+                    src[i] = bcol + (row >= 0 ? (int64_t)row * a.b_ld : 0);
                 }
                 if (!mbar_wait(empty_bar(s), ph ^ 1u, abort_flag, a.status, a.wait_ns)) { ok = false; break; }
                 const uint32_t sb = base + s * L::kStageBytes + L::kABytes + lane_off;
 #pragma unroll
                 for (int i = 0; i < kRowsPerWarp; ++i) {
                     const int r = gw + kGatherWarps * i;
-                    int row = __shfl_sync(0xffffffffu, rows, ((kb - kb0) & 3) * 8 + i);
-                    if (row >= a.b_rows || (row < 0 && (int64_t)kb * BK + r < a.k)) {
-                        atomicExch(a.status, (int)RMM_ERR_BOUNDS);
-                        row = -1;
-                    }
                     const uint32_t dst = sb + r * 128 + (((uint32_t)(lane & 7) ^ (uint32_t)(r & 7)) << 4);
-                    cp_async_16(dst, row >= 0 ? bcol + (int64_t)row * a.b_ld : bcol, row >= 0 ? col_bytes : 0u);
+                    cp_async_16(dst, src[i], live >> i & 1u ? col_bytes : 0u);
                 }
                 cp_async_arrive_noinc(full_bar(s));
                 if (++s == kStages) { s = 0; ph ^= 1u; }
@@ -602,14 +611,14 @@ int launch_variant(const CUtensorMap &ma, const CUtensorMap &mb, const CUtensorM
     if (cudaError_t e = configured.smem(L::kTotal, kern)) return fail(RMM_ERR_CUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e));
     const int64_t tiles = a.batch * a.tiles_m * a.tiles_n, num_kb = ceil_div(a.k, FP8 ? 2 * BK : BK);
     const int64_t slots = sm_count() / CTAS;
-    const int64_t blocks = B_GATHER ? ceil_div(tiles * num_kb, a.seg_kb) : (tiles < slots ? tiles : slots);
+    const int64_t blocks = B_GATHER && a.seg_kb > 0 ? ceil_div(tiles * num_kb, a.seg_kb) : (tiles < slots ? tiles : slots);
     prof_begin("reduced_gemm_tc_kernel", stream);
     cudaError_t e = launch_kernel(kern, dim3((unsigned)(blocks * CTAS)),
                                   dim3(B_GATHER ? kThreadsTc + 32 * kGatherWarps : (a.epi_sets == 2 ? kThreadsTc2 : kThreadsTc)), L::kTotal, stream,
                                   CTAS, ma, mb, my, a);
     if (e != cudaSuccess) return fail(RMM_ERR_CUDA, "reduced_gemm_tc_kernel: launch: %s", cudaGetErrorString(e));
     int rc = check_launch("reduced_gemm_tc_kernel", stream);
-    if (!B_GATHER || rc != RMM_OK || a.seg_kb % num_kb == 0) return rc;
+    if (!B_GATHER || rc != RMM_OK || a.seg_kb == 0) return rc;
     prof_begin("gemm_meet_kernel", stream);
     launch_kernel(gemm_meet_kernel<OUT_BF16>, dim3((unsigned)tiles, (unsigned)ceil_div(a.M < BM ? a.M : BM, kMeetRows)), dim3(32 * kMeetRows), 0,
                   stream, 1, a, (int)num_kb);
@@ -749,7 +758,7 @@ int launch_gemm_tc_problem(const TcProblem &p, cudaStream_t stream)
         if (a.seg_kb < 2) a.seg_kb = 2;
         const double whole = (double)(ceil_div(n_tiles, sms) * num_kb), cut = 1.27 * (double)a.seg_kb + 2.0 + 15.0 * (double)(p.M < BM ? p.M : BM) / BM;
         const size_t sums = (size_t)(2 * ceil_div(n_tiles * num_kb, a.seg_kb) * (p.M < BM ? p.M : BM)) * 256 * 4;
-        if (whole <= cut || sums > p.partials_bytes) a.seg_kb = ceil_div(n_tiles, sms) * num_kb;
+        if (whole <= cut || a.seg_kb % num_kb == 0 || sums > p.partials_bytes || p.col_energy != nullptr) a.seg_kb = 0;
         a.partials = p.partials;
         if (p.col_energy != nullptr)
             return fail(RMM_ERR_INVALID_ARG, "reduced_gemm_tc: the in-kernel row gather cuts tiles and leaves no column energies");
