@@ -750,13 +750,15 @@ int launch_gemm_tc_problem(const TcProblem &p, cudaStream_t stream)
     if (p.b_idx != nullptr) {
         // A product of few rows is bound by how fast the SMs pull rows of B, so none may idle: equal shares of all tiles'
         // k-blocks, one per SM (at least two k-blocks each), where whole tiles would leave too many without work.  Cutting
-        // costs the partial sums (measured, in k-blocks of 0.94 us: 2 + 15 for 128 rows) and a k-block takes 1.27 times as
-        // long with every SM pulling.  48 x 28672 (half kept) x 8192, 32 tiles: 216 us whole, 70 cut; 128 x 8192 (a quarter)
-        // x 28672, 112 tiles: 41.6 whole, 54 cut.
+        // costs the partial sums and their meeting (measured, in k-blocks of 0.94 us: 4 + 15 for 128 rows and 0.4 more for each
+        // piece of a tile) and a k-block takes 1.27 of them with every SM pulling, 0.88 with whole tiles.  Whole calls, a quarter
+        // or half of the rows kept: 48 x 28672 (half) x 8192, 32 tiles: 75 us cut; 128 x 8192 (a quarter) x 8192: 42 cut, 32
+        // whole; 48 x 8192 (half) x 28672, 112 tiles: 64.5 whole.
         const int64_t num_kb = ceil_div(p.k, (int64_t)BK), sms = sm_count();
         a.seg_kb = ceil_div(n_tiles * num_kb, sms);
         if (a.seg_kb < 2) a.seg_kb = 2;
-        const double whole = (double)(ceil_div(n_tiles, sms) * num_kb), cut = 1.27 * (double)a.seg_kb + 2.0 + 15.0 * (double)(p.M < BM ? p.M : BM) / BM;
+        const double whole = 0.88 * (double)(ceil_div(n_tiles, sms) * num_kb), pieces = (double)num_kb / (double)a.seg_kb;
+        const double cut = 1.27 * (double)a.seg_kb + 4.0 + (15.0 + 0.4 * pieces) * (double)(p.M < BM ? p.M : BM) / BM;
         const size_t sums = (size_t)(2 * ceil_div(n_tiles * num_kb, a.seg_kb) * (p.M < BM ? p.M : BM)) * 256 * 4;
         if (whole <= cut || a.seg_kb % num_kb == 0 || sums > p.partials_bytes || p.col_energy != nullptr) a.seg_kb = 0;
         a.partials = p.partials;
