@@ -157,6 +157,7 @@ struct TcPlan {
     int b_kmajor;       // 0: B rows (contraction slices) contiguous, kept rows copied; 1: B is K-contiguous, packed like A
     int64_t ldp;        // leading dimension of the packed operands (multiple of 8)
     bool gathers;       // with an index list the kernel fetches the kept rows of B itself (no column energies in that form)
+    bool few_rows;      // gathers, by the kernel for few rows (gemm_skinny.cu)
     size_t off_ap, off_bp, off_colen, total_bytes;
     size_t least_bytes;    // what a call needs: where the kernel gathers B, a workspace without room for all partial sums does with
                            // fewer pieces, from the size on that the packed rows of B would take

@@ -628,6 +628,19 @@ int launch_variant(const CUtensorMap &ma, const CUtensorMap &mb, const CUtensorM
 // Products of few rows fetch the kept rows of B inside the kernel (see the file header)
 bool gathers_b(const TcPlan &plan, int64_t M, int64_t N) { return !plan.b_kmajor && M <= 2 * BM && N > 128; }
 
+// The few-row kernel (gemm_skinny.cu) or 128-row tiles?  Up to 24 rows the former throughout (behind the kernel that selects and
+// packs A it starts sooner); with a fourth tile of eight rows it falls behind whole tiles that nearly fill the GPU, the more so where
+// its own 128-column blocks fill one block an SM but not two.  Estimates in microseconds, gather of A included (32 x 8192 x
+// 28672, a quarter and half kept: 46 and 75 us by the few-row kernel, 40 and 64.5 by whole tiles; 32 x 4096 x 20000, half: 46 and 42).
+bool few_rows_win(int64_t batch, int64_t M, int64_t N, int64_t k)
+{
+    const int64_t tiles = batch * ceil_div(N, 256), sms = sm_count();
+    if (M <= 24 || M > kSkinnyRows || 2 * tiles < sms) return M <= kSkinnyRows;
+    const int64_t blocks = batch * ceil_div(N, 128);
+    const double rate = blocks > sms && blocks < 2 * sms ? 3.5e6 : 4.3e6, few = 1.1 * (15.0 + 2.0 * (double)(batch * k * N) / rate);
+    return few + 2.0 <= 13.0 + 0.85 * (double)(ceil_div(tiles, sms) * ceil_div(k, BK));
+}
+
 // Two slots (first and last piece) per block, and no more blocks than SMs or pairs of k-blocks: enough for every cut of up
 // to k kept rows.
 size_t gather_partial_bytes(int64_t batch, int64_t M, int64_t N, int64_t k)
@@ -666,9 +679,10 @@ bool tc_eligible(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k, const rmm_ma
         off += align_up((size_t)batch * M * plan->ldp * 2, 256);
         plan->off_bp = off;  // packed B, or the sums of cut tiles
         plan->gathers = gathers_b(*plan, M, N);
+        plan->few_rows = plan->gathers && few_rows_win(batch, M, N, k);
         const size_t packed_b = align_up(b_kmajor ? (size_t)batch * N * plan->ldp * 2 : (size_t)batch * k * N * 2, 256);
         size_t third = packed_b;
-        if (plan->gathers && M <= kSkinnyRows) third = gemm_skinny_partial_bytes(batch, M, N, k);
+        if (plan->few_rows) third = gemm_skinny_partial_bytes(batch, M, N, k);
         else if (plan->gathers) third = gather_partial_bytes(batch, M, N, k);
         off += third;
         // column energies from the epilogue: bf16 output with an even number of columns (the pairs are stored as float2)
@@ -865,7 +879,7 @@ int launch_gemm_tc(const rmm_mat_t *A, const rmm_mat_t *B, const int32_t *idx, i
         p.partials = reinterpret_cast<float *>(w + plan.off_bp);
         p.partials_bytes = ws_bytes > plan.off_bp ? ws_bytes - plan.off_bp : 0;
         if (!a_packed && (rc = launch_pack(specs, 1, status, stream)) != RMM_OK) return rc;
-        if (idx != nullptr && M <= kSkinnyRows) return launch_gemm_skinny(p, stream);
+        if (idx != nullptr && plan.few_rows) return launch_gemm_skinny(p, stream);
         return launch_gemm_tc_problem(p, stream);
     }
     if (plan.b_kmajor) {

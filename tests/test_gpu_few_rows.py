@@ -50,3 +50,14 @@ def test_few_rows_batches_strides_and_bad_indices(M):
     Y = rmm.rmm_reduced_gemm(A[0].cuda(), B[0].cuda(), bad.int().cuda(), out_dtype=torch.float32)
     assert torch.equal(Y.cpu(), A[0][:, lists[0][keep]].float() @ B[0][lists[0][keep]].float())
     assert rmm.rmm_status_read() == 6
+
+
+@pytest.mark.parametrize("M", [24, 25, 32])
+@pytest.mark.parametrize("k", [40, 111, 600])
+def test_wide_outputs_by_either_kernel_are_exact_on_whole_numbers(M, k):
+    """19208 columns: from 25 rows on whole 128-row tiles take over, for the longer of these contractions."""
+    A, B = ints((M, 700), 6), ints((700, 19208), 7)
+    idx = torch.randperm(700, generator=torch.Generator().manual_seed(8))[:k].sort().values
+    Y = rmm.rmm_reduced_gemm(A.cuda(), B.cuda(), idx.int().cuda(), out_dtype=torch.float32)
+    assert torch.equal(Y.cpu(), A[:, idx].float() @ B[idx].float())
+    assert rmm.rmm_status_read() == 0
