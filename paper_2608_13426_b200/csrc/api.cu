@@ -350,21 +350,33 @@ int rmm_reduced_gemm_q8(const rmm_mat_t *A, const rmm_mat_t *B, float b_scale, c
 }
 
 // ---- product that also scores its output ---------------------------------------------------------------
+// Outputs of up to 256 rows whose kernel fetches the kept rows of B (plan.gathers): is a pass over Y worth what the product
+// gains by cutting the contraction, or by the few-row kernel, neither of which leaves column energies?  Estimates in
+// microseconds, gather of A included, fitted to calls of 5 to 256 rows on 256 to 28672 columns (24 x 8192, half kept, x 28672: 89 us with the
+// pass, 67 without; x 8192: 41 and 61).
+static bool scored_apart(int64_t batch, int64_t M, int64_t N, int64_t k)
+{
+    const double tiles = (double)(batch * ceil_div(M, 128) * ceil_div(N, 256)), kb = (double)ceil_div(k, 64), sms = (double)sm_count();
+    const double whole = 13.0 + 0.85 * kb * ceil(tiles / sms), pass = 5.5 + (double)(batch * N) / 2300.0;
+    const double share = fmax(2.0, ceil(tiles * kb / sms)), rows = (double)(M < 128 ? M : 128) / 128.0;
+    const double few = 15.0 + 2.0 * (double)(batch * k * N) / 4.3e6, cut = 13.0 + 0.94 * (1.27 * share + 4.0 + (15.0 + 0.4 * kb / share) * rows);
+    return (M <= kSkinnyRows ? few : cut) + pass < whole + 1.0;
+}
+
 size_t rmm_reduced_gemm_scored_workspace_bytes(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k, const rmm_mat_t *Y)
 {
     if (A == nullptr || B == nullptr || Y == nullptr) return 0;
     rmm_mat_t b = shared_b(A, B);
     GemvPlan gplan;
     TcPlan plan;
-    size_t need;
-    if (!gemv_eligible(A, &b, k, Y, &gplan) && tc_eligible(A, &b, k, Y, &plan, true)) {
-        if (plan.epilogue_energy && !plan.gathers) return plan.total_bytes;
+    size_t need = 0;
+    if (!gemv_eligible(A, &b, k, Y, &gplan) && tc_eligible(A, &b, k, Y, &plan, true) && plan.epilogue_energy) {
         need = plan.total_bytes;
-    } else {
-        need = rmm_reduced_gemm_workspace_bytes(A, B, k, Y);
+        if (!plan.gathers || !scored_apart(A->batch, A->rows, B->cols, k)) return need;
     }
-    const size_t s = rmm_score_workspace_bytes(Y, 1);  // the output is scored by a pass of its own
-    if (need == 0 || s == 0) return 0;
+    const size_t p = rmm_reduced_gemm_workspace_bytes(A, B, k, Y), s = rmm_score_workspace_bytes(Y, 1);  // the output is scored by a pass of its own
+    if (p == 0 || s == 0) return 0;
+    if (p > need) need = p;
     return need > s ? need : s;
 }
 
@@ -375,16 +387,17 @@ int rmm_reduced_gemm_scored(const rmm_mat_t *A, const rmm_mat_t *B, const int32_
     int rc = check_gemm(A, B, idx, k, Y);
     if (rc != RMM_OK) return rc;
     rmm_mat_t b = shared_b(A, B);
+    const size_t s1 = rmm_score_workspace_bytes(Y, 1), s2 = gemm_least_bytes(A, B, k, Y), apart = s1 > s2 ? s1 : s2;
     GemvPlan gplan;
     TcPlan plan;
-    if (!gemv_eligible(A, &b, k, Y, &gplan) && tc_eligible(A, &b, k, Y, &plan, true) && plan.epilogue_energy && !(plan.gathers && idx != nullptr)) {
-        rc = check_ws(ws, ws_bytes, plan.total_bytes, "reduced_gemm_scored");
+    if (!gemv_eligible(A, &b, k, Y, &gplan) && tc_eligible(A, &b, k, Y, &plan, true) && plan.epilogue_energy &&
+        !(plan.gathers && idx != nullptr && ws_bytes >= apart && scored_apart(A->batch, A->rows, B->cols, k))) {
+        rc = check_ws(ws, ws_bytes, plan.least_bytes, "reduced_gemm_scored");
         if (rc != RMM_OK) return rc;
         return launch_gemm_tc(A, &b, idx, k, scale, Y, plan, ws, ws_bytes, static_cast<cudaStream_t>(stream), energy_out);
     }
     // every other form of the product: the output is scored by the ordinary pass once it has been written
-    const size_t s1 = rmm_score_workspace_bytes(Y, 1), s2 = gemm_least_bytes(A, B, k, Y);
-    rc = check_ws(ws, ws_bytes, s1 > s2 ? s1 : s2, "reduced_gemm_scored");
+    rc = check_ws(ws, ws_bytes, apart, "reduced_gemm_scored");
     if (rc != RMM_OK) return rc;
     rc = rmm_reduced_gemm(A, B, idx, k, scale, Y, ws, ws_bytes, stream);
     if (rc != RMM_OK) return rc;

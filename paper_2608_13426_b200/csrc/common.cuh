@@ -156,7 +156,7 @@ int launch_gemv(const rmm_mat_t *A, const rmm_mat_t *B, const int32_t *idx, int6
 struct TcPlan {
     int b_kmajor;       // 0: B rows (contraction slices) contiguous, kept rows copied; 1: B is K-contiguous, packed like A
     int64_t ldp;        // leading dimension of the packed operands (multiple of 8)
-    bool gathers;       // with an index list the kernel fetches the kept rows of B itself (no column energies in that form)
+    bool gathers;       // with an index list the kernel fetches the kept rows of B itself (column energies: from whole tiles only)
     bool few_rows;      // gathers, by the kernel for few rows (gemm_skinny.cu)
     size_t off_ap, off_bp, off_colen, total_bytes;
     size_t least_bytes;    // what a call needs: where the kernel gathers B, a workspace without room for all partial sums does with

@@ -681,12 +681,13 @@ bool tc_eligible(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k, const rmm_ma
         plan->gathers = gathers_b(*plan, M, N);
         plan->few_rows = plan->gathers && few_rows_win(batch, M, N, k);
         const size_t packed_b = align_up(b_kmajor ? (size_t)batch * N * plan->ldp * 2 : (size_t)batch * k * N * 2, 256);
+        // column energies from the epilogue: bf16 output with an even number of columns (the pairs are stored as float2), whole tiles
+        plan->epilogue_energy = with_energy && Y->dtype == RMM_BF16 && N % 2 == 0;
         size_t third = packed_b;
-        if (plan->few_rows) third = gemm_skinny_partial_bytes(batch, M, N, k);
+        if (plan->gathers && plan->epilogue_energy) third = 0;
+        else if (plan->few_rows) third = gemm_skinny_partial_bytes(batch, M, N, k);
         else if (plan->gathers) third = gather_partial_bytes(batch, M, N, k);
         off += third;
-        // column energies from the epilogue: bf16 output with an even number of columns (the pairs are stored as float2)
-        plan->epilogue_energy = with_energy && Y->dtype == RMM_BF16 && N % 2 == 0;
         plan->off_colen = off;
         if (plan->epilogue_energy) off += align_up((size_t)batch * ceil_div(M, 32) * N * 4, 256);
         plan->total_bytes = off;
@@ -776,8 +777,6 @@ int launch_gemm_tc_problem(const TcProblem &p, cudaStream_t stream)
         const size_t sums = (size_t)(2 * ceil_div(n_tiles * num_kb, a.seg_kb) * (p.M < BM ? p.M : BM)) * 256 * 4;
         if (whole <= cut || a.seg_kb % num_kb == 0 || sums > p.partials_bytes || p.col_energy != nullptr) a.seg_kb = 0;
         a.partials = p.partials;
-        if (p.col_energy != nullptr)
-            return fail(RMM_ERR_INVALID_ARG, "reduced_gemm_tc: the in-kernel row gather cuts tiles and leaves no column energies");
         if (p.b_kmajor || ctas != 1 || BN != 256)
             return fail(RMM_ERR_UNSUPPORTED, "reduced_gemm_tc: in-kernel row gather needs single-CTA 128 x 256 tiles and row-contiguous B");
         CUtensorMap my_g = ma;  // (the tensor map of B is unused in this form; A's stands in)
@@ -879,7 +878,7 @@ int launch_gemm_tc(const rmm_mat_t *A, const rmm_mat_t *B, const int32_t *idx, i
         p.partials = reinterpret_cast<float *>(w + plan.off_bp);
         p.partials_bytes = ws_bytes > plan.off_bp ? ws_bytes - plan.off_bp : 0;
         if (!a_packed && (rc = launch_pack(specs, 1, status, stream)) != RMM_OK) return rc;
-        if (idx != nullptr && plan.few_rows) return launch_gemm_skinny(p, stream);
+        if (idx != nullptr && plan.few_rows && !plan.epilogue_energy) return launch_gemm_skinny(p, stream);
         return launch_gemm_tc_problem(p, stream);
     }
     if (plan.b_kmajor) {

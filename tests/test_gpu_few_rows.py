@@ -1,8 +1,10 @@
 """Products of 5 to 256 rows that fetch the kept rows of B themselves (gemm_skinny.cu, the cut tiles of gemm_sm100.cu)."""
+import numpy as np
 import pytest
 import torch
 
 import paper_2608_13426_b200 as rmm
+from paper_2608_13426_b200 import binding, synth
 
 pytestmark = pytest.mark.gpu
 
@@ -60,4 +62,29 @@ def test_wide_outputs_by_either_kernel_are_exact_on_whole_numbers(M, k):
     idx = torch.randperm(700, generator=torch.Generator().manual_seed(8))[:k].sort().values
     Y = rmm.rmm_reduced_gemm(A.cuda(), B.cuda(), idx.int().cuda(), out_dtype=torch.float32)
     assert torch.equal(Y.cpu(), A[:, idx].float() @ B[idx].float())
+    assert rmm.rmm_status_read() == 0
+
+
+@pytest.mark.parametrize("M, K, N, k, apart", [
+    (64, 1024, 28672, 512, False),     # tiles enough for the GPU: the epilogue leaves the energies
+    (200, 512, 264, 100, False),       # two row tiles, a last tile of eight columns, a ragged k-block
+    (24, 1024, 14336, 512, False),     # few rows, as above
+    (24, 4096, 2048, 2048, True),      # the few-row kernel and a pass over Y
+    (48, 8192, 2048, 4096, True),      # cut tiles and a pass over Y
+])
+def test_scored_products_of_few_rows_keep_their_energies_where_tiles_are_whole(oracle, M, K, N, k, apart):
+    A, B = synth.mlp_product(M, K, N, seed=M + k)
+    idx = torch.randperm(K, generator=torch.Generator().manual_seed(k))[:k].sort().values.int()
+    Ad, Bd, ix = A.cuda(), B.cuda(), idx.cuda()
+    rmm.rmm_reduced_gemm(Ad, Bd, ix, want_energy=True)
+    timer = binding.KernelTimer(16)
+    with timer:
+        Y, e = rmm.rmm_reduced_gemm(Ad, Bd, ix, want_energy=True)
+    assert any("score" in name for name, _ in timer.times_ms()) == apart
+    cols = np.r_[0:min(N, 300), N - 40:N]
+    want = oracle.reduced_gemm(A, B[:, cols].contiguous(), idx.numpy())
+    got = Y.float().cpu().numpy()
+    assert np.linalg.norm(got[:, cols] - want) <= 1e-2 * np.linalg.norm(want)
+    # exact squares, fp32 chains of 16: 16 roundings of 2^-24 at most
+    assert np.allclose(e.cpu().numpy(), (got.astype(np.float64) ** 2).sum(0), rtol=1e-6, atol=0)
     assert rmm.rmm_status_read() == 0
