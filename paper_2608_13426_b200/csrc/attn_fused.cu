@@ -53,6 +53,7 @@ constexpr int kOffQ = 0, kOffKv = kGroups * kQTile, kOffP = kOffKv + kKvStages *
 constexpr int kFusedSmem = kOffBar + 512;
 constexpr int kTmemCols = 512;        // per group: S~ (128 columns); then O (128 columns per group)
 constexpr uint32_t kTmemO = kGroups * FN;
+constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kGrowLimit = 40.f;    // log2 of the largest p taken against a stale maximum
 
 // Debug aid (-DRMM_ATTN_STAMPS): clocks spent per phase by the MMA issuer of group 0 and by one softmax warp of
@@ -113,6 +114,8 @@ struct MaskTileArgs {
 
 __global__ void __launch_bounds__(kMaskThreads) mask_tiles_kernel(const MaskTileArgs a)
 {
+    __shared__ int s_seen[kMaskThreads / 32];
+    static_assert(kMaskThreads == FM, "a thread per row of the tile");
     pdl_wait();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned rb = blockIdx.x / (unsigned)a.kind_ld, tile = blockIdx.x % (unsigned)a.kind_ld;
@@ -150,23 +153,43 @@ __global__ void __launch_bounds__(kMaskThreads) mask_tiles_kernel(const MaskTile
         }
         if (__any_sync(0xffffffffu, some) && __any_sync(0xffffffffu, live)) break;
     }
-    const bool any_some = __syncthreads_or(some), any_live = __syncthreads_or(live), any_low = __syncthreads_or(low);
-    bool lone = false;  // a row of a low tile that sees no ordinary key
-    if (!any_live && any_low) {
-        const int64_t last = min((int64_t)FM, a.Lq - r0);
-        for (int64_t r = warp; r < last && !lone; r += kMaskThreads / 32) {
-            const float *row = m + (r0 + r) * a.mask.sr;
-            const int64_t seen = a.causal ? min(a.Lk, r0 + r + a.diag + 1) : a.Lk;
-            if (seen <= 0) continue;
-            bool ordinary = __any_sync(0xffffffffu, __ldg(row + (seen - 1) * lane / 31) >= kMaskOrdinary);  // 32 keys spread evenly, then all
-            for (int64_t c = 0; c < seen && !ordinary; c += 32)
-                ordinary = __any_sync(0xffffffffu, c + lane < seen && __ldg(row + c + lane) >= kMaskOrdinary);
+    const bool w_some = __any_sync(0xffffffffu, some), w_live = __any_sync(0xffffffffu, live), w_low = __any_sync(0xffffffffu, low);
+    if (lane == 0) s_seen[warp] = (w_some ? 1 : 0) | (w_live ? 2 : 0) | (w_low ? 4 : 0);
+    __syncthreads();
+    int seen = 0;
+#pragma unroll
+    for (int w = 0; w < kMaskThreads / 32; ++w) seen |= s_seen[w];
+    int kind = seen & 2 ? (seen & 1 ? TILE_ADD : TILE_CLEAR) : TILE_HIDDEN;
+    if ((seen & 6) == 4) {  // (block-uniform) low values only: does every row see an ordinary key?
+        // a row per thread looks at four keys: the first, the last that it sees and two between; what that leaves open is
+        // read row by row, until a row has no such key
+        const int64_t r = r0 + threadIdx.x, visible = a.causal ? min(a.Lk, r + a.diag + 1) : a.Lk;
+        const float *row = m + r * a.mask.sr;
+        bool open = r < a.Lq && visible > 0;
+        if (open) {
+            float v[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) v[i] = __ldg(row + (visible - 1) * i / 3);
+            open = !(fmaxf(fmaxf(v[0], v[1]), fmaxf(v[2], v[3])) >= kMaskOrdinary);
+        }
+        bool lone = false;
+        for (unsigned left = __ballot_sync(0xffffffffu, open); left != 0 && !lone; left &= left - 1) {
+            const int src = __ffs(left) - 1;
+            const int64_t rr = r0 + warp * 32 + src, vis = a.causal ? min(a.Lk, rr + a.diag + 1) : a.Lk;
+            const float *p = m + rr * a.mask.sr;
+            bool ordinary = false;
+            for (int64_t c = 0; c < vis && !ordinary; c += 256) {
+                float top = -INFINITY;
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+                    if (c + 32 * i + lane < vis) top = fmaxf(top, __ldg(p + c + 32 * i + lane));
+                ordinary = __any_sync(0xffffffffu, top >= kMaskOrdinary);
+            }
             lone = !ordinary;
         }
+        if (__syncthreads_or(lone)) kind = TILE_ADD;
     }
-    lone = __syncthreads_or(lone);
-    if (threadIdx.x == 0)
-        a.kind[(plane * a.kind_rb + rb) * a.kind_ld + tile] = any_live ? (any_some ? TILE_ADD : TILE_CLEAR) : (lone ? TILE_ADD : TILE_HIDDEN);
+    if (threadIdx.x == 0) a.kind[(plane * a.kind_rb + rb) * a.kind_ld + tile] = (uint8_t)kind;
 }
 
 template <int MODE, bool MASK>
@@ -516,14 +539,10 @@ fused_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             // past the last key read nothing.  The tile then holds x = scaled logit + M in the log2 domain, rounded: equal
             // sums give equal x, however large M is, so that x - max is what it would be in exact arithmetic (the product
             // with the scale taken inside the subtraction leaves 2^-24 of x, which an M of -1e30 turns into infinities).
-            // A finite M stays finite.
+            // A low finite M stays finite.
             [[maybe_unused]] auto add_mask_tile = [&](int j) {
                 const int64_t c0 = (int64_t)j * FN;
                 const float *mrow = a.mask.p + (head / a.mask.seq_heads) * a.mask.sb + (head % a.mask.seq_heads) * a.mask.sh + (int64_t)i * a.mask.sr + c0;
-                auto log2_of = [&](float v) -> float {
-                    const float t = v * 1.4426950408889634f;
-                    return fabsf(t) < INFINITY || !(fabsf(v) < INFINITY) ? t : copysignf(FLT_MAX, t);
-                };
 #pragma unroll 1
                 for (int c = 0; c < FN; c += 16) {
                     float m4[16];
@@ -541,7 +560,11 @@ fused_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                     tmem_ld16_issue(t_s + c, s16);
                     tmem_ld_wait();
 #pragma unroll
-                    for (int e = 0; e < 16; ++e) s16[e] = __float_as_uint(fmaf(__uint_as_float(s16[e]), a.scale_log2, log2_of(m4[e])));
+                    for (int e = 0; e < 16; ++e) {
+                        float t = m4[e] * kLog2e;
+                        if (m4[e] >= -FLT_MAX) t = fmaxf(t, -FLT_MAX);
+                        s16[e] = __float_as_uint(fmaf(__uint_as_float(s16[e]), a.scale_log2, t));
+                    }
                     tmem_st16_issue(t_s + c, s16);
                 }
                 tmem_st_wait();
