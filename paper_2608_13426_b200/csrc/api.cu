@@ -328,7 +328,7 @@ int rmm_reduced_gemm_q8(const rmm_mat_t *A, const rmm_mat_t *B, float b_scale, c
     int *status = &reinterpret_cast<WsHeader *>(w)->status;
     uint8_t *Aq = reinterpret_cast<uint8_t *>(w + q.off_aq), *Bq = reinterpret_cast<uint8_t *>(w + q.off_bq);
     float *row_scale = a_scale != nullptr ? a_scale : reinterpret_cast<float *>(w + q.off_scale);
-    if (gather_q8_streams(A->cols, q.ldq)) {
+    if (gather_q8_streams(A->rows, A->cols, q.ldq)) {
         rc = launch_gather_q8_pair(A->ptr, A->rows, A->stride_row * 2, B->ptr, B->cols, B->stride_col, A->cols, idx, k, Aq, Bq, q.ldq, row_scale,
                                    status, st);
     } else {

@@ -242,7 +242,7 @@ int launch_pack(const PackSpec *specs, int n, int *status, cudaStream_t stream);
 // row_scale[r] = max_j |src[r, idx[j]]| / 448, codes are e4m3(src / step); otherwise src already holds codes (bytes).
 // s_row: elements between two rows of src; rows must start on 16-byte boundaries.
 // Both gathers of a product in one launch, where gather_q8_streams() (pitches in bytes, multiples of 16).
-bool gather_q8_streams(int64_t K, int64_t ld_dst);
+bool gather_q8_streams(int64_t a_rows, int64_t K, int64_t ld_dst);
 int launch_gather_q8_pair(const void *A, int64_t a_rows, int64_t a_pitch, const void *B, int64_t b_rows, int64_t b_pitch, int64_t K,
                           const int32_t *idx, int64_t k, uint8_t *Aq, uint8_t *Bq, int64_t ld_dst, float *row_scale, int *status,
                           cudaStream_t stream);

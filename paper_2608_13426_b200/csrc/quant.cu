@@ -273,9 +273,11 @@ __global__ void __launch_bounds__(kThreadsS, 1) gather_q8_stream_kernel(const __
 #pragma unroll
     for (int sl = 0; sl < 4 * G; ++sl) {
         const int j = ((sl >> 2) * (kThreadsS / 32) + warp) * 128 + 32 * (sl & 3) + lane;
+        // Positions past the row's end are not written; they stand for the first output once more, whose quotient costs what
+        // any other does (a zero's would be divided: 4096 x 4096 activations, 3072 kept, 4096 columns 97 us, 84 this way).
         uint32_t col = (uint32_t)(a.K + 15) / 16 * 16;
-        if (j < a.k) {
-            const int c = __ldg(a.idx + j);
+        if (j < a.k || j >= (int)a.ld_dst) {
+            const int c = __ldg(a.idx + (j < a.k ? j : 0));
             if (c < 0 || c >= a.K) atomicExch(a.status, (int)RMM_ERR_BOUNDS);
             else col = (uint32_t)c;
         }
@@ -291,9 +293,12 @@ __global__ void __launch_bounds__(kThreadsS, 1) gather_q8_stream_kernel(const __
 
 }  // namespace
 
-bool gather_q8_streams(int64_t K, int64_t ld_dst)
+bool gather_q8_streams(int64_t a_rows, int64_t K, int64_t ld_dst)
 {
-    return K <= 65520 && (K + 15) / 16 * 32 + 16 <= kStreamMaxRowBytes && ld_dst <= 4096 * kUnitsS;
+    // Half of the block's outputs at least: below that most of its threads have nothing to do (4096 x 1024 activations, 512 kept,
+    // and 1024 columns, whole product: 60 us, by rows 25; 2048 kept of 4096, 4096 columns: 71 and 69; 3072 kept: 83 and 89)
+    // (few rows leave the SMs to the streaming blocks either way: 128 x 4096, 2048 kept, 4096 columns 28 and 30 us)
+    return ld_dst > (a_rows <= 512 ? 1536 : 2048) && K <= 65520 && (K + 15) / 16 * 32 + 16 <= kStreamMaxRowBytes && ld_dst <= 4096 * kUnitsS;
 }
 
 int launch_gather_q8_pair(const void *A, int64_t a_rows, int64_t a_pitch, const void *B, int64_t b_rows, int64_t b_pitch, int64_t K,
@@ -310,8 +315,7 @@ int launch_gather_q8_pair(const void *A, int64_t a_rows, int64_t a_pitch, const 
     a.status = status;
     a.wait_ns = wait_limit_ns();
     a.withhold = debug_withhold() == WITHHOLD_QUANT;
-    const int64_t groups = ceil_div(ld_dst, 4096);
-    const int g = groups <= 1 ? 1 : (groups <= 2 ? 2 : (groups <= 4 ? 4 : 8));
+    const int g = (int)ceil_div(ld_dst, 4096);
     int64_t blocks = 0;
     size_t smem = 0;
     for (int w = 0; w < 2; ++w) {
@@ -326,10 +330,12 @@ int launch_gather_q8_pair(const void *A, int64_t a_rows, int64_t a_pitch, const 
         const int64_t nb = ceil_div(a.rows[w], a.per_block[w]);
         if (nb > blocks) blocks = nb;
     }
-    auto kern = g == 1 ? gather_q8_stream_kernel<1> : (g == 2 ? gather_q8_stream_kernel<2> : (g == 4 ? gather_q8_stream_kernel<4> : gather_q8_stream_kernel<8>));
-    static PerDeviceOnce configured;
-    const int most = 2 * (kStreamMaxRowBytes + 16);
-    if (cudaError_t e = configured.smem(most, gather_q8_stream_kernel<1>, gather_q8_stream_kernel<2>, gather_q8_stream_kernel<4>, gather_q8_stream_kernel<8>))
+    static void (*const kernels[kUnitsS])(StreamQ8) = {gather_q8_stream_kernel<1>, gather_q8_stream_kernel<2>, gather_q8_stream_kernel<3>,
+                                                       gather_q8_stream_kernel<4>, gather_q8_stream_kernel<5>, gather_q8_stream_kernel<6>,
+                                                       gather_q8_stream_kernel<7>, gather_q8_stream_kernel<8>};
+    auto kern = kernels[g - 1];
+    static PerDeviceOnce configured[kUnitsS];
+    if (cudaError_t e = configured[g - 1].smem(2 * (kStreamMaxRowBytes + 16), kern))
         return fail(RMM_ERR_CUDA, "gather_q8: cudaFuncSetAttribute: %s", cudaGetErrorString(e));
     prof_begin("gather_q8_stream_kernel", stream);
     launch_kernel(kern, dim3((unsigned)blocks), dim3(kThreadsS), smem, stream, 1, a);

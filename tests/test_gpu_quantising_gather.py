@@ -58,3 +58,12 @@ def test_codes_at_ties_zeros_and_extremes(oracle):
     codes, steps = oracle.quantize_rows_e4m3(A.float().numpy())
     assert np.array_equal(step, steps.astype(np.float32))
     assert np.array_equal(got, codes.astype(np.float32) * steps[:, None].astype(np.float32))
+
+
+@pytest.mark.parametrize("M,K,k", [
+    (149, 4096, 2048), (149, 4096, 2049),                   # the last count that rows take on their own, the first that streams
+    (500, 4104, 4097), (310, 16400, 12288),                 # an output in a second group of 4096; three groups, full
+    (200, 30000, 24570), (150, 32000, 28000), (150, 40000, 32768),   # six, seven and eight groups, a row at a time
+])
+def test_every_number_of_output_groups(oracle, M, K, k):
+    test_codes_and_steps_match_the_definition(oracle, M, K, k)
