@@ -29,6 +29,7 @@ constexpr int kThreads = 1024;     // one block per SM: its tail (the select) th
 constexpr int kUnroll = 4;       // rows in flight per thread (1024 threads x 4 x 16 B = 64 KB in flight per SM)
 constexpr int kFlushEvery = 4;   // loop trips between fp32 -> fp64 flushes (kUnroll * kFlushEvery = 16 terms)
 constexpr int kFusedSelectMax = 8192;    // largest K whose select runs in the score kernel's tail
+constexpr int kCachedSelectMax = 49152;  // largest K that one selecting block caches in shared memory (192 KB)
 
 using namespace sel;
 
@@ -859,6 +860,16 @@ __global__ void __launch_bounds__(kThreads, 1) rmm_front_kernel(const __grid_con
 // matrices (and up to eight rows of 4096 columns) take one block, CTAS = 1: 1 x 512 10.5 us, 5.3.
 constexpr int kSelCtas = 8, kSelThreads = 512;
 constexpr int64_t kClusterSelectMax = (int64_t)kSelCtas * kSelThreads * 16;
+// Many lists at once keep the GPU busy with one block each, the keys in shared memory: the blocks of a cluster repeat per list what
+// does not shrink with its share of the keys.  One block a list takes about 8 us (4 from 32768 keys on) and 6.2 + K / 1270 a round
+// of lists over the SMs; a cluster 9 us and 0.175, 0.26 or 0.36 a list (4, 8 or 16 keys a thread).  32 x 28672 keys 18 us by clusters, 36 by blocks;
+// 96: 33 and 36; 128: 43 and 37; 160: 51 and 64; 256: 76 and 65; 128 x 8200: 29 and 20.
+bool select_by_cluster(int64_t batch, int64_t K)
+{
+    if (K <= kFusedSelectMax || K > kClusterSelectMax) return false;
+    const double list = K <= 16384 ? 0.175 : (K <= 32768 ? 0.26 : 0.36);
+    return K > kCachedSelectMax || 9.0 + list * (double)batch <= (K <= 32768 ? 8.0 : 4.0) + (double)ceil_div(batch, sm_count()) * (6.2 + (double)K / 1270.0);
+}
 
 struct ClusterSelectArgs {
     const float *keys;       // [batch, K], or
@@ -1120,12 +1131,14 @@ int launch_cluster_select(const ClusterSelectArgs &a, int64_t batch, const char 
     return check_launch(name, stream);
 }
 
-__global__ void __launch_bounds__(1024) select_kernel(const float *keys, int K, int k, int32_t *idx, float *retained)
+__global__ void __launch_bounds__(1024) select_kernel(const float *keys, int K, int k, int32_t *idx, float *retained, int use_cache)
 {
+    extern __shared__ __align__(128) unsigned char s_dyn[];
     __shared__ SelectSmem s_sel;
     pdl_wait();
     const int64_t b = blockIdx.x;
-    block_select_any(keys + b * K, K, k, idx + b * (int64_t)k, retained ? retained + b : nullptr, s_sel);
+    block_select_any(keys + b * K, K, k, idx + b * (int64_t)k, retained ? retained + b : nullptr, s_sel,
+                     use_cache ? reinterpret_cast<unsigned *>(s_dyn) : nullptr);
 }
 
 }  // namespace
@@ -1358,13 +1371,18 @@ int launch_select(const float *keys, int64_t batch, int64_t K, int64_t k, int32_
                   cudaStream_t stream)
 {
     (void)ws;
-    if (K > kFusedSelectMax && K <= kClusterSelectMax) {
+    if (select_by_cluster(batch, K)) {
         ClusterSelectArgs c = {};
         c.keys = keys; c.K = (int)K; c.k = (int)k; c.idx = idx; c.retained = retained;
         return launch_cluster_select<false>(c, batch, "select_kernel", stream);
     }
+    const int use_cache = K > kFusedSelectMax && K <= kCachedSelectMax;
+    static PerDeviceOnce configured;
+    if (cudaError_t e = configured.smem(kCachedSelectMax * 4, select_kernel))
+        return fail(RMM_ERR_CUDA, "select: cudaFuncSetAttribute: %s", cudaGetErrorString(e));
     prof_begin("select_kernel", stream);
-    launch_kernel(select_kernel, dim3((unsigned)batch), dim3(1024), 0, stream, 1, keys, (int)K, (int)k, idx, retained);
+    launch_kernel(select_kernel, dim3((unsigned)batch), dim3(1024), use_cache ? (size_t)K * 4 : (size_t)0, stream, 1, keys, (int)K, (int)k, idx, retained,
+                  use_cache);
     return check_launch("select_kernel", stream);
 }
 

@@ -81,17 +81,18 @@ __device__ __forceinline__ void find_bin(SelectSmem &sm, int nbins, unsigned rem
 
 // Block-wide top-k of keys[0..K): writes idx[0..k) ascending (ties at the threshold go to the lowest indices) and,
 // if asked, the kept fraction of the key mass.  Every thread of the block must call it.  Keys are read through L2
-// (other blocks may have just written them).
+// (other blocks may have just written them).  kcache, if not NULL, is shared memory for K key images: the keys are then
+// fetched once and every later pass runs out of shared memory.
 //
 // Radix select on the order-preserving integer image of the keys: the bits common to all keys are skipped, one
 // digit of up to 11 bits is histogrammed over all keys, the (few) keys that share the threshold's digit are copied
 // to a short list and finished there with 8-bit digits.  The kept indices are then emitted by warps that own
 // consecutive chunks of the index range, ranks coming from ballots.
 inline __device__ void block_select(const float *__restrict__ keys, int K, int k, int32_t *__restrict__ idx, float *retained,
-                             SelectSmem &sm)
+                             SelectSmem &sm, unsigned *kcache)
 {
     const int tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31, warp = tid >> 5, nwarp = nthr >> 5;
-    auto image = [&](int j) -> unsigned { return key_image(__ldcg(keys + j)); };
+    auto image = [&](int j) -> unsigned { return kcache != nullptr ? kcache[j] : key_image(__ldcg(keys + j)); };
     // ---- fetch the keys, eight independent loads at a time; min and max give the common leading bits
     unsigned lo = 0xffffffffu, hi = 0u;
     for (int j0 = tid; j0 < K; j0 += 8 * nthr) {
@@ -105,6 +106,7 @@ inline __device__ void block_select(const float *__restrict__ keys, int K, int k
         for (int i = 0; i < 8; ++i) {
             const int j = j0 + i * nthr;
             if (j < K) {
+                if (kcache != nullptr) kcache[j] = u[i];
                 lo = min(lo, u[i]);
                 hi = max(hi, u[i]);
             }
@@ -554,14 +556,15 @@ __device__ void block_select_blocked(const float *__restrict__ keys, int K, int 
     __syncthreads();
 }
 
-// Dispatch on the problem size: keys in registers when they fit (blocks of 1024 threads), else re-read in every pass.
+// Dispatch on the problem size: keys in registers when they fit (blocks of 1024 threads), else in kcache or, without one,
+// re-read in every pass.
 __device__ __forceinline__ void block_select_any(const float *keys, int K, int k, int32_t *idx, float *retained,
-                                                 SelectSmem &sm)
+                                                 SelectSmem &sm, unsigned *kcache = nullptr)
 {
     if (blockDim.x == 1024 && K <= 1024) block_select_blocked<1>(keys, K, k, idx, retained, sm);
     else if (blockDim.x == 1024 && K <= 4096) block_select_blocked<4>(keys, K, k, idx, retained, sm);
     else if (blockDim.x == 1024 && K <= 8192) block_select_blocked<8>(keys, K, k, idx, retained, sm);
-    else block_select(keys, K, k, idx, retained, sm);
+    else block_select(keys, K, k, idx, retained, sm, kcache);
 }
 
 }  // namespace sel

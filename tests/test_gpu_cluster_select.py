@@ -43,3 +43,16 @@ def test_many_keys_batches_retained_and_alignment(oracle):
         frac = float(keys[b].double()[want].sum() / keys[b].double().sum())
         assert np.array_equal(idx[b].cpu().numpy(), want)
         assert abs(float(kept[b]) - frac) <= 2e-7      # fp64 sums, rounded once to fp32
+
+
+@pytest.mark.parametrize("batch, K", [(79, 8201), (130, 14336), (120, 28672), (149, 9000), (300, 16385), (150, 49152), (140, 49153)])
+def test_many_lists_at_once_match_one_at_a_time(batch, K):
+    """A block per list or a cluster per list, whichever the rule takes: the sets and fractions are the same."""
+    keys = torch.stack([keys_of(("uniform", "concentrated", "ties", "wild")[b % 4], K, b) for b in range(batch)]).cuda()
+    keys[3::4] = keys[3::4].clamp(min=0.0, max=1e30)                       # (fractions of what is finite)
+    idx, kept = rmm.rmm_select(keys, rho=0.3, want_retained=True)
+    for b in range(0, batch, 7):
+        one, frac = rmm.rmm_select(keys[b].contiguous(), rho=0.3, want_retained=True)
+        assert torch.equal(idx[b], one), b
+        assert abs(float(kept[b]) - float(frac)) <= 2.0 ** -23
+    assert rmm.rmm_status_read() == 0
