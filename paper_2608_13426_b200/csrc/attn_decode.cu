@@ -1,7 +1,7 @@
 // Reduced attention for decode steps (paper Sec. 3.3 with rho_t = 1 and a handful of query rows): feature selection,
 // S~ = Q[:, I] K[:, I]^T / sqrt(Dh), softmax and P V in one pass over the key/value cache, plus a small combine.
 //
-// Bound: HBM.  K and V are each read once, 4 bytes per (key, column); the kept features of a 2-byte row touch every
+// Bound: HBM.  K and V are read once per 16 query rows that share a kv head, 4 bytes per (key, column); the kept features of a 2-byte row touch every
 // 32-byte sector of it, so there is nothing to gain from gathering and the packed copies of K per query head that the
 // prefill form makes would multiply the traffic (8 sequences x 32 / 8 heads x 4096 keys x 128: 80 us of packing and
 // 97 us of a kernel whose 128-row tiles hold one row; 33 us
@@ -110,7 +110,7 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, kDecodeBlocks) attn_decode_
             if (f < a.Dh)
                 for (int r = 0; r < a.Lq; ++r) {
                     const float x = __bfloat162float(qp[(int64_t)r * a.q_sr + f]);
-                    e += (double)(x * x);  // the square of a bf16 number is exact in fp32
+                    e += (double)(x * x);  // exact for magnitudes from 2^-63 to 2^64, as in every score pass
                 }
             u[i] = f < a.Dh ? sel::key_image((float)e) : 0u;  // 0: below every key
         }
@@ -390,10 +390,13 @@ DecodeGrid decode_grid(const rmm_attn_desc_t *d)
     DecodeGrid g;
     const int64_t rows = d->Hq / d->Hkv * d->Lq, slots = (int64_t)sm_count() * kDecodeBlocks;
     g.dh = d->Dh <= 64 ? 64 : (d->Dh <= 128 ? 128 : 256);
-    g.nt = rows <= 8 ? 1 : 2;
+    g.tiles = (int)ceil_div(d->Lk, 16 * kDecodeWarps);
+    // Sixteen rows a block read the cache half as often as eight.  Where even blocks of one tile and eight rows leave the GPU
+    // room, what a block spends on the feature sets of its heads is what counts, and eight rows have half of it (32 heads of
+    // 256 on one kv head, one query, 512 keys: 52 us a call with sixteen, 32 with eight).
+    g.nt = rows <= 8 || d->B * d->Hkv * ceil_div(rows, 8) * g.tiles <= slots ? 1 : 2;
     g.chunks = (int)ceil_div(rows, 8 * g.nt);
     g.jobs = d->B * d->Hkv * g.chunks;
-    g.tiles = (int)ceil_div(d->Lk, 16 * kDecodeWarps);
     int64_t best = INT64_MAX;
     for (int64_t rounds = 0; rounds <= 2; ++rounds) {  // whole jobs, or the most pieces that make one or two rounds
         int64_t s = rounds * slots / g.jobs;
