@@ -316,17 +316,15 @@ struct SimtPlan {
 // costs about 2 us outside its steps, slices another 1.5 for their meeting.  (777 x 1500 kept x 1500: 230 us with one
 // slice, 134 with two, 119 with three, which the rule takes; 1500 x 2000 x 700: 231, 169, 120.)
 // Slices whose partial sums take more than `room` bytes are not considered.
-SimtPlan plan_simt(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k, bool vec, size_t room)
+SimtPlan plan_simt(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k, size_t room)
 {
-    // blocks per SM: what the registers of a variant allow (168 / 226 / 254 a thread with 64 rows, 96 / 128 with 32)
-    const int fits[2] = {vec ? 3 : 2, A->dtype == RMM_BF16 ? 4 : 5};
     static const double step_us[2][5] = {{1.15, 2.4, 2.7}, {0.9, 1.9, 2.1, 2.2, 2.3}};
     SimtPlan best = {8, 1, ceil_div(k, BK) * BK};
     double best_cost = 1e300;
     const int64_t steps = ceil_div(k, BK), sms = sm_count();
     for (int tm = 8; tm >= 4; tm /= 2) {
         if (ceil_div(A->rows, kHi * tm) > 65535) continue;
-        const int fit = fits[tm == 8 ? 0 : 1];
+        const int fit = tm == 8 ? 3 : 5;
         const double *t = step_us[tm == 8 ? 0 : 1];
         const int64_t tiles = simt_tiles(A, B, tm), most = simt_slices_max(tiles, k);
         for (int64_t s = 1; s <= most; ++s) {
@@ -368,9 +366,7 @@ size_t gemm_simt_workspace_bytes(const rmm_mat_t *A, const rmm_mat_t *B, int64_t
 int launch_gemm_simt(const rmm_mat_t *A, const rmm_mat_t *B, const int32_t *idx, int64_t k, float scale,
                      const rmm_mat_t *Y, void *ws, size_t ws_bytes, cudaStream_t stream)
 {
-    auto al16 = [](const void *p) { return reinterpret_cast<uintptr_t>(p) % 16 == 0; };
-    const bool vec = B->dtype == RMM_F32 && B->stride_col == 1 && B->stride_row % 4 == 0 && B->stride_batch % 4 == 0 && B->cols % 4 == 0 && al16(B->ptr);
-    const SimtPlan plan = plan_simt(A, B, k, vec, ws_bytes - RMM_WS_HEADER_BYTES);
+    const SimtPlan plan = plan_simt(A, B, k, ws_bytes - RMM_WS_HEADER_BYTES);
     SimtArgs a;
     a.A = A->ptr; a.B = B->ptr; a.Y = Y->ptr; a.idx = idx;
     a.M = A->rows; a.K = A->cols; a.N = B->cols; a.k = k;
@@ -384,7 +380,9 @@ int launch_gemm_simt(const rmm_mat_t *A, const rmm_mat_t *B, const int32_t *idx,
     a.partials = reinterpret_cast<float4 *>(static_cast<char *>(ws) + RMM_WS_HEADER_BYTES);
     a.counters = reinterpret_cast<WsHeader *>(ws)->counters;
     a.y_bf16 = Y->dtype == RMM_BF16;
+    auto al16 = [](const void *p) { return reinterpret_cast<uintptr_t>(p) % 16 == 0; };
     a.y_vec = !a.y_bf16 && a.y_sc == 1 && a.y_sr % 4 == 0 && a.y_sb % 4 == 0 && al16(a.Y);
+    const bool vec = B->dtype == RMM_F32 && a.b_sc == 1 && a.b_sr % 4 == 0 && a.b_sb % 4 == 0 && a.N % 4 == 0 && al16(a.B);
     dim3 grid((unsigned)ceil_div(a.N, BN), (unsigned)ceil_div(a.M, kHi * plan.tm), (unsigned)(A->batch * plan.splits));
     if (A->batch > 65535 || ceil_div(a.M, 64) > 65535)
         return fail(RMM_ERR_UNSUPPORTED, "reduced_gemm (FMA path): batch or M/64 exceeds 65535");
