@@ -68,8 +68,8 @@ int rmm_keep_count(double rho, int64_t K, int64_t *k);
  *   axis   1: one score per column (the contraction axis of A B); 0: one score per row.
  *   scores fp32 [batch, n] with n = cols (axis 1) or rows (axis 0), or NULL
  *   energy fp32 [batch, n]: the squared scores sum_i A[i,j]^2, which are the selection keys, or NULL
- * Squares of bf16 values are exact in fp32; sums run in short fp32 chains combined in fp64 in a fixed
- * order, so results are deterministic and accurate to about 1e-7 relative. */
+ * Squares of bf16 values of magnitude 2^-63 to 2^64 are exact in fp32 (beyond, they leave fp32's range); sums run in short fp32
+ * chains combined in fp64 in a fixed order, so results are deterministic and accurate to about 1e-7 relative. */
 size_t rmm_score_workspace_bytes(const rmm_mat_t *A, int axis);
 int rmm_score(const rmm_mat_t *A, int axis, float *scores, float *energy, void *ws, size_t ws_bytes, void *stream);
 
@@ -85,7 +85,8 @@ int rmm_select(const float *keys, int64_t batch, int64_t K, double rho, int64_t 
                void *ws, size_t ws_bytes, void *stream);
 
 /* rmm_score followed by rmm_select on the energies, in ONE launch when n <= 8192 (the last thread block to finish
- * a batch element's scores selects its index set; larger n: the select kernel follows as a second launch).
+ * a batch element's scores selects its index set), or when n <= 65536 and the scores sum at most 32 contiguous bf16 rows (the
+ * selecting blocks sum the columns they hold); otherwise the select kernel follows as a second launch.
  * scores / energy / retained may be NULL. */
 size_t rmm_score_select_workspace_bytes(const rmm_mat_t *A, int axis);
 int rmm_score_select(const rmm_mat_t *A, int axis, double rho, int64_t k, int32_t *idx, float *scores, float *energy,
@@ -123,7 +124,10 @@ int rmm_score_select_static_status(int *device_status);
  *   Decode-step shapes (batch 1, M <= 4, bf16, B with contiguous rows; App. "Complexity Analysis", decoding step)
  *   take a gathered GEMV that reads only the kept rows of B (k N 2 bytes) and packs nothing; outputs of up to 256
  *   rows (small decode batches, B with contiguous rows, N > 128) run on the tensor cores with the kept rows of B
- *   fetched by the kernel itself, so W is read once and never copied. */
+ *   fetched by the kernel itself, so W is read once and never copied (up to 32 rows on warp-level products, more on 128-row
+ *   tiles).  These forms and the FMA kernel cut the contraction axis where the output alone would leave multiprocessors idle;
+ *   the pieces' fp32 sums are what most of their workspace is for.  In a smaller one (sized for another shape) they run with fewer
+ *   pieces: what the packed operands would take is enough, for the FMA kernel the header; the order of summation follows. */
 size_t rmm_reduced_gemm_workspace_bytes(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k, const rmm_mat_t *Y);
 int rmm_reduced_gemm(const rmm_mat_t *A, const rmm_mat_t *B, const int32_t *idx, int64_t k, float scale,
                      const rmm_mat_t *Y, void *ws, size_t ws_bytes, void *stream);
@@ -134,7 +138,9 @@ int rmm_reduced_gemm(const rmm_mat_t *A, const rmm_mat_t *B, const int32_t *idx,
  * treatment of selection and reduced multiplication as the way to cut memory movement).  On the tensor-core path with a
  * bf16 Y the epilogue accumulates the sums while it holds the rounded tile (exact squares, fp32 chains of 16, 32-row
  * groups added in fp64 in a fixed order: deterministic, about 1e-7 relative); every other form of the product runs
- * rmm_score on Y afterwards.  Arguments otherwise as rmm_reduced_gemm. */
+ * rmm_score on Y afterwards, and so do outputs of up to 256 rows with an index list where cutting the contraction saves more
+ * time than that pass takes (elsewhere their contraction is not cut, so Y can differ from rmm_reduced_gemm's in the order of
+ * its fp32 sums).  Arguments otherwise as rmm_reduced_gemm. */
 size_t rmm_reduced_gemm_scored_workspace_bytes(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k, const rmm_mat_t *Y);
 int rmm_reduced_gemm_scored(const rmm_mat_t *A, const rmm_mat_t *B, const int32_t *idx, int64_t k, float scale,
                             const rmm_mat_t *Y, float *energy_out, void *ws, size_t ws_bytes, void *stream);
@@ -162,7 +168,8 @@ int rmm_reduced_gemm_q8(const rmm_mat_t *A, const rmm_mat_t *B, float b_scale, c
  *   rho_t == 1: O = P V
  * Q [B,Hq,Lq,Dh], K,V [B,Hkv,Lk,Dh], O [B,Hq,Lq,Dh] are bf16 with explicit element strides
  * (batch, head, row, 1).  idx_feat int32 [B,Hq,kd] and idx_tok int32 [B,Hq,kt] receive the index sets
- * (either may be NULL).  With at most 128 kept features and a head_dim of at most 256, S~ and P stay on the SM (heads wider
+ * (either may be NULL).  Up to 16 query rows per head without a mask and with rho_t == 1 (decode steps, heads up to 256 wide) read
+ * K and V in place, once per 16 query rows that share a kv head.  Otherwise, with at most 128 kept features and a head_dim of at most 256, S~ and P stay on the SM (heads wider
  * than 128 columns in two passes over the columns of V; fused kernel: one pass
  * for rho_t == 1; row normalisers, token scores and a gathered P V pass for rho_t < 1, where the normalised P is
  * what is rounded, scored and multiplied; for rho_t == 1 the bf16 rounding is applied to P times a per-row factor,
@@ -171,9 +178,9 @@ int rmm_reduced_gemm_q8(const rmm_mat_t *A, const rmm_mat_t *B, float b_scale, c
  * mask (device, fp32, or NULL): the additive M of Sec. 3.3, entry (b, h, i, t) at mask[b ms[0] + h ms[1] + i ms[2] + t]
  * with ms = mask_stride in elements (0 shares the mask along that axis; rows contiguous); -inf hides a key; a row with
  * every key hidden gives zeros.  A finite value hides none, however low: S~ + M is taken in fp32, so a row that holds
- * nothing but, say, -1e30 weighs its keys equally.  It composes with `causal`.  With rho_t == 1, a fused-eligible shape and mask rows that are
- * 16-byte aligned (base pointer and all three strides multiples of 4 elements) the one-pass fused kernel adds the mask
- * itself; otherwise a call with a mask runs the composed form (S~ and P in the workspace). */
+ * nothing but, say, -1e30 weighs its keys equally.  It composes with `causal`.  With rho_t == 1 and a fused-eligible shape the one-pass fused kernel
+ * adds the mask itself, whatever its alignment (128 x 128 tiles that the mask hides, or leaves alone, cost no additions);
+ * otherwise a call with a mask runs the composed form (S~ and P in the workspace). */
 typedef struct {
     int64_t B, Hq, Hkv, Lq, Lk, Dh;
     int32_t causal;
@@ -196,7 +203,8 @@ int rmm_reduced_attn(const rmm_attn_desc_t *desc, const void *Q, const void *K, 
  * and both gathers run in ONE launch (every block owns 64 columns of A, a grid-wide barrier makes all column energies
  * visible, every block then selects and gathers its own kept columns and the matching rows of B), followed by the
  * tensor-core product; this form expects the GPU to itself (all of its blocks must be resident at once; if they are
- * not, the barrier's bounded wait expires and RMM_ERR_TIMEOUT is reported).  Everything else runs as the two calls. */
+ * not, the barrier's bounded wait expires and RMM_ERR_TIMEOUT is reported).  Outputs of 5 to 32 rows have their selecting kernel
+ * pack A[:, I] as well, where the product fetches the rows of B itself.  Everything else runs as the two calls. */
 size_t rmm_product_workspace_bytes(const rmm_mat_t *A, const rmm_mat_t *B, const rmm_mat_t *Y);
 int rmm_product(const rmm_mat_t *A, const rmm_mat_t *B, double rho, int64_t k, float scale, const rmm_mat_t *Y, int32_t *idx,
                 float *retained, void *ws, size_t ws_bytes, void *stream);

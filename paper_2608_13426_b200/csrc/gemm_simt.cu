@@ -8,8 +8,9 @@
 // pairs of columns for the packed fp32 FMA (one instruction, two FMAs; with single FMAs the same kernel took 480 us
 // where this takes 380): per contraction index a thread reads TM + 8 floats from shared memory for 8 TM FMAs, one index
 // ahead.  16 indices per step; fp32 elements are gathered by cp.async into a ring of three steps, bf16 ones pass through
-// registers; index lists are loaded a step before they are used.  Small blocks, so that three share an SM and none of
-// them waits at another's barrier.  fp32 accumulation with one partial sum per step of 16, so that rounding error grows
+// registers; index lists are loaded a step before they are used.  Small blocks, so that several share an SM (vectorised fp32:
+// three of 64 rows, five of 32; the registers of the other variants allow two of 64 rows, and in bf16 four of 32) and none
+// of them waits at another's barrier.  fp32 accumulation with one partial sum per step of 16, so that rounding error grows
 // with k/16 rather than k.  Outputs with fewer tiles than the GPU has room for cut the contraction axis (plan_simt): the
 // slices of a tile meet in its last block, which adds them in order.
 // fp32, kernel alone: 777 x 1500 kept x 1500 379 -> 119 us, 2048 x 4096 x 4096 5530 -> 1490 us (46 of the 65 TFLOP/s that
@@ -314,7 +315,10 @@ struct SimtPlan {
 // warp each), so what counts is how many blocks share an SM; a step of 16 indices took about 1.2, 2.4 and 2.7 us for one,
 // two and three blocks of 64 rows (three fit), 0.9, 1.9, 2.1, 2.2 and 2.3 us for one to five of 32 rows.  A round of blocks
 // costs about 2 us outside its steps, slices another 1.5 for their meeting.  (777 x 1500 kept x 1500: 230 us with one
-// slice, 134 with two, 119 with three, which the rule takes; 1500 x 2000 x 700: 231, 169, 120.)
+// slice, 134 with two, 119 with three, which the rule takes; 1500 x 2000 x 700: 231, 169, 120.)  The times are those of the
+// vectorised fp32 variant and stand for all: with each variant's own number of blocks in their place, bf16 on 100 x 3000 x
+// 1500 took 43 us for 59, but fp32 with B by columns took 634 for 435 on 2048 x 4096 x 1023 (32-row tiles), 864 for 650 on 2048 x
+// 2000 x 4094.
 // Slices whose partial sums take more than `room` bytes are not considered.
 SimtPlan plan_simt(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k, size_t room)
 {

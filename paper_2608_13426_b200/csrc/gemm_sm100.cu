@@ -9,7 +9,7 @@
 //             K-contiguous (K^T in attention) it is packed like A and loaded as K-major tiles.  (Fetching the
 //             kept rows inside the producer with TMA gather4 was measured first: at 512 bytes per instruction
 //             the copy engine sustained about one instruction per 70 clocks, 2.5x slower than this form.)
-//             Outputs of 33 to 256 rows (fewer: gemm_skinny.cu) skip the packed copy of B: eight gather warps fetch
+//             Outputs of 33 to 256 rows (some from 25 on; fewer: gemm_skinny.cu) skip the packed copy of B: eight gather warps fetch
 //             the kept rows straight from B with 16-byte cp.async into the same swizzled layout (one row of the tile
 //             = one 512-byte warp request).  There every tile of B is used once, the product is bound by reading the
 //             kept rows from HBM, and the copy would triple that traffic; where whole tiles leave SMs idle the

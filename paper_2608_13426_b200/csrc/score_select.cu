@@ -954,7 +954,8 @@ __global__ void __launch_bounds__(kSelThreads) select_cluster_kernel(const Clust
 #pragma unroll
             for (int i = 0; i < ITEMS; ++i) {
                 const float x = __uint_as_float(i & 1 ? w[i / 2] & 0xffff0000u : w[i / 2] << 16);
-                e[i] += (double)(x * x);  // the square of a bf16 number is exact in fp32
+                // exact for magnitudes from 2^-63 to 2^64; squared in 64 bits, 512 lists of 8192 took 150 us where this takes 119
+                e[i] += (double)(x * x);
             }
         });
 #pragma unroll
@@ -1117,15 +1118,17 @@ int launch_cluster_select(const ClusterSelectArgs &a, int64_t batch, const char 
 {
     void (*kern)(ClusterSelectArgs) = nullptr;
     int ctas = kSelCtas;
-    if (FROM_A && (a.K <= 1024 || (a.K <= 4096 && a.m <= 8))) {
-        ctas = 1;
-        kern = a.K <= 1024 ? select_cluster_kernel<2, 1, FROM_A> : select_cluster_kernel<8, 1, FROM_A>;
-    } else if (FROM_A && a.K <= 8192) {
-        kern = select_cluster_kernel<2, kSelCtas, FROM_A>;
-    } else {
+    if constexpr (FROM_A) {  // (keys that are given are more than 8192 here)
+        if (a.K <= 1024 || (a.K <= 4096 && a.m <= 8)) {
+            ctas = 1;
+            kern = a.K <= 1024 ? select_cluster_kernel<2, 1, true> : select_cluster_kernel<8, 1, true>;
+        } else if (a.K <= 8192) {
+            kern = select_cluster_kernel<2, kSelCtas, true>;
+        }
+    }
+    if (kern == nullptr)
         kern = a.K <= 16384 ? select_cluster_kernel<4, kSelCtas, FROM_A>
                             : (a.K <= 32768 ? select_cluster_kernel<8, kSelCtas, FROM_A> : select_cluster_kernel<16, kSelCtas, FROM_A>);
-    }
     prof_begin(name, stream);
     launch_kernel(kern, dim3((unsigned)(batch * ctas)), dim3(kSelThreads), 0, stream, ctas, a);
     return check_launch(name, stream);
