@@ -10,7 +10,8 @@ With N > 1 every rank runs the same workload on its own GPU (independent replica
 
     python bench.py [--gpus N] [--steps K] [--warmup W] [--impl reference]
 
-prints ONE JSON line.  `--impl reference` times the CPU oracle (the slow fp64 checker) on a bounded
+prints ONE JSON line of a few thousand characters (readers keep no more of the output than that); the sweeps and the
+per-kernel breakdown go to stderr, as one JSON line as well.  `--impl reference` times the CPU oracle (the slow fp64 checker) on a bounded
 sample of the same workload.
 """
 from __future__ import annotations
@@ -36,6 +37,8 @@ RHO = 0.5
 RHOS = (0.25, 0.5, 0.75, 1.0)
 METRIC = "reduced-GEMM retained TFLOP/s (whole RMM op: score + select + reduced product)"
 UNIT = "TFLOP/s"
+LINE_KEYS = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling", "vs_baseline", "dtype",
+             "data", "config", "roofline", "cpu_baseline", "e2e", "gpu_launches", "clocks", "peaks")
 NOMINAL_BF16_TFLOPS = 2250.0          # dense bf16 tensor peak of a B200 as specified (context beside the measured peaks)
 NOMINAL_HBM_GBS = 8000.0
 # dram__bytes_read.sum + dram__bytes_write.sum of ONE launch of the GEMM kernel on the headline workload at rho = 0.5,
@@ -166,6 +169,12 @@ def gemm_roofline(achieved_tflops: float, kernel_ms: float, peaks: dict, clocks:
             "frac_of_sustained_peak": achieved_tflops / peaks["bf16_sustained"],
             "frac_of_nominal_peak": achieved_tflops / NOMINAL_BF16_TFLOPS,
             "kernel_ms": kernel_ms, "sm_mhz_x_kernel_ms": (sm * kernel_ms) if sm else None}
+
+
+def split_line(out: dict):
+    """(the result line, the details): the line holds the measurement itself, everything else is detail."""
+    line = {key: out[key] for key in LINE_KEYS if key in out}
+    return json.dumps(line), json.dumps({"details": {key: v for key, v in out.items() if key not in line}})
 
 
 def time_region(fn, steps: int, world: int) -> float:
@@ -845,7 +854,9 @@ def main():
             "kernel_breakdown": breakdown, "per_rho": per_rho, "peaks": peaks,
         }
         out.update(extras)
-        print(json.dumps(out))
+        line, details = split_line(out)
+        print(details, file=sys.stderr, flush=True)
+        print(line)
     if world > 1:
         import torch.distributed as dist
         dist.destroy_process_group()

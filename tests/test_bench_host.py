@@ -78,3 +78,21 @@ def test_clock_sample_parser():
     s.proc = P()
     r = s.stop()
     assert r["sm_mhz"] == 1320 and r["sm_max_mhz"] == 1965 and r["reasons"] == ["sw_power_cap"] and r["samples"] == 3
+
+
+def test_the_result_line_stays_short_whatever_the_sweeps_hold():
+    import json
+
+    import bench
+
+    peaks = {"bf16_burst": 1643.8123456789, "bf16_sustained": 1386.7123456789, "hbm_gbs": 6450.123456789, "source": "measured"}
+    clocks = {"sm_mhz": 1320.0, "sm_max_mhz": 1965.0, "reasons": ["sw_power_cap"], "samples": 30, "power_w_max": 999.123}
+    cpu = {"value": 0.003118085998796839, "unit": bench.UNIT, "cores": 16, "kind": "oracle", "sample": "x" * 100}
+    out = {key: 1.0 / 3.0 for key in bench.LINE_KEYS}
+    out.update(metric=bench.METRIC, unit=bench.UNIT, data="synthetic", config={"workload": bench.WORKLOAD, "l2_policy": "x" * 100}, peaks=peaks,
+               roofline=bench.gemm_roofline(1000.0 / 3.0, 5.0 / 3.0, peaks, clocks, 1e9 / 3.0), clocks=clocks, cpu_baseline=cpu,
+               e2e={"value": 1.0 / 3.0, "unit": bench.UNIT, "ms_per_step": 1.0 / 3.0, "steps": 5, "h2d_bytes_per_step": 2 ** 31, "d2h_bytes_per_step": 2 ** 29})
+    sweeps = {"per_rho": [{"a": 1.0 / 3.0}] * 1000, "kernel_breakdown": {"k": {}}}
+    line, details = bench.split_line({**out, **sweeps})
+    assert set(json.loads(line)) == set(bench.LINE_KEYS) and len(line) < 4000
+    assert json.loads(details) == {"details": sweeps}
