@@ -260,6 +260,11 @@ int rmm_reduced_gemm(const rmm_mat_t *A, const rmm_mat_t *B, const int32_t *idx,
 {
     int rc = check_gemm(A, B, idx, k, Y);
     if (rc != RMM_OK) return rc;
+    if (idx != nullptr && small_eligible(A, B, Y)) {  // (the same kernel as in rmm_product: the same sums)
+        rc = check_ws(ws, ws_bytes, gemm_least_bytes(A, B, k, Y), "reduced_gemm");
+        if (rc != RMM_OK) return rc;
+        return launch_small_product(A, B, k, scale, Y, nullptr, idx, &static_cast<WsHeader *>(ws)->status, static_cast<cudaStream_t>(stream));
+    }
     rmm_mat_t b = shared_b(A, B);
     GemvPlan gplan;
     if (gemv_eligible(A, &b, k, Y, &gplan)) {  // decode-step shapes: only the kept rows of B are read
@@ -372,7 +377,7 @@ size_t rmm_reduced_gemm_scored_workspace_bytes(const rmm_mat_t *A, const rmm_mat
     size_t need = 0;
     if (!gemv_eligible(A, &b, k, Y, &gplan) && tc_eligible(A, &b, k, Y, &plan, true) && plan.epilogue_energy) {
         need = plan.total_bytes;
-        if (!plan.gathers || !scored_apart(A->batch, A->rows, B->cols, k)) return need;
+        if (!small_eligible(A, B, Y) && (!plan.gathers || !scored_apart(A->batch, A->rows, B->cols, k))) return need;
     }
     const size_t p = rmm_reduced_gemm_workspace_bytes(A, B, k, Y), s = rmm_score_workspace_bytes(Y, 1);  // the output is scored by a pass of its own
     if (p == 0 || s == 0) return 0;
@@ -390,8 +395,9 @@ int rmm_reduced_gemm_scored(const rmm_mat_t *A, const rmm_mat_t *B, const int32_
     const size_t s1 = rmm_score_workspace_bytes(Y, 1), s2 = gemm_least_bytes(A, B, k, Y), apart = s1 > s2 ? s1 : s2;
     GemvPlan gplan;
     TcPlan plan;
-    if (!gemv_eligible(A, &b, k, Y, &gplan) && tc_eligible(A, &b, k, Y, &plan, true) && plan.epilogue_energy &&
-        !(plan.gathers && idx != nullptr && ws_bytes >= apart && scored_apart(A->batch, A->rows, B->cols, k))) {
+    // (small products take the form that rmm_reduced_gemm takes for them: the output is the same with and without its energies)
+    if (!(idx != nullptr && small_eligible(A, B, Y)) && !gemv_eligible(A, &b, k, Y, &gplan) && tc_eligible(A, &b, k, Y, &plan, true) &&
+        plan.epilogue_energy && !(plan.gathers && idx != nullptr && ws_bytes >= apart && scored_apart(A->batch, A->rows, B->cols, k))) {
         rc = check_ws(ws, ws_bytes, plan.least_bytes, "reduced_gemm_scored");
         if (rc != RMM_OK) return rc;
         return launch_gemm_tc(A, &b, idx, k, scale, Y, plan, ws, ws_bytes, static_cast<cudaStream_t>(stream), energy_out);
@@ -406,14 +412,15 @@ int rmm_reduced_gemm_scored(const rmm_mat_t *A, const rmm_mat_t *B, const int32_
 
 // ---- whole operation on device operands ------------------------------------------------------------
 struct ProductPlan {
-    bool fused;
+    bool small, fused;
     FrontPlan front;
     size_t total;
 };
 
-static int plan_product(const rmm_mat_t *A, const rmm_mat_t *B, const rmm_mat_t *Y, int64_t k, ProductPlan *pp)
+static int plan_product(const rmm_mat_t *A, const rmm_mat_t *B, const rmm_mat_t *Y, int64_t k, bool want_retained, ProductPlan *pp)
 {
     rmm_mat_t b = shared_b(A, B);
+    pp->small = !want_retained && small_eligible(A, B, Y);  // (asks for the workspace of the other forms all the same)
     pp->fused = k < A->cols && front_eligible(A, &b, Y, k, &pp->front);
     if (pp->fused) {
         pp->total = pp->front.total_bytes;
@@ -450,11 +457,12 @@ int rmm_product(const rmm_mat_t *A, const rmm_mat_t *B, double rho, int64_t k, f
     rc = check_gemm(A, B, idx, kk, Y);
     if (rc != RMM_OK) return rc;
     ProductPlan pp;
-    rc = plan_product(A, B, Y, kk, &pp);
+    rc = plan_product(A, B, Y, kk, retained != nullptr, &pp);
     if (rc != RMM_OK) return fail(rc, "product: operands not covered");
     rc = check_ws(ws, ws_bytes, pp.total, "product");
     if (rc != RMM_OK) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
+    if (pp.small) return launch_small_product(A, B, kk, scale, Y, idx, nullptr, &static_cast<WsHeader *>(ws)->status, st);
     if (kk == A->cols) {
         // every index is kept: the list is 0 .. K-1 (written by the selection, which also gives `retained`), and the product
         // is the unreduced one, which needs no gather at all
