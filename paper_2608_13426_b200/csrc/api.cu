@@ -241,7 +241,9 @@ size_t rmm_reduced_gemm_workspace_bytes(const rmm_mat_t *A, const rmm_mat_t *B, 
     if (gemv_eligible(A, &b, k, Y, &gplan)) return gplan.total_bytes;
     TcPlan plan;
     if (tc_eligible(A, &b, k, Y, &plan)) return plan.total_bytes;
-    return gemm_simt_workspace_bytes(A, &b, k);
+    const size_t fma = gemm_simt_workspace_bytes(A, &b, k);
+    SplitPlan split;
+    return plan_split(A, &b, k, &split) && split.total_bytes > fma ? split.total_bytes : fma;
 }
 
 // What a call needs: the forms that cut the contraction axis do with fewer pieces in a smaller workspace.  (A caller's one
@@ -280,6 +282,14 @@ int rmm_reduced_gemm(const rmm_mat_t *A, const rmm_mat_t *B, const int32_t *idx,
     }
     rc = check_ws(ws, ws_bytes, RMM_WS_HEADER_BYTES, "reduced_gemm");
     if (rc != RMM_OK) return rc;
+    SplitPlan split;
+    if (plan_split(A, &b, k, &split) && split.cost < gemm_simt_cost(A, &b, k) && ws_bytes >= split.total_bytes) {
+        rc = launch_split_gemm(A, &b, idx, k, scale, Y, split, ws, static_cast<cudaStream_t>(stream));
+        if (rc != RMM_OK) return rc;
+        // elements that cannot be split: the FMA kernel does the product (its scratch ends before the flags)
+        return launch_gemm_simt(A, &b, idx, k, scale, Y, ws, split.off_flags, static_cast<cudaStream_t>(stream),
+                                reinterpret_cast<const int *>(static_cast<char *>(ws) + split.off_flags), (int)(split.gather_blocks * A->batch));
+    }
     return launch_gemm_simt(A, &b, idx, k, scale, Y, ws, ws_bytes, static_cast<cudaStream_t>(stream));
 }
 

@@ -144,10 +144,24 @@ int launch_small_product(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k, floa
 
 // ---- reduced GEMM ------------------------------------------------------------------------------------
 // Plain FMA kernel: any strides, bf16 or fp32 operands, fp32 accumulation, bf16 or fp32 output.
+// n_flags > 0: the kernel returns at once unless one of flags[0 .. n_flags) is set (they must lie outside the workspace).
 int launch_gemm_simt(const rmm_mat_t *A, const rmm_mat_t *B, const int32_t *idx, int64_t k, float scale,
-                     const rmm_mat_t *Y, void *ws, size_t ws_bytes, cudaStream_t stream);
+                     const rmm_mat_t *Y, void *ws, size_t ws_bytes, cudaStream_t stream, const int *flags = nullptr, int n_flags = 0);
+double gemm_simt_cost(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k);  // estimate, microseconds
 // What the slices of the contraction axis want; a smaller workspace (down to the header) gets fewer slices.
 size_t gemm_simt_workspace_bytes(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k);
+
+// fp32 operands as sums of three bf16 numbers on the tensor cores (gemm_split.cu).  Leaves the product to the FMA kernel where a
+// kept element cannot be split: flags [0, gather_blocks * batch) at off_flags.
+struct SplitPlan {
+    int b_kmajor;
+    int64_t lda, ldb, gather_blocks, tiles, cut_first, seg_kb;
+    size_t off_a, off_b, off_partials, off_flags, total_bytes;
+    double cost;   // estimate, microseconds
+};
+bool plan_split(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k, SplitPlan *plan);
+int launch_split_gemm(const rmm_mat_t *A, const rmm_mat_t *B, const int32_t *idx, int64_t k, float scale, const rmm_mat_t *Y,
+                      const SplitPlan &plan, void *ws, cudaStream_t stream);
 
 // Decode-step path (M <= 4 rows of bf16 activations, B rows contiguous): HBM-bound gathered GEMV, no packing.
 struct GemvPlan {

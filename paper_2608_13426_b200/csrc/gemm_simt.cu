@@ -1,8 +1,8 @@
 // Reduced product Y = scale * A[:, I] B[I, :] (paper Sec. 3.2) on the plain FMA pipes.
 //
-// This kernel covers what the tensor-core path does not: fp32 operands (whose 1e-5 accuracy target
-// bf16 tensor-core inputs cannot meet) and bf16 operands with strides or alignments outside the TMA
-// rules.  Any element strides are accepted.
+// This kernel covers what the tensor-core paths do not: fp32 operands that are too small a product for gemm_split.cu, or whose
+// elements cannot be split there, and bf16 operands with strides or alignments outside the TMA rules.  Any element strides
+// are accepted.
 //
 // Bound: FMA issue.  A block of 128 threads owns a tile of 8 TM x 128 outputs and a thread TM x 8 of them, held as
 // pairs of columns for the packed fp32 FMA (one instruction, two FMAs; with single FMAs the same kernel took 480 us
@@ -35,6 +35,8 @@ struct SimtArgs {
     int64_t k_split;      // contraction indices per slice (a multiple of BK)
     float4 *partials;     // [tile][slice][TM * 2][THREADS]
     unsigned *counters;   // one per tile
+    const int *flags;     // n_flags > 0: nothing is done unless one of them is set
+    int n_flags;
 };
 
 template <bool BF16>
@@ -62,6 +64,11 @@ __global__ void __launch_bounds__(THREADS) reduced_gemm_simt_kernel(const SimtAr
     __shared__ __align__(16) float sB[kRing][BK][PB];
     __shared__ int s_last;
     pdl_wait();
+    if (a.n_flags > 0) {
+        int set = 0;
+        for (int i = threadIdx.x; i < a.n_flags; i += THREADS) set |= __ldg(a.flags + i);
+        if (!__syncthreads_or(set)) return;
+    }
 
     const int tid = threadIdx.x;
     const int64_t b = blockIdx.z / a.splits, slice = blockIdx.z % a.splits;
@@ -320,7 +327,7 @@ struct SimtPlan {
 // 1500 took 43 us for 59, but fp32 with B by columns took 634 for 435 on 2048 x 4096 x 1023 (32-row tiles), 864 for 650 on 2048 x
 // 2000 x 4094.
 // Slices whose partial sums take more than `room` bytes are not considered.
-SimtPlan plan_simt(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k, size_t room)
+SimtPlan plan_simt(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k, size_t room, double *estimate = nullptr)
 {
     static const double step_us[2][5] = {{1.15, 2.4, 2.7}, {0.9, 1.9, 2.1, 2.2, 2.3}};
     SimtPlan best = {8, 1, ceil_div(k, BK) * BK};
@@ -342,6 +349,7 @@ SimtPlan plan_simt(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k, size_t roo
             }
         }
     }
+    if (estimate != nullptr) *estimate = best_cost;
     return best;
 }
 
@@ -367,11 +375,19 @@ size_t gemm_simt_workspace_bytes(const rmm_mat_t *A, const rmm_mat_t *B, int64_t
     return RMM_WS_HEADER_BYTES + most;
 }
 
+double gemm_simt_cost(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k)
+{
+    double cost;
+    plan_simt(A, B, k, SIZE_MAX, &cost);
+    return cost;
+}
+
 int launch_gemm_simt(const rmm_mat_t *A, const rmm_mat_t *B, const int32_t *idx, int64_t k, float scale,
-                     const rmm_mat_t *Y, void *ws, size_t ws_bytes, cudaStream_t stream)
+                     const rmm_mat_t *Y, void *ws, size_t ws_bytes, cudaStream_t stream, const int *flags, int n_flags)
 {
     const SimtPlan plan = plan_simt(A, B, k, ws_bytes - RMM_WS_HEADER_BYTES);
-    SimtArgs a;
+    SimtArgs a = {};
+    a.flags = flags; a.n_flags = n_flags;
     a.A = A->ptr; a.B = B->ptr; a.Y = Y->ptr; a.idx = idx;
     a.M = A->rows; a.K = A->cols; a.N = B->cols; a.k = k;
     a.a_sb = A->stride_batch; a.a_sr = A->stride_row; a.a_sc = A->stride_col;

@@ -1,0 +1,89 @@
+"""fp32 products as sums of bf16 products on the tensor cores (gemm_split.cu)."""
+import pytest
+import torch
+
+import paper_2608_13426_b200 as rmm
+
+pytestmark = pytest.mark.gpu
+
+# sizes at which the split form is the cheaper one: edges of its 128 x 128 tiles, 64-index k-blocks, 8-column rows of the packed
+# parts; few tiles (the contraction cut into shares) and many
+SIZES = [(777, 3000, 1500, 1500), (385, 9000, 520, 8191), (384, 8192, 512, 8192), (1024, 1025, 1023, 1025), (2048, 2048, 1280, 449), (600, 4100, 513, 4097)]
+
+
+def operands(M, K, N, form, seed=0):
+    g = torch.Generator().manual_seed(seed + M + N)
+    A, B = torch.randn(M, K, generator=g).cuda(), (torch.randn(K, N, generator=g) * 0.02).cuda()
+    if form == "wide":                      # rows of B off 16 bytes, columns of A apart
+        return torch.stack([A, A], 2)[:, :, 0], torch.cat([B, B[:, :1]], 1)[:, :N]
+    if form == "columns":                   # both with the other axis contiguous
+        return A.t().contiguous().t(), B.t().contiguous().t()
+    return A, B
+
+
+def fma(A, B, idx):
+    """The same product by the FMA kernel: a workspace of the header only."""
+    ws = torch.zeros(4096 + 256, dtype=torch.uint8, device="cuda")
+    return rmm.rmm_reduced_gemm(A, B, idx, ws=ws)
+
+
+@pytest.mark.parametrize("form", ["rows", "wide", "columns"])
+@pytest.mark.parametrize("M, K, N, k", SIZES)
+def test_split_product_is_as_close_as_the_fma_kernel(M, K, N, k, form):
+    A, B = operands(M, K, N, form)
+    idx = torch.randperm(K, generator=torch.Generator().manual_seed(k))[:k].sort().values.int().cuda()
+    n0 = rmm.rmm_launch_count()
+    Y = rmm.rmm_reduced_gemm(A, B, idx)
+    assert rmm.rmm_launch_count() - n0 == 3
+    want = A[:, idx.long()].double() @ B[idx.long()].double()
+    err, ref = [float((y.double() - want).norm() / want.norm()) for y in (Y, fma(A, B, idx))]
+    assert err <= ref * 1.05 and err <= 2.0 ** -22, (err, ref)
+    assert torch.equal(Y, rmm.rmm_reduced_gemm(A, B, idx))          # pieces are added in order
+    half = rmm.rmm_reduced_gemm(A, B, idx, scale=0.5, out_dtype=torch.bfloat16)
+    assert torch.equal(half, (Y * 0.5).bfloat16())
+    assert rmm.rmm_status_read() == 0
+
+
+def test_batches_shared_weights_and_no_list():
+    A, B = torch.randn(3, 500, 2000, device="cuda"), torch.randn(3, 2000, 400, device="cuda")
+    idx = torch.stack([torch.randperm(2000)[:1500].sort().values for _ in range(3)]).int().cuda()
+    for b in (B, B[0]):
+        Y = rmm.rmm_reduced_gemm(A, b, idx)
+        for i in range(3):
+            want = A[i][:, idx[i].long()].double() @ (b if b.dim() == 2 else b[i])[idx[i].long()].double()
+            assert float((Y[i].double() - want).norm() / want.norm()) <= 2.0 ** -22
+    Y = rmm.rmm_reduced_gemm(A[0], B[0], None)
+    want = A[0].double() @ B[0].double()
+    assert float((Y.double() - want).norm() / want.norm()) <= 2.0 ** -22
+
+
+@pytest.mark.parametrize("value", [float("inf"), -float("inf"), float("nan"), 3e38, 1e-38, 1e-44, 2e12])
+@pytest.mark.parametrize("where", ["A", "B"])
+def test_elements_that_cannot_be_split_take_the_fma_kernel(value, where):
+    M, K, N, k = 777, 3000, 1500, 1500
+    A, B = operands(M, K, N, "rows", seed=5)
+    idx = torch.arange(0, 3000, 2, dtype=torch.int32, device="cuda")
+    plain = rmm.rmm_reduced_gemm(A, B, idx)
+    (A if where == "A" else B)[501 if where == "A" else 1001, 1001 if where == "A" else 501] = value    # not kept: nothing changes
+    assert torch.equal(rmm.rmm_reduced_gemm(A, B, idx), plain)
+    (A if where == "A" else B)[500, 500] = value
+    ws = torch.zeros(1 << 28, dtype=torch.uint8, device="cuda")
+    Y = rmm.rmm_reduced_gemm(A, B, idx, ws=ws)
+    want = A[:, ::2].double() @ B[::2].double()
+    assert torch.equal(Y.isfinite(), want.float().isfinite()) and torch.equal(Y.isnan(), want.float().isnan())
+    ok = want.float().isfinite()
+    assert torch.allclose(Y[ok].double(), want[ok], rtol=1e-5, atol=1e-5 * float(want[ok].abs().max()))
+    assert torch.equal(rmm.rmm_reduced_gemm(A, B, idx, ws=ws).nan_to_num(1.0), Y.nan_to_num(1.0))
+
+
+def test_bad_index_is_reported():
+    A, B = operands(777, 3000, 1500, "rows", seed=6)
+    idx = torch.arange(0, 3000, 2, dtype=torch.int32, device="cuda")
+    idx[3], idx[700] = -1, 3000
+    Y = rmm.rmm_reduced_gemm(A, B, idx)
+    assert rmm.rmm_status_read() == 6 and rmm.rmm_status_read() == 0
+    keep = torch.ones(1500, dtype=torch.bool)
+    keep[3] = keep[700] = False
+    kept = idx.cpu().long()[keep].cuda()
+    want = A[:, kept].double() @ B[kept].double()
+    assert float((Y.double() - want).norm() / want.norm()) <= 2.0 ** -22
