@@ -326,7 +326,7 @@ static int plan_q8(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k, const rmm_
 size_t rmm_reduced_gemm_q8_workspace_bytes(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k, const rmm_mat_t *Y)
 {
     Q8Plan q = {};
-    return plan_q8(A, B, k, Y, &q) == RMM_OK ? q.total : 0;
+    return plan_q8(A, B, k, Y, &q) == RMM_OK ? q.total + gemm_cut_bytes(1, A->rows, B->cols, ceil_div(k, 128)) : 0;
 }
 
 int rmm_reduced_gemm_q8(const rmm_mat_t *A, const rmm_mat_t *B, float b_scale, const int32_t *idx, int64_t k, float scale,
@@ -361,6 +361,8 @@ int rmm_reduced_gemm_q8(const rmm_mat_t *A, const rmm_mat_t *B, float b_scale, c
     p.y = Y->ptr; p.y_bf16 = Y->dtype == RMM_BF16; p.y_sb = Y->stride_batch; p.y_sr = Y->stride_row;
     p.scale = scale * b_scale;
     p.status = status;
+    p.partials = reinterpret_cast<float *>(w + q.total);
+    p.partials_bytes = ws_bytes - q.total;
     return launch_gemm_tc_problem(p, st);
 }
 

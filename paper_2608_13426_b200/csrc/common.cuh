@@ -127,6 +127,11 @@ int launch_select(const float *keys, int64_t batch, int64_t K, int64_t k, int32_
                   cudaStream_t stream);
 
 // Front end of a whole product in one launch (scores, selection, packed A[:, I] and B[I, :]); see score_select.cu.
+// The largest products it takes.  Tall or wide ones gather faster through the separate gather launches (whole rows of A per
+// block with full-line stores; rows of B spread over every SM) than through the front end's 64-byte pieces per row and its 16
+// copying warps per block.  Measured at 8192 columns of A, rho = 0.5: ahead by 4 to 6 us up to 8192 rows when B has 2048
+// columns, level at 16384 rows, behind by 15 % at 32768; behind at every row count when B has 8192 columns.
+constexpr int64_t kFrontMaxRows = 8192, kFrontMaxK = 8192, kFrontMaxCols = 4096;
 struct FrontPlan {
     int col_blocks;
     int64_t ldp;  // row pitch of the packed A (multiple of 8)
@@ -178,7 +183,7 @@ struct TcPlan {
     int64_t ldp;        // leading dimension of the packed operands (multiple of 8)
     bool gathers;       // with an index list the kernel fetches the kept rows of B itself (column energies: from whole tiles only)
     bool few_rows;      // gathers, by the kernel for few rows (gemm_skinny.cu)
-    size_t off_ap, off_bp, off_colen, total_bytes;
+    size_t off_ap, off_bp, off_colen, off_cut, total_bytes;
     size_t least_bytes;    // what a call needs: where the kernel gathers B, a workspace without room for all partial sums does with
                            // fewer pieces, from the size on that the packed rows of B would take
     bool epilogue_energy;  // the plan reserves the per-group column energies of Y and the epilogue fills them
@@ -203,7 +208,7 @@ struct TcProblem {
     // kept rows b_idx[i * b_idx_stride + 0 .. k-1] itself (no packed copy of B; outputs of up to 128 rows)
     const int32_t *b_idx;
     int64_t b_idx_stride, b_rows;
-    float *partials;         // with b_idx: room for the fp32 sums of pieces of the contraction; what does not fit is not cut
+    float *partials;         // or NULL: room for the fp32 sums of pieces of the contraction; what does not fit is not cut
     size_t partials_bytes;
     void *y;
     int y_bf16;
@@ -219,6 +224,7 @@ struct TcProblem {
     float *col_energy;
 };
 int launch_gemm_tc_problem(const TcProblem &p, cudaStream_t stream);
+size_t gemm_cut_bytes(int64_t batch, int64_t M, int64_t N, int64_t k_blocks);   // what it uses of partials without b_idx
 // The same for at most kSkinnyRows rows with b_idx set (gemm_skinny.cu).
 constexpr int64_t kSkinnyRows = 32;
 size_t gemm_skinny_partial_bytes(int64_t batch, int64_t M, int64_t N, int64_t k);

@@ -73,7 +73,7 @@ struct TcArgs {
     const int32_t *b_idx;
     int64_t b_ld, b_sb, b_idx_stride, b_rows;
     int64_t seg_kb;              // k-blocks per block: the k-blocks of all tiles form one axis that is cut into equal shares; 0: whole tiles
-    float *partials;             // [2 x blocks][min(M, 128)][256] unscaled sums of the tiles that were cut
+    float *partials;             // [2 x blocks][min(M, 128)][256] unscaled sums of the tiles that were cut; CUT: [2 x CTAs][64][128] float4
 };
 
 // BN = tile columns (MMA N, accumulator columns); CTAS = CTAs per tile.  With CTAS == 2 a pair of CTAs on one TPC
@@ -110,7 +110,9 @@ __device__ __forceinline__ void tile_coords(int64_t t, int tiles_m, int tiles_n,
 // FP8: both operands are e4m3 bytes, K-major (tcgen05.mma kind::f8f6f4, 32 contraction indices per instruction); a
 // pipeline stage is still 128 bytes per row, i.e. 128 indices instead of 64, and the epilogue multiplies every output
 // row by its own scale (the activation row's quantisation step times the weight's).
-template <int BN, bool B_KMAJOR, bool OUT_BF16, int CTAS, bool B_GATHER, bool FP8>
+// CUT: CTA pairs that take equal shares of all tiles' k-blocks instead of whole tiles (outputs of few tiles); a form of its own, since
+// its epilogue made the ordinary one 10 % slower.
+template <int BN, bool B_KMAJOR, bool OUT_BF16, int CTAS, bool B_GATHER, bool FP8, bool CUT>
 __global__ void __launch_bounds__(B_GATHER ? kThreadsTc + 32 * kGatherWarps : kThreadsTc2, 1)
 reduced_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                        const __grid_constant__ CUtensorMap map_y, TcArgs a)
@@ -138,11 +140,11 @@ reduced_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
     constexpr int UK = FP8 ? 2 * UMMA_K : UMMA_K;   // contraction indices per MMA instruction (32 bytes per row)
     static_assert(!FP8 || (B_KMAJOR && !B_GATHER), "8-bit operands: both K-major, packed");
     const int num_kb = (int)((a.k + BKE - 1) / BKE);
-    // The n-th piece of work of this block: k-blocks [kb0, kb1) of a tile.  Whole tiles, round robin; where the gather form
-    // cuts them, what its share of the joint (tile, k-block) axis holds (only the first and the last of its tiles are cut).
+    // The n-th piece of work of this block (or pair): k-blocks [kb0, kb1) of a tile.  Whole tiles, round robin; where tiles are cut,
+    // what its share of the joint (tile, k-block) axis holds (only the first and the last of its tiles are cut).
     auto piece = [&](int64_t n, int64_t &tile, int &kb0, int &kb1) -> bool {
-        if (B_GATHER && a.seg_kb > 0) {
-            const int64_t begin = (int64_t)blockIdx.x * a.seg_kb, end = min(num_tiles * num_kb, begin + a.seg_kb);
+        if (CUT || (B_GATHER && a.seg_kb > 0)) {
+            const int64_t begin = (int64_t)(blockIdx.x / CTAS) * a.seg_kb, end = min(num_tiles * num_kb, begin + a.seg_kb);
             const int64_t pos = n == 0 ? begin : (begin / num_kb + n) * num_kb;
             if (pos >= end) return false;
             tile = pos / num_kb;
@@ -434,6 +436,19 @@ reduced_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
                                    make_float4(__uint_as_float(r[4 * v]), __uint_as_float(r[4 * v + 1]), __uint_as_float(r[4 * v + 2]), __uint_as_float(r[4 * v + 3])));
                     }
                 }
+            } else if (CUT && kb1 - kb0 < num_kb) {
+                // part of the contraction (pair_meet_kernel adds the parts up): 32 rows of four columns are 512 contiguous bytes
+                float4 *dst = reinterpret_cast<float4 *>(a.partials) + (2 * (int64_t)blockIdx.x + (n > 0 ? 1 : 0)) * (BN / 4) * BM + q * 32 + lane;
+#pragma unroll 1
+                for (int c = eset; c < BN / 32; c += a.epi_sets) {
+                    uint32_t r[32];
+                    tmem_ld32_issue(t_row + c * 32, r);
+                    tmem_ld_wait();
+#pragma unroll
+                    for (int v = 0; v < 8; ++v)
+                        __stcg(dst + (c * 8 + v) * BM, make_float4(__uint_as_float(r[4 * v]), __uint_as_float(r[4 * v + 1]), __uint_as_float(r[4 * v + 2]),
+                                                                   __uint_as_float(r[4 * v + 3])));
+                }
             } else if constexpr (OUT_BF16) {
                 // 64 columns at a time: two TMEM loads, scale and round, one 32 x 64 slab per warp through a TMA store
 #pragma unroll 1
@@ -599,26 +614,107 @@ __global__ void __launch_bounds__(32 * kMeetRows) gemm_meet_kernel(const TcArgs 
     }
 }
 
+// The same for tiles of CTA pairs: 32 rows of a 256 x 256 tile per block; a thread adds 32 columns of one row, and the rows are
+// written out through shared memory.
+template <bool OUT_BF16>
+__global__ void __launch_bounds__(256) pair_meet_kernel(const TcArgs a, int num_kb)
+{
+    __shared__ __align__(16) float s_out[32][256 + 4];
+    pdl_wait();
+    const int64_t tile = blockIdx.x, per_batch = (int64_t)a.tiles_n * a.tiles_m, b = tile / per_batch;
+    const int64_t u0 = tile * num_kb / a.seg_kb, u1 = ((tile + 1) * num_kb - 1) / a.seg_kb;
+    if (u0 == u1) return;  // written by its only pair
+    int tm, tn;
+    tile_coords(tile - b * per_batch, a.tiles_m, a.tiles_n, a.raster, tm, tn);
+    const int r0 = blockIdx.y * 32, rank = r0 / BM, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t m0 = (int64_t)tm * 2 * BM + r0, n0 = (int64_t)tn * 256;
+    if (m0 >= a.M) return;
+    float4 v[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 2
+    for (int64_t u = u0; u <= u1; ++u) {  // only a tile's first pair can hold it as its last piece
+        const int64_t slot = 2 * (2 * u + rank) + (u == u0 && u0 * a.seg_kb < tile * num_kb ? 1 : 0);
+        const float4 *src = reinterpret_cast<const float4 *>(a.partials) + (slot * 64 + warp * 8) * BM + (r0 % BM) + lane;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const float4 x = __ldcg(src + i * BM);
+            v[i].x += x.x; v[i].y += x.y; v[i].z += x.z; v[i].w += x.w;
+        }
+    }
+    float scale = a.scale;
+    if (a.row_scale != nullptr && m0 + lane < a.M) scale *= __ldg(a.row_scale + b * a.M + m0 + lane);
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+        *reinterpret_cast<float4 *>(&s_out[lane][warp * 32 + 4 * i]) = make_float4(v[i].x * scale, v[i].y * scale, v[i].z * scale, v[i].w * scale);
+    __syncthreads();
+    if (OUT_BF16 && a.col_energy != nullptr && n0 + threadIdx.x < a.N) {  // as the epilogue has them: even and odd rows apart
+        float ea = 0.f, eb = 0.f;
+#pragma unroll
+        for (int r = 0; r < 32; r += 2) {
+            const float x = __bfloat162float(__float2bfloat16_rn(s_out[r][threadIdx.x])), y = __bfloat162float(__float2bfloat16_rn(s_out[r + 1][threadIdx.x]));
+            ea = fmaf(x, x, ea);
+            eb = fmaf(y, y, eb);
+        }
+        a.col_energy[(b * ((a.M + 31) / 32) + m0 / 32) * a.N + n0 + threadIdx.x] = ea + eb;
+    }
+    for (int r = warp; r < 32 && m0 + r < a.M; r += 8) {
+        const int64_t n = n0 + lane * 8, off = b * a.y_sb + (m0 + r) * a.y_sr + n;   // rows of Y start on 16 bytes
+        const float4 x = *reinterpret_cast<const float4 *>(&s_out[r][lane * 8]), y = *reinterpret_cast<const float4 *>(&s_out[r][lane * 8 + 4]);
+        const float w[8] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w};
+        if constexpr (OUT_BF16) {
+            __nv_bfloat16 *d = static_cast<__nv_bfloat16 *>(a.Y) + off;
+            if (n + 8 <= a.N) {
+                uint32_t q[4];
+#pragma unroll
+                for (int p = 0; p < 4; ++p) {
+                    const __nv_bfloat162 h = __floats2bfloat162_rn(w[2 * p], w[2 * p + 1]);
+                    q[p] = *reinterpret_cast<const uint32_t *>(&h);
+                }
+                *reinterpret_cast<uint4 *>(d) = make_uint4(q[0], q[1], q[2], q[3]);
+            } else {
+                for (int e = 0; e < 8 && n + e < a.N; ++e) d[e] = __float2bfloat16_rn(w[e]);
+            }
+        } else {
+            float *d = static_cast<float *>(a.Y) + off;
+            if (n + 8 <= a.N) {
+                reinterpret_cast<float4 *>(d)[0] = x;
+                reinterpret_cast<float4 *>(d)[1] = y;
+            } else {
+                for (int e = 0; e < 8 && n + e < a.N; ++e) d[e] = w[e];
+            }
+        }
+    }
+}
+
 // ----------------------------------------------------------------------------------------------
 // host side
 // ----------------------------------------------------------------------------------------------
-template <int BN, bool B_KMAJOR, bool OUT_BF16, int CTAS, bool B_GATHER = false, bool FP8 = false>
+template <int BN, bool B_KMAJOR, bool OUT_BF16, int CTAS, bool B_GATHER = false, bool FP8 = false, bool CUT = false>
 int launch_variant(const CUtensorMap &ma, const CUtensorMap &mb, const CUtensorMap &my, const TcArgs &a, cudaStream_t stream)
 {
-    auto kern = reduced_gemm_tc_kernel<BN, B_KMAJOR, OUT_BF16, CTAS, B_GATHER, FP8>;
+    if constexpr (CTAS == 2 && !CUT) {
+        if (a.seg_kb > 0) return launch_variant<BN, B_KMAJOR, OUT_BF16, CTAS, B_GATHER, FP8, true>(ma, mb, my, a, stream);
+    }
+    auto kern = reduced_gemm_tc_kernel<BN, B_KMAJOR, OUT_BF16, CTAS, B_GATHER, FP8, CUT>;
     using L = SmemLayout<BN, CTAS>;
     static PerDeviceOnce configured;
     if (cudaError_t e = configured.smem(L::kTotal, kern)) return fail(RMM_ERR_CUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e));
     const int64_t tiles = a.batch * a.tiles_m * a.tiles_n, num_kb = ceil_div(a.k, FP8 ? 2 * BK : BK);
     const int64_t slots = sm_count() / CTAS;
-    const int64_t blocks = B_GATHER && a.seg_kb > 0 ? ceil_div(tiles * num_kb, a.seg_kb) : (tiles < slots ? tiles : slots);
+    const int64_t blocks = a.seg_kb > 0 ? ceil_div(tiles * num_kb, a.seg_kb) : (tiles < slots ? tiles : slots);
     prof_begin("reduced_gemm_tc_kernel", stream);
     cudaError_t e = launch_kernel(kern, dim3((unsigned)(blocks * CTAS)),
                                   dim3(B_GATHER ? kThreadsTc + 32 * kGatherWarps : (a.epi_sets == 2 ? kThreadsTc2 : kThreadsTc)), L::kTotal, stream,
                                   CTAS, ma, mb, my, a);
     if (e != cudaSuccess) return fail(RMM_ERR_CUDA, "reduced_gemm_tc_kernel: launch: %s", cudaGetErrorString(e));
     int rc = check_launch("reduced_gemm_tc_kernel", stream);
-    if (!B_GATHER || rc != RMM_OK || a.seg_kb == 0) return rc;
+    if (rc != RMM_OK || a.seg_kb == 0) return rc;
+    if constexpr (CUT) {
+        prof_begin("pair_meet_kernel", stream);
+        launch_kernel(pair_meet_kernel<OUT_BF16>, dim3((unsigned)tiles, 2 * BM / 32), dim3(256), 0, stream, 1, a, (int)num_kb);
+        return check_launch("pair_meet_kernel", stream);
+    }
     prof_begin("gemm_meet_kernel", stream);
     launch_kernel(gemm_meet_kernel<OUT_BF16>, dim3((unsigned)tiles, (unsigned)ceil_div(a.M < BM ? a.M : BM, kMeetRows)), dim3(32 * kMeetRows), 0,
                   stream, 1, a, (int)num_kb);
@@ -650,6 +746,21 @@ size_t gather_partial_bytes(int64_t batch, int64_t M, int64_t N, int64_t k)
 }
 
 }  // namespace
+
+// Outputs of fewer pair tiles than there are pairs: each pair takes an equal share of all k-blocks instead, where that saves more
+// than writing the pieces and adding them up costs, about 18 us (300 x 10000 kept x 2048, 16 tiles: 99 -> 71 us a call).  Cutting only the
+// last of several rounds gains nothing: its few tiles run faster than those of a full one (32768 x 14336 kept x 8192 lost 9 %).
+// Room for two pieces of a 128 x 256 tile per CTA, 0 where tiles stay whole (more k-blocks never need less).
+size_t gemm_cut_bytes(int64_t batch, int64_t M, int64_t N, int64_t k_blocks)
+{
+    if (M <= BM || N <= 128) return 0;
+    const int64_t slots = sm_count() / 2, tiles = batch * ceil_div(M, 2 * BM) * ceil_div(N, 256);
+    if (tiles >= slots || (1.0 - (double)tiles / (double)slots) * 0.37 * (double)k_blocks <= 18.0) return 0;
+    return (size_t)(2 * (slots * 2)) * BM * 256 * 4;
+}
+
+// Shapes that the one-launch front end may take stay with whole tiles, there and here: a product is the same in both forms.
+static bool may_cut(int64_t M, int64_t K, int64_t N) { return K > kFrontMaxK || M > kFrontMaxRows || N > kFrontMaxCols; }
 
 bool tc_eligible(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k, const rmm_mat_t *Y, TcPlan *plan, bool with_energy)
 {
@@ -690,8 +801,10 @@ bool tc_eligible(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k, const rmm_ma
         off += third;
         plan->off_colen = off;
         if (plan->epilogue_energy) off += align_up((size_t)batch * ceil_div(M, 32) * N * 4, 256);
-        plan->total_bytes = off;
         plan->least_bytes = off - third + (third < packed_b ? third : packed_b);
+        plan->off_cut = off;
+        if (!plan->gathers && may_cut(M, K, N)) off += gemm_cut_bytes(batch, M, N, ceil_div(k, BK));
+        plan->total_bytes = off;
     }
     return true;
 }
@@ -712,13 +825,16 @@ int launch_gemm_tc_problem(const TcProblem &p, cudaStream_t stream)
         if (rc != RMM_OK) return rc;
     }
     const int BN = p.N <= 128 ? 128 : 256;
-    // CTA pairs (256 x 256 tiles, a third fewer operand bytes per flop) pay off once there are enough pair tiles to
-    // keep every SM pair busy: measured 1.81-1.87 PFLOP/s against 1.51-1.59 for single CTAs on 8192 x 8192 outputs,
-    // while on a 2048 x 2048 output (64 pair tiles for 74 SM pairs) the pair's longer set-up and epilogue lose about
-    // 2 us.  RMM_GEMM_CTAS=1 or 2 forces a form (for measurements).
+    // CTA pairs (256 x 256 tiles, a third fewer operand bytes per flop) or single CTAs (128 x 256, two of them where the pair has
+    // one): whichever takes less by rounds of blocks.  Microseconds a k-block 0.37 for pairs, 0.42 for single CTAs, 3 a round, and
+    // the longer set-up of a pair, which 8-bit operands (k-blocks of 128) feel more.  One round, 64 pairs: 2048 x 4096 kept x
+    // 2048 29.6 us by pairs, 31.8 by single CTAs, 300 x 4096 x 8192 29.7 and 33; 2048 kept: level; 20000 x 750 x 256 49.6 and 50.2 (whole calls); 8-bit 2048 x 4096 x 2048 18.6 and
+    // 17.5.  Several rounds: 3000 x 4000 x 4096 70.7 and 82.  RMM_GEMM_CTAS=1 or 2 forces a form (for measurements).
     static const int forced = []() { const char *e = getenv("RMM_GEMM_CTAS"); return e ? atoi(e) : 0; }();
-    const int64_t pair_tiles = p.batch * ceil_div(p.M, 2 * BM) * ceil_div(p.N, 256);
-    int ctas = (BN == 256 && p.M > BM && pair_tiles >= sm_count() / 2) ? 2 : 1;
+    const int64_t sms = sm_count(), k_blocks = ceil_div(p.k, (int64_t)bke), pair_tiles = p.batch * ceil_div(p.M, 2 * BM) * ceil_div(p.N, 256);
+    const double singles_us = (double)ceil_div(p.batch * ceil_div(p.M, BM) * ceil_div(p.N, 256), sms) * (3.0 + 0.42 * (double)k_blocks);
+    const double pairs_us = (double)ceil_div(pair_tiles, sms / 2) * (3.0 + 0.37 * (double)k_blocks) + (p.fp8 ? 2.5 : 1.0);
+    int ctas = BN == 256 && p.M > BM && pairs_us < singles_us ? 2 : 1;
     if (forced == 1) ctas = 1;
     if (forced == 2 && BN == 256 && p.M > BM) ctas = 2;
     if (p.b_idx != nullptr) ctas = 1;  // the in-kernel row gather exists for single-CTA tiles
@@ -762,6 +878,12 @@ int launch_gemm_tc_problem(const TcProblem &p, cudaStream_t stream)
     a.epi_sets = (p.y_bf16 && p.b_idx == nullptr && (ceil_div(p.k, (int64_t)bke) <= 4 || n_tiles <= sm_count() / ctas)) ? 2 : 1;
     a.b_src = p.b; a.b_idx = p.b_idx; a.b_ld = p.b_ld; a.b_sb = p.b_batches > 1 ? p.b_sb : 0; a.b_idx_stride = p.b_idx_stride;
     a.b_rows = p.b_rows;
+    a.seg_kb = 0; a.partials = nullptr;
+    const size_t cut_bytes = gemm_cut_bytes(p.batch, p.M, p.N, k_blocks);
+    if (ctas == 2 && p.b_idx == nullptr && p.partials != nullptr && cut_bytes > 0 && p.partials_bytes >= cut_bytes) {
+        a.seg_kb = ceil_div(n_tiles * k_blocks, sms / 2);
+        a.partials = p.partials;
+    }
     if (p.b_idx != nullptr) {
         // A product of few rows is bound by how fast the SMs pull rows of B, so none may idle: equal shares of all tiles'
         // k-blocks, one per SM (at least two k-blocks each), where whole tiles would leave too many without work.  Cutting
@@ -769,7 +891,7 @@ int launch_gemm_tc_problem(const TcProblem &p, cudaStream_t stream)
         // piece of a tile) and a k-block takes 1.27 of them with every SM pulling, 0.88 with whole tiles.  Whole calls, a quarter
         // or half of the rows kept: 48 x 28672 (half) x 8192, 32 tiles: 75 us cut; 128 x 8192 (a quarter) x 8192: 42 cut, 32
         // whole; 48 x 8192 (half) x 28672, 112 tiles: 64.5 whole.
-        const int64_t num_kb = ceil_div(p.k, (int64_t)BK), sms = sm_count();
+        const int64_t num_kb = ceil_div(p.k, (int64_t)BK);
         a.seg_kb = ceil_div(n_tiles * num_kb, sms);
         if (a.seg_kb < 2) a.seg_kb = 2;
         const double whole = 0.88 * (double)(ceil_div(n_tiles, sms) * num_kb), pieces = (double)num_kb / (double)a.seg_kb;
@@ -853,6 +975,10 @@ int launch_gemm_tc(const rmm_mat_t *A, const rmm_mat_t *B, const int32_t *idx, i
     p.scale = scale; p.status = status;
     p.col_energy = plan.epilogue_energy ? reinterpret_cast<float *>(w + plan.off_colen) : nullptr;
     p.b_batch_off = 0; p.b_batch_div = 1; p.b_batches = batch;
+    if (!plan.gathers && may_cut(M, K, N)) {
+        p.partials = reinterpret_cast<float *>(w + plan.off_cut);
+        p.partials_bytes = ws_bytes > plan.off_cut ? ws_bytes - plan.off_cut : 0;
+    }
 
     // the unreduced product (idx NULL, k == K) on TMA-loadable operands needs no gather at all
     const bool in_place = idx == nullptr && !plan.b_kmajor && reinterpret_cast<uintptr_t>(A->ptr) % 16 == 0 &&

@@ -28,7 +28,7 @@ namespace {
 constexpr int kThreads = 1024;     // one block per SM: its tail (the select) then has 32 warps to work with
 constexpr int kUnroll = 4;       // rows in flight per thread (1024 threads x 4 x 16 B = 64 KB in flight per SM)
 constexpr int kFlushEvery = 4;   // loop trips between fp32 -> fp64 flushes (kUnroll * kFlushEvery = 16 terms)
-constexpr int kFusedSelectMax = 8192;    // largest K whose select runs in the score kernel's tail
+constexpr int kFusedSelectMax = (int)kFrontMaxK;    // largest K whose select runs in the score kernel's tail
 constexpr int kCachedSelectMax = 49152;  // largest K that one selecting block caches in shared memory (192 KB)
 
 using namespace sel;
@@ -471,11 +471,6 @@ struct FrontArgs {
     int rows_per_chunk;       // rows of A per chunk of the gather: 64 KB / (2 n)
 };
 
-// Tall or wide products gather faster through the separate gather launches (whole rows of A per block with full-line
-// stores; rows of B spread over every SM) than through this kernel's 64-byte pieces per row and its 16 copying warps
-// per block.  Measured at 8192 columns of A, rho = 0.5: ahead by 4 to 6 us up to 8192 rows when B has 2048 columns,
-// level at 16384 rows, behind by 15 % at 32768; behind at every row count when B has 8192 columns.
-constexpr int64_t kFrontMaxRows = 8192, kFrontMaxCols = 4096;
 constexpr int kChunkSlots = 3;                         // row chunks in the ring
 constexpr int kChunkBytes = 2 * kTmaStageBytes;        // 64 KB: rows_per_chunk = 64 KB / row bytes
 constexpr int kGroupsPerThread = 4;                    // 8-byte output groups per gathering thread and row: k <= 4 * 4 * 512
