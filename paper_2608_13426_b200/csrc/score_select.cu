@@ -940,19 +940,45 @@ __global__ void __launch_bounds__(kSelThreads) select_cluster_kernel(const Clust
                 if (r0 + q < a.m) use(r0 + q, w[q]);
         }
     };
+    // Two columns a thread (lists of up to 8192): all rows are requested at once and stay in registers, so that the gather below does
+    // not fetch them again.
+    constexpr bool kHeld = FROM_A && ITEMS == 2;
+    unsigned held[kHeld ? kFewRows : 1];
     if constexpr (FROM_A) {
         col = a.A + b * a.s_batch + j0;
         double e[ITEMS];
 #pragma unroll
         for (int i = 0; i < ITEMS; ++i) e[i] = 0.0;
-        each_row([&](int, const unsigned (&w)[ITEMS / 2]) {
+        auto add = [&](int, const unsigned (&w)[ITEMS / 2]) {
 #pragma unroll
             for (int i = 0; i < ITEMS; ++i) {
                 const float x = __uint_as_float(i & 1 ? w[i / 2] & 0xffff0000u : w[i / 2] << 16);
                 // exact for magnitudes from 2^-63 to 2^64; squared in 64 bits, 512 lists of 8192 took 150 us where this takes 119
                 e[i] += (double)(x * x);
             }
-        });
+        };
+        if constexpr (kHeld) {
+            const bool wide = a.vec && nvalid == ITEMS;
+#pragma unroll
+            for (int r0 = 0; r0 < kFewRows; r0 += 8) {
+                if (r0 >= a.m) break;
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                    const __nv_bfloat16 *p = col + (r0 + q < a.m ? r0 + q : r0) * a.s_row;
+                    const unsigned short *p2 = reinterpret_cast<const unsigned short *>(p);
+                    if (wide) held[r0 + q] = __ldg(reinterpret_cast<const unsigned *>(p));
+                    else held[r0 + q] = (nvalid > 0 ? (unsigned)__ldg(p2) : 0u) | (nvalid > 1 ? (unsigned)__ldg(p2 + 1) << 16 : 0u);
+                }
+            }
+#pragma unroll
+            for (int r = 0; r < kFewRows; ++r) {
+                if (r >= a.m) break;
+                const unsigned w[1] = {held[r]};
+                add(r, reinterpret_cast<const unsigned (&)[ITEMS / 2]>(w));
+            }
+        } else {
+            each_row(add);
+        }
 #pragma unroll
         for (int i = 0; i < ITEMS; ++i) {
             u[i] = i < nvalid ? key_image((float)e[i]) : 0u;
@@ -1068,11 +1094,21 @@ __global__ void __launch_bounds__(kSelThreads) select_cluster_kernel(const Clust
     if constexpr (FROM_A) {
         if (a.Ap != nullptr) {
             unsigned short *dst = reinterpret_cast<unsigned short *>(a.Ap) + b * a.m * a.ldp;
-            each_row([&](int r, const unsigned (&w)[ITEMS / 2]) {
+            auto put = [&](int r, const unsigned (&w)[ITEMS / 2]) {
 #pragma unroll
                 for (int i = 0; i < ITEMS; ++i)
                     if (pos[i] >= 0) dst[r * a.ldp + pos[i]] = (unsigned short)(i & 1 ? w[i / 2] >> 16 : w[i / 2]);
-            });
+            };
+            if constexpr (kHeld) {
+#pragma unroll
+                for (int r = 0; r < kFewRows; ++r) {
+                    if (r >= a.m) break;
+                    const unsigned w[1] = {held[r]};
+                    put(r, reinterpret_cast<const unsigned (&)[ITEMS / 2]>(w));
+                }
+            } else {
+                each_row(put);
+            }
             const int pad = (int)(a.ldp - k);
             for (int i = tid; rank == 0 && i < a.m * pad; i += kSelThreads) dst[i / pad * a.ldp + k + i % pad] = 0;
         }
