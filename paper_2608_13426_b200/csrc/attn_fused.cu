@@ -250,14 +250,24 @@ fused_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
     const int kq = (a.kd + 63) / 64, nv = (a.Dh + 63) / 64;       // 64-column chunks of Q/K and of V
     const int blocks_r = (int)((a.Lr + kGroups * FM - 1) / (kGroups * FM));
     const int64_t items = a.heads * blocks_r;
-    // kept keys (GATHERED) with position <= limit: T is ascending
+    // kept keys (GATHERED) with position <= limit (the same for the whole warp): T is ascending.  The lanes look at 32 places at a
+    // time: every item starts with four such searches one after the other, and a memory latency per halving was a fifth of the kernel.
     auto kept_upto = [&](const int32_t *T, int64_t limit) -> int64_t {
         int64_t lo = 0, hi = a.Lc;
         while (lo < hi) {
-            const int64_t mid = (lo + hi) >> 1;
-            if ((int64_t)__ldg(T + mid) <= limit) lo = mid + 1; else hi = mid;
+            const int64_t step = (hi - lo + 31) / 32, at = lo + (lane + 1) * step - 1;  // the last place of the lane's part
+            const int whole = __popc(__ballot_sync(0xffffffffu, at < hi && (int64_t)__ldg(T + at) <= limit));
+            lo += whole * step;
+            hi = min(hi, lo + step - 1);
         }
         return lo;
+    };
+    // the same for limit + lane
+    auto kept_upto_rows = [&](const int32_t *T, int64_t limit) -> int64_t {
+        const int64_t first = kept_upto(T, limit);
+        const int64_t ahead = first + lane < a.Lc ? (int64_t)__ldg(T + first + lane) - limit : 32;   // at least 1; 31 of them at most matter
+        const unsigned marks = __reduce_or_sync(0xffffffffu, ahead < 32 ? 1u << ahead : 0u);
+        return first + __popc(marks & (0xffffffffu >> (31 - lane)));
     };
     // Column tiles [jb, je) that the 128 rows starting at r0 need (empty: jb = je = 0).
     auto tile_range = [&](int64_t head, int64_t r0, int *jb, int *je) {
@@ -351,7 +361,7 @@ fused_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             if (++ks == kKvStages) { ks = 0; kph ^= 1u; }
             return true;
         };
-        for (int64_t n = 0; lane == 0 && n < rounds && ok; ++n) {
+        for (int64_t n = 0; n < rounds && ok; ++n) {
             int64_t head, r0;
             if (!item_of(n, &head, &r0)) continue;
             int jb, je;
@@ -359,20 +369,25 @@ fused_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             Tiles tiles = tiles_of(head, r0, true);
             jb = tiles.next(jb, je);
             if (je <= jb) continue;
-            const int vb = (int)((head + a.v_off) / a.v_div);
-            if (!mbar_wait_sleepy(q_empty, (n_item & 1u) ^ 1u, abort_flag, a.status, a.wait_ns)) { ok = false; break; }
-            mbar_arrive_expect_tx(q_full, (uint32_t)(kGroups * kq) * kQChunk);
-            for (int g = 0; g < kGroups; ++g)
-                for (int c = 0; c < kq; ++c)
-                    tma_load_3d(base + kOffQ + g * kQTile + c * kQChunk, &map_q, c * 64, (int)(r0 + g * FM), (int)head, q_full);
-            ok = load_kv(&map_k, kq, (int64_t)jb * FN, (int)head);
-            for (int j = jb, nj; j < je && ok; j = nj) {
-                nj = tiles.next(j + 1, je);
-                if (nj < je) ok = load_kv(&map_k, kq, (int64_t)nj * FN, (int)head);
-                if constexpr (kHasV) {
-                    if (ok) ok = load_kv(&map_v, nv, (int64_t)j * FN, vb);
+            if (lane == 0) {
+                const int vb = (int)((head + a.v_off) / a.v_div);
+                ok = mbar_wait_sleepy(q_empty, (n_item & 1u) ^ 1u, abort_flag, a.status, a.wait_ns);
+                if (ok) {
+                    mbar_arrive_expect_tx(q_full, (uint32_t)(kGroups * kq) * kQChunk);
+                    for (int g = 0; g < kGroups; ++g)
+                        for (int c = 0; c < kq; ++c)
+                            tma_load_3d(base + kOffQ + g * kQTile + c * kQChunk, &map_q, c * 64, (int)(r0 + g * FM), (int)head, q_full);
+                    ok = load_kv(&map_k, kq, (int64_t)jb * FN, (int)head);
+                }
+                for (int j = jb, nj; j < je && ok; j = nj) {
+                    nj = tiles.next(j + 1, je);
+                    if (nj < je) ok = load_kv(&map_k, kq, (int64_t)nj * FN, (int)head);
+                    if constexpr (kHasV) {
+                        if (ok) ok = load_kv(&map_v, nv, (int64_t)j * FN, vb);
+                    }
                 }
             }
+            ok = __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
             ++n_item;  // counts the items that reach the tensor cores (those with at least one tile)
         }
         __syncwarp();
@@ -512,7 +527,7 @@ fused_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             int first_col = 0, last_col = (int)a.Lc - 1;
             if (a.causal) {
                 if constexpr (MODE == MODE_ENERGY) first_col = max(0, i - (int)a.diag);
-                else if constexpr (MODE == MODE_GATHERED) last_col = (int)kept_upto(a.tok + head * a.Lc, i + a.diag) - 1;
+                else if constexpr (MODE == MODE_GATHERED) last_col = (int)kept_upto_rows(a.tok + head * a.Lc, r0 + q * 32 + a.diag) - 1;
                 else last_col = min((int)a.Lc - 1, i + (int)a.diag);
             }
             float m = -INFINITY, l = 0.f;  // FULL / STATS: the maximum that p is taken against (log2 domain), the row sum
