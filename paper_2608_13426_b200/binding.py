@@ -9,6 +9,7 @@ refused, an exception is raised.
 from __future__ import annotations
 
 import ctypes
+import functools
 import os
 from typing import Optional, Tuple
 
@@ -115,27 +116,28 @@ def _check(rc: int) -> None:
         raise RmmError(rc, lib().rmm_last_error().decode())
 
 
+_DTYPE_CODES = {torch.bfloat16: RMM_BF16, torch.float32: RMM_F32, torch.float8_e4m3fn: RMM_F8E4M3}
+
+
 def _dtype_code(t: torch.Tensor) -> int:
-    if t.dtype == torch.bfloat16:
-        return RMM_BF16
-    if t.dtype == torch.float32:
-        return RMM_F32
-    if t.dtype == torch.float8_e4m3fn:
-        return RMM_F8E4M3
-    raise RmmError(RMM_ERR_UNSUPPORTED, f"dtype {t.dtype} (bf16, fp32, and e4m3 codes for the 8-bit product)")
+    code = _DTYPE_CODES.get(t.dtype)
+    if code is None:
+        raise RmmError(RMM_ERR_UNSUPPORTED, f"dtype {t.dtype} (bf16, fp32, and e4m3 codes for the 8-bit product)")
+    return code
 
 
 def as_mat(t: torch.Tensor) -> rmm_mat_t:
     """Describe a 2-D [rows, cols] or 3-D [batch, rows, cols] CUDA tensor (any strides) as an rmm_mat_t."""
     if not t.is_cuda:
         raise RmmError(RMM_ERR_INVALID_ARG, "tensor is not on a CUDA device")
-    if t.dim() == 2:
-        b, (r, c), sb, (sr, sc) = 1, t.shape, 0, t.stride()
-    elif t.dim() == 3:
-        b, r, c = t.shape
-        sb, sr, sc = t.stride()
-    else:
+    shape = t.shape
+    if len(shape) == 2:
+        (r, c), (sr, sc) = shape, t.stride()
+        return rmm_mat_t(t.data_ptr(), _dtype_code(t), 1, r, c, 0, sr, sc)
+    if len(shape) != 3:
         raise RmmError(RMM_ERR_INVALID_ARG, "expected a 2-D or 3-D tensor")
+    b, r, c = shape
+    sb, sr, sc = t.stride()
     return rmm_mat_t(t.data_ptr(), _dtype_code(t), b, r, c, sb, sr, sc)
 
 
@@ -166,9 +168,10 @@ _ws_cache = {}
 
 def workspace(nbytes: int, device: torch.device) -> torch.Tensor:
     """A zero-initialised, cached, growing workspace per device (torch owns the memory)."""
-    key = (device.type, device.index if device.index is not None else torch.cuda.current_device())
+    index = device.index
+    key = (device.type, index if index is not None else torch.cuda.current_device())
     ws = _ws_cache.get(key)
-    nbytes = max(int(nbytes), RMM_WS_HEADER_BYTES)
+    nbytes = max(nbytes, RMM_WS_HEADER_BYTES)
     if ws is None or ws.numel() < nbytes:
         ws = torch.zeros(nbytes + 256, dtype=torch.uint8, device=device)
         _ws_cache[key] = ws
@@ -181,10 +184,15 @@ def _ws_ptr(ws: torch.Tensor) -> Tuple[int, int]:
     return a, ws.numel() - (a - p)
 
 
-def rmm_keep_count(rho: float, K: int) -> int:
+@functools.lru_cache(maxsize=1024)
+def _keep_count(rho: float, K: int) -> int:
     k = ctypes.c_int64(0)
-    _check(lib().rmm_keep_count(float(rho), int(K), ctypes.byref(k)))
+    _check(lib().rmm_keep_count(rho, K, ctypes.byref(k)))
     return int(k.value)
+
+
+def rmm_keep_count(rho: float, K: int) -> int:
+    return _keep_count(float(rho), int(K))
 
 
 def rmm_debug_control(key: str, value: float) -> None:
@@ -247,15 +255,15 @@ def rmm_score(A: torch.Tensor, axis: int = 1, want_scores: bool = True, want_ene
     """(scores, energy) fp32 [batch, n] (2-D input: [n]); either may be None if not requested."""
     m = as_mat(A)
     n = m.cols if axis == 1 else m.rows
-    need = lib().rmm_score_workspace_bytes(ctypes.byref(m), axis)
+    need = lib().rmm_score_workspace_bytes(m, axis)
     if need == 0:
-        _check(lib().rmm_score(ctypes.byref(m), axis, None, None, None, 0, None) or RMM_ERR_INVALID_ARG)
+        _check(lib().rmm_score(m, axis, None, None, None, 0, None) or RMM_ERR_INVALID_ARG)
     ws = workspace(need, A.device) if ws is None else ws
     p, nb = _ws_ptr(ws)
     shape = (m.batch, n) if A.dim() == 3 else (n,)
     scores = _out(shape, torch.float32, A) if want_scores else None
     energy = _out(shape, torch.float32, A) if want_energy else None
-    _check(lib().rmm_score(ctypes.byref(m), axis, scores.data_ptr() if want_scores else None,
+    _check(lib().rmm_score(m, axis, scores.data_ptr() if want_scores else None,
                            energy.data_ptr() if want_energy else None, p, nb, _stream()))
     return scores, energy
 
@@ -283,7 +291,7 @@ def rmm_score_select(A: torch.Tensor, rho: float = 0.0, k: int = 0, axis: int = 
     m = as_mat(A)
     n = m.cols if axis == 1 else m.rows
     kk = int(k) if k > 0 else rmm_keep_count(rho, n)
-    need = lib().rmm_score_select_workspace_bytes(ctypes.byref(m), axis)
+    need = lib().rmm_score_select_workspace_bytes(m, axis)
     ws = workspace(need, A.device) if ws is None else ws
     p, nb = _ws_ptr(ws)
     three = A.dim() == 3
@@ -293,7 +301,7 @@ def rmm_score_select(A: torch.Tensor, rho: float = 0.0, k: int = 0, axis: int = 
     scores = _out(shape, torch.float32, A) if want_scores else None
     energy = _out(shape, torch.float32, A) if want_energy else None
     ret = _out((m.batch,), torch.float32, A) if want_retained else None
-    _check(lib().rmm_score_select(ctypes.byref(m), axis, float(rho), int(k), idx.data_ptr(),
+    _check(lib().rmm_score_select(m, axis, float(rho), int(k), idx.data_ptr(),
                                   scores.data_ptr() if want_scores else None,
                                   energy.data_ptr() if want_energy else None,
                                   ret.data_ptr() if want_retained else None, p, nb, _stream()))
@@ -318,7 +326,7 @@ def rmm_score_select_static(A: torch.Tensor, idx: torch.Tensor, rho: float = 0.0
         buf(energy, torch.float32, m.batch * n, "energy")
     if retained is not None:
         buf(retained, torch.float32, m.batch, "retained")
-    _check(lib().rmm_score_select_static(ctypes.byref(m), axis, float(rho), int(k), idx.data_ptr(), None,
+    _check(lib().rmm_score_select_static(m, axis, float(rho), int(k), idx.data_ptr(), None,
                                          energy.data_ptr() if energy is not None else None,
                                          retained.data_ptr() if retained is not None else None, _stream()))
 
@@ -356,18 +364,18 @@ def rmm_reduced_gemm(A: torch.Tensor, B: torch.Tensor, idx: Optional[torch.Tenso
         out = _out(shape, dt, A)
     my = as_mat(out)
     if want_energy:
-        need = lib().rmm_reduced_gemm_scored_workspace_bytes(ctypes.byref(ma), ctypes.byref(mb), k, ctypes.byref(my))
+        need = lib().rmm_reduced_gemm_scored_workspace_bytes(ma, mb, k, my)
         ws = workspace(need, A.device) if ws is None else ws
         p, nb = _ws_ptr(ws)
         energy = _out((ma.batch, mb.cols) if A.dim() == 3 else (mb.cols,), torch.float32, A)
-        _check(lib().rmm_reduced_gemm_scored(ctypes.byref(ma), ctypes.byref(mb), idx.data_ptr() if idx is not None else None, k,
-                                             float(scale), ctypes.byref(my), energy.data_ptr(), p, nb, _stream()))
+        _check(lib().rmm_reduced_gemm_scored(ma, mb, idx.data_ptr() if idx is not None else None, k,
+                                             float(scale), my, energy.data_ptr(), p, nb, _stream()))
         return out, energy
-    need = lib().rmm_reduced_gemm_workspace_bytes(ctypes.byref(ma), ctypes.byref(mb), k, ctypes.byref(my))
+    need = lib().rmm_reduced_gemm_workspace_bytes(ma, mb, k, my)
     ws = workspace(need, A.device) if ws is None else ws
     p, nb = _ws_ptr(ws)
-    _check(lib().rmm_reduced_gemm(ctypes.byref(ma), ctypes.byref(mb), idx.data_ptr() if idx is not None else None, k, float(scale),
-                                  ctypes.byref(my), p, nb, _stream()))
+    _check(lib().rmm_reduced_gemm(ma, mb, idx.data_ptr() if idx is not None else None, k, float(scale),
+                                  my, p, nb, _stream()))
     return out
 
 
@@ -386,13 +394,13 @@ def rmm_reduced_gemm_q8(A: torch.Tensor, Bq_nk: torch.Tensor, b_scale: float, id
     if out is None:
         out = _out((ma.rows, mb.cols), out_dtype if out_dtype is not None else torch.bfloat16, A)
     my = as_mat(out)
-    need = lib().rmm_reduced_gemm_q8_workspace_bytes(ctypes.byref(ma), ctypes.byref(mb), k, ctypes.byref(my))
+    need = lib().rmm_reduced_gemm_q8_workspace_bytes(ma, mb, k, my)
     if need == 0:
         raise RmmError(RMM_ERR_UNSUPPORTED, lib().rmm_last_error().decode())
     ws = workspace(need, A.device) if ws is None else ws
     p, nb = _ws_ptr(ws)
     a_scale = _out((ma.rows,), torch.float32, A) if want_scales else None
-    _check(lib().rmm_reduced_gemm_q8(ctypes.byref(ma), ctypes.byref(mb), float(b_scale), idx.data_ptr(), k, float(scale), ctypes.byref(my),
+    _check(lib().rmm_reduced_gemm_q8(ma, mb, float(b_scale), idx.data_ptr(), k, float(scale), my,
                                      a_scale.data_ptr() if want_scales else None, p, nb, _stream()))
     return (out, a_scale) if want_scales else out
 
@@ -421,7 +429,7 @@ def rmm_reduced_attn(Q: torch.Tensor, K: torch.Tensor, V: torch.Tensor, causal: 
             raise RmmError(RMM_ERR_INVALID_ARG, "mask must be an fp32 CUDA tensor broadcastable to [B,Hq,Lq,Lk], last dim contiguous")
         d.mask = m.data_ptr()
         d.mask_stride = (ctypes.c_int64 * 3)(*[0 if m.shape[a] == 1 else m.stride(a) for a in range(3)])
-    need = lib().rmm_reduced_attn_workspace_bytes(ctypes.byref(d))
+    need = lib().rmm_reduced_attn_workspace_bytes(d)
     if need == 0:
         raise RmmError(RMM_ERR_INVALID_ARG, "reduced_attn: invalid description (check shapes and retention ratios)")
     ws = workspace(need, Q.device) if ws is None else ws
@@ -431,7 +439,7 @@ def rmm_reduced_attn(Q: torch.Tensor, K: torch.Tensor, V: torch.Tensor, causal: 
         idx_feat = _out((B, Hq, rmm_keep_count(rho_d, Dh)), torch.int32, Q)
         if rho_t < 1.0:
             idx_tok = _out((B, Hq, rmm_keep_count(rho_t, Lk)), torch.int32, Q)
-    _check(lib().rmm_reduced_attn(ctypes.byref(d), Q.data_ptr(), K.data_ptr(), V.data_ptr(), O.data_ptr(),
+    _check(lib().rmm_reduced_attn(d, Q.data_ptr(), K.data_ptr(), V.data_ptr(), O.data_ptr(),
                                   idx_feat.data_ptr() if idx_feat is not None else None,
                                   idx_tok.data_ptr() if idx_tok is not None else None, p, nb, _stream()))
     return (O, idx_feat, idx_tok) if want_idx else O
@@ -467,12 +475,12 @@ def rmm_product(A: torch.Tensor, B: torch.Tensor, rho: float = 0.0, k: int = 0, 
         raise RmmError(RMM_ERR_INVALID_ARG, "idx must be a contiguous int32 CUDA tensor of batch * k elements")
     ret = _out((ma.batch,), torch.float32, A) if want_retained else None
     my = as_mat(out)
-    need = lib().rmm_product_workspace_bytes(ctypes.byref(ma), ctypes.byref(mb), ctypes.byref(my))
+    need = lib().rmm_product_workspace_bytes(ma, mb, my)
     if need == 0:
         raise RmmError(RMM_ERR_UNSUPPORTED, "rmm_product: operands not covered")
     ws = workspace(need, A.device) if ws is None else ws
     p, nb = _ws_ptr(ws)
-    _check(lib().rmm_product(ctypes.byref(ma), ctypes.byref(mb), float(rho), int(k), float(scale), ctypes.byref(my),
+    _check(lib().rmm_product(ma, mb, float(rho), int(k), float(scale), my,
                              idx.data_ptr(), ret.data_ptr() if want_retained else None, p, nb, _stream()))
     return (out, idx, ret) if want_retained else (out, idx)
 
