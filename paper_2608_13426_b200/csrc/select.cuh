@@ -19,7 +19,7 @@ constexpr int kCandMax = 1024;   // keys that share the threshold's first digit 
 
 struct SelectSmem {
     __align__(16) unsigned hist[kBins];
-    unsigned cand[kCandMax];
+    __align__(16) unsigned cand[kCandMax];
     unsigned warp_a[32], warp_b[32], warp_lo[32], warp_hi[32];
     unsigned bin, remaining, count, n_cand;
     double red[64];
@@ -556,12 +556,68 @@ __device__ void block_select_blocked(const float *__restrict__ keys, int K, int 
     __syncthreads();
 }
 
+// Whole selection of at most 128 keys (attention heads), blockDim.x == 1024: every key is compared with every other one, an eighth of
+// them per thread, and kept if fewer than k come before it (larger, or equal with a lower index).  Four barriers instead of some
+// fifteen for the digits: attention of 8 heads x 700 x 64 30.0 -> 29.1 us a call, 16 heads x 2048 x 128 84.1 -> 83.1; at 256 keys level.
+static __device__ __noinline__ void block_select_short(const float *__restrict__ keys, int K, int k, int32_t *__restrict__ idx, float *retained, SelectSmem &sm)
+{
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, j = tid & 127, part = tid >> 7;
+    const float key = j < K ? __ldcg(keys + j) : 0.f;
+    const unsigned u = j < K ? key_image(key) : 0u;
+    if (tid < 128) sm.cand[tid] = u;
+    __syncthreads();
+    unsigned before = 0;   // the zeros past K come after every key: they are no larger, and their indices are higher
+    for (int i = part * 16; i < min(K, part * 16 + 16); i += 4) {
+        const uint4 q = *reinterpret_cast<const uint4 *>(&sm.cand[i]);
+        before += (q.x > u || (q.x == u && i < j)) ? 1u : 0u;
+        before += (q.y > u || (q.y == u && i + 1 < j)) ? 1u : 0u;
+        before += (q.z > u || (q.z == u && i + 2 < j)) ? 1u : 0u;
+        before += (q.w > u || (q.w == u && i + 3 < j)) ? 1u : 0u;
+    }
+    sm.hist[tid] = before;
+    __syncthreads();
+    unsigned rank = 0;
+#pragma unroll
+    for (int p = 0; p < 8; ++p) rank += sm.hist[p * 128 + j];
+    const bool keep = tid < K && rank < (unsigned)k;
+    const unsigned kept = __ballot_sync(0xffffffffu, keep);
+    double sum_kept = keep ? (double)key : 0.0, sum_all = tid < K ? (double)key : 0.0;
+    if (retained != nullptr) {
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) {
+            sum_kept += __shfl_down_sync(0xffffffffu, sum_kept, d);
+            sum_all += __shfl_down_sync(0xffffffffu, sum_all, d);
+        }
+    }
+    if (lane == 0) {
+        sm.warp_a[warp] = __popc(kept);
+        sm.red[warp] = sum_kept;
+        sm.red[32 + warp] = sum_all;
+    }
+    __syncthreads();
+    if (keep) {
+        unsigned at = __popc(kept & ((1u << lane) - 1u));
+        for (int w = 0; w < warp; ++w) at += sm.warp_a[w];
+        idx[at] = tid;
+    }
+    if (retained != nullptr && tid == 0) {
+        double a = 0.0, b = 0.0;
+        for (int w = 0; w < 32; ++w) {  // fixed order
+            a += sm.red[w];
+            b += sm.red[32 + w];
+        }
+        *retained = (b > 0.0) ? (float)(a / b) : 1.0f;
+    }
+    __syncthreads();
+}
+
 // Dispatch on the problem size: keys in registers when they fit (blocks of 1024 threads), else in kcache or, without one,
 // re-read in every pass.
 __device__ __forceinline__ void block_select_any(const float *keys, int K, int k, int32_t *idx, float *retained,
                                                  SelectSmem &sm, unsigned *kcache = nullptr)
 {
-    if (blockDim.x == 1024 && K <= 1024) block_select_blocked<1>(keys, K, k, idx, retained, sm);
+    if (blockDim.x == 1024 && K <= 128) block_select_short(keys, K, k, idx, retained, sm);
+    else if (blockDim.x == 1024 && K <= 1024) block_select_blocked<1>(keys, K, k, idx, retained, sm);
     else if (blockDim.x == 1024 && K <= 4096) block_select_blocked<4>(keys, K, k, idx, retained, sm);
     else if (blockDim.x == 1024 && K <= 8192) block_select_blocked<8>(keys, K, k, idx, retained, sm);
     else block_select(keys, K, k, idx, retained, sm, kcache);
