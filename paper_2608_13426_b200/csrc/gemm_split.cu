@@ -312,14 +312,16 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
                 float4 *mine = slot(unit);
 #pragma unroll
                 for (int c = 0; c < 16; ++c) __stcg(mine + c * kTile, make_float4(acc[2 * c].x, acc[2 * c].y, acc[2 * c + 1].x, acc[2 * c + 1].y));
-                __threadfence();
                 if (!epilogue_meet()) { ok = false; break; }
-                if (tid == 128) s_last = atomicInc(a.counters + 2 * u0 + rank, (unsigned)(u1 - u0)) == (unsigned)(u1 - u0);
+                if (tid == 128) {  // (fences are cumulative: one thread's stand for all that it has met)
+                    __threadfence();
+                    s_last = atomicInc(a.counters + 2 * u0 + rank, (unsigned)(u1 - u0)) == (unsigned)(u1 - u0);
+                    __threadfence();
+                }
                 if (!epilogue_meet()) { ok = false; break; }
                 const bool last = *const_cast<volatile int *>(&s_last) != 0;
                 if (!epilogue_meet()) { ok = false; break; }   // (s_last is written again for the next cut tile)
                 if (!last) continue;
-                __threadfence();
 #pragma unroll
                 for (int i = 0; i < 32; ++i) acc[i] = make_float2(0.f, 0.f);
                 for (int64_t u = u0; u <= u1; ++u) {
