@@ -685,7 +685,7 @@ __global__ void __launch_bounds__(kThreads, 1) rmm_front_kernel(const __grid_con
     if (tid < kSelThreads) {
         unsigned u[kSelItems];
         const int nvalid = load_keys_blocked<kSelItems>(a.energy, (int)a.n, u);
-        const Threshold th = block_threshold<kSelItems, kSelThreads>(u, nvalid, a.k, s_sel);
+        const Threshold th = block_threshold<kSelItems, kSelThreads, true>(u, nvalid, a.k, s_sel);
         const unsigned before = block_rank_blocked<kSelItems, kSelThreads>(u, nvalid, th.tau, s_sel);
         unsigned gt_before = before >> 16, eq_before = before & 0xffffu;
         const bool writer = blockIdx.x == 0;

@@ -350,7 +350,10 @@ __device__ __forceinline__ void find_bin8(SelectSmem &sm, int nbins, unsigned re
 // the keys that share the prefix found so far count (a per-thread bit mask of those keys is carried along, and warps
 // without any skip the pass).  With 32 warps on four schedulers every instruction that all warps execute costs eight
 // issue clocks, so the code paths below are kept short rather than general.
-template <int ITEMS, int NTHR = 1024>
+// LIST: keys that share the first digit and are few enough are finished from a list, one to a thread.  For the front end, where
+// every block selects: 2048 x 8192 x 2048 56.9 -> 56.2 us a call.  In the tail of a score pass, where one block does, the code that it adds
+// is fetched for the first time in each call and costs more than it saves (512 x 8192 x 8192 73.4 -> 75.0).
+template <int ITEMS, int NTHR = 1024, bool LIST = false>
 __device__ __forceinline__ Threshold block_threshold(const unsigned (&u)[ITEMS], int nvalid, int k, SelectSmem &sm)
 {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -381,6 +384,7 @@ __device__ __forceinline__ Threshold block_threshold(const unsigned (&u)[ITEMS],
         uint4 *h4 = reinterpret_cast<uint4 *>(sm.hist);
         for (int i = tid; i < kBins / 4; i += nthr) h4[i] = make_uint4(0, 0, 0, 0);
     }
+    if (LIST && tid == 0) sm.count = 0;
     group_sync<NTHR>();
     SEL_STAMP(0);
     {
@@ -421,8 +425,63 @@ __device__ __forceinline__ Threshold block_threshold(const unsigned (&u)[ITEMS],
 #pragma unroll
     for (int i = 0; i < ITEMS; ++i) live |= (i < nvalid && (u[i] & mask) == prefix) ? (1u << i) : 0u;
 
-    // ---- remaining bits, eight at a time, over the keys that share the prefix
     [[maybe_unused]] int pass = 1;
+    if (LIST && n_same <= (unsigned)(NTHR < kCandMax ? NTHR : kCandMax) && shift > 0) {
+        // one to a thread from here on: with eight keys a thread, few of them among these, the second pass took 2500 clocks
+        const unsigned cnt = __popc(live);
+        unsigned incl = cnt;
+#pragma unroll
+        for (int e = 1; e < 32; e <<= 1) {
+            const unsigned v = __shfl_up_sync(0xffffffffu, incl, e);
+            if (lane >= e) incl += v;
+        }
+        unsigned at = 0;
+        if (lane == 31 && incl > 0) at = atomicAdd(&sm.count, incl);
+        at = __shfl_sync(0xffffffffu, at, 31) + incl - cnt;
+#pragma unroll
+        for (int i = 0; i < ITEMS; ++i)
+            if (live & (1u << i)) sm.cand[at++] = u[i];   // (their order does not matter)
+        if (tid < 64) reinterpret_cast<uint4 *>(sm.hist)[tid] = make_uint4(0, 0, 0, 0);
+        group_sync<NTHR>();
+        const bool held = tid < (int)n_same;
+        const unsigned c = held ? sm.cand[tid] : 0u;
+        while (shift > 0 && n_same != remaining) {
+            d = shift < 8 ? shift : 8;
+            shift -= d;
+            m = (1u << d) - 1u;
+            if (held && (c & mask) == prefix) atomicAdd(&sm.hist[(c >> shift) & m], 1u);
+            group_sync<NTHR>();
+            SEL_STAMP(1 + 2 * pass);
+            find_bin8<NTHR>(sm, 256, remaining);
+            SEL_STAMP(2 + 2 * pass);
+            ++pass;
+            prefix |= sm.bin << shift;
+            mask |= m << shift;
+            remaining = sm.remaining;
+            n_same = sm.n_cand;
+            if (shift > 0 && n_same != remaining) {
+                if (tid < 64) reinterpret_cast<uint4 *>(sm.hist)[tid] = make_uint4(0, 0, 0, 0);
+                group_sync<NTHR>();
+            }
+        }
+        t.tau = prefix;
+        t.need_eq = remaining;
+        if (shift > 0) {
+            // all that share the prefix are kept: the threshold is the smallest of them, and need_eq how many equal it
+            const bool same = held && (c & mask) == prefix;
+            const unsigned w_min = __reduce_min_sync(0xffffffffu, same ? c : 0xffffffffu);
+            if (lane == 0) sm.warp_lo[warp] = w_min;
+            group_sync<NTHR>();
+            t.tau = __reduce_min_sync(0xffffffffu, lane < nwarp ? sm.warp_lo[lane] : 0xffffffffu);
+            const unsigned equal = __popc(__ballot_sync(0xffffffffu, same && c == t.tau));
+            if (lane == 0) sm.warp_hi[warp] = equal;
+            group_sync<NTHR>();
+            t.need_eq = __reduce_add_sync(0xffffffffu, lane < nwarp ? sm.warp_hi[lane] : 0u);
+        }
+        return t;
+    }
+
+    // ---- remaining bits, eight at a time, over the keys that share the prefix
     while (shift > 0 && n_same != remaining) {
         d = shift < 8 ? shift : 8;
         shift -= d;
