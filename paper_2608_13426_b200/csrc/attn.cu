@@ -252,7 +252,7 @@ int rmm_reduced_attn(const rmm_attn_desc_t *desc, const void *Q, const void *K, 
 
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     char *w = static_cast<char *>(ws);
-    if (p.decode) return launch_decode_attn(d, p.kd, Q, K, V, O, idx_feat, w + RMM_WS_HEADER_BYTES, st);
+    if (p.decode) return launch_decode_attn(d, p.kd, Q, K, V, O, idx_feat, w + RMM_WS_HEADER_BYTES, static_cast<WsHeader *>(ws)->counters, st);
     int *status = &reinterpret_cast<WsHeader *>(w)->status;
     const __nv_bfloat16 *q = static_cast<const __nv_bfloat16 *>(Q), *kk = static_cast<const __nv_bfloat16 *>(K),
                         *v = static_cast<const __nv_bfloat16 *>(V);

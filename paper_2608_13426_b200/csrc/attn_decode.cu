@@ -17,6 +17,8 @@
 // attn_fused.cu), rounded once to bf16; row sums, maxima and O stay fp32.  Pieces of one head meet in a fixed order.
 #include <math.h>
 
+#include <type_traits>
+
 #include "common.cuh"
 #include "select.cuh"
 #include "sm100_ptx.cuh"
@@ -36,6 +38,7 @@ struct DecodeArgs {
     float scale_log2;            // log2(e) / sqrt(Dh)
     int32_t *idx_feat;           // [B, Hq, kd] or NULL
     float *part_o, *part_ml;     // pieces > 1: [blocks][row tile][Dh padded], [blocks][row tile][2]
+    unsigned *counters;          // an arrival counter per job, where its last block adds the pieces up
 };
 
 constexpr int kDecodeWarps = 4, kDecodeBlocks = 2;  // warps per block, blocks per SM
@@ -52,8 +55,63 @@ struct DecodeShape {
     static_assert(kRows * DH * 4 <= kRing, "the merge of the warps reuses the rings");
 };
 
+// A job of few pieces: whichever of its blocks comes last adds them up, in order.  (A second launch for it took 3 us.)  Out of line,
+// so that the loop over the keys keeps its registers.
 template <int DH, int NT>
-__global__ void __launch_bounds__(kDecodeWarps * 32, kDecodeBlocks) attn_decode_kernel(const DecodeArgs a)
+__device__ __noinline__ void decode_meet(const DecodeArgs &a, int *final_piece)
+{
+    constexpr int WARPS = kDecodeWarps, kRows = 8 * NT;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, pieces = a.pieces;
+    const int64_t job = blockIdx.x / pieces;
+    const int row0 = (int)(job % a.chunks) * kRows, nrows = min(kRows, a.rows - row0);
+    const int64_t bh = job / a.chunks, b = bh / a.Hkv, hk = bh % a.Hkv;
+    __syncthreads();
+    if (tid == 0) {  // (fences are cumulative: one thread's stand for all that the barrier has ordered before it)
+        __threadfence();
+        *final_piece = atomicInc(a.counters + job, (unsigned)a.pieces - 1u) == (unsigned)a.pieces - 1u;
+        __threadfence();
+    }
+    __syncthreads();
+    if (*final_piece == 0) return;
+    const int64_t slot0 = job * a.pieces;
+    for (int r = warp; r < nrows; r += WARPS) {   // a warp per row, four columns a lane; lane p looks after piece p
+        const float *pm = a.part_ml + ((slot0 + lane) * kRows + r) * 2;
+        const float mw = lane < a.pieces ? __ldcg(pm) : -INFINITY, lw = lane < a.pieces ? __ldcg(pm + 1) : 0.f;
+        float mx = mw;
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, d));
+        const float f = mw > -INFINITY ? ptx::ex2(mw - mx) : 0.f;
+        float lsum = 0.f;
+        float4 acc[DH <= 128 ? 1 : 2] = {};
+#pragma unroll 4
+        for (int p = 0; p < pieces; ++p) {
+            const float fp = __shfl_sync(0xffffffffu, f, p), mp = __shfl_sync(0xffffffffu, mw, p);
+            lsum += fp * __shfl_sync(0xffffffffu, lw, p);
+            const float4 *src = reinterpret_cast<const float4 *>(a.part_o + ((slot0 + p) * kRows + r) * DH);
+#pragma unroll
+            for (int i = 0; i < (DH <= 128 ? 1 : 2); ++i) {
+                if (mp > -INFINITY && (i * 32 + lane) * 4 < DH) {
+                    const float4 x = __ldcg(src + i * 32 + lane);
+                    acc[i].x += fp * x.x; acc[i].y += fp * x.y; acc[i].z += fp * x.z; acc[i].w += fp * x.w;
+                }
+            }
+        }
+        const float inv = lsum == 0.f ? 0.f : 1.f / lsum;  // 0: the row sees no key; a NaN stays one
+        const int row = row0 + r;
+        __nv_bfloat16 *o = a.o + b * a.o_sb + (hk * a.group + row / a.Lq) * a.o_sh + (int64_t)(row % a.Lq) * a.o_sr;
+#pragma unroll
+        for (int i = 0; i < (DH <= 128 ? 1 : 2); ++i) {
+            const int c = (i * 32 + lane) * 4;
+            if (c < a.Dh) {   // Dh and the strides are multiples of 8
+                const __nv_bfloat162 lo = __floats2bfloat162_rn(acc[i].x * inv, acc[i].y * inv), hi = __floats2bfloat162_rn(acc[i].z * inv, acc[i].w * inv);
+                *reinterpret_cast<uint2 *>(o + c) = make_uint2(*reinterpret_cast<const uint32_t *>(&lo), *reinterpret_cast<const uint32_t *>(&hi));
+            }
+        }
+    }
+}
+
+template <int DH, int NT, bool MEET>
+__global__ void __launch_bounds__(kDecodeWarps * 32, kDecodeBlocks) attn_decode_kernel(const __grid_constant__ DecodeArgs a)
 {
     using S = DecodeShape<DH, NT>;
     constexpr int WARPS = kDecodeWarps, kRows = S::kRows, U = S::kUnits, CPR = DH / 8;  // 16-byte vectors per row
@@ -321,6 +379,7 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, kDecodeBlocks) attn_decode_
             }
         }
     }
+    if constexpr (MEET) decode_meet<DH, NT>(a, reinterpret_cast<int *>(smem + S::kOffMl));
 }
 
 // Jobs cut into pieces: a block per row; its warps take every fourth piece each, and meet in order.
@@ -412,17 +471,17 @@ DecodeGrid decode_grid(const rmm_attn_desc_t *d)
     return g;
 }
 
-template <int DH, int NT>
+template <int DH, int NT, bool MEET>
 int launch_shape(const DecodeArgs &a, const DecodeGrid &g, cudaStream_t stream)
 {
     using S = DecodeShape<DH, NT>;
-    auto kern = attn_decode_kernel<DH, NT>;
+    auto kern = attn_decode_kernel<DH, NT, MEET>;
     static PerDeviceOnce configured;
     if (cudaError_t e = configured.smem(S::kSmem, kern)) return fail(RMM_ERR_CUDA, "attn_decode: cudaFuncSetAttribute: %s", cudaGetErrorString(e));
     prof_begin("attn_decode_kernel", stream);
     launch_kernel(kern, dim3((unsigned)g.blocks), dim3(kDecodeWarps * 32), S::kSmem, stream, 1, a);
     int rc = check_launch("attn_decode_kernel", stream);
-    if (rc != RMM_OK || g.pieces == 1) return rc;
+    if (MEET || rc != RMM_OK || g.pieces == 1) return rc;
     prof_begin("attn_decode_combine_kernel", stream);
     launch_kernel(attn_decode_combine_kernel<DH, NT>, dim3((unsigned)(g.jobs * S::kRows)), dim3(kCombineWarps * 32), 0, stream, 1, a);
     return check_launch("attn_decode_combine_kernel", stream);
@@ -443,7 +502,7 @@ size_t decode_attn_workspace_bytes(const rmm_attn_desc_t *d)
 }
 
 int launch_decode_attn(const rmm_attn_desc_t *d, int64_t kd, const void *Q, const void *K, const void *V, void *O, int32_t *idx_feat,
-                       void *scratch, cudaStream_t stream)
+                       void *scratch, unsigned *counters, cudaStream_t stream)
 {
     const DecodeGrid g = decode_grid(d);
     DecodeArgs a = {};
@@ -460,9 +519,22 @@ int launch_decode_attn(const rmm_attn_desc_t *d, int64_t kd, const void *Q, cons
     a.idx_feat = idx_feat;
     a.part_o = static_cast<float *>(scratch);
     a.part_ml = a.part_o + (size_t)g.blocks * 8 * g.nt * g.dh;
-    if (g.dh == 64) return g.nt == 1 ? launch_shape<64, 1>(a, g, stream) : launch_shape<64, 2>(a, g, stream);
-    if (g.dh == 128) return g.nt == 1 ? launch_shape<128, 1>(a, g, stream) : launch_shape<128, 2>(a, g, stream);
-    return g.nt == 1 ? launch_shape<256, 1>(a, g, stream) : launch_shape<256, 2>(a, g, stream);
+    // Short pieces of up to 1024 keys are added up in the last block of their job, where a warp then has at most 16 pieces of rows
+    // (4 x 8 heads x 2048 keys 17.6 -> 16.0 us, 16 x 8 / 4 heads x 512 17.5 -> 14.7, 8 x 32 / 8 heads x 4096 32.0 -> 31.8) and each job has
+    // its counter (the header's last four belong to the products).  Others keep a launch of their own, with a block per row: 32 pieces
+    // of rows a warp took 22.7 us for 17.6 (32 / 8 heads x 4096), and pieces of 4096 keys 96 for 90 (16 x 32 / 8 heads x 8192).
+    const int64_t rows_a_warp = ceil_div(a.rows < 8 * g.nt ? a.rows : 8 * g.nt, kDecodeWarps);
+    const bool meet = g.pieces > 1 && g.per <= 16 && g.pieces * rows_a_warp <= 16 && g.jobs <= kHeaderCounters - 4;
+    if (meet) a.counters = counters;
+    auto launch = [&](auto dh, auto nt) {
+        constexpr int kDh = decltype(dh)::value, kNt = decltype(nt)::value;
+        return meet ? launch_shape<kDh, kNt, true>(a, g, stream) : launch_shape<kDh, kNt, false>(a, g, stream);
+    };
+    using std::integral_constant;
+    auto launch_dh = [&](auto dh) { return g.nt == 1 ? launch(dh, integral_constant<int, 1>{}) : launch(dh, integral_constant<int, 2>{}); };
+    if (g.dh == 64) return launch_dh(integral_constant<int, 64>{});
+    if (g.dh == 128) return launch_dh(integral_constant<int, 128>{});
+    return launch_dh(integral_constant<int, 256>{});
 }
 
 }  // namespace rmm

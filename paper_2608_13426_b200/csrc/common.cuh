@@ -301,7 +301,7 @@ constexpr int64_t kDecodeMaxRows = 16;
 bool decode_attn_eligible(const rmm_attn_desc_t *d);
 size_t decode_attn_workspace_bytes(const rmm_attn_desc_t *d);
 int launch_decode_attn(const rmm_attn_desc_t *d, int64_t kd, const void *Q, const void *K, const void *V, void *O, int32_t *idx_feat,
-                       void *scratch, cudaStream_t stream);
+                       void *scratch, unsigned *counters, cudaStream_t stream);
 // lse == tok == NULL: O = softmax(Qp Kp^T / sqrt(Dh) + mask) V.  With lse [heads, lse_ld] and tok [heads, Lk] given,
 // Kp and V hold the kept keys only (Lk of them, at positions tok): O = P V with P = bf16(2^(x + lse)), not
 // renormalised.  diag = Lk - Lq of the unpacked problem (causal: query i sees key t iff t <= i + diag).
