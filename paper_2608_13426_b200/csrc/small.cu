@@ -88,23 +88,18 @@ __global__ void __launch_bounds__(kSmallThreads) small_product_kernel(const Smal
             s_list[i] = (unsigned short)j;
         }
     } else {
-        // ---- scores: two columns a thread, rows in up to 16 per fp32 chain (their squares are exact), chains and row ranges in fp64
-        const int pairs = (a.K + 1) / 2, span = ((a.M + lay.splits - 1) / lay.splits + 15) / 16 * 16;
+        // ---- scores: two columns a thread; the squares are exact in fp32 and added up in fp64, as in every score pass of so few rows
+        const int pairs = (a.K + 1) / 2, span = (a.M + lay.splits - 1) / lay.splits;
         for (int w = tid; w < pairs * lay.splits; w += kSmallThreads) {
             const int s = w / pairs, p = w - s * pairs, r1 = min(a.M, (s + 1) * span);
             const unsigned char *col = s_dyn + p * 4;
             double e0 = 0.0, e1 = 0.0;
-            for (int r = s * span; r < r1; r += 16) {
-                float f0 = 0.f, f1 = 0.f;
-#pragma unroll
-                for (int i = 0; i < 16; ++i) {
-                    const uint32_t x = r + i < r1 ? *reinterpret_cast<const uint32_t *>(col + (r + i) * lay.a_pitch) : 0u;
-                    const float x0 = __uint_as_float(x << 16), x1 = __uint_as_float(x & 0xffff0000u);
-                    f0 = fmaf(x0, x0, f0);
-                    f1 = fmaf(x1, x1, f1);
-                }
-                e0 += (double)f0;
-                e1 += (double)f1;
+#pragma unroll 8
+            for (int r = s * span; r < r1; ++r) {
+                const uint32_t x = *reinterpret_cast<const uint32_t *>(col + r * lay.a_pitch);
+                const float x0 = __uint_as_float(x << 16), x1 = __uint_as_float(x & 0xffff0000u);
+                e0 += (double)(x0 * x0);
+                e1 += (double)(x1 * x1);
             }
             s_sum[(s * pairs + p) * 2] = e0;
             s_sum[(s * pairs + p) * 2 + 1] = e1;
