@@ -265,7 +265,7 @@ int rmm_reduced_gemm(const rmm_mat_t *A, const rmm_mat_t *B, const int32_t *idx,
     if (idx != nullptr && small_eligible(A, B, Y)) {  // (the same kernel as in rmm_product: the same sums)
         rc = check_ws(ws, ws_bytes, gemm_least_bytes(A, B, k, Y), "reduced_gemm");
         if (rc != RMM_OK) return rc;
-        return launch_small_product(A, B, k, scale, Y, nullptr, idx, &static_cast<WsHeader *>(ws)->status, static_cast<cudaStream_t>(stream));
+        return launch_small_product(A, B, k, scale, Y, nullptr, nullptr, idx, &static_cast<WsHeader *>(ws)->status, static_cast<cudaStream_t>(stream));
     }
     rmm_mat_t b = shared_b(A, B);
     GemvPlan gplan;
@@ -429,10 +429,10 @@ struct ProductPlan {
     size_t total;
 };
 
-static int plan_product(const rmm_mat_t *A, const rmm_mat_t *B, const rmm_mat_t *Y, int64_t k, bool want_retained, ProductPlan *pp)
+static int plan_product(const rmm_mat_t *A, const rmm_mat_t *B, const rmm_mat_t *Y, int64_t k, ProductPlan *pp)
 {
     rmm_mat_t b = shared_b(A, B);
-    pp->small = !want_retained && small_eligible(A, B, Y);  // (asks for the workspace of the other forms all the same)
+    pp->small = small_eligible(A, B, Y);  // (asks for the workspace of the other forms all the same)
     pp->fused = k < A->cols && front_eligible(A, &b, Y, k, &pp->front);
     if (pp->fused) {
         pp->total = pp->front.total_bytes;
@@ -469,12 +469,12 @@ int rmm_product(const rmm_mat_t *A, const rmm_mat_t *B, double rho, int64_t k, f
     rc = check_gemm(A, B, idx, kk, Y);
     if (rc != RMM_OK) return rc;
     ProductPlan pp;
-    rc = plan_product(A, B, Y, kk, retained != nullptr, &pp);
+    rc = plan_product(A, B, Y, kk, &pp);
     if (rc != RMM_OK) return fail(rc, "product: operands not covered");
     rc = check_ws(ws, ws_bytes, pp.total, "product");
     if (rc != RMM_OK) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if (pp.small) return launch_small_product(A, B, kk, scale, Y, idx, nullptr, &static_cast<WsHeader *>(ws)->status, st);
+    if (pp.small) return launch_small_product(A, B, kk, scale, Y, idx, retained, nullptr, &static_cast<WsHeader *>(ws)->status, st);
     if (kk == A->cols) {
         // every index is kept: the list is 0 .. K-1 (written by the selection, which also gives `retained`), and the product
         // is the unreduced one, which needs no gather at all

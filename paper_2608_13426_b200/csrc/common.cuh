@@ -145,7 +145,7 @@ int launch_front(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k, int32_t *idx
 // `given` list; see small.cu.
 bool small_eligible(const rmm_mat_t *A, const rmm_mat_t *B, const rmm_mat_t *Y);
 int launch_small_product(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k, float scale, const rmm_mat_t *Y, int32_t *idx,
-                         const int32_t *given, int *status, cudaStream_t stream);
+                         float *retained, const int32_t *given, int *status, cudaStream_t stream);
 
 // ---- reduced GEMM ------------------------------------------------------------------------------------
 // Plain FMA kernel: any strides, bf16 or fp32 operands, fp32 accumulation, bf16 or fp32 output.

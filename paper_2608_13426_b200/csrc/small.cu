@@ -26,6 +26,7 @@ struct SmallArgs {
     float scale;
     int32_t *idx;            // the selection, written by the first block, or
     const int32_t *given;    // ... the caller's list: nothing is scored
+    float *retained;         // or NULL: with idx, the kept share of the energies
     int *status;
 };
 
@@ -119,16 +120,42 @@ __global__ void __launch_bounds__(kSmallThreads) small_product_kernel(const Smal
         const sel::Threshold th = sel::block_threshold<ITEMS, kSmallThreads>(u, nvalid, a.k, s_sel);
         const unsigned before = sel::block_rank_blocked<ITEMS, kSmallThreads>(u, nvalid, th.tau, s_sel);
         unsigned gt_before = before >> 16, eq_before = before & 0xffffu;
+        double sum_kept = 0.0, sum_all = 0.0;
 #pragma unroll
         for (int i = 0; i < ITEMS; ++i) {
-            const bool gt = i < nvalid && u[i] > th.tau, eq = i < nvalid && u[i] == th.tau;
-            if (gt || (eq && eq_before < th.need_eq)) {
+            const bool gt = i < nvalid && u[i] > th.tau, eq = i < nvalid && u[i] == th.tau, keep = gt || (eq && eq_before < th.need_eq);
+            if (keep) {
                 const unsigned pos = gt_before + min(eq_before, th.need_eq);
                 s_list[pos] = (unsigned short)(j0 + i);
                 if (blockIdx.x == 0) a.idx[pos] = j0 + i;
             }
             gt_before += gt ? 1u : 0u;
             eq_before += eq ? 1u : 0u;
+            if (a.retained != nullptr && i < nvalid) {
+                const double f = (double)sel::key_value(u[i]);
+                sum_all += f;
+                if (keep) sum_kept += f;
+            }
+        }
+        if (a.retained != nullptr && blockIdx.x == 0) {   // the whole block: sums in a fixed order
+#pragma unroll
+            for (int d = 16; d > 0; d >>= 1) {
+                sum_kept += __shfl_down_sync(0xffffffffu, sum_kept, d);
+                sum_all += __shfl_down_sync(0xffffffffu, sum_all, d);
+            }
+            if (lane == 0) {
+                s_sel.red[warp] = sum_kept;
+                s_sel.red[32 + warp] = sum_all;
+            }
+            __syncthreads();
+            if (tid == 0) {
+                double kept = 0.0, all = 0.0;
+                for (int w = 0; w < kSmallWarps; ++w) {
+                    kept += s_sel.red[w];
+                    all += s_sel.red[32 + w];
+                }
+                *a.retained = all > 0.0 ? (float)(kept / all) : 1.0f;
+            }
         }
     }
     if (tid < 16) s_list[a.k + tid] = (unsigned short)a.K;   // the zero column / row
@@ -218,7 +245,7 @@ bool small_eligible(const rmm_mat_t *A, const rmm_mat_t *B, const rmm_mat_t *Y)
 }
 
 int launch_small_product(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k, float scale, const rmm_mat_t *Y, int32_t *idx,
-                         const int32_t *given, int *status, cudaStream_t stream)
+                         float *retained, const int32_t *given, int *status, cudaStream_t stream)
 {
     SmallArgs a;
     a.A = static_cast<const __nv_bfloat16 *>(A->ptr); a.B = static_cast<const __nv_bfloat16 *>(B->ptr); a.Y = Y->ptr;
@@ -226,7 +253,7 @@ int launch_small_product(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k, floa
     a.y_bf16 = Y->dtype == RMM_BF16;
     a.M = (int)A->rows; a.K = (int)A->cols; a.N = (int)B->cols; a.k = (int)k;
     a.scale = scale;
-    a.idx = idx; a.given = given; a.status = status;
+    a.idx = idx; a.retained = retained; a.given = given; a.status = status;
     const bool wide = small_columns(a.N) == 32;
     if (a.K <= 512) return wide ? launch_small_as<1, 32>(a, stream) : launch_small_as<1, 16>(a, stream);
     if (a.K <= 1024) return wide ? launch_small_as<2, 32>(a, stream) : launch_small_as<2, 16>(a, stream);

@@ -38,3 +38,21 @@ def test_the_index_set_is_that_of_the_score_pass(M, K):
     A, B = A.cuda()[:, :K], torch.ones(K, 64, device="cuda", dtype=torch.bfloat16)
     for k in sorted({1, K // 3, K // 2, K - 1}):
         assert torch.equal(rmm.rmm_product(A, B, k=k)[1], rmm.rmm_score_select(A, k=k)[0]), k
+
+
+@pytest.mark.parametrize("M, K", SHAPES)
+def test_the_kept_share_changes_nothing_else(M, K):
+    """Asking for the kept share of the energies leaves Y and the list as they are, and so does the list when it is given."""
+    g = torch.Generator().manual_seed(M * K)
+    wide = (K + 7) // 8 * 8
+    A, B = torch.randn(M, wide, generator=g).bfloat16().cuda()[:, :K], torch.randn(K, 264, generator=g).bfloat16().cuda()
+    for k in sorted({1, K // 2, K}):
+        Y, idx = rmm.rmm_product(A, B, k=k, out=torch.empty(M, 264, device="cuda"))
+        Y2, idx2, kept = rmm.rmm_product(A, B, k=k, out=torch.empty(M, 264, device="cuda"), want_retained=True)
+        assert torch.equal(Y, Y2) and torch.equal(idx, idx2)
+        assert torch.equal(Y, rmm.rmm_reduced_gemm(A, B, idx, out_dtype=torch.float32))
+        want_idx, _, energy, want = rmm.rmm_score_select(A, k=k, want_energy=True, want_retained=True)
+        assert torch.equal(idx, want_idx) and abs(float(kept) - float(want)) <= 2.0 ** -23
+        share = float(energy[idx.long()].double().sum() / energy.double().sum())
+        assert abs(float(kept) - share) <= 2.0 ** -23          # fp64 sums, rounded once to fp32
+    assert rmm.rmm_status_read() == 0
