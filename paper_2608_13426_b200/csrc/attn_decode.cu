@@ -55,12 +55,16 @@ struct DecodeShape {
     static_assert(kRows * DH * 4 <= kRing, "the merge of the warps reuses the rings");
 };
 
-// A job of few pieces: whichever of its blocks comes last adds them up, in order.  (A second launch for it took 3 us.)  Out of line,
-// so that the loop over the keys keeps its registers.
+// A job of few pieces: whichever of its blocks comes last adds them up, in order.  (A second launch takes 3 us of the host.)  Out of
+// line, so that the loop over the keys keeps its registers, and short: what runs once a call is fetched from memory.  A warp takes a
+// row, or one or two rows' pieces are shared out among the four.
 template <int DH, int NT>
-__device__ __noinline__ void decode_meet(const DecodeArgs &a, int *final_piece)
+__device__ __noinline__ void decode_meet(const DecodeArgs &a, uint8_t *smem)
 {
-    constexpr int WARPS = kDecodeWarps, kRows = 8 * NT;
+    constexpr int WARPS = kDecodeWarps, kRows = 8 * NT, V = DH <= 128 ? 1 : 2;
+    float *s_inv = reinterpret_cast<float *>(smem);              // [WARPS], the flag behind it
+    float4 *s_acc = reinterpret_cast<float4 *>(smem) + 2;        // [warp][32 V]
+    int *s_last = reinterpret_cast<int *>(smem) + WARPS;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, pieces = a.pieces;
     const int64_t job = blockIdx.x / pieces;
     const int row0 = (int)(job % a.chunks) * kRows, nrows = min(kRows, a.rows - row0);
@@ -68,46 +72,71 @@ __device__ __noinline__ void decode_meet(const DecodeArgs &a, int *final_piece)
     __syncthreads();
     if (tid == 0) {  // (fences are cumulative: one thread's stand for all that the barrier has ordered before it)
         __threadfence();
-        *final_piece = atomicInc(a.counters + job, (unsigned)a.pieces - 1u) == (unsigned)a.pieces - 1u;
+        *s_last = atomicInc(a.counters + job, (unsigned)pieces - 1u) == (unsigned)pieces - 1u;
         __threadfence();
     }
     __syncthreads();
-    if (*final_piece == 0) return;
-    const int64_t slot0 = job * a.pieces;
-    for (int r = warp; r < nrows; r += WARPS) {   // a warp per row, four columns a lane; lane p looks after piece p
-        const float *pm = a.part_ml + ((slot0 + lane) * kRows + r) * 2;
-        const float mw = lane < a.pieces ? __ldcg(pm) : -INFINITY, lw = lane < a.pieces ? __ldcg(pm + 1) : 0.f;
-        float mx = mw;
-#pragma unroll
-        for (int d = 16; d > 0; d >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, d));
-        const float f = mw > -INFINITY ? ptx::ex2(mw - mx) : 0.f;
-        float lsum = 0.f;
-        float4 acc[DH <= 128 ? 1 : 2] = {};
-#pragma unroll 4
-        for (int p = 0; p < pieces; ++p) {
-            const float fp = __shfl_sync(0xffffffffu, f, p), mp = __shfl_sync(0xffffffffu, mw, p);
-            lsum += fp * __shfl_sync(0xffffffffu, lw, p);
-            const float4 *src = reinterpret_cast<const float4 *>(a.part_o + ((slot0 + p) * kRows + r) * DH);
-#pragma unroll
-            for (int i = 0; i < (DH <= 128 ? 1 : 2); ++i) {
-                if (mp > -INFINITY && (i * 32 + lane) * 4 < DH) {
-                    const float4 x = __ldcg(src + i * 32 + lane);
-                    acc[i].x += fp * x.x; acc[i].y += fp * x.y; acc[i].z += fp * x.z; acc[i].w += fp * x.w;
-                }
-            }
-        }
-        const float inv = lsum == 0.f ? 0.f : 1.f / lsum;  // 0: the row sees no key; a NaN stays one
+    if (*s_last == 0) return;
+    const int64_t slot0 = job * pieces;
+    const int parts = nrows >= 3 ? 1 : WARPS / nrows;
+    float4 acc[V];
+    auto put = [&](int r, float inv) {
         const int row = row0 + r;
         __nv_bfloat16 *o = a.o + b * a.o_sb + (hk * a.group + row / a.Lq) * a.o_sh + (int64_t)(row % a.Lq) * a.o_sr;
 #pragma unroll
-        for (int i = 0; i < (DH <= 128 ? 1 : 2); ++i) {
+        for (int i = 0; i < V; ++i) {
             const int c = (i * 32 + lane) * 4;
             if (c < a.Dh) {   // Dh and the strides are multiples of 8
                 const __nv_bfloat162 lo = __floats2bfloat162_rn(acc[i].x * inv, acc[i].y * inv), hi = __floats2bfloat162_rn(acc[i].z * inv, acc[i].w * inv);
                 *reinterpret_cast<uint2 *>(o + c) = make_uint2(*reinterpret_cast<const uint32_t *>(&lo), *reinterpret_cast<const uint32_t *>(&hi));
             }
         }
+    };
+    for (int u = warp; u < nrows * parts; u += WARPS) {
+        const int r = u / parts;
+        const float *pm = a.part_ml + ((slot0 + lane) * kRows + r) * 2;    // lane p looks after piece p
+        const float mw = lane < pieces ? __ldcg(pm) : -INFINITY, lw = lane < pieces ? __ldcg(pm + 1) : 0.f;
+        const float4 *src = reinterpret_cast<const float4 *>(a.part_o + (slot0 * kRows + r) * DH) + lane;
+        float mx = mw;
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, d));
+        const float f = mw > -INFINITY ? ptx::ex2(mw - mx) : 0.f;   // (a piece without a key has zeros for its sums)
+        float lsum = f * lw;
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, d);
+#pragma unroll
+        for (int i = 0; i < V; ++i) acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll (V == 1 ? 8 : 4)
+        for (int p = u % parts; p < pieces; p += parts) {
+            const float fp = __shfl_sync(0xffffffffu, f, p);
+#pragma unroll
+            for (int i = 0; i < V; ++i)
+                if ((i * 32 + lane) * 4 < DH) {
+                    const float4 x = __ldcg(src + (int64_t)p * kRows * (DH / 4) + i * 32);
+                    acc[i].x += fp * x.x; acc[i].y += fp * x.y; acc[i].z += fp * x.z; acc[i].w += fp * x.w;
+                }
+        }
+        const float inv = lsum == 0.f ? 0.f : 1.f / lsum;  // 0: the row sees no key; a NaN stays one
+        if (parts == 1) {
+            put(r, inv);
+        } else {
+#pragma unroll
+            for (int i = 0; i < V; ++i) s_acc[(u * V + i) * 32 + lane] = acc[i];
+            if (lane == 0) s_inv[r] = inv;
+        }
     }
+    if (parts == 1) return;
+    __syncthreads();
+    if (warp >= nrows) return;
+#pragma unroll
+    for (int i = 0; i < V; ++i) {
+        acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int s = 0; s < parts; ++s) {
+            const float4 x = s_acc[((warp * parts + s) * V + i) * 32 + lane];
+            acc[i].x += x.x; acc[i].y += x.y; acc[i].z += x.z; acc[i].w += x.w;
+        }
+    }
+    put(warp, s_inv[warp]);
 }
 
 template <int DH, int NT, bool MEET>
@@ -379,7 +408,7 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, kDecodeBlocks) attn_decode_
             }
         }
     }
-    if constexpr (MEET) decode_meet<DH, NT>(a, reinterpret_cast<int *>(smem + S::kOffMl));
+    if constexpr (MEET) decode_meet<DH, NT>(a, smem);
 }
 
 // Jobs cut into pieces: a block per row; its warps take every fourth piece each, and meet in order.
@@ -519,12 +548,15 @@ int launch_decode_attn(const rmm_attn_desc_t *d, int64_t kd, const void *Q, cons
     a.idx_feat = idx_feat;
     a.part_o = static_cast<float *>(scratch);
     a.part_ml = a.part_o + (size_t)g.blocks * 8 * g.nt * g.dh;
-    // Short pieces of up to 1024 keys are added up in the last block of their job, where a warp then has at most 16 pieces of rows
-    // (4 x 8 heads x 2048 keys 17.6 -> 16.0 us, 16 x 8 / 4 heads x 512 17.5 -> 14.7, 8 x 32 / 8 heads x 4096 32.0 -> 31.8) and each job has
-    // its counter (the header's last four belong to the products).  Others keep a launch of their own, with a block per row: 32 pieces
-    // of rows a warp took 22.7 us for 17.6 (32 / 8 heads x 4096), and pieces of 4096 keys 96 for 90 (16 x 32 / 8 heads x 8192).
-    const int64_t rows_a_warp = ceil_div(a.rows < 8 * g.nt ? a.rows : 8 * g.nt, kDecodeWarps);
-    const bool meet = g.pieces > 1 && g.per <= 16 && g.pieces * rows_a_warp <= 16 && g.jobs <= kHeaderCounters - 4;
+    // Where the last block of a job adds the pieces up (each job then has its counter; the header's last four belong to the
+    // products).  Measured on 420 shapes against a launch of its own, through the binding and as a replayed graph.  Heads of up to
+    // 128: the meeting takes 0.5 to 1.5 us of the GPU more than that launch, which starts early, and saves 3.5 us of the host.
+    // So it is for short pieces of few rows, whose calls the host bounds (per <= 4 and up to four rows: 18.4 -> 14.9 to 17 us a
+    // call, 9.9 -> 10.9 replayed); six tiles a piece gain nothing (level, 7 % replayed), eight rows lose 7 to 16 %.  Heads of 256,
+    // whose second launch starts late: 2 to 13 % faster either way, but for short pieces of more than four rows (6 % slower).
+    const int64_t rows = a.rows < 8 * g.nt ? a.rows : 8 * g.nt;
+    const bool worth = g.dh <= 128 ? rows <= kDecodeWarps && g.per <= 4 : rows <= kDecodeWarps || g.per >= 6;
+    const bool meet = g.pieces > 1 && worth && g.per <= 16 && g.pieces * ceil_div(rows, kDecodeWarps) <= 16 && g.jobs <= kHeaderCounters - 4;
     if (meet) a.counters = counters;
     auto launch = [&](auto dh, auto nt) {
         constexpr int kDh = decltype(dh)::value, kNt = decltype(nt)::value;

@@ -12,9 +12,14 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("B, Hq, Hkv, Lq, Lk, Dh, launches", [
     (8, 32, 8, 1, 1000, 128, 1),     # four pieces of four rows
     (4, 16, 8, 1, 1500, 64, 1),      # eight pieces of two rows, half a warp per row
-    (20, 4, 2, 4, 1100, 256, 1),     # six pieces of eight rows, wide heads
-    (10, 4, 2, 4, 1100, 256, 2),     # nine of them
-    (30, 16, 2, 2, 900, 128, 1),     # sixteen rows a block
+    (8, 24, 8, 1, 1000, 128, 1),     # three rows: a warp without one
+    (9, 2, 2, 1, 2000, 64, 1),       # sixteen pieces of one row, shared out among the warps
+    (20, 4, 2, 1, 1100, 256, 1),     # two rows of wide heads
+    (20, 4, 2, 4, 4000, 256, 1),     # long pieces of eight rows, wide heads
+    (20, 4, 2, 4, 1100, 256, 2),     # short ones
+    (10, 4, 2, 4, 1100, 256, 2),
+    (30, 16, 2, 2, 900, 128, 2),     # sixteen rows a block
+    (4, 4, 4, 1, 6092, 128, 2),      # pieces of six tiles
     (2, 4, 2, 1, 3000, 128, 2),      # one row per warp, more than 32 pieces
     (1, 32, 2, 1, 4000, 64, 2),      # sixteen rows, many pieces
 ])
