@@ -286,9 +286,9 @@ int rmm_reduced_gemm(const rmm_mat_t *A, const rmm_mat_t *B, const int32_t *idx,
     if (plan_split(A, &b, k, &split) && split.cost < gemm_simt_cost(A, &b, k) && ws_bytes >= split.total_bytes) {
         rc = launch_split_gemm(A, &b, idx, k, scale, Y, split, ws, static_cast<cudaStream_t>(stream));
         if (rc != RMM_OK) return rc;
-        // elements that cannot be split: the FMA kernel does the product (its scratch ends before the flags)
-        return launch_gemm_simt(A, &b, idx, k, scale, Y, ws, split.off_flags, static_cast<cudaStream_t>(stream),
-                                reinterpret_cast<const int *>(static_cast<char *>(ws) + split.off_flags), (int)(split.gather_blocks * A->batch));
+        // elements that cannot be split: the FMA kernel does the outputs that see them (its scratch ends before the flags)
+        const SplitFlags left = split_flags(A, &b, k, split, ws);
+        return launch_gemm_simt(A, &b, idx, k, scale, Y, ws, split.off_flags, static_cast<cudaStream_t>(stream), &left);
     }
     return launch_gemm_simt(A, &b, idx, k, scale, Y, ws, ws_bytes, static_cast<cudaStream_t>(stream));
 }

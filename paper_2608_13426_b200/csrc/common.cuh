@@ -149,22 +149,32 @@ int launch_small_product(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k, floa
 
 // ---- reduced GEMM ------------------------------------------------------------------------------------
 // Plain FMA kernel: any strides, bf16 or fp32 operands, fp32 accumulation, bf16 or fp32 output.
-// n_flags > 0: the kernel returns at once unless one of flags[0 .. n_flags) is set (they must lie outside the workspace).
+// `behind`: what gemm_split.cu left to it (flags and verdict lie outside the workspace given here).
+struct SplitFlags;
 int launch_gemm_simt(const rmm_mat_t *A, const rmm_mat_t *B, const int32_t *idx, int64_t k, float scale,
-                     const rmm_mat_t *Y, void *ws, size_t ws_bytes, cudaStream_t stream, const int *flags = nullptr, int n_flags = 0);
-double gemm_simt_cost(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k);  // estimate, microseconds
+                     const rmm_mat_t *Y, void *ws, size_t ws_bytes, cudaStream_t stream, const SplitFlags *behind = nullptr);
+// Estimate, microseconds; tile_us: of a block that shares its SM.
+double gemm_simt_cost(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k, double *tile_us = nullptr);
 // What the slices of the contraction axis want; a smaller workspace (down to the header) gets fewer slices.
 size_t gemm_simt_workspace_bytes(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k);
 
-// fp32 operands as sums of three bf16 numbers on the tensor cores (gemm_split.cu).  Leaves the product to the FMA kernel where a
-// kept element cannot be split: flags [0, gather_blocks * batch) at off_flags.
+// fp32 operands as sums of three bf16 numbers on the tensor cores (gemm_split.cu).  Outputs that see a kept element which cannot be
+// split are left to the FMA kernel: a flag per gathering block (per batch element those of A, [16 rows][256 kept columns], then
+// those of B, [16 kept rows][256 columns] or, K-major, [16 columns][256 kept rows]) and a verdict (0: nothing is left, 1: what the
+// flags say, 2: everything).
+struct SplitFlags {
+    const int *flags;
+    int *verdict;
+    int per_batch, a_blocks, a_cols, b_rows, b_cols, b_kmajor;   // flags per batch element, those of A, blocks per row of blocks
+};
 struct SplitPlan {
     int b_kmajor;
-    int64_t lda, ldb, gather_blocks, tiles, cut_first, seg_kb;
+    int64_t lda, ldb, a_blocks, gather_blocks, tiles, cut_first, seg_kb;
     size_t off_a, off_b, off_partials, off_flags, total_bytes;
     double cost;   // estimate, microseconds
 };
 bool plan_split(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k, SplitPlan *plan);
+SplitFlags split_flags(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k, const SplitPlan &plan, void *ws);
 int launch_split_gemm(const rmm_mat_t *A, const rmm_mat_t *B, const int32_t *idx, int64_t k, float scale, const rmm_mat_t *Y,
                       const SplitPlan &plan, void *ws, cudaStream_t stream);
 

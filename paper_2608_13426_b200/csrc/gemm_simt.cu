@@ -35,8 +35,8 @@ struct SimtArgs {
     int64_t k_split;      // contraction indices per slice (a multiple of BK)
     float4 *partials;     // [tile][slice][TM * 2][THREADS]
     unsigned *counters;   // one per tile
-    const int *flags;     // n_flags > 0: nothing is done unless one of them is set
-    int n_flags;
+    int behind;           // only what the split product left over
+    SplitFlags left;
 };
 
 template <bool BF16>
@@ -64,15 +64,27 @@ __global__ void __launch_bounds__(THREADS) reduced_gemm_simt_kernel(const SimtAr
     __shared__ __align__(16) float sB[kRing][BK][PB];
     __shared__ int s_last;
     pdl_wait();
-    if (a.n_flags > 0) {
-        int set = 0;
-        for (int i = threadIdx.x; i < a.n_flags; i += THREADS) set |= __ldg(a.flags + i);
-        if (!__syncthreads_or(set)) return;
-    }
-
     const int tid = threadIdx.x;
     const int64_t b = blockIdx.z / a.splits, slice = blockIdx.z % a.splits;
     const int64_t m0 = (int64_t)blockIdx.y * BM, n0 = (int64_t)blockIdx.x * BN;
+    if (a.behind) {
+        const SplitFlags &f = a.left;
+        const int verdict = __ldg(f.verdict);
+        if (verdict == 0) return;
+        if (verdict == 1) {   // (all slices of a tile find the same)
+            const int *fa = f.flags + b * f.per_batch, *fb = fa + f.a_blocks;
+            const int a_end = (int)min((int64_t)f.a_blocks, (m0 + BM) / 16 * f.a_cols);
+            int set = 0;
+            for (int i = (int)(m0 / 16) * f.a_cols + tid; i < a_end; i += THREADS) set |= __ldg(fa + i);
+            if (f.b_kmajor) {
+                const int b_end = (int)min((int64_t)f.b_rows, (n0 + BN) / 16) * f.b_cols;
+                for (int i = (int)(n0 / 16) * f.b_cols + tid; i < b_end; i += THREADS) set |= __ldg(fb + i);
+            } else {
+                for (int r = tid; r < f.b_rows; r += THREADS) set |= __ldg(fb + r * f.b_cols + n0 / 256);
+            }
+            if (!__syncthreads_or(set)) return;
+        }
+    }
     const int64_t k_begin = slice * a.k_split, k_end = min(a.k, k_begin + a.k_split);
     const int hi = tid / 16, lo = tid % 16;   // compute: row group hi, column group lo
     const int32_t *idx = a.idx != nullptr ? a.idx + b * a.k : nullptr;
@@ -375,19 +387,21 @@ size_t gemm_simt_workspace_bytes(const rmm_mat_t *A, const rmm_mat_t *B, int64_t
     return RMM_WS_HEADER_BYTES + most;
 }
 
-double gemm_simt_cost(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k)
+double gemm_simt_cost(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k, double *tile_us)
 {
     double cost;
-    plan_simt(A, B, k, SIZE_MAX, &cost);
+    const SimtPlan plan = plan_simt(A, B, k, SIZE_MAX, &cost);
+    if (tile_us != nullptr) *tile_us = (double)(plan.k_split / BK) * (plan.tm == 8 ? 2.7 : 2.3);
     return cost;
 }
 
 int launch_gemm_simt(const rmm_mat_t *A, const rmm_mat_t *B, const int32_t *idx, int64_t k, float scale,
-                     const rmm_mat_t *Y, void *ws, size_t ws_bytes, cudaStream_t stream, const int *flags, int n_flags)
+                     const rmm_mat_t *Y, void *ws, size_t ws_bytes, cudaStream_t stream, const SplitFlags *behind)
 {
     const SimtPlan plan = plan_simt(A, B, k, ws_bytes - RMM_WS_HEADER_BYTES);
     SimtArgs a = {};
-    a.flags = flags; a.n_flags = n_flags;
+    a.behind = behind != nullptr;
+    if (behind != nullptr) a.left = *behind;
     a.A = A->ptr; a.B = B->ptr; a.Y = Y->ptr; a.idx = idx;
     a.M = A->rows; a.K = A->cols; a.N = B->cols; a.k = k;
     a.a_sb = A->stride_batch; a.a_sr = A->stride_row; a.a_sc = A->stride_col;

@@ -128,8 +128,10 @@ struct SplitGemmArgs {
     float scale;
     float4 *partials;     // [2 x CTAs][32][128]: the sums of a CTA's first and last tile where those are cut, rows of four columns
     unsigned *counters;   // [CTAs]
-    const int *flags;
-    int n_flags;
+    SplitFlags f;
+    int n_flags;          // of all batch elements
+    int cost_a, cost_b;   // tiles of the FMA kernel that a flag of a block of A or B stands for
+    int64_t most_lost;    // from more than these on that kernel does everything
     int *status;
     unsigned long long wait_ns;
     int withhold;
@@ -141,6 +143,7 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
 {
     extern __shared__ uint8_t smem_raw[];
     __shared__ int s_last;
+    __shared__ unsigned long long s_lost;
     const uint32_t rank = cluster_rank();
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t *base_ptr = smem_raw + (base - smem_u32(smem_raw));
@@ -171,9 +174,21 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
     const uint32_t tmem_base = *tmem_slot;
     pdl_wait();
 
-    int odd = 0;
-    for (int i = tid; i < a.n_flags; i += kSplitThreads) odd |= __ldg(a.flags + i);
-    const bool run = !__syncthreads_or(odd);   // (the same in both CTAs)
+    // Elements that cannot be split: the FMA kernel behind does the outputs that see them, or everything if those are too many (the
+    // verdict is the same in every CTA).
+    if (tid == 0) s_lost = 0;
+    __syncthreads();
+    {
+        unsigned long long lost = 0;
+        for (int i = tid; i < a.n_flags; i += kSplitThreads)
+            if (__ldg(a.f.flags + i) != 0) lost += i % a.f.per_batch < a.f.a_blocks ? a.cost_a : a.cost_b;
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) lost += __shfl_xor_sync(0xffffffffu, lost, d);
+        if (lane == 0 && lost > 0) atomicAdd(&s_lost, lost);
+    }
+    __syncthreads();
+    const bool run = s_lost <= (unsigned long long)a.most_lost;
+    if (blockIdx.x == 0 && tid == 0) *a.f.verdict = run ? (s_lost > 0 ? 1 : 0) : 2;
 
     const int num_kb = (int)((a.k + kBk - 1) / kBk);
     // The n-th piece of work of this pair: k-blocks [kb0, kb1) of a tile.  Whole tiles round robin, then the pair's share of the rest,
@@ -394,15 +409,30 @@ bool plan_split(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k, SplitPlan *p)
     p->lda = ceil_div(k, 8) * 8;
     p->ldb = p->b_kmajor ? p->lda : ceil_div(N, 8) * 8;
     const int64_t b_rows = p->b_kmajor ? N : k;
-    p->gather_blocks = ceil_div(M, kGatherRows) * ceil_div(p->lda, kGatherCols) + ceil_div(b_rows, kGatherRows) * ceil_div(p->ldb, kGatherCols);
+    p->a_blocks = ceil_div(M, kGatherRows) * ceil_div(p->lda, kGatherCols);
+    p->gather_blocks = p->a_blocks + ceil_div(b_rows, kGatherRows) * ceil_div(p->ldb, kGatherCols);
     if (p->gather_blocks * batch > (1 << 20)) return false;
     size_t off = RMM_WS_HEADER_BYTES;
     p->off_a = off; off += align_up((size_t)batch * kPlanes * M * p->lda * 2, 256);
     p->off_b = off; off += align_up((size_t)batch * kPlanes * b_rows * p->ldb * 2, 256);
     p->off_partials = off; off += (size_t)(2 * pairs) * 2 * kTile * kTile * 4;
-    p->off_flags = off; off += align_up((size_t)(p->gather_blocks * batch) * 4, 256);
+    p->off_flags = off; off += align_up((size_t)(p->gather_blocks * batch + 1) * 4, 256);   // and the verdict
     p->total_bytes = off;
     return true;
+}
+
+SplitFlags split_flags(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k, const SplitPlan &p, void *ws)
+{
+    SplitFlags f;
+    f.flags = reinterpret_cast<const int *>(static_cast<char *>(ws) + p.off_flags);
+    f.per_batch = (int)p.gather_blocks;
+    f.verdict = const_cast<int *>(f.flags) + p.gather_blocks * A->batch;
+    f.a_blocks = (int)p.a_blocks;
+    f.a_cols = (int)ceil_div(p.lda, kGatherCols);
+    f.b_rows = (int)ceil_div(p.b_kmajor ? B->cols : k, kGatherRows);
+    f.b_cols = (int)ceil_div(p.ldb, kGatherCols);
+    f.b_kmajor = p.b_kmajor;
+    return f;
 }
 
 int launch_split_gemm(const rmm_mat_t *A, const rmm_mat_t *B, const int32_t *idx, int64_t k, float scale, const rmm_mat_t *Y, const SplitPlan &p,
@@ -457,7 +487,16 @@ int launch_split_gemm(const rmm_mat_t *A, const rmm_mat_t *B, const int32_t *idx
     a.scale = scale;
     a.partials = reinterpret_cast<float4 *>(w + p.off_partials);
     a.counters = h->counters;
-    a.flags = g.flags; a.n_flags = (int)(p.gather_blocks * batch);
+    a.f = split_flags(A, B, k, p, ws);
+    a.n_flags = (int)(p.gather_blocks * batch);
+    // (64 x 128 tiles; a block of A has 16 rows, one of B 16 or 256 columns)
+    a.cost_a = (int)ceil_div(N, 128); a.cost_b = (int)ceil_div(M, 64) * (p.b_kmajor ? 1 : 2);
+    // A few tiles take the FMA kernel as long as its slowest block does, on an SM with two others: only products of several rounds of
+    // its blocks gain by leaving the rest to the tensor cores, and not from half of the tiles on.  (One element of 1e-20: 2048 x
+    // 4096 kept x 4096 1552 us -> 1064, 8192 x 4096 x 8192 11460 -> 4441; 777 x 1500 x 1500 would take 139 for 127.)
+    double tile_us;
+    const double fma_us = gemm_simt_cost(A, B, k, &tile_us);
+    a.most_lost = p.cost + tile_us < fma_us ? batch * ceil_div(M, 64) * ceil_div(N, 128) / 2 : 0;
     a.status = &h->status;
     a.wait_ns = wait_limit_ns();
     a.withhold = debug_withhold() == WITHHOLD_GEMM;

@@ -57,23 +57,78 @@ def test_batches_shared_weights_and_no_list():
     assert float((Y.double() - want).norm() / want.norm()) <= 2.0 ** -22
 
 
-@pytest.mark.parametrize("value", [float("inf"), -float("inf"), float("nan"), 3e38, 1e-38, 1e-44, 2e12])
-@pytest.mark.parametrize("where", ["A", "B"])
+def fma_rows(A, B, idx):
+    """The same product by the FMA kernel with room for the slices that it takes behind the split product."""
+    M, N, k = A.shape[0], B.shape[1], len(idx)
+    # the split product wants the header and its flags besides
+    ws = torch.zeros(6 * (M + N) * k + 2 * 148 * 65536, dtype=torch.uint8, device="cuda")
+    n0 = rmm.rmm_launch_count()
+    Y = rmm.rmm_reduced_gemm(A, B, idx, ws=ws)
+    assert rmm.rmm_launch_count() - n0 == 1
+    return Y
+
+
+# the last two of either side lie just inside 2^-50 .. 2^40, the ones before them just outside
+@pytest.mark.parametrize("value", [float("inf"), -float("inf"), float("nan"), 3e38, 1e-38, 1e-44, -(2.0 ** 40) * (1 + 2.0 ** -23), 2.0 ** -50 * (1 - 2.0 ** -24)])
+@pytest.mark.parametrize("where", ["A", "B", "B by columns"])
 def test_elements_that_cannot_be_split_take_the_fma_kernel(value, where):
+    """The outputs that see such an element, in tiles of 64 x 128, are the FMA kernel's bit for bit; the others stay.  (A product of
+    several rounds of the FMA kernel's blocks; a smaller one is all its.)"""
+    M, K, N, k = 4000, 3000, 4100, 1500
+    A, B = operands(M, K, N, "rows", seed=5)
+    if where == "B by columns":
+        B = B.t().contiguous().t()
+    X = A if where == "A" else B
+    idx = torch.arange(0, 3000, 2, dtype=torch.int32, device="cuda")
+    plain = rmm.rmm_reduced_gemm(A, B, idx)
+    X[501 if where == "A" else 1001, 1001 if where == "A" else 501] = value    # not kept: nothing changes
+    assert torch.equal(rmm.rmm_reduced_gemm(A, B, idx), plain)
+    X[500, 500] = value
+    Y, want = rmm.rmm_reduced_gemm(A, B, idx), fma_rows(A, B, idx)
+    left = torch.zeros(M, N, dtype=torch.bool, device="cuda")
+    if where == "A":
+        left[448:512] = True                                                    # rows 496 .. 511 share a flag, a tile has 64
+    elif where == "B":
+        left[:, 256:512] = True                                                # 256 columns share a flag
+    else:
+        left[:, 384:512] = True                                                 # 16 columns do, a tile has 128
+    same = (Y == want) | (Y.isnan() & want.isnan())
+    assert bool(same[left].all()) and torch.equal(Y[~left], plain[~left])
+    assert not bool(same[~left].all())                                          # the two forms do differ
+    A, B = A[:777], B[:, :1500]
+    Y, want = rmm.rmm_reduced_gemm(A, B, idx), fma_rows(A, B, idx)
+    assert bool(((Y == want) | (Y.isnan() & want.isnan())).all()) and rmm.rmm_status_read() == 0
+
+
+@pytest.mark.parametrize("value", [2.0 ** 40, -(2.0 ** 40), 2.0 ** -50, 0.0])
+@pytest.mark.parametrize("where", ["A", "B"])
+def test_elements_at_the_ends_of_the_range_are_split(value, where):
     M, K, N, k = 777, 3000, 1500, 1500
     A, B = operands(M, K, N, "rows", seed=5)
     idx = torch.arange(0, 3000, 2, dtype=torch.int32, device="cuda")
-    plain = rmm.rmm_reduced_gemm(A, B, idx)
-    (A if where == "A" else B)[501 if where == "A" else 1001, 1001 if where == "A" else 501] = value    # not kept: nothing changes
-    assert torch.equal(rmm.rmm_reduced_gemm(A, B, idx), plain)
     (A if where == "A" else B)[500, 500] = value
-    ws = torch.zeros(1 << 28, dtype=torch.uint8, device="cuda")
-    Y = rmm.rmm_reduced_gemm(A, B, idx, ws=ws)
-    want = A[:, ::2].double() @ B[::2].double()
-    assert torch.equal(Y.isfinite(), want.float().isfinite()) and torch.equal(Y.isnan(), want.float().isnan())
-    ok = want.float().isfinite()
-    assert torch.allclose(Y[ok].double(), want[ok], rtol=1e-5, atol=1e-5 * float(want[ok].abs().max()))
-    assert torch.equal(rmm.rmm_reduced_gemm(A, B, idx, ws=ws).nan_to_num(1.0), Y.nan_to_num(1.0))
+    Y, other = rmm.rmm_reduced_gemm(A, B, idx), fma_rows(A, B, idx)
+    rows = slice(500, 501) if where == "A" else slice(None)
+    cols = slice(500, 501) if where == "B" else slice(None)
+    assert not torch.equal(Y[448:512, 256:512], other[448:512, 256:512])
+    # per output, against the sum of the products' magnitudes (3 parts: 2^-22 of it, as everywhere)
+    want = A[rows][:, idx.long()].double() @ B[idx.long()][:, cols].double()
+    size = A[rows][:, idx.long()].double().abs() @ B[idx.long()][:, cols].double().abs()
+    assert bool(((Y[rows, cols].double() - want).abs() <= size * 2.0 ** -22).all())
+
+
+@pytest.mark.parametrize("M, K, N, every", [(777, 3000, 1500, 1), (777, 3000, 1500, 40), (1100, 2000, 640, 1), (4000, 3000, 4100, 64)])
+def test_many_elements_that_cannot_be_split(M, K, N, every):
+    """From half of the tiles on, everything is the FMA kernel's."""
+    A, B = operands(M, K, N, "rows", seed=6)
+    idx = torch.arange(0, K, 2, dtype=torch.int32, device="cuda")
+    A[::every, 0] = 1e-30
+    Y, want = rmm.rmm_reduced_gemm(A, B, idx), fma_rows(A, B, idx)
+    assert torch.equal(Y, want)
+    exact = A[:, ::2].double() @ B[::2].double()
+    assert bool(((Y.double() - exact).norm(dim=1) <= exact.norm(dim=1) * 2.0 ** -22).all())     # every row by itself
+    again = rmm.rmm_reduced_gemm(A, B, idx)
+    assert torch.equal(Y, again) and rmm.rmm_status_read() == 0
 
 
 def test_bad_index_is_reported():
