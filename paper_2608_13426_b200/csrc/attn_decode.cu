@@ -551,11 +551,12 @@ int launch_decode_attn(const rmm_attn_desc_t *d, int64_t kd, const void *Q, cons
     // Where the last block of a job adds the pieces up (each job then has its counter; the header's last four belong to the
     // products).  Measured on 420 shapes against a launch of its own, through the binding and as a replayed graph.  Heads of up to
     // 128: the meeting takes 0.5 to 1.5 us of the GPU more than that launch, which starts early, and saves 3.5 us of the host.
-    // So it is for short pieces of few rows, whose calls the host bounds (per <= 4 and up to four rows: 18.4 -> 14.9 to 17 us a
-    // call, 9.9 -> 10.9 replayed); six tiles a piece gain nothing (level, 7 % replayed), eight rows lose 7 to 16 %.  Heads of 256,
-    // whose second launch starts late: 2 to 13 % faster either way, but for short pieces of more than four rows (6 % slower).
+    // So it is for short pieces of few rows, whose calls the host bounds (four tiles of heads of 128, eight of 64, up to four rows:
+    // 17.9 -> 14.5 to 16.4 us a call, 10 to 14 -> 11 to 15 replayed); longer ones gain nothing (level or slower, 7 % replayed), eight
+    // rows lose 7 to 16 %.  Heads of 256, whose second launch starts late: 2 to 13 % faster either way, but for short pieces of more
+    // than four rows (6 % slower).
     const int64_t rows = a.rows < 8 * g.nt ? a.rows : 8 * g.nt;
-    const bool worth = g.dh <= 128 ? rows <= kDecodeWarps && g.per <= 4 : rows <= kDecodeWarps || g.per >= 6;
+    const bool worth = g.dh <= 128 ? rows <= kDecodeWarps && g.per * g.dh <= 512 : rows <= kDecodeWarps || g.per >= 6;
     const bool meet = g.pieces > 1 && worth && g.per <= 16 && g.pieces * ceil_div(rows, kDecodeWarps) <= 16 && g.jobs <= kHeaderCounters - 4;
     if (meet) a.counters = counters;
     auto launch = [&](auto dh, auto nt) {

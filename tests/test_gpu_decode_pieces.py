@@ -20,6 +20,7 @@ pytestmark = pytest.mark.gpu
     (10, 4, 2, 4, 1100, 256, 2),
     (30, 16, 2, 2, 900, 128, 2),     # sixteen rows a block
     (4, 4, 4, 1, 6092, 128, 2),      # pieces of six tiles
+    (4, 4, 4, 1, 6092, 64, 1),
     (2, 4, 2, 1, 3000, 128, 2),      # one row per warp, more than 32 pieces
     (1, 32, 2, 1, 4000, 64, 2),      # sixteen rows, many pieces
 ])
