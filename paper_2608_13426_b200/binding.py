@@ -475,7 +475,11 @@ def rmm_product(A: torch.Tensor, B: torch.Tensor, rho: float = 0.0, k: int = 0, 
         raise RmmError(RMM_ERR_INVALID_ARG, "idx must be a contiguous int32 CUDA tensor of batch * k elements")
     ret = _out((ma.batch,), torch.float32, A) if want_retained else None
     my = as_mat(out)
-    need = lib().rmm_product_workspace_bytes(ma, mb, my)
+    if ma.dtype == RMM_F32:  # by the kept count (six bytes a kept element): the query without one covers every count
+        parts = lib().rmm_score_select_workspace_bytes(ma, 1), lib().rmm_reduced_gemm_workspace_bytes(ma, mb, kk, my)
+        need = max(parts) if min(parts) > 0 else 0
+    else:
+        need = lib().rmm_product_workspace_bytes(ma, mb, my)
     if need == 0:
         raise RmmError(RMM_ERR_UNSUPPORTED, "rmm_product: operands not covered")
     ws = workspace(need, A.device) if ws is None else ws

@@ -233,6 +233,11 @@ static rmm_mat_t shared_b(const rmm_mat_t *A, const rmm_mat_t *B)
     return b;
 }
 
+static bool split_wins(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k, SplitPlan *plan)
+{
+    return plan_split(A, B, k, plan) && plan->cost < gemm_simt_cost(A, B, k);
+}
+
 size_t rmm_reduced_gemm_workspace_bytes(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k, const rmm_mat_t *Y)
 {
     if (A == nullptr || B == nullptr || Y == nullptr) return 0;
@@ -243,7 +248,7 @@ size_t rmm_reduced_gemm_workspace_bytes(const rmm_mat_t *A, const rmm_mat_t *B, 
     if (tc_eligible(A, &b, k, Y, &plan)) return plan.total_bytes;
     const size_t fma = gemm_simt_workspace_bytes(A, &b, k);
     SplitPlan split;
-    return plan_split(A, &b, k, &split) && split.total_bytes > fma ? split.total_bytes : fma;
+    return split_wins(A, &b, k, &split) && split.total_bytes > fma ? split.total_bytes : fma;
 }
 
 // What a call needs: the forms that cut the contraction axis do with fewer pieces in a smaller workspace.  (A caller's one
@@ -283,13 +288,8 @@ int rmm_reduced_gemm(const rmm_mat_t *A, const rmm_mat_t *B, const int32_t *idx,
     rc = check_ws(ws, ws_bytes, RMM_WS_HEADER_BYTES, "reduced_gemm");
     if (rc != RMM_OK) return rc;
     SplitPlan split;
-    if (plan_split(A, &b, k, &split) && split.cost < gemm_simt_cost(A, &b, k) && ws_bytes >= split.total_bytes) {
-        rc = launch_split_gemm(A, &b, idx, k, scale, Y, split, ws, static_cast<cudaStream_t>(stream));
-        if (rc != RMM_OK) return rc;
-        // elements that cannot be split: the FMA kernel does the outputs that see them (its scratch ends before the flags)
-        const SplitFlags left = split_flags(A, &b, k, split, ws);
-        return launch_gemm_simt(A, &b, idx, k, scale, Y, ws, split.off_flags, static_cast<cudaStream_t>(stream), &left);
-    }
+    if (split_wins(A, &b, k, &split) && ws_bytes >= split.total_bytes)
+        return launch_split_gemm(A, &b, idx, k, scale, Y, split, ws, static_cast<cudaStream_t>(stream));
     return launch_gemm_simt(A, &b, idx, k, scale, Y, ws, ws_bytes, static_cast<cudaStream_t>(stream));
 }
 
@@ -455,6 +455,10 @@ size_t rmm_product_workspace_bytes(const rmm_mat_t *A, const rmm_mat_t *B, const
     rmm_mat_t b = shared_b(A, B);
     FrontPlan fp;
     if (front_eligible(A, &b, Y, A->cols, &fp) && fp.total_bytes > need) need = fp.total_bytes;
+    // (fp32: the estimates may prefer the parts for some counts of kept indices only)
+    SplitPlan split;
+    for (int64_t q = 3; q > 0; --q)
+        if (A->cols >= 4 && split_wins(A, &b, A->cols * q / 4, &split) && split.total_bytes > need) need = split.total_bytes;
     return need;
 }
 

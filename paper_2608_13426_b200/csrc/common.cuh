@@ -169,12 +169,12 @@ struct SplitFlags {
 };
 struct SplitPlan {
     int b_kmajor;
+    int64_t batch, rows, cols;   // of a panel: large products run in several
     int64_t lda, ldb, a_blocks, gather_blocks, tiles, cut_first, seg_kb;
     size_t off_a, off_b, off_partials, off_flags, total_bytes;
-    double cost;   // estimate, microseconds
+    double cost;   // estimate, microseconds, of all panels
 };
 bool plan_split(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k, SplitPlan *plan);
-SplitFlags split_flags(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k, const SplitPlan &plan, void *ws);
 int launch_split_gemm(const rmm_mat_t *A, const rmm_mat_t *B, const int32_t *idx, int64_t k, float scale, const rmm_mat_t *Y,
                       const SplitPlan &plan, void *ws, cudaStream_t stream);
 

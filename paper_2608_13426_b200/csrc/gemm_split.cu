@@ -381,24 +381,19 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
 
 }  // namespace
 
+// The layout of one panel: batch x rows of A times batch x cols columns of B.
 // Whole tiles round robin over the CTA pairs; a last round (or an only one) of few tiles is cut into one equal share per pair, where
 // that saves more than the meeting of the pieces costs.  (Cutting everything instead took 476 us for 440 on 2048 x 4096 kept x
 // 4096: pairs at different places of the contraction share no operands.)  Estimate in microseconds: 1.2 a k-block, 3 a round, 8
 // for cut tiles, and 10 for the launches of the gather and of the idle FMA kernel behind.
-bool plan_split(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k, SplitPlan *p)
+static void panel_layout(int64_t batch, int64_t rows, int64_t cols, int64_t k, SplitPlan *p)
 {
-    const int64_t M = A->rows, N = B->cols, batch = A->batch;
-    if (A->dtype != RMM_F32 || B->dtype != RMM_F32) return false;
-    if ((double)batch * (double)M * (double)N * (double)k < 1.5e8) return false;   // 10 us of the FMA kernel
-    const int64_t tm = ceil_div(M, 2 * kTile), tn = ceil_div(N, kTile), num_kb = ceil_div(k, kBk), sms = sm_count();
-    if (M > INT32_MAX / 2 || N > INT32_MAX / 2 || A->cols > INT32_MAX / 2 || batch > 65535 / kPlanes) return false;
-    const int64_t tiles = batch * tm * tn;
-    const int64_t pairs = sms / 2;
-    p->b_kmajor = B->stride_col != 1 && B->stride_row == 1;
+    const int64_t num_kb = ceil_div(k, kBk), pairs = sm_count() / 2, tiles = batch * ceil_div(rows, 2 * kTile) * ceil_div(cols, kTile);
+    p->batch = batch; p->rows = rows; p->cols = cols;
     p->tiles = p->cut_first = tiles;
     p->seg_kb = 0;
     const int64_t rest = tiles % pairs;
-    p->cost = 10.0 + (double)ceil_div(tiles, pairs) * (3.0 + 1.2 * (double)num_kb) + (double)(batch * (M + N) * k) * 10.0 / 5.0e6;  // the gather: four bytes read, six written
+    p->cost = 10.0 + (double)ceil_div(tiles, pairs) * (3.0 + 1.2 * (double)num_kb) + (double)(batch * (rows + cols) * k) * 10.0 / 5.0e6;  // the gather: four bytes read, six written
     const double saved = (1.0 - (double)rest / (double)pairs) * 1.2 * (double)num_kb - 8.0;
     if (rest > 0 && saved > 0.0) {
         p->cut_first = tiles - rest;
@@ -407,21 +402,43 @@ bool plan_split(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k, SplitPlan *p)
         p->cost -= saved;
     }
     p->lda = ceil_div(k, 8) * 8;
-    p->ldb = p->b_kmajor ? p->lda : ceil_div(N, 8) * 8;
-    const int64_t b_rows = p->b_kmajor ? N : k;
-    p->a_blocks = ceil_div(M, kGatherRows) * ceil_div(p->lda, kGatherCols);
+    p->ldb = p->b_kmajor ? p->lda : ceil_div(cols, 8) * 8;
+    const int64_t b_rows = p->b_kmajor ? cols : k;
+    p->a_blocks = ceil_div(rows, kGatherRows) * ceil_div(p->lda, kGatherCols);
     p->gather_blocks = p->a_blocks + ceil_div(b_rows, kGatherRows) * ceil_div(p->ldb, kGatherCols);
-    if (p->gather_blocks * batch > (1 << 20)) return false;
     size_t off = RMM_WS_HEADER_BYTES;
-    p->off_a = off; off += align_up((size_t)batch * kPlanes * M * p->lda * 2, 256);
+    p->off_a = off; off += align_up((size_t)batch * kPlanes * rows * p->lda * 2, 256);
     p->off_b = off; off += align_up((size_t)batch * kPlanes * b_rows * p->ldb * 2, 256);
     p->off_partials = off; off += (size_t)(2 * pairs) * 2 * kTile * kTile * 4;
     p->off_flags = off; off += align_up((size_t)(p->gather_blocks * batch + 1) * 4, 256);   // and the verdict
     p->total_bytes = off;
+}
+
+// The parts take six bytes an element of the kept operands, beside a user's own memory: products whose operands are larger than
+// kSplitParts allows run in panels (of batch elements, then of rows and columns), one after the other in the same scratch.  The
+// panels follow from the whole operands, not from the kept count, so that a workspace for more kept indices holds fewer.
+// 8192 x 4096 kept x 8192 2888 us a call in one panel, 2830 in four; 16384 x 4096 kept x 8192 5966 and, in eight, 6150 to 6290.
+constexpr double kSplitParts = 512.0 * 1024 * 1024;
+bool plan_split(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k, SplitPlan *p)
+{
+    const int64_t M = A->rows, N = B->cols, batch = A->batch;
+    if (A->dtype != RMM_F32 || B->dtype != RMM_F32) return false;
+    if ((double)batch * (double)M * (double)N * (double)k < 1.5e8) return false;   // 10 us of the FMA kernel
+    if (M > INT32_MAX / 2 || N > INT32_MAX / 2 || A->cols > INT32_MAX / 2 || batch > 65535 / kPlanes || ceil_div(M, 64) > 65535) return false;
+    int64_t nb = batch, rows = M, cols = N;
+    while ((double)nb * (double)(rows + cols) * (double)A->cols * 2.0 * kPlanes > kSplitParts) {
+        if (nb > 1) nb = ceil_div(nb, 2);
+        else if (rows >= cols && rows > 2 * kTile) rows = ceil_div(rows, 4 * kTile) * 2 * kTile;
+        else if (cols > 2 * kTile) cols = ceil_div(cols, 4 * kTile) * 2 * kTile;
+        else return false;
+    }
+    p->b_kmajor = B->stride_col != 1 && B->stride_row == 1;
+    panel_layout(nb, rows, cols, k, p);
+    p->cost *= (double)(ceil_div(batch, nb) * ceil_div(M, rows) * ceil_div(N, cols));
     return true;
 }
 
-SplitFlags split_flags(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k, const SplitPlan &p, void *ws)
+static SplitFlags split_flags(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k, const SplitPlan &p, void *ws)
 {
     SplitFlags f;
     f.flags = reinterpret_cast<const int *>(static_cast<char *>(ws) + p.off_flags);
@@ -435,8 +452,8 @@ SplitFlags split_flags(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k, const 
     return f;
 }
 
-int launch_split_gemm(const rmm_mat_t *A, const rmm_mat_t *B, const int32_t *idx, int64_t k, float scale, const rmm_mat_t *Y, const SplitPlan &p,
-                      void *ws, cudaStream_t stream)
+static int launch_panel(const rmm_mat_t *A, const rmm_mat_t *B, const int32_t *idx, int64_t k, float scale, const rmm_mat_t *Y, const SplitPlan &p,
+                        void *ws, cudaStream_t stream)
 {
     char *w = static_cast<char *>(ws);
     WsHeader *h = static_cast<WsHeader *>(ws);
@@ -508,6 +525,34 @@ int launch_split_gemm(const rmm_mat_t *A, const rmm_mat_t *B, const int32_t *idx
     e = launch_kernel(kern, dim3(2 * (unsigned)(p.tiles < pairs && p.seg_kb == 0 ? p.tiles : pairs)), dim3(kSplitThreads), kSplitSmem, stream, 2, ma, mb, a);
     if (e != cudaSuccess) return fail(RMM_ERR_CUDA, "split_gemm_kernel: launch: %s", cudaGetErrorString(e));
     return check_launch("split_gemm_kernel", stream);
+}
+
+int launch_split_gemm(const rmm_mat_t *A, const rmm_mat_t *B, const int32_t *idx, int64_t k, float scale, const rmm_mat_t *Y, const SplitPlan &plan,
+                      void *ws, cudaStream_t stream)
+{
+    const auto at = [](const rmm_mat_t *X, int64_t b, int64_t r, int64_t c) -> void * {
+        const int64_t e = b * X->stride_batch + r * X->stride_row + c * X->stride_col;
+        return static_cast<char *>(X->ptr) + e * (int64_t)dtype_size(X->dtype);
+    };
+    for (int64_t b = 0; b < A->batch; b += plan.batch)
+        for (int64_t c = 0; c < B->cols; c += plan.cols)
+            for (int64_t r = 0; r < A->rows; r += plan.rows) {
+                const int64_t nb = A->batch - b < plan.batch ? A->batch - b : plan.batch, rows = A->rows - r < plan.rows ? A->rows - r : plan.rows,
+                              cols = B->cols - c < plan.cols ? B->cols - c : plan.cols;
+                SplitPlan p = plan;
+                panel_layout(nb, rows, cols, k, &p);
+                rmm_mat_t pa = *A, pb = *B, py = *Y;
+                pa.ptr = at(A, b, r, 0); pb.ptr = at(B, b, 0, c); py.ptr = at(Y, b, r, c);
+                pa.batch = pb.batch = py.batch = nb; pa.rows = py.rows = rows; pb.cols = py.cols = cols;
+                const int32_t *list = idx != nullptr ? idx + b * k : nullptr;
+                int rc = launch_panel(&pa, &pb, list, k, scale, &py, p, ws, stream);
+                if (rc != RMM_OK) return rc;
+                // elements that cannot be split: the FMA kernel does the outputs that see them (its scratch ends before the flags)
+                const SplitFlags left = split_flags(&pa, &pb, k, p, ws);
+                rc = launch_gemm_simt(&pa, &pb, list, k, scale, &py, ws, p.off_flags, stream, &left);
+                if (rc != RMM_OK) return rc;
+            }
+    return RMM_OK;
 }
 
 }  // namespace rmm
