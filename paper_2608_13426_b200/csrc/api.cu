@@ -407,8 +407,10 @@ int rmm_reduced_gemm_scored(const rmm_mat_t *A, const rmm_mat_t *B, const int32_
     const size_t s1 = rmm_score_workspace_bytes(Y, 1), s2 = gemm_least_bytes(A, B, k, Y), apart = s1 > s2 ? s1 : s2;
     GemvPlan gplan;
     TcPlan plan;
-    // (small products take the form that rmm_reduced_gemm takes for them: the output is the same with and without its energies)
-    if (!(idx != nullptr && small_eligible(A, B, Y)) && !gemv_eligible(A, &b, k, Y, &gplan) && tc_eligible(A, &b, k, Y, &plan, true) &&
+    // small products take the form that rmm_reduced_gemm takes for them (the output is the same with and without its energies), unless
+    // the workspace has room for whole tiles only, whose epilogue leaves the energies
+    const bool small = idx != nullptr && ws_bytes >= apart && small_eligible(A, B, Y);
+    if (!small && !gemv_eligible(A, &b, k, Y, &gplan) && tc_eligible(A, &b, k, Y, &plan, true) &&
         plan.epilogue_energy && !(plan.gathers && idx != nullptr && ws_bytes >= apart && scored_apart(A->batch, A->rows, B->cols, k))) {
         rc = check_ws(ws, ws_bytes, plan.least_bytes, "reduced_gemm_scored");
         if (rc != RMM_OK) return rc;

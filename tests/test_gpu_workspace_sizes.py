@@ -64,3 +64,15 @@ def test_the_reserve_follows_the_problem():
     assert sized_for(A, B, 256) <= 4096 + 48 * 512 * 2 + 4 * 48 * 1024
     sizes = [sized_for(A, B, k) for k in (64, 128, 256, 512)]
     assert sizes == sorted(sizes)
+
+
+def test_a_small_scored_product_in_what_whole_tiles_take():
+    """Packed A and the epilogue's column energies: no room for a pass over the output."""
+    M, K, N, k = 64, 512, 256, 256
+    A, B = synth.mlp_product(M, K, N, seed=183)
+    Ad, Bd, idx = A.cuda(), B.cuda(), kept(K, k)
+    Y, e = rmm.rmm_reduced_gemm(Ad, Bd, idx, want_energy=True)
+    ws = buffer(4096 + M * k * 2 + M // 32 * N * 4)
+    Y2, e2 = rmm.rmm_reduced_gemm(Ad, Bd, idx, want_energy=True, ws=ws)
+    assert float((Y2.double() - Y.double()).norm() / Y.double().norm()) <= 2.0 ** -8        # a rounding to bf16 apart
+    assert torch.allclose(e2.double(), Y2.double().square().sum(0), rtol=3e-7, atol=0) and rmm.rmm_status_read(ws=ws) == 0
