@@ -829,12 +829,16 @@ int launch_gemm_tc_problem(const TcProblem &p, cudaStream_t stream)
     // one): whichever takes less by rounds of blocks.  Microseconds a k-block 0.37 for pairs, 0.42 for single CTAs, 3 a round, and
     // the longer set-up of a pair, which 8-bit operands (k-blocks of 128) feel more.  One round, 64 pairs: 2048 x 4096 kept x
     // 2048 29.6 us by pairs, 31.8 by single CTAs, 300 x 4096 x 8192 29.7 and 33; 2048 kept: level; 20000 x 750 x 256 49.6 and 50.2 (whole calls); 8-bit 2048 x 4096 x 2048 18.6 and
-    // 17.5.  Several rounds: 3000 x 4000 x 4096 70.7 and 82.  RMM_GEMM_CTAS=1 or 2 forces a form (for measurements).
+    // 17.5.  Several rounds: 3000 x 4000 x 4096 70.7 and 82; from six k-blocks on single CTAs have to be ahead by 5 % there (blocks
+    // do not take rounds in step: 8242 x 560 kept x 6848 66 us by pairs and 72 by single CTAs, estimated at 83 and 81; 8-bit 14344 x 656 x
+    // 1600 33 and 37; with two to five k-blocks single CTAs are ahead, 5793 x 128 x 4288 25 and 21, and where a round less does for
+    // them, 542 x 7680 x 6272 88 and 62).  RMM_GEMM_CTAS=1 or 2 forces a form (for measurements).
     static const int forced = []() { const char *e = getenv("RMM_GEMM_CTAS"); return e ? atoi(e) : 0; }();
     const int64_t sms = sm_count(), k_blocks = ceil_div(p.k, (int64_t)bke), pair_tiles = p.batch * ceil_div(p.M, 2 * BM) * ceil_div(p.N, 256);
     const double singles_us = (double)ceil_div(p.batch * ceil_div(p.M, BM) * ceil_div(p.N, 256), sms) * (3.0 + 0.42 * (double)k_blocks);
     const double pairs_us = (double)ceil_div(pair_tiles, sms / 2) * (3.0 + 0.37 * (double)k_blocks) + (p.fp8 ? 2.5 : 1.0);
-    int ctas = BN == 256 && p.M > BM && pairs_us < singles_us ? 2 : 1;
+    const double ahead = k_blocks >= 6 && pair_tiles >= sms / 2 ? 0.95 : 1.0;
+    int ctas = BN == 256 && p.M > BM && pairs_us * ahead < singles_us ? 2 : 1;
     if (forced == 1) ctas = 1;
     if (forced == 2 && BN == 256 && p.M > BM) ctas = 2;
     if (p.b_idx != nullptr) ctas = 1;  // the in-kernel row gather exists for single-CTA tiles
