@@ -44,6 +44,29 @@ def test_split_product_is_as_close_as_the_fma_kernel(M, K, N, k, form):
     assert rmm.rmm_status_read() == 0
 
 
+VALUES = {"uniform": lambda t: t.uniform_(), "exponential": lambda t: t.exponential_(), "absolute": lambda t: t.normal_().abs_(),
+          "spread": lambda t: t.normal_().mul_(2).exp_()}
+
+
+@pytest.mark.parametrize("k", [51, 64, 96, 449, 1024, 4100])
+@pytest.mark.parametrize("values", sorted(VALUES))
+def test_operands_of_one_sign(values, k):
+    """The tensor cores' sums round toward zero, which operands of one sign show: an accumulator of 64 indices is cut four times at its
+    full size (16 indices an instruction), half a unit of 2^-23 each, so 2^-22 whatever k is.  Where values lie far apart each of an
+    instruction's 17 terms is cut at a unit of the largest: 17 times that at the most."""
+    M = N = 2048 if k < 1024 else 1024
+    fill = VALUES[values]
+    A, B = torch.empty(M, k, device="cuda"), torch.empty(k, N, device="cuda")
+    torch.manual_seed(k)
+    fill(A), fill(B)
+    n0 = rmm.rmm_launch_count()
+    Y = rmm.rmm_reduced_gemm(A, B, None)
+    assert rmm.rmm_launch_count() - n0 == 3
+    want = A.double() @ B.double()
+    err = float((Y.double() - want).norm() / want.norm())
+    assert err <= 2.0 ** -22 * (17 if values == "spread" else 1), err
+
+
 def test_batches_shared_weights_and_no_list():
     A, B = torch.randn(3, 500, 2000, device="cuda"), torch.randn(3, 2000, 400, device="cuda")
     idx = torch.stack([torch.randperm(2000)[:1500].sort().values for _ in range(3)]).int().cuda()

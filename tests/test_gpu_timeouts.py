@@ -47,6 +47,34 @@ Y = rmm.rmm_reduced_gemm(Ad, Bd, idx)
 assert rel(Y.float().cpu().numpy(), oracle.reduced_gemm(A, B, idx.cpu().numpy())) <= 1e-2
 assert rmm.rmm_status_read() == 0
 """,
+    "gemm_cut_pair_tiles": """
+A, B = synth.mlp_product(300, 9000, 264, seed=9)
+Ad, Bd = A.cuda(), B.cuda()
+idx = torch.arange(0, 9000, 2, dtype=torch.int32, device="cuda")
+n0 = rmm.rmm_launch_count()
+rmm.rmm_reduced_gemm(Ad, Bd, idx)
+assert rmm.rmm_launch_count() - n0 == 3       # gathers, product, meeting: a tile's pieces lie with several CTA pairs
+expect_timeout(lambda: rmm.rmm_reduced_gemm(Ad, Bd, idx), 1)
+Y = rmm.rmm_reduced_gemm(Ad, Bd, idx)
+assert rel(Y.float().cpu().numpy(), oracle.reduced_gemm(A, B, idx.cpu().numpy())) <= 1e-2
+assert rmm.rmm_status_read() == 0
+""",
+    "gemm_fp32_parts": """
+A, B = synth.mlp_product(777, 3000, 1500, seed=10, dtype=torch.float32)
+Ad, Bd = A.cuda(), B.cuda()
+idx = torch.arange(0, 3000, 2, dtype=torch.int32, device="cuda")
+n0 = rmm.rmm_launch_count()
+rmm.rmm_reduced_gemm(Ad, Bd, idx)
+assert rmm.rmm_launch_count() - n0 == 3       # gather, product (its cut tiles meet through the header's counters), what is left of it
+expect_timeout(lambda: rmm.rmm_reduced_gemm(Ad, Bd, idx), 1)
+want = oracle.reduced_gemm(A, B, idx.cpu().numpy())
+assert rel(rmm.rmm_reduced_gemm(Ad, Bd, idx).cpu().numpy(), want) <= 1e-5
+expect_timeout(lambda: rmm.rmm_reduced_gemm(Ad, Bd, idx), 1)
+A[5, 0] = Ad[5, 0] = 1e-30                    # left to the FMA kernel, whose slices meet through the same counters
+want = oracle.reduced_gemm(A, B, idx.cpu().numpy())
+assert rel(rmm.rmm_reduced_gemm(Ad, Bd, idx).cpu().numpy(), want) <= 1e-5
+assert rmm.rmm_status_read() == 0
+""",
     "gemm_rows_of_b_fetched_in_kernel": """
 A, B = synth.mlp_product(100, 512, 512, seed=2)
 Ad, Bd = A.cuda(), B.cuda()
