@@ -171,7 +171,7 @@ def workspace(nbytes: int, device: torch.device) -> torch.Tensor:
     index = device.index
     key = (device.type, index if index is not None else torch.cuda.current_device())
     ws = _ws_cache.get(key)
-    nbytes = max(nbytes, RMM_WS_HEADER_BYTES)
+    nbytes = max(int(nbytes), RMM_WS_HEADER_BYTES)
     if ws is None or ws.numel() < nbytes:
         ws = torch.zeros(nbytes + 256, dtype=torch.uint8, device=device)
         _ws_cache[key] = ws

@@ -7,6 +7,7 @@ import re
 from fractions import Fraction
 
 import pytest
+import torch
 
 from paper_2608_13426_b200 import binding
 from paper_2608_13426_b200 import build as rmm_build
@@ -103,3 +104,12 @@ def test_workspace_sizes(L):
     assert L.rmm_reduced_attn_workspace_bytes(ctypes.byref(d)) > 4096
     d.rho_d = 0.0
     assert L.rmm_reduced_attn_workspace_bytes(ctypes.byref(d)) == 0
+
+
+def test_a_workspace_size_may_be_any_number():
+    device = torch.device("cpu", 0)
+    try:
+        assert binding.workspace(5000.0, device).numel() >= 5000
+        assert binding.workspace(1e4, device).numel() >= 10000
+    finally:
+        binding._ws_cache.pop(("cpu", 0), None)
