@@ -119,15 +119,28 @@ int rmm_score_select_static_status(int *device_status);
  *        the paper's static / random controls); order fixes the summation order
  *   bf16 operands run on the tensor cores (fp32 accumulation) when A has stride_col 1, B has
  *   stride_col 1 (slices of the contraction axis contiguous) or stride_row 1, Y has stride_col 1, and
- *   pointers / leading strides are 16-byte aligned; Y may be bf16 or fp32.  Every other layout, and
- *   fp32 operands, run on a plain FMA kernel (fp32 accumulation).  A and B must share a dtype.
+ *   pointers / leading strides are 16-byte aligned; Y may be bf16 or fp32.  Every other bf16 layout runs on a plain FMA
+ *   kernel (fp32 accumulation).  A and B must share a dtype.
+ *   fp32 operands (any strides) run on the tensor cores, every element as the sum of three bf16 numbers (six products of
+ *   parts, accumulators of 64 indices added up in fp32), or on the FMA kernel where that is estimated to be faster (few rows,
+ *   small products) or the workspace has no room for the parts (6 bytes per kept element of both operands, at most 512 MB: larger
+ *   products run in panels; 20 MB beside them).  The outputs that see a kept element which is not finite, or not zero and
+ *   outside 2^-50 .. 2^40, come from the FMA kernel, and all of them where there are many such elements or the product is small.
+ *   Distance from 64 bits (2-norm, unit normal operands): 0.8e-7 at 64 indices, 1.5e-7 at 8192, where the FMA kernel has 0.8e-7
+ *   and 4.1e-7.  The tensor cores' sums round toward zero, which operands of one sign show: up to 1.3e-7 (uniform, exponential,
+ *   |Student t|, any number of indices; FMA kernel 0.5e-7 at 64, level at about 1000, 3e-7 at 8192), 5.6e-7 at values spread over
+ *   many powers of two (e^(2 z), z normal; FMA kernel 0.6e-7 to 3.1e-7).
  *   Decode-step shapes (batch 1, M <= 4, bf16, B with contiguous rows; App. "Complexity Analysis", decoding step)
  *   take a gathered GEMV that reads only the kept rows of B (k N 2 bytes) and packs nothing; outputs of up to 256
  *   rows (small decode batches, B with contiguous rows, N > 128) run on the tensor cores with the kept rows of B
  *   fetched by the kernel itself, so W is read once and never copied (up to 32 rows on warp-level products, more on 128-row
- *   tiles).  These forms and the FMA kernel cut the contraction axis where the output alone would leave multiprocessors idle;
- *   the pieces' fp32 sums are what most of their workspace is for.  In a smaller one (sized for another shape) they run with fewer
- *   pieces: what the packed operands would take is enough, for the FMA kernel the header; the order of summation follows. */
+ *   tiles).  These forms, outputs of few tiles of more rows, and the FMA kernel cut the contraction axis where the output alone
+ *   would leave multiprocessors idle; the pieces' fp32 sums are what most of their workspace is for.  In a smaller one (sized for
+ *   another shape) they run with fewer pieces: what the packed operands would take is enough, for fp32 operands the header; the
+ *   order of summation follows.
+ *   With a list, small bf16 products (batch 1, 5 to 64 rows, K <= 2048, N a multiple of 8 and at most 32 columns per
+ *   multiprocessor, rows 16-byte aligned, operands that fit a multiprocessor's shared memory) run in one launch without scratch,
+ *   all of B being read; they ask for the workspace of the forms above all the same. */
 size_t rmm_reduced_gemm_workspace_bytes(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k, const rmm_mat_t *Y);
 int rmm_reduced_gemm(const rmm_mat_t *A, const rmm_mat_t *B, const int32_t *idx, int64_t k, float scale,
                      const rmm_mat_t *Y, void *ws, size_t ws_bytes, void *stream);
@@ -140,7 +153,8 @@ int rmm_reduced_gemm(const rmm_mat_t *A, const rmm_mat_t *B, const int32_t *idx,
  * groups added in fp64 in a fixed order: deterministic, about 1e-7 relative); every other form of the product runs
  * rmm_score on Y afterwards, and so do outputs of up to 256 rows with an index list where cutting the contraction saves more
  * time than that pass takes (elsewhere their contraction is not cut, so Y can differ from rmm_reduced_gemm's in the order of
- * its fp32 sums).  Arguments otherwise as rmm_reduced_gemm. */
+ * its fp32 sums), and small products, unless the workspace only has room for the epilogue's sums.  Arguments otherwise as
+ * rmm_reduced_gemm. */
 size_t rmm_reduced_gemm_scored_workspace_bytes(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k, const rmm_mat_t *Y);
 int rmm_reduced_gemm_scored(const rmm_mat_t *A, const rmm_mat_t *B, const int32_t *idx, int64_t k, float scale,
                             const rmm_mat_t *Y, float *energy_out, void *ws, size_t ws_bytes, void *stream);
@@ -169,7 +183,8 @@ int rmm_reduced_gemm_q8(const rmm_mat_t *A, const rmm_mat_t *B, float b_scale, c
  * Q [B,Hq,Lq,Dh], K,V [B,Hkv,Lk,Dh], O [B,Hq,Lq,Dh] are bf16 with explicit element strides
  * (batch, head, row, 1).  idx_feat int32 [B,Hq,kd] and idx_tok int32 [B,Hq,kt] receive the index sets
  * (either may be NULL).  Up to 16 query rows per head without a mask and with rho_t == 1 (decode steps, heads up to 256 wide) read
- * K and V in place, once per 16 query rows that share a kv head.  Otherwise, with at most 128 kept features and a head_dim of at most 256, S~ and P stay on the SM (heads wider
+ * K and V in place, once per 16 query rows that share a kv head (a cache cut into pieces is added up in order, by a second launch
+ * or, short pieces, by the last block of each job, which counts arrivals in the workspace header).  Otherwise, with at most 128 kept features and a head_dim of at most 256, S~ and P stay on the SM (heads wider
  * than 128 columns in two passes over the columns of V; fused kernel: one pass
  * for rho_t == 1; row normalisers, token scores and a gathered P V pass for rho_t < 1, where the normalised P is
  * what is rounded, scored and multiplied; for rho_t == 1 the bf16 rounding is applied to P times a per-row factor,
@@ -196,15 +211,20 @@ int rmm_reduced_attn(const rmm_attn_desc_t *desc, const void *Q, const void *K, 
 
 /* The whole operation of Sec. 3.2 on device operands: I = TopK of the column norms of A with |I| = k (k == 0:
  * ceil(rho K)), Y = scale * A[:, I] B[I, :].  The result is that of rmm_score_select followed by rmm_reduced_gemm
- * (in the one-launch form below the column energies are summed in a different fixed order, which can move a key by one
- * fp64 rounding before it is rounded to fp32); idx [batch, k] and retained [batch] (or NULL) as there.  For one small bf16 product (batch 1, A with 2368 to
+ * (in the one-launch forms below the column energies are summed in a different fixed order, which can move a key by one
+ * fp64 rounding before it is rounded to fp32); idx [batch, k] and retained [batch] (or NULL, which changes nothing else) as there.
+ * At k = K the list is 0 .. K-1 and nothing is gathered: Y is rmm_reduced_gemm's without a list (for small products with it; the
+ * two can differ in the order of their fp32 sums).  Small products (as there: 5 to 64 rows, K <= 2048) are one launch, in which
+ * every block scores and selects for itself.  For one bf16 product of medium size (batch 1, A with 2368 to
  * 8192 columns and 257 to 8192 rows, B with at most 4096 columns) whose operands meet the tensor-core layout rules (the
  * regime where launch and hand-off latencies weigh most), the scores, the selection
  * and both gathers run in ONE launch (every block owns 64 columns of A, a grid-wide barrier makes all column energies
  * visible, every block then selects and gathers its own kept columns and the matching rows of B), followed by the
  * tensor-core product; this form expects the GPU to itself (all of its blocks must be resident at once; if they are
  * not, the barrier's bounded wait expires and RMM_ERR_TIMEOUT is reported).  Outputs of 5 to 32 rows have their selecting kernel
- * pack A[:, I] as well, where the product fetches the rows of B itself.  Everything else runs as the two calls. */
+ * pack A[:, I] as well, where the product fetches the rows of B itself.  Everything else runs as the two calls.
+ * rmm_product_workspace_bytes is enough for every k.  For fp32 operands the larger of rmm_score_select_workspace_bytes and
+ * rmm_reduced_gemm_workspace_bytes(k) is enough at that k, and usually much less. */
 size_t rmm_product_workspace_bytes(const rmm_mat_t *A, const rmm_mat_t *B, const rmm_mat_t *Y);
 int rmm_product(const rmm_mat_t *A, const rmm_mat_t *B, double rho, int64_t k, float scale, const rmm_mat_t *Y, int32_t *idx,
                 float *retained, void *ws, size_t ws_bytes, void *stream);

@@ -167,7 +167,12 @@ _ws_cache = {}
 
 
 def workspace(nbytes: int, device: torch.device) -> torch.Tensor:
-    """A zero-initialised, cached, growing workspace per device (torch owns the memory)."""
+    """A zero-initialised, cached, growing workspace per device (torch owns the memory).
+
+    Calls that share a workspace must be ordered on one stream.  The cached one is shared by all calls of a device that are not given
+    another, so calls that may overlap (several streams or threads) need a `ws` of their own each: a uint8 CUDA tensor of zeros.
+    Overlapping calls on one workspace spoil each other's scratch, and can leave an arrival counter of its header half way, which
+    spoils later calls as well."""
     index = device.index
     key = (device.type, index if index is not None else torch.cuda.current_device())
     ws = _ws_cache.get(key)

@@ -3,20 +3,27 @@
 // Every operand is written as the sum of three bf16 numbers, a = a1 + a2 + a3 (each the rounding of what the ones before it
 // leave: 24 bits and the signs, so the sum is exact up to 2^-26 of a), and the product of two of them as the six products
 // a1 b1 + a1 b2 + a2 b1 + a2 b2 + a1 b3 + a3 b1; what is left out is below 2^-24 of |a b|.  Products of bf16 numbers are
-// exact in the tensor cores, but their fp32 accumulators round toward zero: 64 indices cost 6.6e-8 of the result (2-norm,
-// normal operands), 1504 of them 1.5e-6, where the FMA pipes with a partial sum per 16 indices give 8.5e-8 and 1.2e-7.  So an
-// accumulator takes 64 indices only, the small products first, and is then added to fp32 registers that round to nearest:
-// the error stays below that of the FMA pipes for every number of indices.
-// The split is exact only for ordinary magnitudes: where a kept element is not finite, or neither zero nor within 2^-50 .. 2^40
-// (so that no product or sum of the parts leaves the normal range), the gather says so, this kernel returns at once, and the
-// FMA kernel behind it, which otherwise returns at once, runs.
+// exact in the tensor cores, but their fp32 accumulators round toward zero: 1504 indices in one cost 1.5e-6 of the result
+// (2-norm, normal operands).  So an accumulator takes 64 indices only, the small products first, and is then added to fp32
+// registers that round to nearest.  Measured against 64 bits (2-norm) at 64, 1500 and 8192 indices, the FMA kernel (a partial sum
+// per 16 indices, one slice) in brackets: normal operands 0.8e-7 1.2e-7 1.5e-7 (0.8e-7 1.9e-7 4.1e-7).  Operands of one sign show
+// the rounding toward zero, a mean of -0.7e-7 to -1.2e-7 that the FMA kernel does not have: uniform 0.8e-7 1.1e-7 1.0e-7 (0.5e-7
+// 1.5e-7 3.0e-7), exponential 1.0e-7 1.2e-7 1.2e-7 (0.5e-7 1.5e-7 3.0e-7), level at about 1000 indices; e^(2 z), z normal, whose
+// largest products hide the others, 5.6e-7 2.9e-7 3.4e-7 (0.8e-7 2.7e-7 3.1e-7).  (A second accumulator, for the products of first
+// parts alone, took 6 % off the uniform figure, nothing off the others, and 15 % more time: the loss is inside an instruction.)
+// The split is exact only for ordinary magnitudes: a kept element that is not finite, or neither zero nor within 2^-50 .. 2^40,
+// is flagged by the gather.  (Within, products of first parts are normal numbers, and what products of later parts lose below
+// 2^-126 is less than 2^-26 of them.)  The FMA kernel behind this one, which otherwise returns at once, does the outputs that see
+// a flag, or all of them where that is cheaper.  777 x 1500 kept x 1500 with one such element 128 us, 117 by the FMA kernel alone.
 //
-// Bound: tensor cores (six bf16 products a multiplication: 270 TFLOP/s at best, where the FMA pipes reach 46), 1.0 us per 64
-// indices of a 256 x 128 tile, of which the copies hide all but 0.2 to 0.4 us.  CTA pairs, since a tensor instruction reads both
+// Bound: tensor cores (six bf16 products a multiplication: 280 TFLOP/s at the burst rate, where the FMA pipes reach 46), 1.1 us per
+// 64 indices of a 256 x 128 tile at that rate.  The tensor pipe is busy for 61 % of 338 us on 2048 x 4096 kept x 4096 (203 TFLOP/s,
+// 1.5 us per 64 indices: the copies and the additions are not all hidden), for 32 % of 41.5 us on 777 x 1500 x 1500 (48 tiles for 74
+// pairs, a quarter of them nine rows high; pieces and their meeting).  CTA pairs, since a tensor instruction reads both
 // its operands from shared memory: 128 bytes a clock for a lone CTA's 128 x 128, all there is, 96 for each CTA of a pair.  Where a
 // round of tiles would leave pairs idle its tiles are cut along the contraction; the pieces meet in whichever pair comes last.
-// Whole calls, FMA kernel before: 777 x 3000 (half kept) x 1500 123 -> 55.6 us, 2048 x 8192 (half) x 4096 1517 -> 406, 500 x 700
-// (three quarters) x 4000 74.5 -> 35.7.
+// Whole calls, FMA kernel before: 777 x 3000 (half kept) x 1500 123 -> 56 us, 2048 x 8192 (half) x 4096 1486 -> 376 (on a given list),
+// 500 x 700 (half) x 4000 48.6 -> 23.2.
 #include <cuda.h>
 
 #include "common.cuh"

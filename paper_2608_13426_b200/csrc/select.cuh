@@ -350,7 +350,8 @@ __device__ __forceinline__ void find_bin8(SelectSmem &sm, int nbins, unsigned re
 // the keys that share the prefix found so far count (a per-thread bit mask of those keys is carried along, and warps
 // without any skip the pass).  With 32 warps on four schedulers every instruction that all warps execute costs eight
 // issue clocks, so the code paths below are kept short rather than general.
-// LIST: keys that share the first digit and are few enough are finished from a list, one to a thread.  For the front end, where
+// LIST: keys that share the first digit are finished from a list, one to a thread, where they are no more than the threads (512 in the
+// front end).  For the front end, where
 // every block selects: 2048 x 8192 x 2048 56.9 -> 56.2 us a call.  In the tail of a score pass, where one block does, the code that it adds
 // is fetched for the first time in each call and costs more than it saves (512 x 8192 x 8192 73.4 -> 75.0).
 template <int ITEMS, int NTHR = 1024, bool LIST = false>
@@ -617,7 +618,8 @@ __device__ void block_select_blocked(const float *__restrict__ keys, int K, int 
 
 // Whole selection of at most 128 keys (attention heads), blockDim.x == 1024: every key is compared with every other one, an eighth of
 // them per thread, and kept if fewer than k come before it (larger, or equal with a lower index).  Four barriers instead of some
-// fifteen for the digits: attention of 8 heads x 700 x 64 30.0 -> 29.1 us a call, 16 heads x 2048 x 128 84.1 -> 83.1; at 256 keys level.
+// fifteen for the digits: the score pass of 2 x 8 heads x 700 x 64 16.7 -> 14.7 us by itself (whole calls of 33 to 36 us vary by more);
+// at 256 keys level.
 static __device__ __noinline__ void block_select_short(const float *__restrict__ keys, int K, int k, int32_t *__restrict__ idx, float *retained, SelectSmem &sm)
 {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, j = tid & 127, part = tid >> 7;

@@ -231,8 +231,12 @@ int launch_small_as(const SmallArgs &a, cudaStream_t stream)
 }  // namespace
 
 // Whole calls through the binding, two launches (up to 32 rows) or three before and one now: 16 x 1024 x 2048 19.3 -> 17.2 us,
-// 24 x 2048 x 512 21.6 -> 17.3, 64 x 512 x 256 22.5 -> 17.1, 64 x 1024 x 2048 22.7 -> 17.3; what is left is the host.  Up to four
-// rows stay with the GEMV, whose sums round to nearest; one round of blocks at most, so that A is fetched once per SM.
+// 24 x 2048 x 512 21.6 -> 17.3, 64 x 512 x 256 22.5 -> 17.1, 64 x 1024 x 2048 22.7 -> 17.3; what is left is the host.  On a given list
+// (rmm_reduced_gemm) 13.5 to 15.8 -> 9.2 to 10.2, and 22 to 25 -> 18 to 19 where the output is scored by a pass of its own (epilogue
+// energies before).  Replayed from a graph, 1292 shapes: 1.0 to 3.3 times as fast on six in seven; slower where few indices of a
+// wide B are kept, since all of its rows are read: at most 16 rows, 256 kept indices or fewer, 1536 columns or more (8 x 1024 (a
+// quarter) x 4096 6.3 -> 7.8 us, 9.6 -> 11.8 for the whole product).  Up to four rows stay with the GEMV, whose sums round to
+// nearest; one round of blocks at most, so that A is fetched once per SM.
 bool small_eligible(const rmm_mat_t *A, const rmm_mat_t *B, const rmm_mat_t *Y)
 {
     auto al16 = [](const void *p) { return reinterpret_cast<uintptr_t>(p) % 16 == 0; };
