@@ -429,7 +429,7 @@ constexpr double kSplitParts = 512.0 * 1024 * 1024;
 bool plan_split(const rmm_mat_t *A, const rmm_mat_t *B, int64_t k, SplitPlan *p)
 {
     const int64_t M = A->rows, N = B->cols, batch = A->batch;
-    if (A->dtype != RMM_F32 || B->dtype != RMM_F32) return false;
+    if (A->dtype != RMM_F32 || B->dtype != RMM_F32 || k > A->cols) return false;
     if ((double)batch * (double)M * (double)N * (double)k < 1.5e8) return false;   // 10 us of the FMA kernel
     if (M > INT32_MAX / 2 || N > INT32_MAX / 2 || A->cols > INT32_MAX / 2 || batch > 65535 / kPlanes || ceil_div(M, 64) > 65535) return false;
     int64_t nb = batch, rows = M, cols = N;

@@ -38,3 +38,7 @@ def test_products_of_the_fma_kernel_do_not_ask_for_parts():
     # few rows: estimates prefer the FMA kernel, whose slices fit in far less than the parts of B
     assert gemm(64, 4096, 4096, 2048) < 6 * 4096 * 2048
     assert gemm(64, 28672, 8192, 14336) < 6 * 8192 * 14336
+
+
+def test_a_kept_count_that_the_call_refuses_asks_for_no_parts():
+    assert gemm(777, 3000, 1500, 10 ** 7) < 64 << 20
