@@ -81,6 +81,7 @@ struct FusedArgs {
     int64_t heads, Lr, Lc;       // rows and columns per head (GATHERED: Lc = kept keys)
     int64_t diag;                // Lk - Lq of the unpacked problem: query i sees key t iff t <= i + diag (causal)
     int kd, Dh, causal;
+    int groups;                  // groups of 128 rows a block owns: 2, or 1 where that keeps more SMs busy (see block_groups)
     int64_t v_off, v_div;        // V batch entry of head h = (h + v_off) / v_div
     __nv_bfloat16 *O;
     int64_t o_sh, o_sr;          // element strides of O: head, row
@@ -255,7 +256,7 @@ fused_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
     pdl_wait();
 
     const int kq = (a.kd + 63) / 64, nv = (a.Dh + 63) / 64;       // 64-column chunks of Q/K and of V
-    const int blocks_r = (int)((a.Lr + kGroups * FM - 1) / (kGroups * FM));
+    const int rows_blk = a.groups * FM, blocks_r = (int)((a.Lr + rows_blk - 1) / rows_blk);
     const int64_t items = a.heads * blocks_r;
     // kept keys (GATHERED) with position <= limit (the same for the whole warp): T is ascending.  The lanes look at 32 places at a
     // time: every item starts with four such searches one after the other, and a memory latency per halving was a fifth of the kernel.
@@ -299,6 +300,7 @@ fused_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
     auto block_range = [&](int64_t head, int64_t r0, int *jb, int *je) {
         int b0, e0, b1, e1;
         tile_range(head, r0, &b0, &e0);
+        if (a.groups == 1) { *jb = b0; *je = e0; return; }
         tile_range(head, r0 + FM, &b1, &e1);
         if (e0 <= b0) { *jb = b1; *je = e1; }
         else if (e1 <= b1) { *jb = b0; *je = e0; }
@@ -347,7 +349,7 @@ fused_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         if (item >= items) return false;
         *head = item % a.heads;
         const int64_t rb = item / a.heads;
-        *r0 = (MODE == MODE_ENERGY ? rb : blocks_r - 1 - rb) * (kGroups * FM);
+        *r0 = (MODE == MODE_ENERGY ? rb : blocks_r - 1 - rb) * rows_blk;
         return true;
     };
     const int64_t rounds = (items + gridDim.x - 1) / gridDim.x;
@@ -373,15 +375,15 @@ fused_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             if (!item_of(n, &head, &r0)) continue;
             int jb, je;
             block_range(head, r0, &jb, &je);
-            Tiles tiles = tiles_of(head, r0, true);
+            Tiles tiles = tiles_of(head, r0, a.groups == 2);
             jb = tiles.next(jb, je);
             if (je <= jb) continue;
             if (lane == 0) {
                 const int vb = (int)((head + a.v_off) / a.v_div);
                 ok = mbar_wait_sleepy(q_empty, (n_item & 1u) ^ 1u, abort_flag, a.status, a.wait_ns);
                 if (ok) {
-                    mbar_arrive_expect_tx(q_full, (uint32_t)(kGroups * kq) * kQChunk);
-                    for (int g = 0; g < kGroups; ++g)
+                    mbar_arrive_expect_tx(q_full, (uint32_t)(a.groups * kq) * kQChunk);
+                    for (int g = 0; g < a.groups; ++g)
                         for (int c = 0; c < kq; ++c)
                             tma_load_3d(base + kOffQ + g * kQTile + c * kQChunk, &map_q, c * 64, (int)(r0 + g * FM), (int)head, q_full);
                     ok = load_kv(&map_k, kq, (int64_t)jb * FN, (int)head);
@@ -448,10 +450,11 @@ fused_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             if (!item_of(n, &head, &r0)) continue;
             int jb, je;
             block_range(head, r0, &jb, &je);
-            Tiles tiles = tiles_of(head, r0, true), own = tiles_of(head, r0 + g * FM, false);
+            Tiles tiles = tiles_of(head, r0, a.groups == 2), own = tiles_of(head, r0 + g * FM, false);
             jb = tiles.next(jb, je);
             if (je <= jb) continue;
-            tile_range(head, r0 + g * FM, &gb, &ge);
+            if (g < a.groups) tile_range(head, r0 + g * FM, &gb, &ge);
+            else gb = ge = 0;   // nothing of the item is this group's: it only hands the ring entries back
             gn = gb = own.next(gb, ge);
             if (!mbar_wait(q_full, n_item & 1u, abort_flag, a.status, a.wait_ns)) { ok = false; break; }
             ok = step_s(jb);
@@ -512,7 +515,7 @@ fused_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             int64_t head, r0;
             if (!item_of(n, &head, &r0)) continue;
             r0 += g * FM;
-            if (r0 >= a.Lr) continue;                  // this group has no rows in the last block
+            if (g >= a.groups || r0 >= a.Lr) continue; // this group has no rows in the block, or none in the last block
             int jb, je;
             tile_range(head, r0, &jb, &je);
             Tiles tiles = tiles_of(head, r0, false);
@@ -822,6 +825,13 @@ fused_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
     if (warp == 1) tmem_dealloc<1>(tmem_base, kTmemCols);
 }
 
+// Groups of 128 rows per block.  Two share every K and V tile and hide each other's waits (3400 clocks a step of 256 x 128), but
+// where blocks of 128 rows do not outnumber the SMs there is nothing to share an SM with: one group alone takes 2330 a step of
+// 128 x 128, and a row block's keys are the serial chain that the launch waits for.  Kernels of 2, 8 and 16 heads x 4096, 2048 and
+// 1000 x 128, causal: 63.8 -> 47.5, 39.2 -> 31.1 and 24.9 -> 20.7 us; the sweeps of the token reduction likewise (8 x 2048: 31.0 / 41.3 /
+// 26.9 -> 24.8 / 33.1 / 20.7).  Beyond one block an SM two groups are ahead for most (8 x 4096 without mask 74 against 95).
+int block_groups(int64_t heads, int64_t rows, int sms) { return heads * ceil_div(rows, FM) <= sms ? 1 : 2; }
+
 template <int MODE, bool MASK = false>
 int launch_mode(const CUtensorMap &mq, const CUtensorMap &mk, const CUtensorMap &mv, const FusedArgs &a, const char *name,
                 cudaStream_t stream)
@@ -832,10 +842,12 @@ int launch_mode(const CUtensorMap &mq, const CUtensorMap &mk, const CUtensorMap 
     int dev = 0, sms = 148;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int64_t items = a.heads * ceil_div(a.Lr, kGroups * FM);
+    FusedArgs args = a;
+    args.groups = block_groups(a.heads, a.Lr, sms);
+    const int64_t items = a.heads * ceil_div(a.Lr, args.groups * FM);
     prof_begin(name, stream);
     cudaError_t e = launch_kernel(kern, dim3((unsigned)(items < sms ? items : sms)), dim3(kFusedThreads), kFusedSmem, stream, 1,
-                                  mq, mk, mv, a);
+                                  mq, mk, mv, args);
     if (e != cudaSuccess) return fail(RMM_ERR_CUDA, "%s: launch: %s", name, cudaGetErrorString(e));
     return check_launch(name, stream);
 }
