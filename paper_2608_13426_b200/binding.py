@@ -1,4 +1,5 @@
-"""Thin ctypes binding of librmm_b200.so: argument marshalling only.
+"""Thin binding of librmm_b200.so: argument marshalling only, by ctypes and, for the plain form of the two calls that
+the host can bound (rmm_product, rmm_reduced_attn), by a small native module (csrc/marshal.c).
 
 Every function has the name of the C entry point it calls (include/rmm.h).  Tensors are torch CUDA
 tensors used as plain device memory; the current torch stream is the launch stream.  Workspaces are
@@ -17,6 +18,7 @@ import torch
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "librmm_b200.so")
+MARSHAL_PATH = os.path.join(_HERE, "rmm_marshal.so")
 
 RMM_OK, RMM_ERR_INVALID_ARG, RMM_ERR_UNSUPPORTED, RMM_ERR_WORKSPACE, RMM_ERR_CUDA, RMM_ERR_TIMEOUT, RMM_ERR_BOUNDS = range(7)
 RMM_BF16, RMM_F32, RMM_F8E4M3 = 0, 1, 2
@@ -146,6 +148,24 @@ def _stream() -> int:
     return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
+_marshal = None
+
+
+def _native():
+    """The native marshalling module, bound to the library and to this module's allocations."""
+    global _marshal
+    if _marshal is None:
+        L = lib()
+        if not os.path.exists(MARSHAL_PATH):
+            raise RuntimeError(f"{MARSHAL_PATH} is missing: build it with `python -m paper_2608_13426_b200.build`")
+        from . import rmm_marshal
+        rmm_marshal.init(L._name, (torch.Tensor, torch.nn.Parameter), (torch.bfloat16, torch.float32, torch.int32),
+                         (torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice, workspace, _check, _out), _ws_cache)
+        rmm_marshal.set_poison(_poison)
+        _marshal = rmm_marshal
+    return _marshal
+
+
 _poison = os.environ.get("RMM_POISON_OUTPUTS", "0") not in ("", "0")
 
 
@@ -154,6 +174,8 @@ def poison_outputs(on: bool) -> None:
     INT32_MIN (indices) before the library is called, so that an element no kernel wrote cannot pass for a result."""
     global _poison
     _poison = bool(on)
+    if _marshal is not None:
+        _marshal.set_poison(_poison)
 
 
 def _out(shape, dtype: torch.dtype, like: torch.Tensor) -> torch.Tensor:
@@ -415,6 +437,10 @@ def rmm_reduced_attn(Q: torch.Tensor, K: torch.Tensor, V: torch.Tensor, causal: 
     """Reduced attention.  Q [B,Hq,Lq,Dh], K,V [B,Hkv,Lk,Dh] bf16 with contiguous last dim; mask (optional): additive
     fp32 CUDA tensor [.., Lq, Lk] with up to four dims, size-1 batch / head / row dims shared, contiguous last dim.
     Returns O [B,Hq,Lq,Dh] bf16, or (O, idx_feat, idx_tok) with want_idx (idx_tok None when rho_t == 1)."""
+    if mask is None and ws is None and not want_idx:
+        done = (_marshal or _native()).attn(Q, K, V, causal, rho_d, rho_t)
+        if done is not None:
+            return done
     for t in (Q, K, V):
         if t.dim() != 4 or t.dtype != torch.bfloat16 or not t.is_cuda or t.stride(3) != 1:
             raise RmmError(RMM_ERR_UNSUPPORTED, "Q, K, V must be 4-D bf16 CUDA tensors with a contiguous last dim")
@@ -469,6 +495,10 @@ def rmm_product(A: torch.Tensor, B: torch.Tensor, rho: float = 0.0, k: int = 0, 
                 out: Optional[torch.Tensor] = None, idx: Optional[torch.Tensor] = None, want_retained: bool = False,
                 ws: Optional[torch.Tensor] = None):
     """RMM_rho(A, B) of Sec. 3.2 on device tensors in one call: (Y, idx) or (Y, idx, retained)."""
+    if out is None and idx is None and ws is None and not want_retained:
+        done = (_marshal or _native()).product(A, B, rho, k, scale)
+        if done is not None:
+            return done
     ma, mb = as_mat(A), as_mat(B)
     kk = int(k) if k > 0 else rmm_keep_count(rho, ma.cols)
     three = A.dim() == 3

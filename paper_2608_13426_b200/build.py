@@ -1,15 +1,18 @@
-"""Build librmm_b200.so in-tree with nvcc for sm_100a (cross-compiles without a GPU)."""
+"""Build librmm_b200.so in-tree with nvcc for sm_100a (cross-compiles without a GPU), and the binding's marshalling module."""
 from __future__ import annotations
 
 import glob
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "librmm_b200.so")
+MARSHAL = os.path.join(HERE, "rmm_marshal.so")
+MARSHAL_SRC = os.path.join(CSRC, "marshal.c")
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -22,10 +25,10 @@ def sources():
 
 
 def stale() -> bool:
-    if not os.path.exists(LIB):
+    if not os.path.exists(LIB) or not os.path.exists(MARSHAL):
         return True
-    t = os.path.getmtime(LIB)
-    deps = sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(ROOT, "include", "*.h"))
+    t = min(os.path.getmtime(LIB), os.path.getmtime(MARSHAL))
+    deps = [MARSHAL_SRC] + sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(ROOT, "include", "*.h"))
     return any(os.path.getmtime(d) > t for d in deps)
 
 
@@ -41,7 +44,14 @@ def build(force: bool = False, verbose: bool = False) -> str:
         cmd.insert(2, "-v")
         print(" ".join(cmd), file=sys.stderr)
     subprocess.run(cmd, check=True)
+    build_marshal()
     return LIB
+
+
+def build_marshal() -> str:
+    subprocess.run([os.environ.get("CC", "gcc"), "-O2", "-Wall", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"],
+                    "-I", os.path.join(ROOT, "include"), "-o", MARSHAL, MARSHAL_SRC], check=True)
+    return MARSHAL
 
 
 if __name__ == "__main__":
