@@ -1,6 +1,6 @@
 // Reduced attention (paper Sec. 3.3) composed from the library's own kernels, one group of query heads
 // at a time:
-//   score + select on Q          -> I per query head              (score_tma_kernel / score_select_kernel)
+//   score + select on Q          -> I per query head              (attn_features_kernel, score_tma_kernel or score_select_kernel)
 //   pack Q[:, I], K_g[:, I]      -> K-major operands              (pack_kernel)
 //   S~ = Q[:, I] K[:, I]^T / sqrt(Dh), fp32                        (reduced_gemm_tc_kernel, K-major B)
 //   P  = bf16(softmax(S~ + causal mask))                            (softmax_rows_kernel)
@@ -274,9 +274,14 @@ int rmm_reduced_attn(const rmm_attn_desc_t *desc, const void *Q, const void *K, 
             // feature scores on Q only, one index set per query head
             rmm_mat_t qm = {const_cast<__nv_bfloat16 *>(q + b * d->q_stride[0] + h0 * d->q_stride[1]), RMM_BF16, hg, d->Lq, d->Dh,
                             d->q_stride[1], d->q_stride[2], 1};
-            ScorePlan sq;
-            if ((rc = plan_score(&qm, 1, &sq)) != RMM_OK) return rc;
-            if ((rc = launch_score_select(&qm, sq, true, p.kd, If, nullptr, nullptr, nullptr, w, st)) != RMM_OK) return rc;
+            if (attn_features_eligible(hg, d->Lq, d->Dh)) {
+                rc = launch_attn_features(static_cast<const __nv_bfloat16 *>(qm.ptr), d->q_stride[1], d->q_stride[2], hg, d->Lq, d->Dh, p.kd, If, st);
+                if (rc != RMM_OK) return rc;
+            } else {
+                ScorePlan sq;
+                if ((rc = plan_score(&qm, 1, &sq)) != RMM_OK) return rc;
+                if ((rc = launch_score_select(&qm, sq, true, p.kd, If, nullptr, nullptr, nullptr, w, st)) != RMM_OK) return rc;
+            }
 
             // Q[:, I_h] and K_{g(h)}[:, I_h]
             PackSpec qk[2];

@@ -285,6 +285,11 @@ int launch_gather_q8_pair(const void *A, int64_t a_rows, int64_t a_pitch, const 
 int launch_gather_q8(bool quantise, const void *src, int64_t rows, int64_t s_row, int64_t K, const int32_t *idx, int64_t k, uint8_t *dst,
                      int64_t ld_dst, float *row_scale, int *status, cudaStream_t stream);
 
+// Kept features of attention heads, from the column energies of Q, in one launch (attn_features.cu).
+bool attn_features_eligible(int64_t heads, int64_t Lq, int64_t Dh);
+int launch_attn_features(const __nv_bfloat16 *q, int64_t q_sh, int64_t q_sr, int64_t heads, int64_t Lq, int64_t Dh, int64_t kd, int32_t *idx,
+                         cudaStream_t stream);
+
 // ---- attention helpers --------------------------------------------------------------------------------
 // Row softmax of fp32 logits S [heads, Lq, ld_s] with optional end-aligned causal mask and optional additive mask
 // (row (h, i) at mask + h m_sh + i m_sr, fp32); writes bf16 P [heads, Lq, ld_p] (columns Lk .. ld_p zeroed).
