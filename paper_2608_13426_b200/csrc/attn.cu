@@ -1,7 +1,7 @@
 // Reduced attention (paper Sec. 3.3) composed from the library's own kernels, one group of query heads
 // at a time:
 //   score + select on Q          -> I per query head              (attn_features_kernel, score_tma_kernel or score_select_kernel)
-//   pack Q[:, I], K_g[:, I]      -> K-major operands              (pack_kernel)
+//   pack Q[:, I], K_g[:, I]      -> K-major operands              (pack_heads_kernel or pack_kernel)
 //   S~ = Q[:, I] K[:, I]^T / sqrt(Dh), fp32                        (reduced_gemm_tc_kernel, K-major B)
 //   P  = bf16(softmax(S~ + causal mask))                            (softmax_rows_kernel)
 //   rho_t < 1: score + select on P -> T; pack P[:, T] and V_g[T, :]; O = P[:, T] V_g[T, :]
@@ -289,7 +289,8 @@ int rmm_reduced_attn(const rmm_attn_desc_t *desc, const void *Q, const void *K, 
                                    If, p.kd, p.kd, Qp, p.ldd);
             qk[1] = pack_cols_spec(kk + b * d->k_stride[0], hg, d->Lk, d->Dh, d->k_stride[1], d->k_stride[2], h0, group, If, p.kd,
                                    p.kd, Kp, p.ldd);
-            if ((rc = launch_pack(qk, 2, status, st)) != RMM_OK) return rc;
+            const bool heads = pack_heads_eligible(d->Dh);
+            if ((rc = heads ? launch_pack_heads(qk, status, st) : launch_pack(qk, 2, status, st)) != RMM_OK) return rc;
 
             if (p.fused) {
                 __nv_bfloat16 *og = o + b * d->o_stride[0] + h0 * d->o_stride[1];
@@ -299,7 +300,7 @@ int rmm_reduced_attn(const rmm_attn_desc_t *desc, const void *Q, const void *K, 
                     rc = launch_fused_attn(Qp, Kp, p.ldd, p.kd, v, d->v_stride[2], d->v_stride[1], d->B * d->Hkv, b * d->Hq + h0, group,
                                            og, d->o_stride[1], d->o_stride[2], hg, d->Lq, d->Lk, d->Dh, d->causal, d->Lk - d->Lq,
                                            nullptr, 0, nullptr, d->mask != nullptr ? &mask : nullptr,
-                                           reinterpret_cast<uint8_t *>(w + p.off_kind), status, st);
+                                           reinterpret_cast<uint8_t *>(w + p.off_kind), heads, status, st);
                     if (rc != RMM_OK) return rc;
                     continue;
                 }
@@ -317,7 +318,7 @@ int rmm_reduced_attn(const rmm_attn_desc_t *desc, const void *Q, const void *K, 
                 if ((rc = launch_pack(kv, 2, status, st)) != RMM_OK) return rc;
                 // sweep 3: O = P[:, T] V[T, :] against the full-row normalisers
                 rc = launch_fused_attn(Qp, KpT, p.ldd, p.kd, Vp, d->Dh, p.kt * d->Dh, hg, 0, 1, og, d->o_stride[1], d->o_stride[2], hg,
-                                       d->Lq, p.kt, d->Dh, d->causal, d->Lk - d->Lq, lse, p.lse_ld, It, nullptr, nullptr, status, st);
+                                       d->Lq, p.kt, d->Dh, d->causal, d->Lk - d->Lq, lse, p.lse_ld, It, nullptr, nullptr, false, status, st);
                 if (rc != RMM_OK) return rc;
                 continue;
             }

@@ -118,13 +118,18 @@ struct MaskTileArgs {
     int causal, vec;   // vec: rows are 16-byte aligned
     uint8_t *kind;
     int64_t kind_rb, kind_ld;
+    int behind_heads;  // pack_heads_kernel is the launch before
 };
 
 __global__ void __launch_bounds__(kMaskThreads) mask_tiles_kernel(const MaskTileArgs a)
 {
     __shared__ int s_seen[kMaskThreads / 32];
     static_assert(kMaskThreads == FM, "a thread per row of the tile");
-    pdl_wait();
+    // pack_heads_kernel started this one after everything before itself was complete, the mask included, and nothing here reads what
+    // it writes: the two run side by side, and this one waits before it ends, so that the next kernel finds both complete (2 x 16
+    // heads x 2048, padded: 81 -> 76.5 us a call).
+    if (a.behind_heads) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    else pdl_wait();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned rb = blockIdx.x / (unsigned)a.kind_ld, tile = blockIdx.x % (unsigned)a.kind_ld;
     const int64_t t0 = (int64_t)tile * FN, r0 = (int64_t)rb * FM, plane = blockIdx.z;
@@ -198,6 +203,7 @@ __global__ void __launch_bounds__(kMaskThreads) mask_tiles_kernel(const MaskTile
         if (__syncthreads_or(lone)) kind = TILE_ADD;
     }
     if (threadIdx.x == 0) a.kind[(plane * a.kind_rb + rb) * a.kind_ld + tile] = (uint8_t)kind;
+    if (a.behind_heads) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 template <int MODE, bool MASK>
@@ -893,7 +899,7 @@ size_t mask_tiles_bytes(const MaskView &m, int64_t seqs, int64_t Lq, int64_t Lk)
 int launch_fused_attn(const __nv_bfloat16 *Qp, const __nv_bfloat16 *Kp, int64_t ldd, int64_t kd, const __nv_bfloat16 *V,
                       int64_t v_ld, int64_t v_sb, int64_t v_batches, int64_t v_off, int64_t v_div, __nv_bfloat16 *O,
                       int64_t o_sh, int64_t o_sr, int64_t heads, int64_t Lq, int64_t Lk, int64_t Dh, int causal, int64_t diag,
-                      const float *lse, int64_t lse_ld, const int32_t *tok, const MaskView *mask, uint8_t *tile_kind,
+                      const float *lse, int64_t lse_ld, const int32_t *tok, const MaskView *mask, uint8_t *tile_kind, bool behind_heads,
                       int *status, cudaStream_t stream)
 {
     CUtensorMap mq, mk, mv;
@@ -902,7 +908,7 @@ int launch_fused_attn(const __nv_bfloat16 *Qp, const __nv_bfloat16 *Kp, int64_t 
     if (mask != nullptr) {
         const int64_t planes = (mask->plane_step > 0 ? heads / mask->seq_heads : 1) * mask->plane_heads;
         if (kind_ld * kind_rb > INT32_MAX || planes > 65535) return fail(RMM_ERR_UNSUPPORTED, "fused_attn: mask too large");
-        MaskTileArgs t = {*mask, Lq, Lk, diag, causal, mask->vec, tile_kind, kind_rb, kind_ld};
+        MaskTileArgs t = {*mask, Lq, Lk, diag, causal, mask->vec, tile_kind, kind_rb, kind_ld, behind_heads ? 1 : 0};
         prof_begin("mask_tiles_kernel", stream);
         launch_kernel(mask_tiles_kernel, dim3((unsigned)(kind_ld * kind_rb), 1, (unsigned)planes), dim3(kMaskThreads), 0, stream, 1, t);
         if ((rc = check_launch("mask_tiles_kernel", stream)) != RMM_OK) return rc;

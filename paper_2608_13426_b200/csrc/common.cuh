@@ -270,6 +270,10 @@ static inline PackSpec pack_rows_spec(const __nv_bfloat16 *src, int64_t batch, i
     PackSpec s = {1, src, dst, idx, batch, 0, K, n, s_batch, s_row, b_off, b_div, idx_stride, k, ld_dst};
     return s;
 }
+// Column gathers of two heads' operands (Q and K of attention): rows of 64, 128 or 256 columns, batch and row strides multiples of
+// 8, in one launch.  Its blocks let the next kernel start only once everything before this one is complete.
+bool pack_heads_eligible(int64_t K);
+int launch_pack_heads(const PackSpec (&specs)[2], int *status, cudaStream_t stream);
 // One launch for one or two gathers.
 int launch_pack(const PackSpec *specs, int n, int *status, cudaStream_t stream);
 
@@ -323,7 +327,8 @@ int launch_decode_attn(const rmm_attn_desc_t *d, int64_t kd, const void *Q, cons
 int launch_fused_attn(const __nv_bfloat16 *Qp, const __nv_bfloat16 *Kp, int64_t ldd, int64_t kd, const __nv_bfloat16 *V,
                       int64_t v_ld, int64_t v_sb, int64_t v_batches, int64_t v_off, int64_t v_div, __nv_bfloat16 *O,
                       int64_t o_sh, int64_t o_sr, int64_t heads, int64_t Lq, int64_t Lk, int64_t Dh, int causal, int64_t diag,
-                      const float *lse, int64_t lse_ld, const int32_t *tok, const MaskView *mask, uint8_t *tile_kind, int *status, cudaStream_t stream);
+                      const float *lse, int64_t lse_ld, const int32_t *tok, const MaskView *mask, uint8_t *tile_kind, bool behind_heads, int *status,
+                      cudaStream_t stream);
 // Two sweeps: lse [heads, lse_ld] (lse_ld a multiple of 64, >= Lq) = negated log2-domain row normalisers of softmax(S~ + mask);
 // energy [heads, Lk] = squared token scores sum_i bf16(P_it)^2.
 int launch_fused_attn_scores(const __nv_bfloat16 *Qp, const __nv_bfloat16 *Kp, int64_t ldd, int64_t kd, int64_t heads,
