@@ -85,19 +85,20 @@ __global__ void __launch_bounds__(kThreadsQ) gather_q8_kernel(const void *__rest
 }
 
 
-// Both gathers of a product as one streaming kernel: one persistent 1024-thread block per SM owns a contiguous range of the
-// rows of A and one of the rows of B, which share the index list.  Rows arrive by bulk asynchronous copies, several at a
+// Both gathers of a product as one streaming kernel: a persistent block (1024 threads, one an SM, or 512 and two) owns a contiguous
+// range of the rows of A and one of the rows of B, which share the index list.  Rows arrive by bulk asynchronous copies, several at a
 // time (up to 8 rows of up to 4096 kept columns; the next ones land while these are worked on), so that the barriers, the
 // wait and the row maxima's meeting are paid per handful of rows: with one 8 KB row at a time they were most of the time.
-// 4096 x 8192 activations and 8192 x 8192 weights, half kept: 33 + 35 us in two launches of a row at a time, 54 us here,
-// 185 MB.
+// 4096 x 8192 activations and 8192 x 8192 weights, half kept: 33 + 35 us in two launches of a row at a time, 54 us by one block an
+// SM, 44 by two (185 MB): a block's steps follow one another (wait, read, meet, convert, write), so a second one fills what they
+// leave idle.
 //
 // Quotients: a code is e4m3(a / s) with the quotient rounded as IEEE division rounds it.  q = a x (1 / s), both roundings
 // to nearest, is within 3 units in the last place of that quotient, so it yields the same code unless it lies that close to
 // a point where codes change: those sit 20 bits below the leading bit for |q| >= 2^-6 (three mantissa bits, ties), and
 // everything smaller is divided.  Divisions are thus taken for a few elements in 10^4.
-constexpr int kThreadsS = 1024;
-constexpr int kUnitsS = 8;                       // (rows at a time) x (groups of 4096 outputs of a row): k <= 8 * 4096
+constexpr int kThreadsS = 1024;                  // one block an SM, or two of half as many threads
+constexpr int kUnitsS = 8;                       // (rows at a time) x (groups of 4 outputs a thread of a row): k <= 8 * 4096
 constexpr int kStreamMaxRowBytes = 110 * 1024;   // two such rows (and their zero pads) fit in shared memory
 constexpr int kStreamStages = 3;
 
@@ -127,8 +128,8 @@ __device__ __forceinline__ uint32_t e4m3_code2(float x0, float x1, float step, f
 }
 
 // One operand's rows of this block.  `stage` and `parity` run on from one operand to the next.
-template <bool QUANT, int G>
-__device__ __forceinline__ bool stream_rows(const StreamQ8 &a, unsigned char *smem, uint64_t *full, int *abort_flag, unsigned (*s_red)[kThreadsS / 32],
+template <bool QUANT, int G, int T>
+__device__ __forceinline__ bool stream_rows(const StreamQ8 &a, unsigned char *smem, uint64_t *full, int *abort_flag, unsigned (*s_red)[T / 32],
                                             const uint32_t (&cb)[2 * G], int &turn)
 {
     using namespace ptx;
@@ -139,7 +140,7 @@ __device__ __forceinline__ bool stream_rows(const StreamQ8 &a, unsigned char *sm
     const int64_t lo = (int64_t)blockIdx.x * a.per_block[W], hi = min(a.rows[W], lo + a.per_block[W]);
     if (lo >= hi) return true;
     // 16 zero bytes after each staged row: where missing indices point
-    for (int i = tid; i < 4 * nst * at_once; i += kThreadsS) reinterpret_cast<uint32_t *>(smem + (size_t)(i >> 2) * pitch + pad)[i & 3] = 0;
+    for (int i = tid; i < 4 * nst * at_once; i += T) reinterpret_cast<uint32_t *>(smem + (size_t)(i >> 2) * pitch + pad)[i & 3] = 0;
     // B's rows land where A's pads and rows were: this thread's own accesses come before the copies (which are another proxy's)
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     __syncthreads();
@@ -212,7 +213,7 @@ __device__ __forceinline__ bool stream_rows(const StreamQ8 &a, unsigned char *sm
             if (q < n) {
                 float step = 1.f, inv = 1.f;
                 if constexpr (QUANT) {
-                    const float amax = __uint_as_float(__reduce_max_sync(0xffffffffu, s_red[q][lane]));
+                    const float amax = __uint_as_float(__reduce_max_sync(0xffffffffu, s_red[q][lane % (T / 32)]));
                     step = amax > 0.f ? __fdiv_rn(amax, 448.f) : 1.f;
                     inv = __frcp_rn(step);
                     if (!(inv < INFINITY) || !(amax < INFINITY)) inv = 0.f;  // every quotient then counts as small: divided
@@ -234,7 +235,7 @@ __device__ __forceinline__ bool stream_rows(const StreamQ8 &a, unsigned char *sm
                     mine = (rr & 1) ? __byte_perm(mine, other, 0x3715) : __byte_perm(mine, other, 0x6240);
                     other = __shfl_xor_sync(0xffffffffu, mine, 2);
                     mine = (rr & 2) ? __byte_perm(mine, other, 0x3276) : __byte_perm(mine, other, 0x5410);
-                    const int w = (g * (kThreadsS / 32) + warp) * 32 + word_in_warp;
+                    const int w = (g * (T / 32) + warp) * 32 + word_in_warp;
                     if (w < words) drow[w] = mine;
                 }
             }
@@ -253,14 +254,14 @@ __device__ __forceinline__ bool stream_rows(const StreamQ8 &a, unsigned char *sm
 // four lanes per bank).  The four bytes of an output word then sit in the four lanes of a quad and are brought together by
 // two shuffle rounds; the warp's 32 words leave as one 128-byte store.  Column numbers (the zero pad: K rounded up to 16)
 // stay in registers for all rows, two to a register.
-template <int G>
-__global__ void __launch_bounds__(kThreadsS, 1) gather_q8_stream_kernel(const __grid_constant__ StreamQ8 a)
+template <int G, int T>
+__global__ void __launch_bounds__(T, kThreadsS / T) gather_q8_stream_kernel(const __grid_constant__ StreamQ8 a)
 {
     using namespace ptx;
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ uint64_t full[kStreamStages];
     __shared__ int abort_flag;
-    __shared__ unsigned s_red[kUnitsS / G][kThreadsS / 32];
+    __shared__ unsigned s_red[kUnitsS / G][T / 32];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (tid == 0) {
         for (int b = 0; b < kStreamStages; ++b) mbar_init(smem_u32(&full[b]), 1);
@@ -272,7 +273,7 @@ __global__ void __launch_bounds__(kThreadsS, 1) gather_q8_stream_kernel(const __
     uint32_t cb[2 * G];
 #pragma unroll
     for (int sl = 0; sl < 4 * G; ++sl) {
-        const int j = ((sl >> 2) * (kThreadsS / 32) + warp) * 128 + 32 * (sl & 3) + lane;
+        const int j = ((sl >> 2) * (T / 32) + warp) * 128 + 32 * (sl & 3) + lane;
         // Positions past the row's end are not written; they stand for the first output once more, whose quotient costs what
         // any other does (a zero's would be divided: 4096 x 4096 activations, 3072 kept, 4096 columns 97 us, 84 this way).
         uint32_t col = (uint32_t)(a.K + 15) / 16 * 16;
@@ -285,9 +286,9 @@ __global__ void __launch_bounds__(kThreadsS, 1) gather_q8_stream_kernel(const __
         else cb[sl >> 1] = col;
     }
     int turn = 0;
-    if (stream_rows<true, G>(a, smem, full, &abort_flag, s_red, cb, turn)) {
+    if (stream_rows<true, G, T>(a, smem, full, &abort_flag, s_red, cb, turn)) {
         __syncthreads();
-        stream_rows<false, G>(a, smem, full, &abort_flag, s_red, cb, turn);
+        stream_rows<false, G, T>(a, smem, full, &abort_flag, s_red, cb, turn);
     }
 }
 
@@ -315,12 +316,19 @@ int launch_gather_q8_pair(const void *A, int64_t a_rows, int64_t a_pitch, const 
     a.status = status;
     a.wait_ns = wait_limit_ns();
     a.withhold = debug_withhold() == WITHHOLD_QUANT;
-    const int g = (int)ceil_div(ld_dst, 4096);
+    // Two blocks an SM where three rows of A fit in half of the shared memory (by events, one block and two: 4096 x 8192 half kept with
+    // 8192 columns 53.6 and 44.0 us, 16000 x 14336 a quarter with 4096 137.6 and 115.1, 2000 x 17920 four fifths with 8192 93 and 86.4,
+    // 300 x 4096 three quarters with 4096 23.0 and 19.4, 500 x 5120 half with 5120 23.4 and 22.0); with two buffers instead of three
+    // rows would land no sooner than they are worked on.
+    const size_t row_a = (size_t)(K + 15) / 16 * 32 + 16, whole = 2 * (size_t)(kStreamMaxRowBytes + 16), halved = 108 * 1024;
+    const bool two = kStreamStages * row_a <= halved && ld_dst <= kThreadsS / 2 * 4 * kUnitsS;
+    const int threads = two ? kThreadsS / 2 : kThreadsS, g = (int)ceil_div(ld_dst, (int64_t)threads * 4);
+    const size_t room = two ? halved : whole;
     int64_t blocks = 0;
     size_t smem = 0;
     for (int w = 0; w < 2; ++w) {
-        const size_t pitch = (size_t)(K + 15) / 16 * 16 * (w == 0 ? 2 : 1) + 16, room = 2 * (size_t)(kStreamMaxRowBytes + 16);
-        a.per_block[w] = ceil_div(a.rows[w], sm_count());
+        const size_t pitch = (size_t)(K + 15) / 16 * 16 * (w == 0 ? 2 : 1) + 16;
+        a.per_block[w] = ceil_div(a.rows[w], (int64_t)sm_count() * (two ? 2 : 1));
         // as many rows at a time as the registers hold, three buffers of them where they fit, no more than a block has
         int64_t n = kUnitsS / g;
         while (n > 1 && (kStreamStages * n * pitch > room || n > a.per_block[w])) n /= 2;
@@ -330,15 +338,18 @@ int launch_gather_q8_pair(const void *A, int64_t a_rows, int64_t a_pitch, const 
         const int64_t nb = ceil_div(a.rows[w], a.per_block[w]);
         if (nb > blocks) blocks = nb;
     }
-    static void (*const kernels[kUnitsS])(StreamQ8) = {gather_q8_stream_kernel<1>, gather_q8_stream_kernel<2>, gather_q8_stream_kernel<3>,
-                                                       gather_q8_stream_kernel<4>, gather_q8_stream_kernel<5>, gather_q8_stream_kernel<6>,
-                                                       gather_q8_stream_kernel<7>, gather_q8_stream_kernel<8>};
-    auto kern = kernels[g - 1];
-    static PerDeviceOnce configured[kUnitsS];
-    if (cudaError_t e = configured[g - 1].smem(2 * (kStreamMaxRowBytes + 16), kern))
+    using Kernel = void (*)(StreamQ8);
+    static const Kernel kernels[2][kUnitsS] = {
+        {gather_q8_stream_kernel<1, 1024>, gather_q8_stream_kernel<2, 1024>, gather_q8_stream_kernel<3, 1024>, gather_q8_stream_kernel<4, 1024>,
+         gather_q8_stream_kernel<5, 1024>, gather_q8_stream_kernel<6, 1024>, gather_q8_stream_kernel<7, 1024>, gather_q8_stream_kernel<8, 1024>},
+        {gather_q8_stream_kernel<1, 512>, gather_q8_stream_kernel<2, 512>, gather_q8_stream_kernel<3, 512>, gather_q8_stream_kernel<4, 512>,
+         gather_q8_stream_kernel<5, 512>, gather_q8_stream_kernel<6, 512>, gather_q8_stream_kernel<7, 512>, gather_q8_stream_kernel<8, 512>}};
+    auto kern = kernels[two][g - 1];
+    static PerDeviceOnce configured[2][kUnitsS];
+    if (cudaError_t e = configured[two][g - 1].smem((int)room, kern))
         return fail(RMM_ERR_CUDA, "gather_q8: cudaFuncSetAttribute: %s", cudaGetErrorString(e));
     prof_begin("gather_q8_stream_kernel", stream);
-    launch_kernel(kern, dim3((unsigned)blocks), dim3(kThreadsS), smem, stream, 1, a);
+    launch_kernel(kern, dim3((unsigned)blocks), dim3(threads), smem, stream, 1, a);
     return check_launch("gather_q8_stream_kernel", stream);
 }
 
