@@ -206,12 +206,34 @@ __global__ void __launch_bounds__(kMaskThreads) mask_tiles_kernel(const MaskTile
     if (a.behind_heads) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
+// 2^x of two numbers on the FMA and integer pipes: x = n + f with f in [-1/2, 1/2] (adding 1.5 x 2^23 rounds to the integer n), a
+// polynomial of degree 5 for 2^f (fitted for the smallest largest relative error: 9.1e-8, 1.6e-7 as evaluated, where the
+// special-function unit has 2^-22) and 2^n put together in the exponent.  Below -127: 0; NaN stays NaN.
+__device__ __forceinline__ void ex2_fma(float x0, float x1, float &p0, float &p1)
+{
+    const uint64_t magic = pack2(12582912.f, 12582912.f), minus = pack2(-1.f, -1.f);
+    asm("max.NaN.f32 %0, %0, 0fC2FE0000;" : "+f"(x0));
+    asm("max.NaN.f32 %0, %0, 0fC2FE0000;" : "+f"(x1));
+    const uint64_t x = pack2(x0, x1), n = fadd2(x, magic), f = fadd2(x, ffma2(n, minus, magic));
+    uint64_t p = ffma2(pack2(0.001326472731307149f, 0.001326472731307149f), f, pack2(0.009671512991189957f, 0.009671512991189957f));
+    p = ffma2(p, f, pack2(0.05550733581185341f, 0.05550733581185341f));
+    p = ffma2(p, f, pack2(0.24022242426872253f, 0.24022242426872253f));
+    p = ffma2(p, f, pack2(0.6931470036506653f, 0.6931470036506653f));
+    p = ffma2(p, f, pack2(1.f, 1.f));
+    float n0, n1, q0, q1;
+    unpack2(n, n0, n1);
+    unpack2(p, q0, q1);
+    p0 = q0 * __uint_as_float((__float_as_uint(n0) << 23) + 0x3f800000u);
+    p1 = q1 * __uint_as_float((__float_as_uint(n1) << 23) + 0x3f800000u);
+}
+
 template <int MODE, bool MASK>
 __global__ void __launch_bounds__(kFusedThreads, 1)
 fused_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
-                  const __grid_constant__ CUtensorMap map_v, FusedArgs a)
+                  const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_o, FusedArgs a)
 {
     constexpr bool kHasV = MODE == MODE_FULL || MODE == MODE_GATHERED;  // P tiles, P V products and an O accumulator
+    constexpr bool kTileStore = MODE == MODE_GATHERED;                  // O leaves by tile stores
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     const uint32_t base = smem_u32(smem_raw);
     uint8_t *base_ptr = smem_raw;
@@ -237,7 +259,10 @@ fused_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
     if (threadIdx.x == 32) {
         asm volatile("prefetch.tensormap [%0];" ::"l"(&map_q) : "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(&map_k) : "memory");
-        if constexpr (kHasV) asm volatile("prefetch.tensormap [%0];" ::"l"(&map_v) : "memory");
+        if constexpr (kHasV) {
+            asm volatile("prefetch.tensormap [%0];" ::"l"(&map_v) : "memory");
+            if constexpr (kTileStore) asm volatile("prefetch.tensormap [%0];" ::"l"(&map_o) : "memory");
+        }
     }
     if (threadIdx.x == 0) {
         mbar_init(q_full, 1);
@@ -625,7 +650,12 @@ fused_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                     for (int e = 0; e < 32; e += 2) {
                         float x0, x1;
                         unpack2(ffma2(pack2(__uint_as_float(v[e]), __uint_as_float(v[e + 1])), c22, nm2), x0, x1);
-                        const float p0 = ex2(x0), p1 = ex2(x1);
+                        // Every fourth pair on the FMA pipe, where no row maximum of the whole tile is taken: 32 heads x 3001 x 128 (2401
+                        // keys) 82.4 -> 76.2 us, 16 x 8000 (half the features) 176.5 -> 166.4 for the normalisers.  The one-pass form
+                        // gains as many clocks (5 %) and loses them to the clock rate (power); the energies are level.
+                        float p0, p1;
+                        if (MODE != MODE_FULL && (e & 6) == 6) ex2_fma(x0, x1, p0, p1);
+                        else { p0 = ex2(x0); p1 = ex2(x1); }
                         if constexpr (MODE != MODE_GATHERED) (e & 2 ? sum_b : sum_a) = fadd2(e & 2 ? sum_b : sum_a, pack2(p0, p1));
                         if constexpr (kHasV) {
                             __nv_bfloat162 h = __floats2bfloat162_rn(p0, p1);
@@ -648,6 +678,11 @@ fused_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                         *reinterpret_cast<uint4 *>(prow + chunk * kPChunk + ((u ^ (r & 7)) << 4)) =
                             make_uint4(w[4 * u], w[4 * u + 1], w[4 * u + 2], w[4 * u + 3]);
                 }
+            };
+            // the O rows of the item before have left the P tile
+            [[maybe_unused]] auto o_stored = [&]() {
+                if (lane == 0) bulk_wait_read<0>();
+                __syncwarp();
             };
             // m and l follow a new chunk maximum (log2 domain); returns the factor the sums taken so far have to be scaled by
             auto follow_max = [&](float mc, bool *any_grow) -> float {
@@ -733,6 +768,7 @@ fused_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                     load_chunk(j, 0, v0, v1);
                     emit_chunk(v0, v1, neg_m, w);
                     if (!mbar_wait(p_empty(g), (p_it & 1u) ^ 1u, abort_flag, a.status, a.wait_ns)) { ok = false; break; }
+                    if (j == jb) o_stored();
                     store_chunk(0, w);
                     load_chunk(j, 64, v0, v1);
                     release_s();
@@ -792,14 +828,18 @@ fused_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                 if (!mbar_wait(o_full(g), o_it & 1u, abort_flag, a.status, a.wait_ns)) { ok = false; break; }
                 tc_fence_after();
                 const float inv_l = MODE == MODE_GATHERED ? 1.f : (l > 0.f ? 1.f / l : 0.f);
-                for (int c = 0; c < nv * 64; c += 32) {
-                    uint32_t v[32];
-                    tmem_ld32_issue(t_o + c, v);
-                    tmem_ld_wait();
-                    if (i < a.Lr) {
+                if constexpr (kTileStore) {
+                    // The P tile is free (the last P V is complete): the warp's 32 rows go through it, laid out as P is, and leave by a
+                    // tile store, which clips rows and columns past the end: 32 heads x 3001 x 128 (2401 keys) 86.4 -> 82.4 us.  The
+                    // one-pass form, where the maps' set-up and the stores' tail weigh more, keeps direct stores (2 heads x 8192: 90.0
+                    // us a call, 91.7 by tiles; 32 x 4096 level).
+#pragma unroll 1
+                    for (int c = 0; c < nv * 64; c += 32) {
+                        uint32_t v[32];
+                        tmem_ld32_issue(t_o + c, v);
+                        tmem_ld_wait();
 #pragma unroll
                         for (int u = 0; u < 4; ++u) {
-                            if (c + 8 * u >= a.Dh) break;
                             uint32_t ww[4];
 #pragma unroll
                             for (int pp = 0; pp < 4; ++pp) {
@@ -807,16 +847,48 @@ fused_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                                                                          __uint_as_float(v[8 * u + 2 * pp + 1]) * inv_l);
                                 ww[pp] = *reinterpret_cast<uint32_t *>(&h);
                             }
-                            *reinterpret_cast<uint4 *>(orow + c + 8 * u) = make_uint4(ww[0], ww[1], ww[2], ww[3]);
+                            *reinterpret_cast<uint4 *>(prow + (c >> 6) * kPChunk + (((((c >> 3) & 7) + u) ^ (r & 7)) << 4)) = make_uint4(ww[0], ww[1], ww[2], ww[3]);
+                        }
+                    }
+                    fence_proxy_async();
+                } else {
+                    for (int c = 0; c < nv * 64; c += 32) {
+                        uint32_t v[32];
+                        tmem_ld32_issue(t_o + c, v);
+                        tmem_ld_wait();
+                        if (i < a.Lr) {
+#pragma unroll
+                            for (int u = 0; u < 4; ++u) {
+                                if (c + 8 * u >= a.Dh) break;
+                                uint32_t ww[4];
+#pragma unroll
+                                for (int pp = 0; pp < 4; ++pp) {
+                                    __nv_bfloat162 h = __floats2bfloat162_rn(__uint_as_float(v[8 * u + 2 * pp]) * inv_l,
+                                                                             __uint_as_float(v[8 * u + 2 * pp + 1]) * inv_l);
+                                    ww[pp] = *reinterpret_cast<uint32_t *>(&h);
+                                }
+                                *reinterpret_cast<uint4 *>(orow + c + 8 * u) = make_uint4(ww[0], ww[1], ww[2], ww[3]);
+                            }
                         }
                     }
                 }
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(o_empty(g));
+                if (lane == 0) {
+                    mbar_arrive(o_empty(g));
+                    if (kTileStore && r0 + q * 32 < a.Lr) {
+                        for (int c = 0; c < nv; ++c)
+                            tma_store_3d(&map_o, base + kOffP + g * kPTile + c * kPChunk + q * 4096, c * 64, (int)r0 + q * 32, (int)head);
+                        bulk_commit();
+                    }
+                }
                 ++o_it;
             }
             ASTAMP(6);
+        }
+        if constexpr (kTileStore) {
+            if (lane == 0) bulk_wait_read<0>();  // shared memory stays until the stores have read it
+            __syncwarp();
         }
         ASTAMP_FLUSH(8);
     }
@@ -839,7 +911,7 @@ fused_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
 int block_groups(int64_t heads, int64_t rows, int sms) { return heads * ceil_div(rows, FM) <= sms ? 1 : 2; }
 
 template <int MODE, bool MASK = false>
-int launch_mode(const CUtensorMap &mq, const CUtensorMap &mk, const CUtensorMap &mv, const FusedArgs &a, const char *name,
+int launch_mode(const CUtensorMap &mq, const CUtensorMap &mk, const CUtensorMap &mv, const CUtensorMap &mo, const FusedArgs &a, const char *name,
                 cudaStream_t stream)
 {
     auto kern = fused_attn_kernel<MODE, MASK>;
@@ -853,7 +925,7 @@ int launch_mode(const CUtensorMap &mq, const CUtensorMap &mk, const CUtensorMap 
     const int64_t items = a.heads * ceil_div(a.Lr, args.groups * FM);
     prof_begin(name, stream);
     cudaError_t e = launch_kernel(kern, dim3((unsigned)(items < sms ? items : sms)), dim3(kFusedThreads), kFusedSmem, stream, 1,
-                                  mq, mk, mv, args);
+                                  mq, mk, mv, mo, args);
     if (e != cudaSuccess) return fail(RMM_ERR_CUDA, "%s: launch: %s", name, cudaGetErrorString(e));
     return check_launch(name, stream);
 }
@@ -902,7 +974,7 @@ int launch_fused_attn(const __nv_bfloat16 *Qp, const __nv_bfloat16 *Kp, int64_t 
                       const float *lse, int64_t lse_ld, const int32_t *tok, const MaskView *mask, uint8_t *tile_kind, bool behind_heads,
                       int *status, cudaStream_t stream)
 {
-    CUtensorMap mq, mk, mv;
+    CUtensorMap mq, mk, mv, mo;
     int rc;
     const int64_t kind_rb = 2 * ceil_div(Lq, kGroups * FM), kind_ld = ceil_div(Lk, FN * 8) * 8;
     if (mask != nullptr) {
@@ -925,6 +997,14 @@ int launch_fused_attn(const __nv_bfloat16 *Qp, const __nv_bfloat16 *Kp, int64_t 
             const uint32_t box[3] = {64, FN, 1};
             if ((rc = make_map(&mv, const_cast<__nv_bfloat16 *>(V + c0), 3, dims, st, box, true)) != RMM_OK) return rc;
         }
+        if (tok == nullptr) {
+            mo = mq;  // (O leaves without a tensor map)
+        } else {
+            uint64_t dims[3] = {(uint64_t)dh, (uint64_t)Lq, (uint64_t)heads};
+            uint64_t st[2] = {(uint64_t)o_sr * 2, heads > 1 ? (uint64_t)o_sh * 2 : (uint64_t)o_sr * 2 * (uint64_t)Lq};
+            const uint32_t box[3] = {64, 32, 1};  // a warp's rows of a 64-column chunk
+            if ((rc = make_map(&mo, O + c0, 3, dims, st, box, true)) != RMM_OK) return rc;
+        }
         FusedArgs a = {};
         a.heads = heads; a.Lr = Lq; a.Lc = Lk; a.diag = diag;
         a.kd = (int)kd; a.Dh = (int)dh; a.causal = causal;
@@ -936,12 +1016,12 @@ int launch_fused_attn(const __nv_bfloat16 *Qp, const __nv_bfloat16 *Kp, int64_t 
         a.wait_ns = wait_limit_ns();
         a.withhold = debug_withhold() == WITHHOLD_ATTN;
         if (tok != nullptr) {
-            rc = launch_mode<MODE_GATHERED>(mq, mk, mv, a, "fused_attn_gathered_kernel", stream);
+            rc = launch_mode<MODE_GATHERED>(mq, mk, mv, mo, a, "fused_attn_gathered_kernel", stream);
         } else if (mask != nullptr) {
             a.mask = *mask; a.tile_kind = tile_kind; a.kind_rb = kind_rb; a.kind_ld = kind_ld;
-            rc = launch_mode<MODE_FULL, true>(mq, mk, mv, a, "fused_attn_masked_kernel", stream);
+            rc = launch_mode<MODE_FULL, true>(mq, mk, mv, mo, a, "fused_attn_masked_kernel", stream);
         } else {
-            rc = launch_mode<MODE_FULL>(mq, mk, mv, a, "fused_attn_kernel", stream);
+            rc = launch_mode<MODE_FULL>(mq, mk, mv, mo, a, "fused_attn_kernel", stream);
         }
         if (rc != RMM_OK) return rc;
     }
@@ -970,12 +1050,12 @@ int launch_fused_attn_scores(const __nv_bfloat16 *Qp, const __nv_bfloat16 *Kp, i
     if ((rc = packed_map(&mq, Qp, kd, Lq, heads, ldd, FM)) != RMM_OK) return rc;
     if ((rc = packed_map(&mk, Kp, kd, Lk, heads, ldd, FN)) != RMM_OK) return rc;
     a.Lr = Lq; a.Lc = Lk;
-    if ((rc = launch_mode<MODE_STATS>(mq, mk, mk, a, "fused_attn_stats_kernel", stream)) != RMM_OK) return rc;
+    if ((rc = launch_mode<MODE_STATS>(mq, mk, mk, mk, a, "fused_attn_stats_kernel", stream)) != RMM_OK) return rc;
     // sweep 2: rows = keys, tiles of queries stream past
     if ((rc = packed_map(&mq, Kp, kd, Lk, heads, ldd, FM)) != RMM_OK) return rc;
     if ((rc = packed_map(&mk, Qp, kd, Lq, heads, ldd, FN)) != RMM_OK) return rc;
     a.Lr = Lk; a.Lc = Lq;
-    return launch_mode<MODE_ENERGY>(mq, mk, mk, a, "fused_attn_energy_kernel", stream);
+    return launch_mode<MODE_ENERGY>(mq, mk, mk, mk, a, "fused_attn_energy_kernel", stream);
 }
 
 }  // namespace rmm
