@@ -64,7 +64,6 @@ struct TcArgs {
     int *status;
     unsigned long long wait_ns;  // bound of every device-side wait
     int withhold;                // test switch: the producer skips its very first stage, so that the waits behind it expire
-    int sync_kb;                 // the producers also meet every sync_kb k-blocks inside a tile (0: at tile starts only)
     unsigned *wave_ctr;          // [2] in the workspace header (arrivals, exits) or NULL: keeps the blocks of a wave in step
     float *col_energy;           // [batch, ceil(M / 32), N] or NULL: sum of squares of the rounded outputs per 32-row group
     const float *row_scale;      // 8-bit operands: [batch, M] factor of every output row, or NULL
@@ -227,7 +226,6 @@ reduced_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
             int64_t bb = (b + a.b_batch_off) / a.b_batch_div;
             if (bb >= a.b_batches) bb = a.b_batches - 1;
             for (int kb = kb0; kb < kb1; ++kb) {
-                if (meeting && a.sync_kb > 0 && kb > 0 && kb % a.sync_kb == 0) meet();
                 if (!mbar_wait_lane(empty_bar(s), ph ^ 1u, abort_flag, a.status, a.wait_ns)) { ok = false; break; }
                 if (a.withhold && blockIdx.x == 0 && n == 0 && kb == 0) {
                     // (test switch) this stage is never requested: its barrier stays incomplete
@@ -864,12 +862,14 @@ int launch_gemm_tc_problem(const TcProblem &p, cudaStream_t stream)
     a.wait_ns = wait_limit_ns();
     a.withhold = debug_withhold() == WITHHOLD_GEMM;
     {
-        // wave synchronisation: products with several waves of long tiles (measurement switch RMM_GEMM_WAVE_SYNC=0|1)
+        // Wave synchronisation: products with several waves of long tiles.  It keeps DRAM traffic (and with it power, so the clock)
+        // down where operands are far larger than L2 and contractions long, and costs a meeting a tile.  In loops of half a second at
+        // the power cap, without and with: 1531 x 4096 x 14336 151.3 and 154.6 us, 3144 x 4800 x 19776 503.6 and 508.7, 32768 x 4096 x 8192
+        // 1683 and 1699; 8192 x 8192 x 8192 882 and 879, 32768 x 14336 x 8192 6122 and 5987, 2048 x 28672 x 8192 825 and 811.  Meeting
+        // again every 128 k-blocks inside a tile, 32768 x 14336 x 8192 takes 6102.  (Measurement switch RMM_GEMM_WAVE_SYNC=0|1.)
         static const int forced_sync = []() { const char *e = getenv("RMM_GEMM_WAVE_SYNC"); return e ? atoi(e) : -1; }();
         const int64_t tiles = (int64_t)a.batch * a.tiles_m * a.tiles_n, per_wave = sm_count() / ctas;
-        const bool want = p.b_idx == nullptr && (forced_sync >= 0 ? forced_sync != 0 : (tiles > per_wave && p.k * es >= 8192));
-        static const int sync_kb = []() { const char *e = getenv("RMM_GEMM_SYNC_KB"); return e ? atoi(e) : 128; }();
-        a.sync_kb = sync_kb;
+        const bool want = p.b_idx == nullptr && (forced_sync >= 0 ? forced_sync != 0 : (tiles > per_wave && p.k * es >= 16384));
         a.wave_ctr = (want && p.status != nullptr)
                          ? &reinterpret_cast<WsHeader *>(reinterpret_cast<char *>(p.status) - offsetof(WsHeader, status))->counters[kHeaderCounters - 4]
                          : nullptr;
