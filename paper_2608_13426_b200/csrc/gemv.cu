@@ -12,7 +12,7 @@
 namespace rmm {
 namespace {
 
-constexpr int kGemvThreads = 256, kGemvCols = 256, kChunk = 256;
+constexpr int kGemvThreads = 256, kGemvCols = 256;
 
 struct GemvArgs {
     const __nv_bfloat16 *x, *w;
@@ -29,6 +29,11 @@ struct GemvArgs {
 template <int MB>
 __global__ void __launch_bounds__(kGemvThreads) reduced_gemv_kernel(GemvArgs a)
 {
+    // Rows staged at a time: a block's whole slice for most shapes.  (By 256, every refill cost two dependent latencies, the row numbers'
+    // and the activations'.  1 x 8192 half kept x 28672 50.0 -> 48.8 us a call, 2 x 16000 x 8576 54.1 -> 52.4, 2 x 28672 three quarters x
+    // 28672 279 -> 271, 4 rows 57.5 -> 57.1; sixteen rows of W in flight a warp instead of eight, or the next eight requested before
+    // these are used: 57 and 61 for the first, registers cost blocks.)
+    constexpr int kChunk = MB <= 2 ? 1024 : 512;
     extern __shared__ __align__(16) float s_red[];  // [8 warps][MB][256]
     __shared__ float s_x[MB][kChunk];
     __shared__ int s_row[kChunk];
@@ -49,16 +54,26 @@ __global__ void __launch_bounds__(kGemvThreads) reduced_gemv_kernel(GemvArgs a)
     for (int64_t c0 = r_begin; c0 < r_end; c0 += kChunk) {
         const int rows = (int)min((int64_t)kChunk, r_end - c0);
         __syncthreads();
-        if (tid < rows) {
-            int j = a.idx != nullptr ? __ldg(a.idx + c0 + tid) : (int)(c0 + tid);
-            if (j < 0 || j >= a.K) {
-                atomicExch(a.status, (int)RMM_ERR_BOUNDS);
-                j = -1;
-            }
-            s_row[tid] = j;
+        int js[kChunk / kGemvThreads];
 #pragma unroll
-            for (int m = 0; m < MB; ++m)
-                s_x[m][tid] = (j >= 0 && m < a.M) ? __bfloat162float(a.x[(int64_t)m * a.x_sr + j]) : 0.f;
+        for (int i = 0; i < kChunk / kGemvThreads; ++i) {
+            const int r = tid + i * kGemvThreads;
+            js[i] = r < rows ? (a.idx != nullptr ? __ldg(a.idx + c0 + r) : (int)(c0 + r)) : 0;
+        }
+#pragma unroll
+        for (int i = 0; i < kChunk / kGemvThreads; ++i) {
+            const int r = tid + i * kGemvThreads;
+            if (r < rows) {
+                int j = js[i];
+                if (j < 0 || j >= a.K) {
+                    atomicExch(a.status, (int)RMM_ERR_BOUNDS);
+                    j = -1;
+                }
+                s_row[r] = j;
+#pragma unroll
+                for (int m = 0; m < MB; ++m)
+                    s_x[m][r] = (j >= 0 && m < a.M) ? __bfloat162float(a.x[(int64_t)m * a.x_sr + j]) : 0.f;
+            }
         }
         __syncthreads();
         constexpr int U = MB <= 2 ? 8 : 4;  // rows of W in flight per warp
