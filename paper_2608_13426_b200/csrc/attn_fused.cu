@@ -907,8 +907,35 @@ fused_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
 // where blocks of 128 rows do not outnumber the SMs there is nothing to share an SM with: one group alone takes 2330 a step of
 // 128 x 128, and a row block's keys are the serial chain that the launch waits for.  Kernels of 2, 8 and 16 heads x 4096, 2048 and
 // 1000 x 128, causal: 63.8 -> 47.5, 39.2 -> 31.1 and 24.9 -> 20.7 us; the sweeps of the token reduction likewise (8 x 2048: 31.0 / 41.3 /
-// 26.9 -> 24.8 / 33.1 / 20.7).  Beyond one block an SM two groups are ahead for most (8 x 4096 without mask 74 against 95).
-int block_groups(int64_t heads, int64_t rows, int sms) { return heads * ceil_div(rows, FM) <= sms ? 1 : 2; }
+// 26.9 -> 24.8 / 33.1 / 20.7).
+// In up to two rounds a causal block's short rows follow another's long ones (item_of), so one group still wins where the longest
+// sum of a pair is not much longer than the longest item: 8 x 4096 67.9 -> 51.5, 16 x 2048 39.3 -> 33.0, 8 x 3001 51.6 -> 39.2, the
+// normalisers and energies of 8 x 4096 51.5 / 76.1 -> 41.3 / 57.6; 32 x 1100, items of nine tiles at most, 37.0 us a call by two and
+// 38.9 by one; without a mask 8 x 4096 takes 74 by two and 95 by one.  Where the
+// number of tiles is not the rows' (an additive mask, kept keys) only the first rule holds (8 x 4096, padded: 55.7 and 61.7).
+template <int MODE, bool MASK>
+int block_groups(const FusedArgs &a, int64_t sms)
+{
+    const int64_t blocks = ceil_div(a.Lr, FM), items = a.heads * blocks;
+    if (items <= sms) return 1;
+    if (MASK || MODE == MODE_GATHERED || !a.causal || items > 2 * sms) return 2;
+    auto tiles = [&](int64_t rank) -> int64_t {  // of the item of this rank in the order of item_of
+        const int64_t r0 = (MODE == MODE_ENERGY ? rank / a.heads : blocks - 1 - rank / a.heads) * FM;
+        if (MODE == MODE_ENERGY) {
+            const int64_t first = r0 > a.diag ? r0 - a.diag : 0;
+            return first >= a.Lc ? 0 : ceil_div(a.Lc, FN) - first / FN;
+        }
+        const int64_t last = a.Lc - 1 < r0 + FM - 1 + a.diag ? a.Lc - 1 : r0 + FM - 1 + a.diag;
+        return last < 0 ? 0 : last / FN + 1;
+    };
+    constexpr double kItem = 7000.0;  // set-up and epilogue
+    double one = kItem + 2330.0 * (double)tiles(0);
+    for (int64_t pair : {2 * sms - items, sms - 1}) {  // an SM's second item: the ranks of a pair add up to 2 sms - 1
+        const double both = 2.0 * kItem + 2330.0 * (double)(tiles(pair) + tiles(2 * sms - 1 - pair));
+        if (both > one) one = both;
+    }
+    return one < 0.95 * (kItem + 3400.0 * (double)tiles(0)) ? 1 : 2;
+}
 
 template <int MODE, bool MASK = false>
 int launch_mode(const CUtensorMap &mq, const CUtensorMap &mk, const CUtensorMap &mv, const CUtensorMap &mo, const FusedArgs &a, const char *name,
@@ -921,7 +948,7 @@ int launch_mode(const CUtensorMap &mq, const CUtensorMap &mk, const CUtensorMap 
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     FusedArgs args = a;
-    args.groups = block_groups(a.heads, a.Lr, sms);
+    args.groups = block_groups<MODE, MASK>(a, sms);
     const int64_t items = a.heads * ceil_div(a.Lr, args.groups * FM);
     prof_begin(name, stream);
     cudaError_t e = launch_kernel(kern, dim3((unsigned)(items < sms ? items : sms)), dim3(kFusedThreads), kFusedSmem, stream, 1,

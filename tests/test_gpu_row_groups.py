@@ -17,6 +17,9 @@ pytestmark = pytest.mark.gpu
     (2, 4, 2, 17, 300, 128, False),      # one short block a head
     (1, 4, 4, 500, 260, 128, True),      # rows that see nothing
     (1, 2, 1, 900, 900, 256, False),     # two passes over the columns
+    (1, 50, 25, 500, 500, 64, True),     # 200 blocks of 128 rows: two rounds of one group
+    (1, 60, 20, 300, 700, 64, True),     # 180, all of them long: two groups
+    (2, 50, 50, 140, 100, 64, True),     # 200, rows that see nothing among them
 ])
 def test_one_and_two_groups(oracle, B, Hq, Hkv, Lq, Lk, Dh, causal, rho_t, masked):
     mask = padded(B, Lq, Lk, [Lk, 128][:B] if B > 1 else [Lk - 30]) if masked else None
