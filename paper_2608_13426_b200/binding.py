@@ -160,7 +160,7 @@ def _native():
             raise RuntimeError(f"{MARSHAL_PATH} is missing: build it with `python -m paper_2608_13426_b200.build`")
         from . import rmm_marshal
         rmm_marshal.init(L._name, (torch.Tensor, torch.nn.Parameter), (torch.bfloat16, torch.float32, torch.int32),
-                         (torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice, workspace, _check, _out), _ws_cache)
+                         (torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice), globals())
         rmm_marshal.set_poison(_poison)
         _marshal = rmm_marshal
     return _marshal

@@ -13,8 +13,8 @@
 
 static PyTypeObject *type_tensor, *type_parameter;
 static PyObject *dt_bf16, *dt_f32, *dt_i32;
-static PyObject *fn_stream, *fn_device, *fn_workspace, *fn_check, *fn_out, *ws_cache;
-static PyObject *s_is_cuda, *s_dtype, *s_shape, *s_stride, *s_data_ptr, *s_new_empty, *s_get_device, *s_numel, *s_device, *s_cuda, *kw_dtype;
+static PyObject *fn_stream, *fn_device, *names;   /* names: the Python module's, looked up at every call */
+static PyObject *s_is_cuda, *s_dtype, *s_shape, *s_stride, *s_data_ptr, *s_new_empty, *s_get_device, *s_numel, *s_device, *s_cuda, *s_ws_cache, *s_workspace, *s_check, *s_out, *kw_dtype;
 static int poison;
 
 static int (*p_keep_count)(double, int64_t, int64_t *);
@@ -81,6 +81,13 @@ static int read_mat(PyObject *t, rmm_mat_t *m, int *dims)
     return 1;
 }
 
+static PyObject *named(PyObject *name)   /* borrowed */
+{
+    PyObject *v = PyDict_GetItemWithError(names, name);
+    if (v == NULL && !PyErr_Occurred()) PyErr_SetObject(PyExc_NameError, name);
+    return v;
+}
+
 static int number(PyObject *o, double *v)
 {
     if (!PyFloat_CheckExact(o) && !PyLong_CheckExact(o)) return 0;
@@ -99,8 +106,8 @@ static PyObject *new_out(PyObject *like, int dims, const int64_t *size, PyObject
         PyTuple_SET_ITEM(shape, i, v);
     }
     if (poison) {
-        PyObject *args[3] = {shape, dtype, like};
-        t = PyObject_Vectorcall(fn_out, args, 3, NULL);
+        PyObject *args[3] = {shape, dtype, like}, *out = named(s_out);
+        t = out != NULL ? PyObject_Vectorcall(out, args, 3, NULL) : NULL;
     } else {
         PyObject *args[3] = {like, shape, dtype};
         t = PyObject_VectorcallMethod(s_new_empty, args, 2, kw_dtype);
@@ -116,13 +123,15 @@ static PyObject *new_out(PyObject *like, int dims, const int64_t *size, PyObject
 /* The cached workspace of `like`'s device, at least `need` bytes: a new reference, its 256-byte aligned part through *ptr, *bytes */
 static PyObject *workspace_of(PyObject *like, size_t need, void **ptr, size_t *bytes)
 {
-    PyObject *ws = NULL, *v, *key;
+    PyObject *ws = NULL, *v, *key, *cache = named(s_ws_cache), *make = named(s_workspace);
+    if (cache == NULL || make == NULL) return NULL;
+    if (!PyDict_Check(cache)) { PyErr_SetString(PyExc_TypeError, "_ws_cache must be a dict"); return NULL; }
     if (need < RMM_WS_HEADER_BYTES) need = RMM_WS_HEADER_BYTES;
     if ((v = PyObject_CallMethodNoArgs(like, s_get_device)) == NULL) return NULL;
     key = PyTuple_Pack(2, s_cuda, v);
     Py_DECREF(v);
     if (key == NULL) return NULL;
-    ws = PyDict_GetItemWithError(ws_cache, key);
+    ws = PyDict_GetItemWithError(cache, key);
     Py_DECREF(key);
     if (ws == NULL && PyErr_Occurred()) return NULL;
     Py_XINCREF(ws);
@@ -137,7 +146,7 @@ static PyObject *workspace_of(PyObject *like, size_t need, void **ptr, size_t *b
         Py_XDECREF(ws);
         PyObject *dev = PyObject_GetAttr(like, s_device), *n = PyLong_FromSize_t(need);
         PyObject *args[2] = {n, dev};
-        ws = dev != NULL && n != NULL ? PyObject_Vectorcall(fn_workspace, args, 2, NULL) : NULL;
+        ws = dev != NULL && n != NULL ? PyObject_Vectorcall(make, args, 2, NULL) : NULL;
         Py_XDECREF(dev);
         Py_XDECREF(n);
         if (ws == NULL) return NULL;
@@ -170,7 +179,7 @@ static int stream_of(void **stream)
 
 static int raise_status(int rc)   /* the library's text belongs to this thread, as in the Python code */
 {
-    PyObject *n = PyLong_FromLong(rc), *v = n != NULL ? PyObject_CallOneArg(fn_check, n) : NULL;
+    PyObject *n = PyLong_FromLong(rc), *check = named(s_check), *v = n != NULL && check != NULL ? PyObject_CallOneArg(check, n) : NULL;
     Py_XDECREF(n);
     Py_XDECREF(v);
     return v != NULL;
@@ -271,14 +280,14 @@ static PyObject *set_poison(PyObject *self, PyObject *on)
     Py_RETURN_NONE;
 }
 
-/* init(library path, (Tensor, Parameter), (bfloat16, float32, int32), (raw stream, current device, workspace, _check, _out), workspaces) */
+/* init(library path, (Tensor, Parameter), (bfloat16, float32, int32), (raw stream, current device), the module's names) */
 static PyObject *init(PyObject *self, PyObject *args)
 {
     const char *path;
     PyObject *tt, *tp;
     (void)self;
-    if (!PyArg_ParseTuple(args, "s(OO)(OOO)(OOOOO)O!", &path, &tt, &tp, &dt_bf16, &dt_f32, &dt_i32, &fn_stream, &fn_device, &fn_workspace,
-                          &fn_check, &fn_out, &PyDict_Type, &ws_cache))
+    if (!PyArg_ParseTuple(args, "s(OO)(OOO)(OO)O!", &path, &tt, &tp, &dt_bf16, &dt_f32, &dt_i32, &fn_stream, &fn_device, &PyDict_Type,
+                          &names))
         return NULL;
     void *h = dlopen(path, RTLD_NOW);
     if (h == NULL) { PyErr_SetString(PyExc_RuntimeError, dlerror()); return NULL; }
@@ -295,7 +304,7 @@ static PyObject *init(PyObject *self, PyObject *args)
     }
     type_tensor = (PyTypeObject *)tt;
     type_parameter = (PyTypeObject *)tp;
-    PyObject *keep[] = {tt, tp, dt_bf16, dt_f32, dt_i32, fn_stream, fn_device, fn_workspace, fn_check, fn_out, ws_cache};
+    PyObject *keep[] = {tt, tp, dt_bf16, dt_f32, dt_i32, fn_stream, fn_device, names};
     for (size_t i = 0; i < sizeof keep / sizeof *keep; ++i) Py_INCREF(keep[i]);   /* for the life of the process */
     Py_RETURN_NONE;
 }
@@ -311,11 +320,12 @@ static struct PyModuleDef module = {PyModuleDef_HEAD_INIT, "rmm_marshal", NULL, 
 
 PyMODINIT_FUNC PyInit_rmm_marshal(void)
 {
-    struct { PyObject **p; const char *s; } names[] = {
+    struct { PyObject **p; const char *s; } texts[] = {
         {&s_is_cuda, "is_cuda"}, {&s_dtype, "dtype"}, {&s_shape, "shape"}, {&s_stride, "stride"}, {&s_data_ptr, "data_ptr"},
-        {&s_new_empty, "new_empty"}, {&s_get_device, "get_device"}, {&s_numel, "numel"}, {&s_device, "device"}, {&s_cuda, "cuda"}};
-    for (size_t i = 0; i < sizeof names / sizeof *names; ++i)
-        if ((*names[i].p = PyUnicode_InternFromString(names[i].s)) == NULL) return NULL;
+        {&s_new_empty, "new_empty"}, {&s_get_device, "get_device"}, {&s_numel, "numel"}, {&s_device, "device"}, {&s_cuda, "cuda"},
+        {&s_ws_cache, "_ws_cache"}, {&s_workspace, "workspace"}, {&s_check, "_check"}, {&s_out, "_out"}};
+    for (size_t i = 0; i < sizeof texts / sizeof *texts; ++i)
+        if ((*texts[i].p = PyUnicode_InternFromString(texts[i].s)) == NULL) return NULL;
     if ((kw_dtype = PyTuple_Pack(1, s_dtype)) == NULL) return NULL;
     return PyModule_Create(&module);
 }
