@@ -188,7 +188,7 @@ int rmm_reduced_gemm_q8(const rmm_mat_t *A, const rmm_mat_t *B, float b_scale, c
  * than 128 columns in two passes over the columns of V; fused kernel: one pass
  * for rho_t == 1; row normalisers, token scores and a gathered P V pass for rho_t < 1, where the normalised P is
  * what is rounded, scored and multiplied; for rho_t == 1 the bf16 rounding is applied to P times a per-row factor,
- * which changes O by rounding noise only).  Wider heads materialise S~ and P in the workspace one group of heads at a
+ * which changes O by rounding noise only: p up to 2^40, so |V| times the visible keys has to stay below 2^87).  Wider heads materialise S~ and P in the workspace one group of heads at a
  * time.  An evenly strided batch is processed as B * Hq heads in one pass of launches.
  * mask (device, fp32, or NULL): the additive M of Sec. 3.3, entry (b, h, i, t) at mask[b ms[0] + h ms[1] + i ms[2] + t]
  * with ms = mask_stride in elements (0 shares the mask along that axis; rows contiguous); -inf hides a key; a row with

@@ -15,15 +15,16 @@
 // consume the same tiles, so each crosses from L2 to the SM once per 256 rows.  Per tile and group: S~ on the tensor
 // cores (kd of the Dh features; 128 columns of tensor memory, released as soon as the softmax warps hold the tile in
 // registers); one thread per row takes p = 2^(x - m) in two chunks of 64 columns, rounds it once to bf16 and writes it
-// to shared memory as the A operand of O += P V.  In FULL mode m is a reference of the row's own, taken kMargin above the
-// first tile's maximum and renewed (again kMargin above) only when a maximum exceeds it by more than kGrowLimit: p lies
-// between 2^-40 and 2^40 at the row's maximum and row sums below 2^71, far from the bf16 and fp32 range limits, and floating
-// point keeps the same relative precision at any scale.  On renewal l and the O row in tensor
-// memory are multiplied by 2^(m_old - m_new); the epilogue divides by l.  The paper rounds the normalised weight P
+// to shared memory as the A operand of O += P V.  In FULL mode m is the row maximum seen so far, refreshed only when
+// the new maximum exceeds it by more than kGrowLimit: then l and the O row in tensor memory are multiplied by
+// 2^(m_old - m_new); the epilogue divides by l.  The row's largest p thus ends between 1 and 2^40, so that sums of P V are no
+// smaller than V and stay in fp32's range for |V| up to 2^87 / Lk.  (A reference 40 above the maximum saves most of the
+// rescales, 8 us of 132 on 32 heads x 4096 x 128, but hands the small end of V's range to the subnormal numbers: values of
+// 1e-33 came out a few percent off, smaller ones as zero.)  The paper rounds the normalised weight P
 // to bf16; in FULL mode the rounded quantity is p = P * l * 2^(m_row - m), the same weight up to a per-row fp32
 // factor, so O differs by bf16 rounding noise only (nothing is decided from P when rho_t = 1); the modes that score or
 // drop tokens round the normalised P itself.  The row sum takes each tile's largest weight as it was rounded: a row that one
-// key dominates then gets that key's value back whatever the weight's scale (error against 64 bits, see kMargin).
+// key dominates then gets that key's value back whatever the weight's scale.
 // Warp 0 feeds TMA, warps 2-5 and 6-9 are the softmax/epilogue warps of the two groups (every scheduler has two of
 // them to switch between), and one thread of warp 1 and of warp 10 issues the tcgen05.mma of group 0 and 1: a single
 // issuing thread for both groups was the bottleneck.  Every wait is bounded.
@@ -56,12 +57,7 @@ constexpr int kFusedSmem = kOffBar + 512;
 constexpr int kTmemCols = 512;        // per group: S~ (128 columns); then O (128 columns per group)
 constexpr uint32_t kTmemO = kGroups * FN;
 constexpr float kLog2e = 1.4426950408889634f;
-// A renewal waits for the P V product before it and passes the O row through registers, about 1500 clocks of a step of 3400,
-// and the whole group waits for the warp that does it.  With logits of standard deviation 25 (outlier features in Q and K) a
-// group renewed in 30 % of its steps when the reference was the maximum itself, in 0.2 % with the margin: 32 heads x 4096 x
-// 128, half the features, 141 -> 130 us causal and 271 -> 256 without the mask.
-constexpr float kGrowLimit = 40.f;    // log2 of the largest p
-constexpr float kMargin = 40.f;       // and of the inverse of a row's largest p after a renewal
+constexpr float kGrowLimit = 40.f;    // log2 of the largest p taken against a stale maximum
 
 // Debug aid (-DRMM_ATTN_STAMPS): clocks spent per phase by the MMA issuer of group 0 and by one softmax warp of
 // block 0, summed over the launch and read back with rmm_debug_attn_stamps().
@@ -688,10 +684,9 @@ fused_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             auto follow_max = [&](float mc, bool *any_grow) -> float {
                 const bool grow = mc > m + kGrowLimit;
                 *any_grow = __any_sync(0xffffffffu, grow);
-                const float next = MODE == MODE_FULL ? mc + kMargin : mc;
-                const float alpha = (grow && m > -INFINITY) ? ex2(m - next) : 1.f;
+                const float alpha = (grow && m > -INFINITY) ? ex2(m - mc) : 1.f;
                 l *= alpha;
-                if (grow) m = next;
+                if (grow) m = mc;
                 return alpha;
             };
 

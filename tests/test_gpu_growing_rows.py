@@ -1,5 +1,5 @@
 """One-pass attention whose row maxima move from tile to tile: the reference that weights are taken against is renewed, or
-stays up to 2^40 above or below the row's largest weight (attn_fused.cu)."""
+lets them grow to 2^40 (attn_fused.cu), whatever the size of the values that they weigh."""
 import math
 
 import pytest
@@ -11,7 +11,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("peak", [0, 30])        # one key of the highest tile stands out by so much
-@pytest.mark.parametrize("v_scale", [1.0, 1e-20, 1e20])
+@pytest.mark.parametrize("v_scale", [1.0, 1e-20, 1e20, 1e-26, 1e-33])
 @pytest.mark.parametrize("levels", [
     [0, 35, 70, 79],            # within the margin: never renewed
     [0, 79, 81, 160, 162],      # just below and above it
