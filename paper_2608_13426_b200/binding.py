@@ -434,7 +434,7 @@ def rmm_reduced_gemm_q8(A: torch.Tensor, Bq_nk: torch.Tensor, b_scale: float, id
 
 def rmm_reduced_attn(Q: torch.Tensor, K: torch.Tensor, V: torch.Tensor, causal: bool, rho_d: float, rho_t: float = 1.0,
                      want_idx: bool = False, ws: Optional[torch.Tensor] = None, mask: Optional[torch.Tensor] = None):
-    """Reduced attention.  Q [B,Hq,Lq,Dh], K,V [B,Hkv,Lk,Dh] bf16 with contiguous last dim; mask (optional): additive
+    """Reduced attention.  Q [B,Hq,Lq,Dh], K,V [B,Hkv,Lk,Dh] bf16 with contiguous last dim (K gives Hkv and Lk); mask (optional): additive
     fp32 CUDA tensor [.., Lq, Lk] with up to four dims, size-1 batch / head / row dims shared, contiguous last dim.
     Returns O [B,Hq,Lq,Dh] bf16, or (O, idx_feat, idx_tok) with want_idx (idx_tok None when rho_t == 1)."""
     if mask is None and ws is None and not want_idx:
@@ -446,6 +446,9 @@ def rmm_reduced_attn(Q: torch.Tensor, K: torch.Tensor, V: torch.Tensor, causal: 
             raise RmmError(RMM_ERR_UNSUPPORTED, "Q, K, V must be 4-D bf16 CUDA tensors with a contiguous last dim")
     B, Hq, Lq, Dh = Q.shape
     _, Hkv, Lk, _ = K.shape
+    if K.shape[0] < B or K.shape[3] < Dh or any(have < need for have, need in zip(V.shape, (B, Hkv, Lk, Dh))):
+        # (the library sees strides only; a larger K or V is read in part: its first sequences, keys and columns)
+        raise RmmError(RMM_ERR_INVALID_ARG, f"K {tuple(K.shape)} and V {tuple(V.shape)} must hold {(B, Hkv, Lk, Dh)} for Q {tuple(Q.shape)}")
     O = _out((B, Hq, Lq, Dh), torch.bfloat16, Q)
     d = rmm_attn_desc_t(B, Hq, Hkv, Lq, Lk, Dh, int(bool(causal)), float(rho_d), float(rho_t),
                         (ctypes.c_int64 * 3)(*Q.stride()[:3]), (ctypes.c_int64 * 3)(*K.stride()[:3]),

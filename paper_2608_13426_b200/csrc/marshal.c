@@ -246,6 +246,9 @@ static PyObject *attn(PyObject *self, PyObject *const *args, Py_ssize_t n)
     d.B = t[0].shape[0]; d.Hq = t[0].shape[1]; d.Lq = t[0].shape[2]; d.Dh = t[0].shape[3];
     d.Hkv = t[1].shape[1]; d.Lk = t[1].shape[2];
     if (d.B < 1 || d.Hq < 1 || d.Lq < 1 || d.Dh < 1) Py_RETURN_NONE;
+    if (t[1].shape[0] < d.B || t[1].shape[3] < d.Dh || t[2].shape[0] < d.B || t[2].shape[1] < d.Hkv || t[2].shape[2] < d.Lk ||
+        t[2].shape[3] < d.Dh)
+        Py_RETURN_NONE;   /* refused there: the library sees strides only */
     d.causal = args[3] == Py_True;
     for (int i = 0; i < 3; ++i) {
         d.q_stride[i] = t[0].stride[i];
