@@ -12,13 +12,14 @@ from __future__ import annotations
 import ctypes
 import functools
 import os
+import sysconfig
 from typing import Optional, Tuple
 
 import torch
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "librmm_b200.so")
-MARSHAL_PATH = os.path.join(_HERE, "rmm_marshal.so")
+MARSHAL_PATH = os.path.join(_HERE, "rmm_marshal" + sysconfig.get_config_var("EXT_SUFFIX"))  # one interpreter's ABI
 
 RMM_OK, RMM_ERR_INVALID_ARG, RMM_ERR_UNSUPPORTED, RMM_ERR_WORKSPACE, RMM_ERR_CUDA, RMM_ERR_TIMEOUT, RMM_ERR_BOUNDS = range(7)
 RMM_BF16, RMM_F32, RMM_F8E4M3 = 0, 1, 2
@@ -152,12 +153,13 @@ _marshal = None
 
 
 def _native():
-    """The native marshalling module, bound to the library and to this module's allocations."""
+    """The native marshalling module, bound to the library and to this module's allocations; None where it has not been built
+    for this interpreter (the same library calls are then marshalled by ctypes, some 6 us slower)."""
     global _marshal
     if _marshal is None:
         L = lib()
         if not os.path.exists(MARSHAL_PATH):
-            raise RuntimeError(f"{MARSHAL_PATH} is missing: build it with `python -m paper_2608_13426_b200.build`")
+            return None
         from . import rmm_marshal
         rmm_marshal.init(L._name, (torch.Tensor, torch.nn.Parameter), (torch.bfloat16, torch.float32, torch.int32),
                          (torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice), globals())
@@ -437,8 +439,8 @@ def rmm_reduced_attn(Q: torch.Tensor, K: torch.Tensor, V: torch.Tensor, causal: 
     """Reduced attention.  Q [B,Hq,Lq,Dh], K,V [B,Hkv,Lk,Dh] bf16 with contiguous last dim (K gives Hkv and Lk); mask (optional): additive
     fp32 CUDA tensor [.., Lq, Lk] with up to four dims, size-1 batch / head / row dims shared, contiguous last dim.
     Returns O [B,Hq,Lq,Dh] bf16, or (O, idx_feat, idx_tok) with want_idx (idx_tok None when rho_t == 1)."""
-    if mask is None and ws is None and not want_idx:
-        done = (_marshal or _native()).attn(Q, K, V, causal, rho_d, rho_t)
+    if mask is None and ws is None and not want_idx and (native := _marshal or _native()) is not None:
+        done = native.attn(Q, K, V, causal, rho_d, rho_t)
         if done is not None:
             return done
     for t in (Q, K, V):
@@ -498,8 +500,8 @@ def rmm_product(A: torch.Tensor, B: torch.Tensor, rho: float = 0.0, k: int = 0, 
                 out: Optional[torch.Tensor] = None, idx: Optional[torch.Tensor] = None, want_retained: bool = False,
                 ws: Optional[torch.Tensor] = None):
     """RMM_rho(A, B) of Sec. 3.2 on device tensors in one call: (Y, idx) or (Y, idx, retained)."""
-    if out is None and idx is None and ws is None and not want_retained:
-        done = (_marshal or _native()).product(A, B, rho, k, scale)
+    if out is None and idx is None and ws is None and not want_retained and (native := _marshal or _native()) is not None:
+        done = native.product(A, B, rho, k, scale)
         if done is not None:
             return done
     ma, mb = as_mat(A), as_mat(B)

@@ -1,4 +1,7 @@
 """The native marshalling of the plain calls (csrc/marshal.c): what it does not take goes to the Python code, which refuses or runs it."""
+import os
+import sysconfig
+
 import pytest
 import torch
 
@@ -31,6 +34,42 @@ def test_what_is_not_plain_is_left_to_python(native):
     with pytest.raises(binding.RmmError) as e:
         rmm.rmm_reduced_attn(Q, Q, Q, True, 0.5)
     assert e.value.code == binding.RMM_ERR_UNSUPPORTED
+
+
+def test_another_interpreter_builds_its_own(native, tmp_path, monkeypatch):
+    suffix = sysconfig.get_config_var("EXT_SUFFIX")
+    assert binding.MARSHAL_PATH == rmm_build.MARSHAL and binding.MARSHAL_PATH.endswith("rmm_marshal" + suffix) and suffix != ".so"
+    other = tmp_path / "rmm_marshal.cpython-399.so"
+    monkeypatch.setattr(rmm_build, "MARSHAL", str(other))
+    before = os.path.getmtime(rmm_build.LIB)
+    rmm_build.build()                                             # the module alone: the library serves every interpreter
+    assert other.exists() and os.path.getmtime(rmm_build.LIB) == before
+
+
+@pytest.fixture
+def missing(native, monkeypatch):
+    monkeypatch.setattr(binding, "_marshal", None)
+    monkeypatch.setattr(binding, "MARSHAL_PATH", "/nowhere/rmm_marshal.so")
+
+
+def test_without_the_module_calls_reach_python(missing):
+    assert binding._native() is None
+    with pytest.raises(binding.RmmError) as e:
+        rmm.rmm(torch.zeros(4, 8), torch.zeros(8, 8), 0.5)
+    assert e.value.code == binding.RMM_ERR_INVALID_ARG
+    Q = torch.zeros(1, 2, 4, 8, dtype=torch.bfloat16)
+    with pytest.raises(binding.RmmError) as e:
+        rmm.rmm_reduced_attn(Q, Q, Q, True, 0.5)
+    assert e.value.code == binding.RMM_ERR_UNSUPPORTED
+
+
+@pytest.mark.gpu
+def test_without_the_module_results_are_the_same(missing):
+    A, B = synth.mlp_product(40, 512, 72, device="cuda")
+    Q, K, V = synth.attention_qkv(1, 4, 2, 70, 70, 64, seed=1, device="cuda")
+    for got, want in zip(rmm.rmm(A, B, 0.5), rmm.rmm_product(A, B, 0.5, want_retained=True)):
+        assert torch.equal(got, want)
+    assert torch.equal(rmm.rmm_reduced_attn(Q, K, V, True, 0.5), rmm.rmm_reduced_attn(Q, K, V, True, 0.5, want_idx=True)[0])
 
 
 @pytest.mark.gpu
