@@ -223,13 +223,14 @@ __device__ __forceinline__ void ex2_fma(float x0, float x1, float &p0, float &p1
     p1 = q1 * __uint_as_float((__float_as_uint(n1) << 23) + 0x3f800000u);
 }
 
-template <int MODE, bool MASK>
+// O_TILES: O leaves by tile stores (GATHERED, where a tensor map describes O: no negative strides).  Both forms in one
+// kernel, chosen at run time, cost it 3 % (32 heads x 3001 x 128 73.7 -> 75.8 us).
+template <int MODE, bool MASK, bool O_TILES>
 __global__ void __launch_bounds__(kFusedThreads, 1)
 fused_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                   const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_o, FusedArgs a)
 {
     constexpr bool kHasV = MODE == MODE_FULL || MODE == MODE_GATHERED;  // P tiles, P V products and an O accumulator
-    constexpr bool kTileStore = MODE == MODE_GATHERED;                  // O leaves by tile stores
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     const uint32_t base = smem_u32(smem_raw);
     uint8_t *base_ptr = smem_raw;
@@ -257,7 +258,7 @@ fused_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         asm volatile("prefetch.tensormap [%0];" ::"l"(&map_k) : "memory");
         if constexpr (kHasV) {
             asm volatile("prefetch.tensormap [%0];" ::"l"(&map_v) : "memory");
-            if constexpr (kTileStore) asm volatile("prefetch.tensormap [%0];" ::"l"(&map_o) : "memory");
+            if constexpr (O_TILES) asm volatile("prefetch.tensormap [%0];" ::"l"(&map_o) : "memory");
         }
     }
     if (threadIdx.x == 0) {
@@ -763,7 +764,7 @@ fused_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                     load_chunk(j, 0, v0, v1);
                     emit_chunk(v0, v1, neg_m, w);
                     if (!mbar_wait(p_empty(g), (p_it & 1u) ^ 1u, abort_flag, a.status, a.wait_ns)) { ok = false; break; }
-                    if (j == jb) o_stored();
+                    if (O_TILES && j == jb) o_stored();
                     store_chunk(0, w);
                     load_chunk(j, 64, v0, v1);
                     release_s();
@@ -823,7 +824,7 @@ fused_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                 if (!mbar_wait(o_full(g), o_it & 1u, abort_flag, a.status, a.wait_ns)) { ok = false; break; }
                 tc_fence_after();
                 const float inv_l = MODE == MODE_GATHERED ? 1.f : (l > 0.f ? 1.f / l : 0.f);
-                if constexpr (kTileStore) {
+                if constexpr (O_TILES) {
                     // The P tile is free (the last P V is complete): the warp's 32 rows go through it, laid out as P is, and leave by a
                     // tile store, which clips rows and columns past the end: 32 heads x 3001 x 128 (2401 keys) 86.4 -> 82.4 us.  The
                     // one-pass form, where the maps' set-up and the stores' tail weigh more, keeps direct stores (2 heads x 8192: 90.0
@@ -871,7 +872,7 @@ fused_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                 __syncwarp();
                 if (lane == 0) {
                     mbar_arrive(o_empty(g));
-                    if (kTileStore && r0 + q * 32 < a.Lr) {
+                    if (O_TILES && r0 + q * 32 < a.Lr) {
                         for (int c = 0; c < nv; ++c)
                             tma_store_3d(&map_o, base + kOffP + g * kPTile + c * kPChunk + q * 4096, c * 64, (int)r0 + q * 32, (int)head);
                         bulk_commit();
@@ -881,7 +882,7 @@ fused_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             }
             ASTAMP(6);
         }
-        if constexpr (kTileStore) {
+        if constexpr (O_TILES) {
             if (lane == 0) bulk_wait_read<0>();  // shared memory stays until the stores have read it
             __syncwarp();
         }
@@ -932,11 +933,11 @@ int block_groups(const FusedArgs &a, int64_t sms)
     return one < 0.95 * (kItem + 3400.0 * (double)tiles(0)) ? 1 : 2;
 }
 
-template <int MODE, bool MASK = false>
+template <int MODE, bool MASK = false, bool O_TILES = false>
 int launch_mode(const CUtensorMap &mq, const CUtensorMap &mk, const CUtensorMap &mv, const CUtensorMap &mo, const FusedArgs &a, const char *name,
                 cudaStream_t stream)
 {
-    auto kern = fused_attn_kernel<MODE, MASK>;
+    auto kern = fused_attn_kernel<MODE, MASK, O_TILES>;
     static PerDeviceOnce configured;
     if (cudaError_t e = configured.smem(kFusedSmem, kern)) return fail(RMM_ERR_CUDA, "fused_attn: cudaFuncSetAttribute: %s", cudaGetErrorString(e));
     int dev = 0, sms = 148;
@@ -1019,7 +1020,8 @@ int launch_fused_attn(const __nv_bfloat16 *Qp, const __nv_bfloat16 *Kp, int64_t 
             const uint32_t box[3] = {64, FN, 1};
             if ((rc = make_map(&mv, const_cast<__nv_bfloat16 *>(V + c0), 3, dims, st, box, true)) != RMM_OK) return rc;
         }
-        if (tok == nullptr) {
+        const bool o_tiles = tok != nullptr && o_sh >= 0 && o_sr >= 0;
+        if (!o_tiles) {
             mo = mq;  // (O leaves without a tensor map)
         } else {
             uint64_t dims[3] = {(uint64_t)dh, (uint64_t)Lq, (uint64_t)heads};
@@ -1037,7 +1039,9 @@ int launch_fused_attn(const __nv_bfloat16 *Qp, const __nv_bfloat16 *Kp, int64_t 
         a.status = status;
         a.wait_ns = wait_limit_ns();
         a.withhold = debug_withhold() == WITHHOLD_ATTN;
-        if (tok != nullptr) {
+        if (o_tiles) {
+            rc = launch_mode<MODE_GATHERED, false, true>(mq, mk, mv, mo, a, "fused_attn_gathered_kernel", stream);
+        } else if (tok != nullptr) {
             rc = launch_mode<MODE_GATHERED>(mq, mk, mv, mo, a, "fused_attn_gathered_kernel", stream);
         } else if (mask != nullptr) {
             a.mask = *mask; a.tile_kind = tile_kind; a.kind_rb = kind_rb; a.kind_ld = kind_ld;
