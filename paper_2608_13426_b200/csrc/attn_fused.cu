@@ -202,27 +202,6 @@ __global__ void __launch_bounds__(kMaskThreads) mask_tiles_kernel(const MaskTile
     if (a.behind_heads) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
-// 2^x of two numbers on the FMA and integer pipes: x = n + f with f in [-1/2, 1/2] (adding 1.5 x 2^23 rounds to the integer n), a
-// polynomial of degree 5 for 2^f (fitted for the smallest largest relative error: 9.1e-8, 1.6e-7 as evaluated, where the
-// special-function unit has 2^-22) and 2^n put together in the exponent.  Below -127: 0; NaN stays NaN.
-__device__ __forceinline__ void ex2_fma(float x0, float x1, float &p0, float &p1)
-{
-    const uint64_t magic = pack2(12582912.f, 12582912.f), minus = pack2(-1.f, -1.f);
-    asm("max.NaN.f32 %0, %0, 0fC2FE0000;" : "+f"(x0));
-    asm("max.NaN.f32 %0, %0, 0fC2FE0000;" : "+f"(x1));
-    const uint64_t x = pack2(x0, x1), n = fadd2(x, magic), f = fadd2(x, ffma2(n, minus, magic));
-    uint64_t p = ffma2(pack2(0.001326472731307149f, 0.001326472731307149f), f, pack2(0.009671512991189957f, 0.009671512991189957f));
-    p = ffma2(p, f, pack2(0.05550733581185341f, 0.05550733581185341f));
-    p = ffma2(p, f, pack2(0.24022242426872253f, 0.24022242426872253f));
-    p = ffma2(p, f, pack2(0.6931470036506653f, 0.6931470036506653f));
-    p = ffma2(p, f, pack2(1.f, 1.f));
-    float n0, n1, q0, q1;
-    unpack2(n, n0, n1);
-    unpack2(p, q0, q1);
-    p0 = q0 * __uint_as_float((__float_as_uint(n0) << 23) + 0x3f800000u);
-    p1 = q1 * __uint_as_float((__float_as_uint(n1) << 23) + 0x3f800000u);
-}
-
 // O_TILES: O leaves by tile stores (GATHERED, where a tensor map describes O: no negative strides).  Both forms in one
 // kernel, chosen at run time, cost it 3 % (32 heads x 3001 x 128 73.7 -> 75.8 us).
 template <int MODE, bool MASK, bool O_TILES>

@@ -446,6 +446,27 @@ __device__ __forceinline__ float ex2(float x)
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
+// 2^x of two numbers on the FMA and integer pipes: x = n + f with f in [-1/2, 1/2] (adding 1.5 x 2^23 rounds to the integer n), a
+// polynomial of degree 5 for 2^f and 2^n put together in the exponent.  The coefficients minimise the largest relative error over
+// [-1/2, 1/2] with a constant term of 1 (a linear program over 4001 Chebyshev points): 9.1e-8, 1.1e-7 once rounded to fp32, 1.7e-7
+// as evaluated, where the special-function unit has 2^-22.  For x up to 127; 0 from -126.5 down, NaN stays NaN.
+__device__ __forceinline__ void ex2_fma(float x0, float x1, float &p0, float &p1)
+{
+    const uint64_t magic = pack2(12582912.f, 12582912.f), minus = pack2(-1.f, -1.f);
+    asm("max.NaN.f32 %0, %0, 0fC2FE0000;" : "+f"(x0));
+    asm("max.NaN.f32 %0, %0, 0fC2FE0000;" : "+f"(x1));
+    const uint64_t x = pack2(x0, x1), n = fadd2(x, magic), f = fadd2(x, ffma2(n, minus, magic));
+    uint64_t p = ffma2(pack2(0.001326472731307149f, 0.001326472731307149f), f, pack2(0.009671512991189957f, 0.009671512991189957f));
+    p = ffma2(p, f, pack2(0.05550733581185341f, 0.05550733581185341f));
+    p = ffma2(p, f, pack2(0.24022242426872253f, 0.24022242426872253f));
+    p = ffma2(p, f, pack2(0.6931470036506653f, 0.6931470036506653f));
+    p = ffma2(p, f, pack2(1.f, 1.f));
+    float n0, n1, q0, q1;
+    unpack2(n, n0, n1);
+    unpack2(p, q0, q1);
+    p0 = q0 * __uint_as_float((__float_as_uint(n0) << 23) + 0x3f800000u);
+    p1 = q1 * __uint_as_float((__float_as_uint(n1) << 23) + 0x3f800000u);
+}
 // Shared-memory operand descriptor (tcgen05 format): 128-byte swizzle, addresses and offsets in 16-byte units.
 __device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo_bytes, uint32_t sbo_bytes)
 {
