@@ -5,7 +5,7 @@
 // distributed shared memory in rank order, and the first block ranks all features by comparing all pairs (at most 256 keys).
 // Bound by HBM for long prompts and else by the chain of latencies, which is why nothing passes through global memory: the general
 // score pass publishes partial sums, hands them to the last block of a column range and the energies to the last block of a head.
-// Kernel by events: 2 heads x 600 x 128 14.4 -> 10.1 us, 8 x 1172 x 128 18.6 -> 11.5, 8 x 8192 x 64 15.2 -> 11.3, 32 x 4096 x 128 24.7 -> 20.9.
+// Kernel by events: 2 heads x 600 x 128 14.4 -> 10.1 us, 8 x 1172 x 128 18.6 -> 11.5 (attn_features_eligible has whole calls).
 #include "common.cuh"
 #include "select.cuh"
 #include "sm100_ptx.cuh"
@@ -121,10 +121,19 @@ __global__ void __launch_bounds__(kFeatThreads) attn_features_kernel(const FeatA
 
 bool attn_features_eligible(int64_t heads, int64_t Lq, int64_t Dh)
 {
-    // Eight blocks a head: with more than 32 heads (8 of more than 128 columns) they queue, and long heads leave SMs idle or want the
-    // general pass's deeper pipeline.  Both by events: 64 x 1000 x 128 14.0 us by the general pass, 16.5 here; 16 x 1000 x 256 14.0 and
-    // 15.6; 8 x 20000 x 128 19.1 and 32.4; 16 x 8192 x 128 17.7 and 18.6; 32 x 8192 x 64 17.3 and 13.3.
-    return heads <= (Dh <= 128 ? 32 : 8) && Dh <= kFeatMaxDh && Lq * Dh <= 4096 * 128;
+    // Eight blocks a head, each with eight loads a thread in flight: short heads are bound by latency, which is shorter here; long ones
+    // want the general pass's deeper pipeline, and many heads queue.  The lines are the crossings of whole calls on 128 keys, here
+    // against the general pass, us with Q in L2 / with new inputs each time (one figure: new inputs):
+    //   Dh 128,  2 heads: 2500 rows -4.5 / -4.5, 5200 -3.3 / -0.8, 8192 +2.3;  4: 2500 -2.7 / -1.7, 4600 +1.9 / +5.0
+    //            8 heads: 2500 -1.0 / -0.4, 3000 +0.4 / +2.1;  16: 2048 -2.1 / -1.0, 2500 -0.7 / +0.5, 3000 -0.1 / +1.9, 4600 +1.5 / +3.6
+    //           24 heads: 2048 -0.9 / -0.2, 3000 -0.4 / +0.8;  28: 3500 -1.3 / +0.2, 4096 -1.2 / +0.4, 4600 +0.2 / +1.7
+    //           32 heads: 2048 -1.7 / -0.9, 3000 -1.0 / -0.1, 4096 -0.6 / 0.0 (whole call on 4096 keys: -0.8 / -1.2), 4600 +1.5 / +1.5
+    //           40 heads: 2048 -1.0 / 0.0;  48: 2048 +2.6, 4096 +5.4;  64: 2048 +4.9
+    //   Dh 64,   2 heads: 10000 -3.7 / -1.0;  8: 4096 -2.4 / -1.1, 7000 -1.1 / +1.3;  40: 4096 -3.3 / -3.1;  48: 4096 +1.0
+    //   Dh 256,  1 head: 3000 -1.9 / -1.4;  2: 2048 -4.0 / -1.1;  4: 1000 -2.5 / -1.9, 2048 +2.2 / +4.5;  6: 750 -1.6 / -0.8, 1000 +2.4 / +3.3
+    //            8 heads: 250 -3.0 / -1.8, 500 +1.1 / +0.8, 1000 +2.3 / +3.9
+    if (Dh > 128) return Dh <= kFeatMaxDh && heads <= 8 && heads * Lq * Dh <= 1 << 20;
+    return heads <= 40 && Lq * Dh <= (heads <= 2 ? 5120 : heads < 28 ? 2560 : 4352) * 128;
 }
 
 int launch_attn_features(const __nv_bfloat16 *q, int64_t q_sh, int64_t q_sr, int64_t heads, int64_t Lq, int64_t Dh, int64_t kd, int32_t *idx,

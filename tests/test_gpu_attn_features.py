@@ -9,7 +9,9 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("B, Hq, Hkv, Lq, Dh", [
     (1, 32, 8, 40, 128), (1, 8, 8, 17, 256), (1, 3, 1, 129, 72), (2, 2, 2, 1001, 64), (1, 1, 1, 4096, 128), (1, 1, 1, 4097, 128),
-    (1, 33, 1, 64, 64), (1, 9, 9, 130, 136), (3, 5, 1, 300, 8), (1, 4, 2, 2048, 256), (1, 2, 1, 65000, 8)])
+    (1, 33, 1, 64, 64), (1, 9, 9, 130, 136), (3, 5, 1, 300, 8), (1, 4, 2, 2048, 256), (1, 2, 1, 65000, 8),
+    (1, 3, 1, 2560, 128), (1, 3, 1, 2561, 128), (1, 28, 4, 4352, 128), (1, 28, 4, 4353, 128), (1, 2, 1, 5120, 128), (1, 2, 1, 5121, 128), (1, 40, 8, 90, 64), (1, 41, 1, 90, 64),
+    (1, 8, 8, 512, 256), (1, 8, 8, 513, 256)])   # either side of each line of attn_features_eligible
 @pytest.mark.parametrize("rho", [0.5, 0.13, 1.0])
 def test_features_are_those_of_the_general_pass(B, Hq, Hkv, Lq, Dh, rho):
     g = torch.Generator(device="cuda").manual_seed(Lq)
