@@ -866,7 +866,9 @@ int launch_gemm_tc_problem(const TcProblem &p, cudaStream_t stream)
         // down where operands are far larger than L2 and contractions long, and costs a meeting a tile.  In loops of half a second at
         // the power cap, without and with: 1531 x 4096 x 14336 151.3 and 154.6 us, 3144 x 4800 x 19776 503.6 and 508.7, 32768 x 4096 x 8192
         // 1683 and 1699; 8192 x 8192 x 8192 882 and 879, 32768 x 14336 x 8192 6122 and 5987, 2048 x 28672 x 8192 825 and 811.  Meeting
-        // again every 128 k-blocks inside a tile, 32768 x 14336 x 8192 takes 6102.  (Measurement switch RMM_GEMM_WAVE_SYNC=0|1.)
+        // again every 128 k-blocks inside a tile, 32768 x 14336 x 8192 takes 6102.  The line is one of bytes: 8-bit contractions below
+        // 16384, GEMM without and with, 4096 x 8192 x 8192 205 and 214, 8192 x 8200 x 4096 245 and 249, 16384 x 14336 x 8192 1478 and 1516,
+        // 16384 x 16000 x 8192 1672 and 1677 (calls 2207 and 2193).  (Measurement switch RMM_GEMM_WAVE_SYNC=0|1.)
         static const int forced_sync = []() { const char *e = getenv("RMM_GEMM_WAVE_SYNC"); return e ? atoi(e) : -1; }();
         const int64_t tiles = (int64_t)a.batch * a.tiles_m * a.tiles_n, per_wave = sm_count() / ctas;
         const bool want = p.b_idx == nullptr && (forced_sync >= 0 ? forced_sync != 0 : (tiles > per_wave && p.k * es >= 16384));
