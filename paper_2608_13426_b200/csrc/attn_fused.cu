@@ -881,13 +881,15 @@ fused_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
 // Groups of 128 rows per block.  Two share every K and V tile and hide each other's waits (3400 clocks a step of 256 x 128), but
 // where blocks of 128 rows do not outnumber the SMs there is nothing to share an SM with: one group alone takes 2330 a step of
 // 128 x 128, and a row block's keys are the serial chain that the launch waits for.  Kernels of 2, 8 and 16 heads x 4096, 2048 and
-// 1000 x 128, causal: 63.8 -> 47.5, 39.2 -> 31.1 and 24.9 -> 20.7 us; the sweeps of the token reduction likewise (8 x 2048: 31.0 / 41.3 /
-// 26.9 -> 24.8 / 33.1 / 20.7).
+// 1100 x 128, causal, by two and by one: 67.5 and 51.2, 41.0 and 32.7, 26.7 and 24.6 us; the sweeps of the token reduction likewise
+// (8 x 2048: 29.4 / 41.3 / 24.6 and 22.8 / 33.2 / 20.5).
 // In up to two rounds a causal block's short rows follow another's long ones (item_of), so one group still wins where the longest
-// sum of a pair is not much longer than the longest item: 8 x 4096 67.9 -> 51.5, 16 x 2048 39.3 -> 33.0, 8 x 3001 51.6 -> 39.2, the
-// normalisers and energies of 8 x 4096 51.5 / 76.1 -> 41.3 / 57.6; 32 x 1100, items of nine tiles at most, 37.0 us a call by two and
-// 38.9 by one; without a mask 8 x 4096 takes 74 by two and 95 by one.  Where the
-// number of tiles is not the rows' (an additive mask, kept keys) only the first rule holds (8 x 4096, padded: 55.7 and 61.7).
+// sum of a pair is not much longer than the longest item: 8 x 4096 71.6 and 57.3, 16 x 2048 41.8 and 37.0, 4 x 8192 124.9 and 92.2,
+// the normalisers and energies of 8 x 4096 50.1 / 74.1 and 38.9 / 55.8; 32 x 1000, items of eight tiles at most, level; 64 x 500
+// 18.5 and 22.5; without a mask 8 x 4096 takes 73.8 by two and 104.4 by one.  The clocks are those of the one-pass kernel; both
+// sweeps keep about their ratio, and over 20 shapes of 64 and 128 columns the rule's choice was never more than 2 us behind.  Where
+// the number of tiles is not the rows', only the first rule holds: kept keys (8 x 4096 36.9 and 43.0, 5 x 4096 36.9 and 28.7), and an
+// additive mask, of which nothing is known here (8 x 4096 padded, causal 71.7 and 63.5, otherwise 73.8 and 104.5).
 template <int MODE, bool MASK>
 int block_groups(const FusedArgs &a, int64_t sms)
 {
