@@ -26,3 +26,23 @@ def test_packed_heads(oracle, Dh, rho_d, Lq, Lk):
     mask.fill_(0)                                                                 # a new mask in the same place
     assert torch.equal(rmm.rmm_reduced_attn(Q, K, V, False, rho_d, mask=mask), want[0])
     assert rmm.rmm_status_read() == 0
+
+
+@pytest.mark.parametrize("B, Hq, Hkv, L, Dh, causal", [(2, 16, 4, 512, 128, True), (1, 4, 2, 1500, 64, False), (2, 40, 8, 390, 128, False)])
+def test_masked_calls_in_flight(B, Hq, Hkv, L, Dh, causal):
+    """Calls with different masks right behind one another: the pass over a mask runs beside the packing, while the attention kernel of
+    the call before, which reads what that pass wrote for it, must be done."""
+    Q, K, V = synth.attention_qkv(B, Hq, Hkv, L, L, Dh, seed=L, device="cuda")
+    masks = [padded(B, L, L, [n, L - n // 2][:B]).cuda() for n in (40, 129, 300, L - 1)] + [torch.zeros(1, 1, L, L, device="cuda")]
+    want = []
+    for m in masks:
+        want.append(rmm.rmm_reduced_attn(Q, K, V, causal, 0.5, mask=m))
+        torch.cuda.synchronize()
+    rmm.binding.poison_outputs(False)                                             # its fills would keep the calls apart
+    try:
+        got = [rmm.rmm_reduced_attn(Q, K, V, causal, 0.5, mask=masks[i * 2 % 5]) for i in range(60)]
+    finally:
+        rmm.binding.poison_outputs(True)
+    for i, o in enumerate(got):
+        assert torch.equal(o, want[i * 2 % 5])
+    assert rmm.rmm_status_read() == 0
