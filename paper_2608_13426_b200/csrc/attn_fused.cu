@@ -880,7 +880,7 @@ fused_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
 
 // Groups of 128 rows per block.  Two share every K and V tile and hide each other's waits (3400 clocks a step of 256 x 128), but
 // where blocks of 128 rows do not outnumber the SMs there is nothing to share an SM with: one group alone takes 2330 a step of
-// 128 x 128, and a row block's keys are the serial chain that the launch waits for.  Kernels of 2, 8 and 16 heads x 4096, 2048 and
+// 128 x 128 (either a tenth more where logits as spread as those of outlier features make it rescale), and a row block's keys are the serial chain that the launch waits for.  Kernels of 2, 8 and 16 heads x 4096, 2048 and
 // 1100 x 128, causal, by two and by one: 67.5 and 51.2, 41.0 and 32.7, 26.7 and 24.6 us; the sweeps of the token reduction likewise
 // (8 x 2048: 29.4 / 41.3 / 24.6 and 22.8 / 33.2 / 20.5).
 // In up to two rounds a causal block's short rows follow another's long ones (item_of), so one group still wins where the longest
