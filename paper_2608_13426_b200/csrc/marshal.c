@@ -123,15 +123,15 @@ static PyObject *new_out(PyObject *like, int dims, const int64_t *size, PyObject
 /* The cached workspace of `like`'s device, at least `need` bytes: a new reference, its 256-byte aligned part through *ptr, *bytes */
 static PyObject *workspace_of(PyObject *like, size_t need, void **ptr, size_t *bytes)
 {
-    PyObject *ws = NULL, *v, *key, *cache = named(s_ws_cache), *make = named(s_workspace);
-    if (cache == NULL || make == NULL) return NULL;
-    if (!PyDict_Check(cache)) { PyErr_SetString(PyExc_TypeError, "_ws_cache must be a dict"); return NULL; }
+    PyObject *ws = NULL, *v, *key, *cache, *make;
     if (need < RMM_WS_HEADER_BYTES) need = RMM_WS_HEADER_BYTES;
     if ((v = PyObject_CallMethodNoArgs(like, s_get_device)) == NULL) return NULL;
     key = PyTuple_Pack(2, s_cuda, v);
     Py_DECREF(v);
     if (key == NULL) return NULL;
-    ws = PyDict_GetItemWithError(cache, key);
+    /* (borrowed names are used at once: a tensor's methods may run Python code, which may bind them anew) */
+    if ((cache = named(s_ws_cache)) != NULL && !PyDict_Check(cache)) PyErr_SetString(PyExc_TypeError, "_ws_cache must be a dict");
+    ws = cache != NULL && PyDict_Check(cache) ? PyDict_GetItemWithError(cache, key) : NULL;
     Py_DECREF(key);
     if (ws == NULL && PyErr_Occurred()) return NULL;
     Py_XINCREF(ws);
@@ -146,7 +146,8 @@ static PyObject *workspace_of(PyObject *like, size_t need, void **ptr, size_t *b
         Py_XDECREF(ws);
         PyObject *dev = PyObject_GetAttr(like, s_device), *n = PyLong_FromSize_t(need);
         PyObject *args[2] = {n, dev};
-        ws = dev != NULL && n != NULL ? PyObject_Vectorcall(make, args, 2, NULL) : NULL;
+        make = dev != NULL && n != NULL ? named(s_workspace) : NULL;
+        ws = make != NULL ? PyObject_Vectorcall(make, args, 2, NULL) : NULL;
         Py_XDECREF(dev);
         Py_XDECREF(n);
         if (ws == NULL) return NULL;

@@ -126,3 +126,23 @@ def test_the_workspace_grows_and_streams_are_followed(native):
         Y, idx = rmm.rmm(A, B, 0.5)
     s.synchronize()
     assert torch.equal(Y, want[0]) and torch.equal(idx, want[1]) and torch.isfinite(small[0]).all()
+
+
+@pytest.mark.gpu
+def test_names_bound_anew_in_the_middle_of_a_call(native, monkeypatch):
+    """A mode's Python code runs inside the tensors' methods; what the module's names held before may be gone after it."""
+    A, B = synth.mlp_product(40, 512, 72, device="cuda")
+    want = rmm.rmm(A, B, 0.5)
+    original = binding.workspace
+
+    class Mode(torch.overrides.TorchFunctionMode):
+        def __torch_function__(self, func, types, args=(), kwargs=None):
+            binding._ws_cache = {}
+            binding.workspace = original
+            return func(*args, **(kwargs or {}))
+
+    monkeypatch.setattr(binding, "_ws_cache", {})
+    monkeypatch.setattr(binding, "workspace", lambda n, device: original(n, device))
+    with Mode():
+        got = rmm.rmm(A, B, 0.5)
+    assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
